@@ -262,9 +262,10 @@ static int grid_dims_impl(const double box[3], double h, int levels, int n_out[3
 
 static void free_plan(Plan* p) {
   if (!p) return;
-  void* ptrs[] = {p->d_pos_w, p->d_cell_of, p->d_zero, p->d_cell_start, p->d_sorted,
+  void* ptrs[] = {p->d_pos_w, p->d_cell_of, p->d_cell_count, p->d_cell_start, p->d_sorted,
                   p->d_sorted_idx, p->d_e0, p->d_floc, p->d_rows, p->d_wv, p->d_top_T,
-                  p->d_top_V, p->d_epart, p->d_wpart, p->d_out, p->d_tcw, p->d_lbw, p->d_lbpot, p->d_mma_rows, p->d_mma_bv,
+                  p->d_top_V, p->d_epart, p->d_wpart, p->d_out, p->d_flag, p->d_scan,
+                  p->d_q1fx, p->d_tcw, p->d_lbw, p->d_lbpot, p->d_mma_rows, p->d_mma_bv,
                   p->d_mma_be};
   for (void* q : ptrs)
     if (q) cudaFree(q);
@@ -474,12 +475,9 @@ int mls6_set_tuning(mls6_plan_t* plan, int split, int groups) {
   if (!plan) return MLS6_ERR_ARG;
   Plan* p = reinterpret_cast<Plan*>(plan);
   if (split != 0 && split != 1 && split != 2 && split != 4 && split != 8 && split != 16 &&
-      split != 32 && split != 128 && split != 256 && split != 512 && split != kPairCluster &&
-      split != kPairTile)
+      split != 32 && split != 128 && split != 256 && split != 512 && split != kPairCluster)
     return MLS6_ERR_ARG;
-  if (split == kPairCluster ? !pair_cl_ok(p)
-      : split == kPairTile  ? !pair_tile_ok(p)
-                            : (split > 8 && !pair_cluster_ok(p)))
+  if (split == kPairCluster ? !pair_cl_ok(p) : (split > 8 && !pair_cluster_ok(p)))
     return MLS6_ERR_ARG;
   if (groups != 0 && groups != 1 && groups != 2 && groups != 4) return MLS6_ERR_ARG;
   const int s2 = split ? split : p->pair_split;
