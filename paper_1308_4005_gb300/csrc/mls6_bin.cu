@@ -1,7 +1,8 @@
 // Spatial binning of the atoms (the linked-cell structure of Sec. III.D):
 // wrap positions into the box, histogram them over cells of width >= a/2,
 // exclusive scan of the counts, scatter into cell order, and order each
-// cell by input index so that every later sum runs in a reproducible order.
+// cell (FP32 by x, FP64 by input index) so that every later sum runs in a
+// reproducible order.
 #include <algorithm>
 #include <climits>
 
@@ -21,10 +22,13 @@ template <typename T> struct BinArgs {
 // order like the value for non-negative doubles), and, when tsum is given
 // (at most kScanDirect tiles), adds the block's atoms per scan tile of
 // kScanTile cells to tsum (a shared-memory histogram first, then one
-// integer atomic per touched tile).
+// integer atomic per touched tile).  count, flag and tsum start at zero (one
+// memset of the region they share, per evaluation).  cell_of keeps each
+// atom's cell and its place among the cell's atoms (the count it met), so
+// that the scatter needs no atomics of its own.
 template <typename T>
 __device__ __forceinline__ void k_bin_body(const Blk bk,const T* __restrict__ pos, const T* __restrict__ cc, int stride, int N,
-                      BinArgs<T> g, Vec4<T>* __restrict__ posw, int* __restrict__ cell_of,
+                      BinArgs<T> g, Vec4<T>* __restrict__ posw, int2* __restrict__ cell_of,
                       int* __restrict__ count, int* __restrict__ flag, int* __restrict__ tsum,
                       int ntiles) {
   const long z = pdl_begin();
@@ -51,14 +55,13 @@ __device__ __forceinline__ void k_bin_body(const Blk bk,const T* __restrict__ po
     int cy = min(max((int)(y * g.inv_w[1]), 0), g.nc[1] - 1);
     int cz = min(max((int)(z * g.inv_w[2]), 0), g.nc[2] - 1);
     int cell = cx + g.nc[0] * (cy + g.nc[1] * cz);
-    cell_of[i] = cell;
     Vec4<T> v;
     v.x = x;
     v.y = y;
     v.z = z;
     v.w = c;
     posw[i] = v;
-    atomicAdd(&count[cell], 1);
+    cell_of[i] = make_int2(cell, atomicAdd(&count[cell], 1));
     if (tsum) atomicAdd(&hist[cell / kScanTile], 1);
     cabs = fabs(c);
   }
@@ -78,7 +81,7 @@ __device__ __forceinline__ void k_bin_body(const Blk bk,const T* __restrict__ po
 
 template <typename T>
 __global__ void k_bin(const T* __restrict__ pos, const T* __restrict__ cc, int stride, int N,
-                      BinArgs<T> g, Vec4<T>* __restrict__ posw, int* __restrict__ cell_of,
+                      BinArgs<T> g, Vec4<T>* __restrict__ posw, int2* __restrict__ cell_of,
                       int* __restrict__ count, int* __restrict__ flag, int* __restrict__ tsum,
                       int ntiles) {
   k_bin_body<T>(Blk::self(), pos, cc, stride, N, g, posw, cell_of, count, flag, tsum, ntiles);
@@ -151,16 +154,16 @@ __global__ void k_scan_tiles(const int* __restrict__ count, long n, int* __restr
 #endif  // MLS6_DEVICE_ONLY
 
 // Scan inside each tile (256 threads x 8 consecutive cells), write start[],
-// reset count[] for use as fill counters by the scatter, and keep the
-// largest cell population in flag[3] (one atomic maximum per block).  The
+// and keep the largest cell population in flag[3] (one atomic maximum per block).  The
 // tile's offset is tsum[tile] from the tile pass, or (direct: at most
 // kScanDirect tiles, tsum holding the tile sums from the binning) the sum of
 // the preceding tiles' sums, formed by each block; the last tile then also
 // writes the grand total to start[n].
-__device__ __forceinline__ void k_scan_final_body(const Blk bk,int* __restrict__ count, long n, const int* __restrict__ tsum,
+__device__ __forceinline__ void k_scan_final_body(const Blk bk,const int* __restrict__ count, long n, const int* __restrict__ tsum,
                              int* __restrict__ start, int direct, int* __restrict__ flag) {
   const long z = pdl_begin();
   tsum += z;
+  count += z;
   __shared__ int wsum[32], wmx[32];
   __shared__ int toff;
   constexpr int PER = kScanTile / 256;
@@ -206,10 +209,7 @@ __device__ __forceinline__ void k_scan_final_body(const Blk bk,int* __restrict__
   int excl = incl - s + (wid > 0 ? wsum[wid - 1] : 0) + toff;
 #pragma unroll
   for (int k = 0; k < PER; ++k) {
-    if (base + k < n) {
-      start[base + k] = excl;
-      count[base + k] = 0;
-    }
+    if (base + k < n) start[base + k] = excl;
     excl += v[k];
   }
   if (direct && threadIdx.x == blockDim.x - 1 && bk.x == bk.n - 1) start[n] = excl;
@@ -222,107 +222,109 @@ __device__ __forceinline__ void k_scan_final_body(const Blk bk,int* __restrict__
 }
 
 #ifndef MLS6_DEVICE_ONLY  // non-template kernel, left out where another unit includes this file
-__global__ void k_scan_final(int* __restrict__ count, long n, const int* __restrict__ tsum,
+__global__ void k_scan_final(const int* __restrict__ count, long n, const int* __restrict__ tsum,
                              int* __restrict__ start, int direct, int* __restrict__ flag) {
   k_scan_final_body(Blk::self(), count, n, tsum, start, direct, flag);
 }
 #else
-__global__ void k_scan_final(int* __restrict__ count, long n, const int* __restrict__ tsum,
+__global__ void k_scan_final(const int* __restrict__ count, long n, const int* __restrict__ tsum,
                              int* __restrict__ start, int direct, int* __restrict__ flag);
 #endif  // MLS6_DEVICE_ONLY
 
-template <typename T>
-__device__ __forceinline__ void k_scatter_body(const Blk bk,const Vec4<T>* __restrict__ posw, const int* __restrict__ cell_of, int N,
-                          const int* __restrict__ start, int* __restrict__ fill,
-                          Vec4<T>* __restrict__ sorted, int* __restrict__ sidx) {
+// Input indices into cell order; the records follow them in the cell sort.
+__device__ __forceinline__ void k_scatter_body(const Blk bk,const int2* __restrict__ cell_of, int N,
+                          const int* __restrict__ start, int* __restrict__ sidx) {
   const long z = pdl_begin();
-  posw += z; cell_of += z; start += z;
-  int i = bk.x * blockDim.x + threadIdx.x;
+  cell_of += z; start += z;
+  const int i = bk.x * blockDim.x + threadIdx.x;
   if (i >= N) return;
-  int cell = cell_of[i];
-  int slot = start[cell] + atomicAdd(&fill[cell], 1);
-  sorted[slot] = posw[i];
-  sidx[slot] = i;
+  const int2 c = cell_of[i];
+  sidx[start[c.x] + c.y] = i;
+}
+
+#ifndef MLS6_DEVICE_ONLY  // non-template kernel, left out where another unit includes this file
+__global__ void k_scatter(const int2* __restrict__ cell_of, int N, const int* __restrict__ start,
+                          int* __restrict__ sidx) {
+  k_scatter_body(Blk::self(), cell_of, N, start, sidx);
+}
+#else
+__global__ void k_scatter(const int2* __restrict__ cell_of, int N, const int* __restrict__ start,
+                          int* __restrict__ sidx);
+#endif  // MLS6_DEVICE_ONLY
+
+// Cell records in their final order, taken from the input-order records: FP32
+// plans by x (ties by input index), so that consecutive atoms of a row of
+// cells lie close together along x (the tile form of the pair sum evaluates 8
+// of them against their common neighbours: 511 -> 494 candidates and 315 ->
+// 298 listed ones per 8 atoms at a = 3, density 0.85); FP64 plans by input
+// index.  Either way every later sum runs in an order that does not depend on
+// the atomics of the binning.  Cells of up to 8 atoms (nearly all at liquid
+// densities with cells of width a/2) sort 64-bit keys (the bits of x >= 0 over
+// the index) in registers by an odd-even transposition network and only then
+// copy the records; larger cells use an insertion sort of the indices in
+// global memory; cells above 256 atoms are left in scatter order (results stay
+// correct, only bitwise reproducibility is lost for them).
+template <typename T>
+__device__ __forceinline__ unsigned long long record_key(const Vec4<T>* __restrict__ posw, int i) {
+  unsigned long long k = (unsigned)i;
+  if constexpr (sizeof(T) == 4) k |= (unsigned long long)__float_as_uint(posw[i].x) << 32;
+  return k;
 }
 
 template <typename T>
-__global__ void k_scatter(const Vec4<T>* __restrict__ posw, const int* __restrict__ cell_of, int N,
-                          const int* __restrict__ start, int* __restrict__ fill,
-                          Vec4<T>* __restrict__ sorted, int* __restrict__ sidx) {
-  k_scatter_body<T>(Blk::self(), posw, cell_of, N, start, fill, sorted, sidx);
-}
-
-// Each cell's records sorted by input index, so that every later sum runs
-// in an order that does not depend on the scatter's atomics.  Cells of up
-// to 8 atoms (nearly all at liquid densities with cells of width a/2) are
-// loaded into registers together and sorted by an odd-even transposition
-// network; larger cells use an insertion sort in global memory; cells
-// above 256 atoms are left in scatter order (results stay correct, only
-// bitwise reproducibility is lost for them).  Also returns the cell's
-// counter, and the first nreset tile sums, to zero for the next binning.
-template <typename T>
-__device__ __forceinline__ void k_cellsort_body(const Blk bk,const int* __restrict__ start, long ncell, Vec4<T>* __restrict__ sorted,
-                           int* __restrict__ sidx, int* __restrict__ count,
-                           int* __restrict__ tsum, int nreset) {
+__device__ __forceinline__ void k_cellsort_body(const Blk bk,const int* __restrict__ start, long ncell,
+                           const Vec4<T>* __restrict__ posw, Vec4<T>* __restrict__ sorted,
+                           int* __restrict__ sidx) {
   const long z = pdl_begin();
-  start += z;
-  long cell = (long)bk.x * blockDim.x + threadIdx.x;
-  if (cell < nreset) tsum[cell] = 0;
+  start += z; posw += z;
+  const long cell = (long)bk.x * blockDim.x + threadIdx.x;
   if (cell >= ncell) return;
-  count[cell] = 0;
   const int b = start[cell], e = start[cell + 1];
   const int n = e - b;
-  if (n < 2 || n > 256) return;
   if (n <= 8) {
-    int key[8];
-    Vec4<T> v[8];
+    unsigned long long key[8];
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
-      key[k] = INT_MAX;
-      if (k < n) {
-        key[k] = sidx[b + k];
-        v[k] = sorted[b + k];
-      }
+      key[k] = ~0ull;
+      if (k < n) key[k] = record_key(posw, sidx[b + k]);
     }
 #pragma unroll
     for (int r = 0; r < 8; ++r)
 #pragma unroll
       for (int k = r & 1; k + 1 < 8; k += 2)
         if (key[k] > key[k + 1]) {
-          const int tk = key[k];
+          const unsigned long long t = key[k];
           key[k] = key[k + 1];
-          key[k + 1] = tk;
-          const Vec4<T> tv = v[k];
-          v[k] = v[k + 1];
-          v[k + 1] = tv;
+          key[k + 1] = t;
         }
 #pragma unroll
     for (int k = 0; k < 8; ++k)
       if (k < n) {
-        sidx[b + k] = key[k];
-        sorted[b + k] = v[k];
+        const int i = (int)(unsigned)key[k];
+        sidx[b + k] = i;
+        sorted[b + k] = posw[i];
       }
     return;
   }
-  for (int i = b + 1; i < e; ++i) {
-    int key = sidx[i];
-    Vec4<T> v = sorted[i];
-    int j = i - 1;
-    while (j >= b && sidx[j] > key) {
-      sidx[j + 1] = sidx[j];
-      sorted[j + 1] = sorted[j];
-      --j;
+  if (n <= 256)
+    for (int i = b + 1; i < e; ++i) {
+      const int id = sidx[i];
+      const unsigned long long key = record_key(posw, id);
+      int j = i - 1;
+      while (j >= b && record_key(posw, sidx[j]) > key) {
+        sidx[j + 1] = sidx[j];
+        --j;
+      }
+      sidx[j + 1] = id;
     }
-    sidx[j + 1] = key;
-    sorted[j + 1] = v;
-  }
+  for (int i = b; i < e; ++i) sorted[i] = posw[sidx[i]];
 }
 
 template <typename T>
-__global__ void k_cellsort(const int* __restrict__ start, long ncell, Vec4<T>* __restrict__ sorted,
-                           int* __restrict__ sidx, int* __restrict__ count,
-                           int* __restrict__ tsum, int nreset) {
-  k_cellsort_body<T>(Blk::self(), start, ncell, sorted, sidx, count, tsum, nreset);
+__global__ void k_cellsort(const int* __restrict__ start, long ncell,
+                           const Vec4<T>* __restrict__ posw, Vec4<T>* __restrict__ sorted,
+                           int* __restrict__ sidx) {
+  k_cellsort_body<T>(Blk::self(), start, ncell, posw, sorted, sidx);
 }
 
 // Arguments of the binning kernel for a plan.
@@ -342,10 +344,8 @@ template <typename T> int launch_bin(Plan* p, const T* pos, const T* cc, cudaStr
   const BinArgs<T> bg = bin_args<T>(p);
   const long ncell = p->cg.ncell;
   const long ntiles = cdiv(ncell, kScanTile);
-  // direct: tile sums from the binning (kept zero between binnings by the
-  // cell sort; zeroed at plan creation), no tile pass
+  // direct: tile sums from the binning, no tile pass
   const bool direct = ntiles <= kScanDirect;
-  // cell counters start at zero: set at plan creation, reset by k_cellsort
   const int nbin = (int)cdiv(N, kBlock);
   launch_pdl(k_bin<T>, nbin, kBlock, 0, st, pos, cc, cc ? 3 : 4, N, bg, (Vec4<T>*)p->d_pos_w,
              p->d_cell_of, p->d_cell_count, p->d_flag, direct ? p->d_scan : (int*)nullptr,
@@ -353,14 +353,12 @@ template <typename T> int launch_bin(Plan* p, const T* pos, const T* cc, cudaStr
   if (!direct)
     launch_pdl(k_scan_tiles, ntiles, kBlock, 0, st, (const int*)p->d_cell_count, ncell, p->d_scan,
                p->d_cell_start, p->d_flag);
-  launch_pdl(k_scan_final, ntiles, kBlock, 0, st, p->d_cell_count, ncell, (const int*)p->d_scan,
+  launch_pdl(k_scan_final, ntiles, kBlock, 0, st, (const int*)p->d_cell_count, ncell, (const int*)p->d_scan,
              p->d_cell_start, direct ? 1 : 0, p->d_flag);
-  launch_pdl(k_scatter<T>, cdiv(N, kBlock), kBlock, 0, st, (const Vec4<T>*)p->d_pos_w, p->d_cell_of, N,
-                                                  p->d_cell_start, p->d_cell_count,
-                                                  (Vec4<T>*)p->d_sorted, p->d_sorted_idx);
-  launch_pdl(k_cellsort<T>, cdiv(std::max(ncell, ntiles), kBlock), kBlock, 0, st,
-             (const int*)p->d_cell_start, ncell, (Vec4<T>*)p->d_sorted, p->d_sorted_idx,
-             p->d_cell_count, p->d_scan, direct ? (int)ntiles : 0);
+  launch_pdl(k_scatter, cdiv(N, kBlock), kBlock, 0, st, (const int2*)p->d_cell_of, N,
+             (const int*)p->d_cell_start, p->d_sorted_idx);
+  launch_pdl(k_cellsort<T>, cdiv(ncell, kBlock), kBlock, 0, st, (const int*)p->d_cell_start, ncell,
+             (const Vec4<T>*)p->d_pos_w, (Vec4<T>*)p->d_sorted, p->d_sorted_idx);
   return direct ? 4 : 5;
 }
 

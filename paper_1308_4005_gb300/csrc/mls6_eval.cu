@@ -70,10 +70,21 @@ template <typename T> static int upload_tables_t(Plan* p) {
   };
   int rc = 0;
   rc |= A(&p->d_pos_w, sizeof(Vec4<T>) * N);
-  rc |= A((void**)&p->d_cell_of, sizeof(int) * N);
-  rc |= A((void**)&p->d_cell_count, sizeof(int) * p->cg.ncell);
+  rc |= A((void**)&p->d_cell_of, sizeof(int2) * N);
   rc |= A((void**)&p->d_cell_start, sizeof(int) * (p->cg.ncell + 1));
-  rc |= A((void**)&p->d_scan, 2 * sizeof(int) * std::max(1L, cdiv(p->cg.ncell, kScanTile)));
+  {
+    auto up = [](size_t b) { return (b + 255) & ~size_t(255); };
+    const size_t flag = up(sizeof(int) * 8);
+    const size_t scan = up(sizeof(int) * std::max(1L, cdiv(p->cg.ncell, kScanTile)));
+    const size_t count = up(sizeof(int) * p->cg.ncell);
+    const size_t q1 = up(e * p->lv[1].np);  // int32 (FP32 modes) or int64 sums
+    p->zero_bytes = flag + scan + count + q1;
+    if (A((void**)&p->d_zero, p->zero_bytes)) return MLS6_ERR_NOMEM;
+    p->d_flag = (int*)p->d_zero;
+    p->d_scan = (int*)(p->d_zero + flag);
+    p->d_cell_count = (int*)(p->d_zero + flag + scan);
+    p->d_q1fx = p->d_zero + flag + scan + count;
+  }
   rc |= A(&p->d_sorted, sizeof(Vec4<T>) * (N + 3));  // 3 padding records (pair kernel loads)
   rc |= A((void**)&p->d_sorted_idx, sizeof(int) * N);
   rc |= A(&p->d_e0, e * N);
@@ -145,8 +156,6 @@ template <typename T> static int upload_tables_t(Plan* p) {
   rc |= A((void**)&p->d_epart, sizeof(double) * p->n_epart);
   rc |= A((void**)&p->d_wpart, 6 * sizeof(double) * p->n_wpart);
   rc |= A((void**)&p->d_out, (8 + 6 * kReduceGroups) * sizeof(double));
-  rc |= A((void**)&p->d_flag, sizeof(int) * 8);
-  rc |= A(&p->d_q1fx, sizeof(unsigned long long) * p->lv[1].np);
   if (rc) return MLS6_ERR_NOMEM;
   if (cudaMallocHost((void**)&p->h_out, 8 * sizeof(double)) != cudaSuccess) return MLS6_ERR_NOMEM;
 
@@ -171,9 +180,7 @@ template <typename T> static int upload_tables_t(Plan* p) {
   CK(cudaMemcpy(p->d_top_T, p->h_top_T.data(), sizeof(double) * np_top, cudaMemcpyHostToDevice));
   CK(cudaMemcpy(p->d_top_V, p->h_top_V.data(), 6 * sizeof(double) * np_top,
                 cudaMemcpyHostToDevice));
-  CK(cudaMemset(p->d_flag, 0, sizeof(int) * 8));
-  CK(cudaMemset(p->d_cell_count, 0, sizeof(int) * p->cg.ncell));  // reset by each binning
-  CK(cudaMemset(p->d_scan, 0, 2 * sizeof(int) * std::max(1L, cdiv(p->cg.ncell, kScanTile))));
+  CK(cudaMemset(p->d_zero, 0, p->zero_bytes));
   CK(cudaMemset(p->d_wpart, 0, 6 * sizeof(double) * p->n_wpart));
   return MLS6_OK;
 }
@@ -212,12 +219,9 @@ static int enqueue(Plan* p, const T* pos, const T* cc, T* forces, double* energy
   } while (0)
   int nl = 0;
   BEGIN(0, st);
-  // flags, tickets, maxima (see Plan::d_flag); anterpolation sums
-  CK(cudaMemsetAsync(p->d_flag, 0, sizeof(int) * 8, st));
-  if (N > 0)
-    CK(cudaMemsetAsync(p->d_q1fx, 0, sizeof(T) * p->lv[1].np, st));  // int32 or int64 sums
-  else
-    CK(cudaMemsetAsync(p->d_q[1], 0, sizeof(T) * p->lv[1].np, st));
+  // flags, tickets, maxima (see Plan::d_flag), cell counts, anterpolation sums
+  CK(cudaMemsetAsync(p->d_zero, 0, p->zero_bytes, st));
+  if (N == 0) CK(cudaMemsetAsync(p->d_q[1], 0, sizeof(T) * p->lv[1].np, st));
   if (N > 0) nl += launch_bin<T>(p, pos, cc, st);
   END(0, st);
   if (N > 0) {
@@ -382,12 +386,12 @@ static int eval_lb_t(Plan* p, const T* pos, const T* sigma, const T* eps, T* for
   const int l = p->levels;
   CK(cudaEventRecord(p->ev_in, p->stream));
   CK(cudaStreamWaitEvent(st, p->ev_in, 0));
-  CK(cudaMemsetAsync(p->d_flag, 0, sizeof(int) * 8, st));
+  CK(cudaMemsetAsync(p->d_zero, 0, p->zero_bytes, st));
   int nl = launch_bin<T>(p, pos, sigma, st);  // records carry sigma as the coefficient
   nl += launch_lb_weights<T>(p, eps, st);
   nl += launch_pair<T>(p, false, st, true);
   for (int m = 0; m < 7; ++m) {
-    CK(cudaMemsetAsync(p->d_q1fx, 0, sizeof(T) * np1, st));
+    if (m > 0) CK(cudaMemsetAsync(p->d_q1fx, 0, sizeof(T) * np1, st));
     nl += launch_anterp<T>(p, st, m);
     for (int k = 1; k < l; ++k) nl += launch_restrict<T>(p, k, st);
     nl += launch_stencil<T>(p, false, st);

@@ -121,7 +121,11 @@ struct Plan {
 
   // ------------------------------------------------------------ device
   void* d_pos_w = nullptr;     // Vec4<T>[N]: wrapped positions + c, input order
-  int* d_cell_of = nullptr;    // int[N]
+  int2* d_cell_of = nullptr;   // [N]: cell, place among the cell's atoms
+  // what every evaluation starts from zero, one region (zero_bytes):
+  // d_flag | d_scan | d_cell_count | d_q1fx
+  char* d_zero = nullptr;
+  size_t zero_bytes = 0;
   int* d_cell_count = nullptr; // int[ncell]
   int* d_cell_start = nullptr; // int[ncell + 1]
   int* d_scan = nullptr;       // tile sums of the cell-count scan

@@ -53,20 +53,16 @@ enum PStage : int {
   P_FROM_FIXED, P_RESTRICT, P_STENCIL, P_PROLONG, P_INTERP, P_OUT
 };
 
-struct ZeroP { int* a; long na; int* b; long nb; };
+struct ZeroP { int* a; long na; };
 struct BinP {
   const float* pos; const float* cc; int stride, N; BinArgs<float> g;
-  Vec4<float>* posw; int* cell_of; int* count; int* flag; int* tsum; int ntiles;
+  Vec4<float>* posw; int2* cell_of; int* count; int* flag; int* tsum; int ntiles;
 };
 struct ScanTilesP { const int* count; long n; int* tsum; int* start; int* flag; };
-struct ScanFinalP { int* count; long n; const int* tsum; int* start; int direct; int* flag; };
-struct ScatterP {
-  const Vec4<float>* posw; const int* cell_of; int N; const int* start; int* fill;
-  Vec4<float>* sorted; int* sidx;
-};
+struct ScanFinalP { const int* count; long n; const int* tsum; int* start; int direct; int* flag; };
+struct ScatterP { const int2* cell_of; int N; const int* start; int* sidx; };
 struct CellsortP {
-  const int* start; long ncell; Vec4<float>* sorted; int* sidx; int* count; int* tsum;
-  int nreset;
+  const int* start; long ncell; const Vec4<float>* posw; Vec4<float>* sorted; int* sidx;
 };
 struct PairP {
   const Vec4<float>* sp; const int* start; int N; PairArgs<float> g; float* e0; float* floc;
@@ -127,8 +123,6 @@ __device__ __forceinline__ void run_stage(const PStageDesc& d, unsigned b) {
       const ZeroP& a = d.u.z;
       for (long i = (long)b * blockDim.x + threadIdx.x; i < a.na; i += (long)d.nb * blockDim.x)
         a.a[i] = 0;
-      for (long i = (long)b * blockDim.x + threadIdx.x; i < a.nb; i += (long)d.nb * blockDim.x)
-        a.b[i] = 0;
       break;
     }
     case P_BIN: {
@@ -149,12 +143,12 @@ __device__ __forceinline__ void run_stage(const PStageDesc& d, unsigned b) {
     }
     case P_SCATTER: {
       const ScatterP& a = d.u.sc;
-      k_scatter_body<float>(bk, a.posw, a.cell_of, a.N, a.start, a.fill, a.sorted, a.sidx);
+      k_scatter_body(bk, a.cell_of, a.N, a.start, a.sidx);
       break;
     }
     case P_CELLSORT: {
       const CellsortP& a = d.u.cs;
-      k_cellsort_body<float>(bk, a.start, a.ncell, a.sorted, a.sidx, a.count, a.tsum, a.nreset);
+      k_cellsort_body<float>(bk, a.start, a.ncell, a.posw, a.sorted, a.sidx);
       break;
     }
     case P_PAIR: {
@@ -328,8 +322,9 @@ static void replica_stages(Plan* p, const float* pos, const float* cc, float* fo
     return d;
   };
   {
-    PStageDesc& d = add(P_ZERO, cdiv(L1.np, 8L * kBlock));
-    d.u.z = ZeroP{p->d_flag, 8, (int*)p->d_q1fx, L1.np};
+    const long n = (long)(p->zero_bytes / sizeof(int));
+    PStageDesc& d = add(P_ZERO, cdiv(n, 8L * kBlock));
+    d.u.z = ZeroP{(int*)p->d_zero, n};
   }
   const long ncell = p->cg.ncell, ntiles = cdiv(ncell, kScanTile);
   const bool direct = ntiles <= kScanDirect;
@@ -350,13 +345,12 @@ static void replica_stages(Plan* p, const float* pos, const float* cc, float* fo
   }
   {
     PStageDesc& d = add(P_SCATTER, cdiv(N, kBlock));
-    d.u.sc = ScatterP{(const Vec4<float>*)p->d_pos_w, p->d_cell_of, N, p->d_cell_start,
-                      p->d_cell_count, (Vec4<float>*)p->d_sorted, p->d_sorted_idx};
+    d.u.sc = ScatterP{p->d_cell_of, N, p->d_cell_start, p->d_sorted_idx};
   }
   {
-    PStageDesc& d = add(P_CELLSORT, cdiv(std::max(ncell, ntiles), kBlock));
-    d.u.cs = CellsortP{p->d_cell_start, ncell, (Vec4<float>*)p->d_sorted, p->d_sorted_idx,
-                       p->d_cell_count, p->d_scan, direct ? (int)ntiles : 0};
+    PStageDesc& d = add(P_CELLSORT, cdiv(ncell, kBlock));
+    d.u.cs = CellsortP{p->d_cell_start, ncell, (const Vec4<float>*)p->d_pos_w,
+                       (Vec4<float>*)p->d_sorted, p->d_sorted_idx};
   }
   {
     PStageDesc& d = add(P_PAIR, cdiv((long)N * p->pair_split, kBlock));

@@ -262,10 +262,9 @@ static int grid_dims_impl(const double box[3], double h, int levels, int n_out[3
 
 static void free_plan(Plan* p) {
   if (!p) return;
-  void* ptrs[] = {p->d_pos_w, p->d_cell_of, p->d_cell_count, p->d_cell_start, p->d_sorted,
+  void* ptrs[] = {p->d_pos_w, p->d_cell_of, p->d_zero, p->d_cell_start, p->d_sorted,
                   p->d_sorted_idx, p->d_e0, p->d_floc, p->d_rows, p->d_wv, p->d_top_T,
-                  p->d_top_V, p->d_epart, p->d_wpart, p->d_out, p->d_flag, p->d_scan,
-                  p->d_q1fx, p->d_tcw, p->d_lbw, p->d_lbpot, p->d_mma_rows, p->d_mma_bv,
+                  p->d_top_V, p->d_epart, p->d_wpart, p->d_out, p->d_tcw, p->d_lbw, p->d_lbpot, p->d_mma_rows, p->d_mma_bv,
                   p->d_mma_be};
   for (void* q : ptrs)
     if (q) cudaFree(q);
