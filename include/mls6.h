@@ -278,15 +278,19 @@ int mls6_auto_levels(const double box[3], double h);
  * warps); 1024: cluster form (FP32 and mixed plans: a warp pairs 8
  * consecutive sorted atoms with every candidate of their segment's
  * neighbour cells, four candidates per step, branch-free; Lorentz-Berthelot
- * evaluations of such a plan run the one-lane-per-atom kernel).  The warp
- * and queue forms are refused with MLS6_ERR_ARG when the neighbour range
+ * evaluations of such a plan run the one-lane-per-atom kernel); 2048: tile
+ * form (FP32 and mixed plans: a warp lists the candidates near 8 consecutive
+ * sorted atoms and evaluates all pairs of them, two per instruction).  The
+ * warp, queue and tile forms are refused with MLS6_ERR_ARG when the neighbour range
  * spans more than two cells per side or the box has fewer than five cells
- * along x, the cluster form also in FP64 or with fewer than 16 cells along
- * x.  stencil_groups: thread groups of 128 sharing one 8^3 stencil tile (1,
+ * along x or continuity is not 2, the cluster form in FP64 or with fewer than
+ * 16 cells along x, the tile form also in FP64.  stencil_groups: thread groups of 128 sharing one 8^3 stencil tile (1,
  * 2 or 4; ignored when the stencil tile does not fit in shared memory); 0
  * keeps the current value.  Defaults: FP64 the queue form with two atoms per
- * warp where allowed; otherwise the lanes per atom that give about 48
- * resident warps per SM (the cluster form is selected only by this call);
+ * warp where allowed; FP32 and mixed the tile form where allowed, from 8,192
+ * atoms and half an atom per cell on; otherwise the lanes per atom that give
+ * about 48 resident warps per SM (the cluster form is selected only by this
+ * call; replicas of a batch default to the lanes per atom);
  * stencil: 24 warps per SM.  A shape
  * changes the order of floating-point sums (results move at rounding level),
  * never what is summed.  Waits for the plan's streams; the next evaluation

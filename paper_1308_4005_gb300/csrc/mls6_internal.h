@@ -28,6 +28,7 @@ constexpr int kStencilW = 4;      // consecutive x outputs per stencil thread
 constexpr size_t kStencilSmemMax = 200 * 1024;  // dynamic shared memory of a stencil tile
 constexpr double kCellDiv = 2.0;  // cell width >= a / kCellDiv
 constexpr int kPairCluster = 1024;  // pair_split code of the cluster form
+constexpr int kPairTile = 2048;     // pair_split code of the tile form
 constexpr int kPairAtomBlock = 64;  // threads per block of the one-lane-per-atom pair kernel
 constexpr int kPairSplitMax = 32;  // pair-kernel blocks are at most N * kPairSplitMax / kBlock
 
@@ -219,8 +220,10 @@ template <typename T> int prepare_pair_kernels(Plan* p);
 int launch_reduce(Plan* p, bool vir, cudaStream_t st);
 int flag_status(int flag_word);  // mls6_eval.cu
 double lb_coef(int m);           // Lorentz-Berthelot channel coefficient (mls6_grid.cu)
-int pair_split(const Plan* p);  // default lanes per atom of the pair kernel (mls6_pair.cu)
+int pair_split(const Plan* p);  // default pair kernel (mls6_pair.cu)
 int pair_split_atom(const Plan* p);  // the default among the per-atom, warp and queue forms
+bool pair_tile_ok(const Plan* p);    // the tile form (kPairTile) applies (mls6_pair_tile.cu)
+int launch_pair_tile(Plan* p, bool vir, bool lb, cudaStream_t st);
 bool pair_cl_ok(const Plan* p);      // the cluster form (kPairCluster) applies
 bool pair_cluster_ok(const Plan* p);  // warp form usable (mls6_pair.cu)
 // virial partial records summed by the final reduction

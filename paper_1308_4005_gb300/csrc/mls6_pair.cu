@@ -1003,6 +1003,7 @@ long pair_blocks(const Plan* p, int split) {
   const long N = p->N;
   if (N <= 0) return 0;
   if (split == kPairCluster) return cdiv(N, (long)kBlock / 4);  // 8 atoms per warp
+  if (split == kPairTile) return cdiv(N, 32L);  // 8 atoms per warp, 4 warps per block
   if (split >= 64) return cdiv(cdiv(N, split / 64), kQWarps);
   if (split <= 8) return cdiv(N * split, 32L);  // per-atom kernel: one virial partial per warp
   return cdiv(N * split, kBlock);                // warp form: one per block
@@ -1010,14 +1011,21 @@ long pair_blocks(const Plan* p, int split) {
 #endif  // MLS6_DEVICE_ONLY
 
 // Default pair kernel: FP64 the queue form where the cell geometry allows
-// it; otherwise the smallest of 1, 2, 4, 8 lanes per atom that gives about
-// 48 resident warps per SM on a 152-SM GPU.
+// it; FP32 and mixed plans the tile form for systems that fill it; otherwise
+// the smallest of 1, 2, 4, 8 lanes per atom that gives about 48 resident
+// warps per SM on a 152-SM GPU.
 #ifndef MLS6_DEVICE_ONLY  // host code, left out where another unit includes this file
 int pair_split(const Plan* p) {
-  // the cluster form is not a default: on the 1M-atom cube it takes 1.22 ms
-  // against 0.757 ms for the per-atom kernel (every atom of a segment is
-  // evaluated against the union of the segment's candidate cells, which the
-  // full lanes do not make up for)
+  // Tile form from 8,192 atoms (1,024 warps) and half an atom per cell on.
+  // Pair stage against the per-atom kernel, with / without the virial:
+  //   65,536-atom slab 94 / 86 -> 53 / 45 us, 131,072 atoms 141 / 131 -> 88 / 78,
+  //   1,048,576 atoms (a = 3) 731 / 679 -> 524 / 466, 349,983 (a = 3.5)
+  //   401 / 374 -> 240 / 217, 4,194,304-atom slab 2528 / 2353 -> 1915 / 1702;
+  //   8,000 atoms 18.6 / 16.5 -> 18.7 / 16.6 (4,000: 16.4 / 15.8 -> 18.7 / 16.9,
+  //   eight lanes per atom, where the row set-up is not spread over enough work).
+  // Sparser systems spread 8 consecutive atoms over many cells (0.3 atoms per
+  // cell, 500,000 atoms: 199 / 157 us against 158 / 149).
+  if (pair_tile_ok(p) && p->N >= 8192 && 2 * p->N >= p->cg.ncell) return kPairTile;
   return pair_split_atom(p);
 }
 
@@ -1173,6 +1181,8 @@ static void launch_cl(Plan* p, const PairArgs<T>& pg, bool vir, cudaStream_t st)
 }
 
 template <typename T> int launch_pair(Plan* p, bool vir, cudaStream_t st, bool lb) {
+  if constexpr (sizeof(T) == 4)
+    if (p->pair_split == kPairTile) return launch_pair_tile(p, vir, lb, st);
   const PairArgs<T> pg = pair_args<T>(p);
   if (p->pair_split == kPairCluster) {
     // Lorentz-Berthelot and FP64 run the per-atom kernel

@@ -474,9 +474,12 @@ int mls6_set_tuning(mls6_plan_t* plan, int split, int groups) {
   if (!plan) return MLS6_ERR_ARG;
   Plan* p = reinterpret_cast<Plan*>(plan);
   if (split != 0 && split != 1 && split != 2 && split != 4 && split != 8 && split != 16 &&
-      split != 32 && split != 128 && split != 256 && split != 512 && split != kPairCluster)
+      split != 32 && split != 128 && split != 256 && split != 512 && split != kPairCluster &&
+      split != kPairTile)
     return MLS6_ERR_ARG;
-  if (split == kPairCluster ? !pair_cl_ok(p) : (split > 8 && !pair_cluster_ok(p)))
+  if (split == kPairCluster ? !pair_cl_ok(p)
+      : split == kPairTile  ? !pair_tile_ok(p)
+                            : (split > 8 && !pair_cluster_ok(p)))
     return MLS6_ERR_ARG;
   if (groups != 0 && groups != 1 && groups != 2 && groups != 4) return MLS6_ERR_ARG;
   const int s2 = split ? split : p->pair_split;
