@@ -136,11 +136,18 @@ int mls6_plan(mls6_plan_t** out, const double box[3], int64_t N, double a, doubl
  *               changes g_0 .. g_l, the tables and the self term
  *               gamma_n(0)/a^6.  Plans with n != 2 run the per-atom pair
  *               kernel only (pair_split 1..8) and refuse mls6_eval_lb.
- *   stencil     level-stencil kernel of an MLS6_MIXED plan: 0 automatic
- *               (tcgen05 tensor cores when 2a/h_1 < 9 and the levels give
- *               at least two 16^3 tiles per SM of the device, else the FP32
- *               CUDA-core kernel), 1 the FP32 CUDA-core kernel, 2 tcgen05
- *               tensor cores whenever 2a/h_1 < 9.  Ignored in FP64 / FP32.
+ *   stencil     level evaluation of an MLS6_MIXED plan: 0 automatic (the
+ *               transforms below where they apply; else, and for the grids of
+ *               mls6_debug_grid, tcgen05 tensor cores when 2a/h_1 < 9 and the
+ *               levels give at least two 16^3 tiles per SM of the device, or
+ *               the FP32 CUDA-core kernel), 1 the FP32 CUDA-core kernel, 2
+ *               tcgen05 tensor cores whenever 2a/h_1 < 9.  Ignored in FP64 /
+ *               FP32, which evaluate as 0 does with the CUDA cores.
+ * Level evaluation by transforms: with 2 to 5 levels, no prime factor above 19
+ * in the finest grid's axes and an x-y plane that fits in shared memory,
+ * restriction, every level, the coarsest level and prolongation are products
+ * in the discrete Fourier transform of the finest grid, in the plan's
+ * precision (the coarsest level in FP64); the same periodic sums, reassociated.
  * Out-of-range values return MLS6_ERR_ARG. */
 typedef struct {
   int continuity;
@@ -238,7 +245,9 @@ int mls6_plan_info(const mls6_plan_t* p, int* n_grid, double* h_actual, int* lev
 /* Copy one grid of the last evaluation to host memory as doubles (x fastest):
  * which = 0: xi^k (anterpolated / restricted coefficients),
  *         1: e^k (level evaluation), 2: e^{k,tot} (after prolongation).
- * level: 1..l.  Synchronises the plan's stream. */
+ * level: 1..l.  Synchronises the plan's stream.  A plan that evaluates by
+ * transforms keeps only xi^1 (fixed point) and e^{1,tot}; the other grids are
+ * formed by this call, with the plan's stencil kernel. */
 int mls6_debug_grid(mls6_plan_t* p, int level, int which, double* host_out);
 
 /* Per-stage timing with CUDA events (off by default).  While enabled, the
@@ -247,7 +256,8 @@ int mls6_debug_grid(mls6_plan_t* p, int level, int which, double* host_out);
  * and end of each stage:
  * 0 bin (wrap, cell histogram, scan, scatter, per-cell order), 1 pair
  * (local part), 2 anterpolation, 3 restriction, 4 level stencils,
- * 5 coarsest level, 6 prolongation, 7 interpolation/forces, 8 reduction. */
+ * 5 coarsest level, 6 prolongation, 7 interpolation/forces, 8 reduction.
+ * A plan that evaluates by transforms does all of 3..6 in stage 4. */
 int mls6_profile(mls6_plan_t* p, int enable);
 
 /* Waits for the plan's stream and writes the stage durations of the last
@@ -297,7 +307,8 @@ int mls6_auto_levels(const double box[3], double h);
  * re-captures its graph. */
 int mls6_set_tuning(mls6_plan_t* p, int pair_split, int stencil_groups);
 
-/* Which level-stencil kernel the plan runs: 0 shared-memory tiles on the
+/* Which level-stencil kernel the plan has, for the evaluation or (a plan that
+ * evaluates by transforms) for mls6_debug_grid: 0 shared-memory tiles on the
  * CUDA cores (FP64 / FP32, and MLS6_MIXED plans whose grids are too small
  * for the tensor-core tiles), 1 global-memory fallback (tile and taps
  * beyond the shared-memory budget), 2 tensor cores through mma.sync

@@ -252,6 +252,67 @@ __device__ __forceinline__ void coarsest_node(const T* __restrict__ q, int n0, i
   }
 }
 
+// (1/8) sqrt(binom(6, k)), the Lorentz-Berthelot expansion coefficient
+// (Sec. II.D) of channel k.
+__device__ __forceinline__ double lb_coef_d(int k) {
+  const double b = (k == 0 || k == 6) ? 1.0 : (k == 1 || k == 5) ? 6.0 : (k == 2 || k == 4) ? 15.0
+                                                                                           : 20.0;
+  return 0.125 * sqrt(b);
+}
+
+// Fixed-point accumulation of the anterpolation: 32-bit integers for the
+// FP32 modes (sums kept below 2^30), 64-bit for FP64 (below 2^61).  Each
+// contribution is rounded to 2^(e-30) (FP32) or 2^(e-61) (FP64), where 2^e
+// exceeds the worst-case node sum B of fixed_exponent; B is a conservative
+// bound (most atoms in a cell x cells a support box meets x max |c|), so for
+// FP32 the step is ~1e-6 of a typical node sum of order 1: tens of FP32
+// rounding units per contribution, far below the FP32 path's force error
+// but not below FP32 rounding (the bound is tested against the FP64 oracle
+// on the 65,536-atom slab).  For FP64 it is ~1e-15 of a node sum.  The
+// conversions stay in the kernel's own precision: FP64 arithmetic is slow on
+// this GPU.
+template <typename T> struct Fixed;
+template <> struct Fixed<float> {
+  using I = int;
+  using U = unsigned int;
+  static constexpr int kBits = 30;
+  __device__ static float pow2(int s) { return __int_as_float((127 + s) << 23); }
+  __device__ static I to_fixed(float v, float scale) { return __float2int_rn(v * scale); }
+  __device__ static float from_fixed(I v, float iscale) { return (float)v * iscale; }
+};
+template <> struct Fixed<double> {
+  using I = long long;
+  using U = unsigned long long;
+  static constexpr int kBits = 61;
+  __device__ static double pow2(int s) { return __longlong_as_double((long long)(1023 + s) << 52); }
+  __device__ static I to_fixed(double v, double scale) { return __double2ll_rn(v * scale); }
+  __device__ static double from_fixed(I v, double iscale) { return (double)v * iscale; }
+};
+
+// Scale 2^s with s chosen so that no node sum can exceed 2^kBits in
+// magnitude.  |Phi| <= 1, so a node receives at most |c| per atom within 2h
+// of it (per axis; with periodic images), and those atoms lie in at most
+// `span` cells (cells meeting a box of width 4h), each holding at most
+// flag[3] atoms: bound = flag[3] * span * max|c|.
+// Lorentz-Berthelot channel m (lbm >= 0): the coefficient is
+// xi_m = lbc sigma^m sqrt(2 eps), bounded by lbc sigma_max^m (flag[4..5])
+// times the largest sqrt(2 eps) (flag[6..7]).
+template <typename T>
+__device__ __forceinline__ int fixed_exponent(const int* __restrict__ flag, double span,
+                                              int lbm = -1, double lbc = 0.0) {
+  double cmax = *reinterpret_cast<const double*>(flag + 4);
+  if (lbm >= 0) {
+    double sm = 1.0;
+    for (int k = 0; k < lbm; ++k) sm *= cmax;
+    cmax = lbc * sm * *reinterpret_cast<const double*>(flag + 6);
+  }
+  const float bound = (float)((double)flag[3] * span * cmax * (1.0 + 1e-6));
+  if (!(bound > 0.f)) return 0;
+  int e;
+  frexpf(bound, &e);  // bound < 2^e
+  return min(max(Fixed<T>::kBits - e, -120), 120);
+}
+
 // Launch with the programmatic-stream-serialization attribute (see
 // pdl_begin); same semantics as kernel<<<grid, block, smem, st>>>(args...).
 template <typename... KArgs, typename... Args>

@@ -10,6 +10,7 @@
 //   stencil  Eq. (evaluation) on levels k < l (cutoff 2^k a)
 //   top      Eq. (last-grid-periodic-transformed) on level l
 //   prolong  e^{k,tot} = e^k + R^T e^{k+1,tot} (Sec. II.B, prolongation)
+//            (restrict .. prolong at once in Fourier space where that applies)
 //   interp   Eq. (interpolation), its gradient (forces), per-atom energy
 //   reduce   fixed-order sums of energy and virial partials
 #include <algorithm>
@@ -133,6 +134,11 @@ template <typename T> static int upload_tables_t(Plan* p) {
     rc = prepare_stencil_tc(p);
     if (rc) return rc;
   }
+  p->spectral = spectral_eligible(p);
+  if (p->spectral) {
+    rc = prepare_spectral<T>(p);
+    if (rc) return rc;
+  }
   if (l >= 2) {
     rc |= A((void**)&p->d_rows, sizeof(int) * 4 * p->nrows);
     rc |= A(&p->d_wv, sizeof(Vec4<T>) * p->ntaps);
@@ -151,8 +157,9 @@ template <typename T> static int upload_tables_t(Plan* p) {
       std::max(1L, std::max(cdiv(N * 8, (long)kBlock) * (kBlock / 32), cdiv(N * kPairSplitMax, kBlock)));
   p->wpart_stencil = 0;
   p->wpart_top = p->stencil_blocks;
-  p->wpart_pair = p->wpart_top + np_top;
-  p->n_wpart = p->wpart_pair + p->n_pair_blocks;
+  // (spectral form: one record per set of frequencies, i.e. coarsest node)
+  p->wpart_pair = p->spectral ? np_top : p->wpart_top + np_top;
+  p->n_wpart = p->wpart_top + np_top + p->n_pair_blocks;
   rc |= A((void**)&p->d_epart, sizeof(double) * p->n_epart);
   rc |= A((void**)&p->d_wpart, 6 * sizeof(double) * p->n_wpart);
   rc |= A((void**)&p->d_out, (8 + 6 * kReduceGroups) * sizeof(double));
@@ -218,6 +225,7 @@ static int enqueue(Plan* p, const T* pos, const T* cc, T* forces, double* energy
     if (p->prof) CK(cudaEventRecordWithFlags(p->ev_e[i], s, evf)); \
   } while (0)
   int nl = 0;
+  p->lb_last = false;
   BEGIN(0, st);
   // flags, tickets, maxima (see Plan::d_flag), cell counts, anterpolation sums
   CK(cudaMemsetAsync(p->d_zero, 0, p->zero_bytes, st));
@@ -232,7 +240,7 @@ static int enqueue(Plan* p, const T* pos, const T* cc, T* forces, double* energy
     END(1, st2);
     CK(cudaEventRecord(p->ev_join, st2));
     BEGIN(2, st);
-    nl += launch_anterp<T>(p, st);
+    nl += launch_anterp<T>(p, st, -1, !p->spectral);
     END(2, st);
   } else {
     // no atoms: grids stay zero; zero the atom-side partial sums
@@ -242,17 +250,20 @@ static int enqueue(Plan* p, const T* pos, const T* cc, T* forces, double* energy
     BEGIN(2, st);
     END(2, st);
   }
+  // spectral form: every level in the stencil stage, the others empty
   BEGIN(3, st);
-  for (int k = 1; k < l; ++k) nl += launch_restrict<T>(p, k, st);
+  if (!p->spectral)
+    for (int k = 1; k < l; ++k) nl += launch_restrict<T>(p, k, st);
   END(3, st);
   BEGIN(4, st);
-  nl += launch_stencil<T>(p, vir, st);
+  nl += p->spectral ? launch_spectral<T>(p, vir, false, st) : launch_stencil<T>(p, vir, st);
   END(4, st);
   BEGIN(5, st);
-  nl += launch_top<T>(p, vir, st);
+  if (!p->spectral) nl += launch_top<T>(p, vir, st);
   END(5, st);
   BEGIN(6, st);
-  for (int k = l - 1; k >= 1; --k) nl += launch_prolong<T>(p, k, st);
+  if (!p->spectral)
+    for (int k = l - 1; k >= 1; --k) nl += launch_prolong<T>(p, k, st);
   END(6, st);
   if (N > 0) CK(cudaStreamWaitEvent(st, p->ev_join, 0));
   // interpolation; its last block also performs the final reduction
@@ -381,16 +392,30 @@ static int eval_lb_t(Plan* p, const T* pos, const T* sigma, const T* eps, T* for
   if (!p->d_lbw) {
     if (cudaMalloc(&p->d_lbw, sizeof(T) * N) != cudaSuccess) return MLS6_ERR_NOMEM;
     if (cudaMalloc(&p->d_lbpot, sizeof(T) * 7 * np1) != cudaSuccess) return MLS6_ERR_NOMEM;
+    if (p->spectral) {
+      const int* n = p->lv[1].n;
+      const size_t ns = (size_t)n[1] * (n[0] / 2 + 1) * n[2];
+      if (cudaMalloc(&p->d_lbq, sizeof(T) * 7 * np1) != cudaSuccess ||
+          cudaMalloc(&p->d_lbs, 2 * sizeof(T) * 2 * 7 * ns) != cudaSuccess)
+        return MLS6_ERR_NOMEM;
+    }
   }
   cudaStream_t st = p->cs;
   const int l = p->levels;
+  p->lb_last = true;
   CK(cudaEventRecord(p->ev_in, p->stream));
   CK(cudaStreamWaitEvent(st, p->ev_in, 0));
   CK(cudaMemsetAsync(p->d_zero, 0, p->zero_bytes, st));
   int nl = launch_bin<T>(p, pos, sigma, st);  // records carry sigma as the coefficient
   nl += launch_lb_weights<T>(p, eps, st);
   nl += launch_pair<T>(p, false, st, true);
-  for (int m = 0; m < 7; ++m) {
+  if (p->spectral) {
+    CK(cudaMemsetAsync(p->d_lbq, 0, sizeof(T) * 7 * np1, st));
+    for (int m = 0; m < 7; ++m)
+      nl += launch_anterp<T>(p, st, m, false, (T*)p->d_lbq + (size_t)m * np1);
+    nl += launch_spectral<T>(p, false, true, st);
+  }
+  for (int m = 0; m < 7 && !p->spectral; ++m) {
     if (m > 0) CK(cudaMemsetAsync(p->d_q1fx, 0, sizeof(T) * np1, st));
     nl += launch_anterp<T>(p, st, m);
     for (int k = 1; k < l; ++k) nl += launch_restrict<T>(p, k, st);
@@ -452,6 +477,20 @@ using namespace mls6;
 
 template <typename T> static int debug_grid_t(Plan* p, int level, int which, double* out) {
   const Level& Lk = p->lv[level];
+  // spectral form: the evaluation kept q^1 (as fixed-point sums) and
+  // e^{1,tot}; the other grids are formed here, by the direct kernels
+  const bool have = level == 1 && which == 2;
+  if (p->spectral && !have) {
+    cudaStream_t st = p->cs ? p->cs : p->stream;
+    if (cudaStreamSynchronize(p->stream) != cudaSuccess) return MLS6_ERR_CUDA;
+    launch_from_fixed<T>(p, st, p->lb_last ? 6 : -1,
+                         p->lb_last ? (const T*)p->d_lbq + (size_t)6 * p->lv[1].np : nullptr);
+    for (int k = 1; k < p->levels; ++k) launch_restrict<T>(p, k, st);
+    launch_stencil<T>(p, false, st);
+    launch_top<T>(p, false, st);
+    for (int k = p->levels - 1; k >= 2; --k) launch_prolong<T>(p, k, st);
+    if (cudaStreamSynchronize(st) != cudaSuccess) return MLS6_ERR_CUDA;
+  }
   const void* src = which == 0 ? p->d_q[level] : which == 1 ? p->d_e[level] : p->d_et[level];
   std::vector<T> tmp((size_t)Lk.np);
   if (cudaStreamSynchronize(p->stream) != cudaSuccess) return MLS6_ERR_CUDA;

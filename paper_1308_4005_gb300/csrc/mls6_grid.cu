@@ -11,67 +11,6 @@ namespace mls6 {
 
 // ------------------------------------------------------------ anterpolation
 
-// (1/8) sqrt(binom(6, k)), the Lorentz-Berthelot expansion coefficient
-// (Sec. II.D) of channel k.
-__device__ __forceinline__ double lb_coef_d(int k) {
-  const double b = (k == 0 || k == 6) ? 1.0 : (k == 1 || k == 5) ? 6.0 : (k == 2 || k == 4) ? 15.0
-                                                                                           : 20.0;
-  return 0.125 * sqrt(b);
-}
-
-// Fixed-point accumulation of the anterpolation: 32-bit integers for the
-// FP32 modes (sums kept below 2^30), 64-bit for FP64 (below 2^61).  Each
-// contribution is rounded to 2^(e-30) (FP32) or 2^(e-61) (FP64), where 2^e
-// exceeds the worst-case node sum B of fixed_exponent; B is a conservative
-// bound (most atoms in a cell x cells a support box meets x max |c|), so for
-// FP32 the step is ~1e-6 of a typical node sum of order 1: tens of FP32
-// rounding units per contribution, far below the FP32 path's force error
-// but not below FP32 rounding (the bound is tested against the FP64 oracle
-// on the 65,536-atom slab).  For FP64 it is ~1e-15 of a node sum.  The
-// conversions stay in the kernel's own precision: FP64 arithmetic is slow on
-// this GPU.
-template <typename T> struct Fixed;
-template <> struct Fixed<float> {
-  using I = int;
-  using U = unsigned int;
-  static constexpr int kBits = 30;
-  __device__ static float pow2(int s) { return __int_as_float((127 + s) << 23); }
-  __device__ static I to_fixed(float v, float scale) { return __float2int_rn(v * scale); }
-  __device__ static float from_fixed(I v, float iscale) { return (float)v * iscale; }
-};
-template <> struct Fixed<double> {
-  using I = long long;
-  using U = unsigned long long;
-  static constexpr int kBits = 61;
-  __device__ static double pow2(int s) { return __longlong_as_double((long long)(1023 + s) << 52); }
-  __device__ static I to_fixed(double v, double scale) { return __double2ll_rn(v * scale); }
-  __device__ static double from_fixed(I v, double iscale) { return (double)v * iscale; }
-};
-
-// Scale 2^s with s chosen so that no node sum can exceed 2^kBits in
-// magnitude.  |Phi| <= 1, so a node receives at most |c| per atom within 2h
-// of it (per axis; with periodic images), and those atoms lie in at most
-// `span` cells (cells meeting a box of width 4h), each holding at most
-// flag[3] atoms: bound = flag[3] * span * max|c|.
-// Lorentz-Berthelot channel m (lbm >= 0): the coefficient is
-// xi_m = lbc sigma^m sqrt(2 eps), bounded by lbc sigma_max^m (flag[4..5])
-// times the largest sqrt(2 eps) (flag[6..7]).
-template <typename T>
-__device__ __forceinline__ int fixed_exponent(const int* __restrict__ flag, double span,
-                                              int lbm = -1, double lbc = 0.0) {
-  double cmax = *reinterpret_cast<const double*>(flag + 4);
-  if (lbm >= 0) {
-    double sm = 1.0;
-    for (int k = 0; k < lbm; ++k) sm *= cmax;
-    cmax = lbc * sm * *reinterpret_cast<const double*>(flag + 6);
-  }
-  const float bound = (float)((double)flag[3] * span * cmax * (1.0 + 1e-6));
-  if (!(bound > 0.f)) return 0;
-  int e;
-  frexpf(bound, &e);  // bound < 2^e
-  return min(max(Fixed<T>::kBits - e, -120), 120);
-}
-
 // Eq. (anterpolation): q^1_mu += c_j phi_mu(x_j) over the NP^3 nodes of
 // every atom (NP = p + 1: 4x4x4 for the cubic, 6x6x6 for the quintic).  The contributions are rounded to the fixed-point grid 2^-s
 // and added as integers (Fixed<T>): integer addition is associative, so the
@@ -232,15 +171,6 @@ __global__ void k_from_fixed(const typename Fixed<T>::U* __restrict__ qfx, long 
   k_from_fixed_body<T>(Blk::self(), qfx, np, flag, span, q, lbm, lbc);
 }
 
-// Cells (with periodic images) that the support of one node's basis
-// function (width (p + 1) h) can meet, product over the axes.
-static double support_span(const Plan* p) {
-  double s = 1.0;
-  const double width = p->order + 1.0;
-  for (int d = 0; d < 3; ++d) s *= std::ceil(width * p->lv[1].h[d] / p->cg.w[d]) + 1.0;
-  return s;
-}
-
 // lbm >= 0: Lorentz-Berthelot channel m (coefficients computed from the
 // sorted sigma and sqrt(2 eps)); -1: the atoms' own coefficients.
 #ifndef MLS6_DEVICE_ONLY  // host code, left out where another unit includes this file
@@ -250,7 +180,7 @@ double lb_coef(int m) {
 }
 #endif  // MLS6_DEVICE_ONLY
 
-template <typename T> int launch_anterp(Plan* p, cudaStream_t st, int lbm) {
+template <typename T> int launch_anterp(Plan* p, cudaStream_t st, int lbm, bool to_grid, void* qfx) {
   const Level& L1 = p->lv[1];
   const int N = (int)p->N;
   const double span = support_span(p);
@@ -258,10 +188,18 @@ template <typename T> int launch_anterp(Plan* p, cudaStream_t st, int lbm) {
   launch_pdl(p->order == 5 ? k_anterp<T, 6> : k_anterp<T, 4>, cdiv(N, kBlock), kBlock, 0, st,
       (const Vec4<T>*)p->d_sorted, N, L1.n[0], L1.n[1], L1.n[2], (T)(1.0 / L1.h[0]),
       (T)(1.0 / L1.h[1]), (T)(1.0 / L1.h[2]), p->d_flag, span,
-      (typename Fixed<T>::U*)p->d_q1fx, (const T*)p->d_lbw, lbm, lbc);
+      (typename Fixed<T>::U*)(qfx ? qfx : p->d_q1fx), (const T*)p->d_lbw, lbm, lbc);
+  return 1 + (to_grid ? launch_from_fixed<T>(p, st, lbm, qfx) : 0);
+}
+
+// q^1 from the fixed-point sums.
+template <typename T> int launch_from_fixed(Plan* p, cudaStream_t st, int lbm, const void* qfx) {
+  const Level& L1 = p->lv[1];
+  const double span = support_span(p), lbc = lb_coef(lbm);
   launch_pdl(k_from_fixed<T>, cdiv(L1.np, kBlock), kBlock, 0, st, 
-      (const typename Fixed<T>::U*)p->d_q1fx, L1.np, p->d_flag, span, (T*)p->d_q[1], lbm, lbc);
-  return 2;
+      (const typename Fixed<T>::U*)(qfx ? qfx : p->d_q1fx), L1.np, p->d_flag, span, (T*)p->d_q[1],
+      lbm, lbc);
+  return 1;
 }
 
 // sqrt(2 eps) of the atoms in sorted order, and its largest value
@@ -1054,7 +992,8 @@ template <typename T> int prepare_grid_kernels(Plan* p) {
 
 #ifndef MLS6_DEVICE_ONLY  // host code, left out where another unit includes this file
 #define MLS6_INSTANTIATE(T)                                               \
-  template int launch_anterp<T>(Plan*, cudaStream_t, int);                \
+  template int launch_anterp<T>(Plan*, cudaStream_t, int, bool, void*);   \
+  template int launch_from_fixed<T>(Plan*, cudaStream_t, int, const void*); \
   template int launch_lb_weights<T>(Plan*, const T*, cudaStream_t);       \
   template int launch_interp_lb<T>(Plan*, T*, cudaStream_t);              \
   template int launch_restrict<T>(Plan*, int, cudaStream_t);              \

@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <cmath>
 #include <vector>
 
 #include "../../include/mls6.h"
@@ -138,6 +139,16 @@ struct Plan {
   void* d_q1fx = nullptr;      // int32 (FP32 modes) / int64 (FP64) fixed-point anterpolation sums
   void* d_lbw = nullptr;       // T[N]: sqrt(2 eps) in sorted order (Lorentz-Berthelot)
   void* d_lbpot = nullptr;     // T[7 n_1]: level-1 total potential of each LB channel
+  void* d_lbq = nullptr;       // fixed-point sums of the seven channels (spectral form)
+  void* d_lbs = nullptr;       // their transforms
+  // spectral form of the grid part (mls6_spectral.cu)
+  bool spectral = false;
+  bool lb_last = false;        // the last evaluation was a Lorentz-Berthelot one
+  unsigned long long spec_rad[3] = {};  // radices per axis (x: of n/2)
+  void* d_spec_tw = nullptr;   // exp(-2 pi i j / n) per axis
+  void* d_spec_tab = nullptr;  // restriction factors per axis | level-1 factors, 7 octants
+  double* d_spec_top = nullptr;// coarsest-level factors, 7 grids
+  void* d_spec_s = nullptr;    // transforms of q^1 and of e^{1,tot}
   void* d_q[kMaxLevels + 1] = {};
   void* d_e[kMaxLevels + 1] = {};
   void* d_et[kMaxLevels + 1] = {};
@@ -206,7 +217,15 @@ int enqueue_eval(Plan* p, const void* pos, const void* c, void* forces, double* 
 // kernel launchers; each returns the number of kernels it launched
 template <typename T> int launch_bin(Plan* p, const T* pos, const T* c, cudaStream_t st);
 template <typename T> int launch_pair(Plan* p, bool vir, cudaStream_t st, bool lb = false);
-template <typename T> int launch_anterp(Plan* p, cudaStream_t st, int lbm = -1);
+// to_grid: also convert the fixed-point sums to q^1; qfx: sums (default d_q1fx)
+template <typename T>
+int launch_anterp(Plan* p, cudaStream_t st, int lbm = -1, bool to_grid = true, void* qfx = nullptr);
+template <typename T>
+int launch_from_fixed(Plan* p, cudaStream_t st, int lbm = -1, const void* qfx = nullptr);
+// q^1 sums -> e^{1,tot} and the grid part of the virial (lb: the seven channels)
+bool spectral_eligible(const Plan* p);
+template <typename T> int prepare_spectral(Plan* p);
+template <typename T> int launch_spectral(Plan* p, bool vir, bool lb, cudaStream_t st);
 template <typename T> int launch_lb_weights(Plan* p, const T* eps, cudaStream_t st);
 template <typename T> int launch_interp_lb(Plan* p, T* forces, cudaStream_t st);
 template <typename T> int launch_restrict(Plan* p, int k, cudaStream_t st);
@@ -230,6 +249,14 @@ bool pair_cluster_ok(const Plan* p);  // warp form usable (mls6_pair.cu)
 long pair_blocks(const Plan* p, int split);  // blocks of the pair kernel (mls6_pair.cu)
 inline long wpart_used(const Plan* p) { return p->wpart_pair + pair_blocks(p, p->pair_split); }
 bool stencil_fuses_top(const Plan* p);
+// Cells (with periodic images) that the support of one node's basis
+// function (width (p + 1) h) can meet, product over the axes.
+inline double support_span(const Plan* p) {
+  double s = 1.0;
+  const double width = p->order + 1.0;
+  for (int d = 0; d < 3; ++d) s *= std::ceil(width * p->lv[1].h[d] / p->cg.w[d]) + 1.0;
+  return s;
+}
 // tensor-core stencil (mls6_stencil_tc.cu)
 size_t tc_smem_bytes(int P);
 bool stencil_tc_eligible(const Plan* p);

@@ -43,6 +43,7 @@
 #include "mls6_bin.cu"
 #include "mls6_pair.cu"
 #include "mls6_grid.cu"
+#include "mls6_spectral.cu"
 #undef MLS6_DEVICE_ONLY
 #undef __restrict__
 
@@ -50,7 +51,8 @@ namespace mls6 {
 
 enum PStage : int {
   P_ZERO, P_BIN, P_SCAN_TILES, P_SCAN_FINAL, P_SCATTER, P_CELLSORT, P_PAIR, P_ANTERP,
-  P_FROM_FIXED, P_RESTRICT, P_STENCIL, P_PROLONG, P_INTERP, P_OUT
+  P_FROM_FIXED, P_RESTRICT, P_STENCIL, P_PROLONG, P_SPEC_FWD, P_SPEC_Z, P_SPEC_TREE, P_SPEC_IZ,
+  P_SPEC_INV, P_INTERP, P_OUT
 };
 
 struct ZeroP { int* a; long na; };
@@ -95,7 +97,8 @@ struct PStageDesc {
   unsigned dep_nb, dep2_nb; // their block counts
   union U {
     ZeroP z; BinP bin; ScanTilesP st; ScanFinalP sf; ScatterP sc; CellsortP cs; PairP pair;
-    AnterpP an; FromFixedP ff; RestrictP re; StencilP sten; ProlongP pr; InterpP in; OutP out;
+    AnterpP an; FromFixedP ff; RestrictP re; StencilP sten; ProlongP pr; SpecArgs<float> sp;
+    InterpP in; OutP out;
     U() {}
   } u;
 };
@@ -114,6 +117,8 @@ struct PExecArgs {
   int B, S;
   long long total, limit, withhold;
 };
+
+extern __shared__ __align__(16) unsigned char persist_smem[];  // the stencil's and the transforms'
 
 template <bool VIR>
 __device__ __forceinline__ void run_stage(const PStageDesc& d, unsigned b) {
@@ -199,6 +204,11 @@ __device__ __forceinline__ void run_stage(const PStageDesc& d, unsigned b) {
       k_prolong_body<float>(bk, a.ef, a.f0, a.f1, a.f2, a.etc_, a.c0, a.c1, a.c2, a.etf);
       break;
     }
+    case P_SPEC_FWD: spec_fwd_body<float, 19>(bk, 0, d.u.sp, persist_smem); break;
+    case P_SPEC_Z: spec_z_body<float, 19>(bk, 0, d.u.sp, 1.0f, persist_smem); break;
+    case P_SPEC_TREE: spec_tree_body<float, VIR>(bk, 0, d.u.sp, persist_smem); break;
+    case P_SPEC_IZ: spec_z_body<float, 19>(bk, 0, d.u.sp, -1.0f, persist_smem); break;
+    case P_SPEC_INV: spec_inv_body<float, 19>(bk, 0, d.u.sp, persist_smem); break;
     case P_INTERP: {
       const InterpP& a = d.u.in;
       if (a.slices)
@@ -365,12 +375,13 @@ static void replica_stages(Plan* p, const float* pos, const float* cc, float* fo
                      (float)(1.0 / L1.h[0]), (float)(1.0 / L1.h[1]), (float)(1.0 / L1.h[2]),
                      p->d_flag, span, (unsigned*)p->d_q1fx};
   }
+  const bool sp = p->spectral;
   {
-    PStageDesc& d = add(P_FROM_FIXED, cdiv(L1.np, kBlock));
+    PStageDesc& d = add(P_FROM_FIXED, sp ? 0 : cdiv(L1.np, kBlock));
     d.u.ff = FromFixedP{(const unsigned*)p->d_q1fx, L1.np, p->d_flag, span, (float*)p->d_q[1]};
   }
   for (int k = 1; k < lmax; ++k) {  // restriction slots (empty beyond this replica's levels)
-    const bool on = k < l;
+    const bool on = k < l && !sp;
     PStageDesc& d = add(P_RESTRICT, on ? cdiv(p->lv[k + 1].np, kBlock) : 0);
     if (on) {
       const Level &F = p->lv[k], &C = p->lv[k + 1];
@@ -380,18 +391,28 @@ static void replica_stages(Plan* p, const float* pos, const float* cc, float* fo
   }
   {
     const int warps = kStencilThreads * 2 / 32;
-    PStageDesc& d = add(P_STENCIL, p->stencil_blocks + cdiv(p->lv[l].np, warps));
+    PStageDesc& d = add(P_STENCIL, sp ? 0 : p->stencil_blocks + cdiv(p->lv[l].np, warps));
     d.u.sten.A = stencil_args<float>(p);
     d.u.sten.wpart = p->d_wpart + 6 * p->wpart_stencil;
   }
   for (int j = 0; j < lmax - 1; ++j) {  // prolongation slots, coarse to fine
     const int k = l - 1 - j;
-    const bool on = k >= 1;
+    const bool on = k >= 1 && !sp;
     PStageDesc& d = add(P_PROLONG, on ? cdiv(p->lv[k].np, kBlock) : 0);
     if (on) {
       const Level &F = p->lv[k], &C = p->lv[k + 1];
       d.u.pr = ProlongP{(const float*)p->d_e[k], F.n[0], F.n[1], F.n[2],
                         (const float*)p->d_et[k + 1], C.n[0], C.n[1], C.n[2], (float*)p->d_et[k]};
+    }
+  }
+  {  // the transforms, empty for a replica that runs the direct kernels
+    const long planes = sp ? L1.n[2] : 0;
+    const long cols = sp ? cdiv((long)L1.n[1] * (L1.n[0] / 2 + 1), kSpecCols) : 0;
+    const long sets = sp ? p->lv[l].np : 0;
+    const long nb[5] = {planes, cols, sets, cols, planes};
+    for (int k = 0; k < 5; ++k) {
+      PStageDesc& d = add(P_SPEC_FWD + k, nb[k]);
+      if (sp) d.u.sp = spec_args<float>(p, false);
     }
   }
   {
@@ -473,7 +494,14 @@ int persist_build(PersistExec** out, Plan* const* plans, int B, const int64_t* o
     }
   x->total = first.back();
   size_t smem = 0;
-  for (int r = 0; r < B; ++r) smem = std::max(smem, plans[r]->stencil_smem);
+  for (int r = 0; r < B; ++r) {
+    const Plan* p = plans[r];
+    const int* n = p->lv[1].n;
+    smem = std::max(smem, p->spectral ? std::max({spec_plane_smem<float>(n[0], n[1], (n[0] / 2 + 1) | 1),
+                                                  spec_z_smem<float>(n[2]),
+                                                  spec_tree_smem<float>(p->levels)})
+                                      : p->stencil_smem);
+  }
   x->smem = smem;
   int rc = MLS6_OK;
   auto A = [&](void** ptr, size_t bytes) {
