@@ -263,7 +263,8 @@ __global__ void k_scatter(const int2* __restrict__ cell_of, int N, const int* __
 // the index) in registers by an odd-even transposition network and only then
 // copy the records; larger cells use an insertion sort of the indices in
 // global memory; cells above 256 atoms are left in scatter order (results stay
-// correct, only bitwise reproducibility is lost for them).
+// correct, only bitwise reproducibility is lost for them).  FP64 plans also get
+// the positions in FP32, for the cutoff test of the pair sum's queue form.
 template <typename T>
 __device__ __forceinline__ unsigned long long record_key(const Vec4<T>* __restrict__ posw, int i) {
   unsigned long long k = (unsigned)i;
@@ -274,9 +275,14 @@ __device__ __forceinline__ unsigned long long record_key(const Vec4<T>* __restri
 template <typename T>
 __device__ __forceinline__ void k_cellsort_body(const Blk bk,const int* __restrict__ start, long ncell,
                            const Vec4<T>* __restrict__ posw, Vec4<T>* __restrict__ sorted,
-                           int* __restrict__ sidx) {
+                           int* __restrict__ sidx, float4* __restrict__ sortedf) {
   const long z = pdl_begin();
   start += z; posw += z;
+  auto put = [&](int k, const Vec4<T>& v) {
+    sorted[k] = v;
+    if constexpr (sizeof(T) == 8)
+      sortedf[k] = make_float4((float)v.x, (float)v.y, (float)v.z, 0.f);
+  };
   const long cell = (long)bk.x * blockDim.x + threadIdx.x;
   if (cell >= ncell) return;
   const int b = start[cell], e = start[cell + 1];
@@ -302,7 +308,7 @@ __device__ __forceinline__ void k_cellsort_body(const Blk bk,const int* __restri
       if (k < n) {
         const int i = (int)(unsigned)key[k];
         sidx[b + k] = i;
-        sorted[b + k] = posw[i];
+        put(b + k, posw[i]);
       }
     return;
   }
@@ -317,14 +323,14 @@ __device__ __forceinline__ void k_cellsort_body(const Blk bk,const int* __restri
       }
       sidx[j + 1] = id;
     }
-  for (int i = b; i < e; ++i) sorted[i] = posw[sidx[i]];
+  for (int i = b; i < e; ++i) put(i, posw[sidx[i]]);
 }
 
 template <typename T>
 __global__ void k_cellsort(const int* __restrict__ start, long ncell,
                            const Vec4<T>* __restrict__ posw, Vec4<T>* __restrict__ sorted,
-                           int* __restrict__ sidx) {
-  k_cellsort_body<T>(Blk::self(), start, ncell, posw, sorted, sidx);
+                           int* __restrict__ sidx, float4* __restrict__ sortedf) {
+  k_cellsort_body<T>(Blk::self(), start, ncell, posw, sorted, sidx, sortedf);
 }
 
 // Arguments of the binning kernel for a plan.
@@ -358,7 +364,8 @@ template <typename T> int launch_bin(Plan* p, const T* pos, const T* cc, cudaStr
   launch_pdl(k_scatter, cdiv(N, kBlock), kBlock, 0, st, (const int2*)p->d_cell_of, N,
              (const int*)p->d_cell_start, p->d_sorted_idx);
   launch_pdl(k_cellsort<T>, cdiv(ncell, kBlock), kBlock, 0, st, (const int*)p->d_cell_start, ncell,
-             (const Vec4<T>*)p->d_pos_w, (Vec4<T>*)p->d_sorted, p->d_sorted_idx);
+             (const Vec4<T>*)p->d_pos_w, (Vec4<T>*)p->d_sorted, p->d_sorted_idx,
+             (float4*)p->d_sorted_f);
   return direct ? 4 : 5;
 }
 

@@ -87,6 +87,7 @@ template <typename T> static int upload_tables_t(Plan* p) {
     p->d_q1fx = p->d_zero + flag + scan + count;
   }
   rc |= A(&p->d_sorted, sizeof(Vec4<T>) * (N + 3));  // 3 padding records (pair kernel loads)
+  if (e == 8) rc |= A(&p->d_sorted_f, sizeof(float4) * N);
   rc |= A((void**)&p->d_sorted_idx, sizeof(int) * N);
   rc |= A(&p->d_e0, e * N);
   rc |= A(&p->d_floc, 3 * e * N);

@@ -132,6 +132,7 @@ struct Plan {
   int* d_cell_start = nullptr; // int[ncell + 1]
   int* d_scan = nullptr;       // tile sums of the cell-count scan
   void* d_sorted = nullptr;    // Vec4<T>[N] sorted by cell
+  void* d_sorted_f = nullptr;  // float4[N]: the same positions in FP32 (FP64 plans)
   int* d_sorted_idx = nullptr; // int[N] original index of sorted atom
   int pair_split = 1;          // lanes per atom in the pair kernel
   void* d_e0 = nullptr;        // T[N] local potential (sorted order)

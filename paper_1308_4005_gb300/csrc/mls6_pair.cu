@@ -19,6 +19,10 @@ template <typename T> struct PairArgs {
   T a2, ia2, ia6, ia8;
   T margin;  // absolute slack of the row trimming (covers rounding of x, x/w)
   T Lhi[3], Llo[3];  // box length as an unevaluated sum hi + lo (exact image shifts)
+  // queue form, FP32 set-up and test: box, (a + slack)^2, cells, slack of the
+  // row trimming; half the box (virial)
+  float Lf[3], a2f, wf[3], iwf, marginf;
+  T mL[3], near2;  // and (a/16)^2
   // smoothing function of continuity other than C^2 (GEN kernels):
   // gamma = sum gc[k] u^k, u = rho^12; gamma'(rho)/rho = -12 rho^10 ... as
   // g_0'/r = -6 r^-8 + a^-8 rho^10 sum gd[k] u^k with gd[k] = -12 (k+1) gc[k+1]
@@ -658,19 +662,45 @@ __global__ void __launch_bounds__(kBlock) k_pair_cl(const Vec4<float>* __restric
   }
 }
 
+// 1/x for x > 0: FP64 from the hardware's approximation (about 20 bits) by two
+// Newton steps y += y (1 - x y), each of which doubles the correct bits: four
+// FP64 operations where the compiler's division spends about ten.
+__device__ __forceinline__ float q_rcp(float x) { return rcp(x); }
+__device__ __forceinline__ double q_rcp(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  y = fma(y, fma(-x, y, 1.0), y);
+  return fma(y, fma(-x, y, 1.0), y);
+}
+
+// 0 < r2 < a2 on the bits (FP64 comparisons take the FP64 pipe).
+__device__ __forceinline__ bool q_inside(float r2, float a2) { return r2 < a2 && r2 > 0.f; }
+__device__ __forceinline__ bool q_inside(double r2, double a2) {
+  const long long b = __double_as_longlong(r2);
+  return b < __double_as_longlong(a2) && b > 0;
+}
+
 // One queued pair of the queue form: displacement with an exact image shift,
-// then Eq. (g_0) and its derivative accumulated into the lane's sums.
+// then Eq. (g_0) and its derivative accumulated into the lane's sums, in units
+// of a: with s = (r/a)^2, e += C a^6 g_0 and f += C (-a^8 g_0'/6r) d (a pair
+// that only the FP32 test let through adds zero).
 // en = {j, image code (mx+8) | (my+8) << 4 | (mz+8) << 8}: the neighbour is
 // x_j + m L.  The box length is the unevaluated sum Lhi + Llo, and the
 // shift is applied to whichever of x_i, x_j lies near the far face
 // (x_i - Lhi for m = +1, x_j - Lhi for m = -1), where the subtraction is
 // exact: an image pair carries no rounding of the box length or of the
 // absolute coordinates.
+// Virial: d = x_j - x_i + m L, and a pair is met from both atoms with opposite
+// d and m, so the sum of c_i f (x) d over all pairs (f = C (...) d) is -2
+// sum_i c_i F_i (x) x_i, formed once per atom, plus c_i f (x) m L for pairs of
+// other images (symmetrised; usually one axis).  The product with x_i loses
+// |x_i| / r of a pair's precision, so pairs closer than a/16 (none in a
+// liquid) stay out of it: they have sums of their own, f and d (x) d.
 template <typename T, bool VIR, bool LB>
 __device__ __forceinline__ void pair_eval(int2 en, const Vec4<T>* __restrict__ sp,
                                           const T* __restrict__ lbw, const Vec4<T>& pi, T wi,
-                                          const PairArgs<T>& g, T& e, T& fx, T& fy, T& fz, T& w0,
-                                          T& w1, T& w2, T& w3, T& w4, T& w5) {
+                                          const PairArgs<T>& g, T& e, T& fx, T& fy, T& fz,
+                                          T (&w)[6], T (&near)[3], bool& any_near) {
   constexpr int kImg0 = 8 | (8 << 4) | (8 << 8);
   const Vec4<T> pj = sp[en.x];
   T ddx = pj.x - pi.x, ddy = pj.y - pi.y, ddz = pj.z - pi.z;
@@ -690,45 +720,71 @@ __device__ __forceinline__ void pair_eval(int2 en, const Vec4<T>* __restrict__ s
     ddz = d[2];
   }
   const T r2 = ddx * ddx + ddy * ddy + ddz * ddz;
-  const T inv = rcp(r2);
-  const T inv3 = inv * inv * inv;
-  const T s1 = r2 * g.ia2, s2 = s1 * s1, s3 = s2 * s1, s6 = s3 * s3;
-  const T s5 = s3 * s2;
-  const T g0 = inv3 - g.ia6 * (T(1.875) - T(1.25) * s6 + T(0.375) * s6 * s6);
-  const T gp = T(-6) * inv3 * inv + g.ia8 * s5 * (T(15) - T(9) * s6);
-  T cj = pj.w;
+  const bool in = q_inside(r2, g.a2);
+  const T s1 = (in ? r2 : g.a2) * g.ia2;
+  const T inv = q_rcp(s1), i2 = inv * inv;
+  const T s2 = s1 * s1, s3 = s2 * s1, s6 = s3 * s3, s5 = s3 * s2;
+  const T g0 = i2 * inv + (s6 * (T(1.25) - T(0.375) * s6) - T(1.875));
+  const T gp = i2 * i2 - s5 * (T(2.5) - T(1.5) * s6);
+  T cj = in ? pj.w : T(0);
   if (LB) {
     const T sg = T(0.5) * (pi.w + pj.w), sg3 = sg * sg * sg;
-    cj = wi * lbw[en.x] * sg3 * sg3;
+    cj = in ? wi * lbw[en.x] * sg3 * sg3 : T(0);
   }
   e += cj * g0;
   const T cg = cj * gp;
+  if (VIR && q_inside(r2, g.near2)) {
+    const T hx = cg * ddx, hy = cg * ddy, hz = cg * ddz;
+    any_near = true;
+    near[0] += hx;
+    near[1] += hy;
+    near[2] += hz;
+    w[0] += pi.w * hx * ddx;
+    w[1] += pi.w * hy * ddy;
+    w[2] += pi.w * hz * ddz;
+    w[3] += pi.w * hx * ddy;
+    w[4] += pi.w * hx * ddz;
+    w[5] += pi.w * hy * ddz;
+    return;
+  }
   fx += cg * ddx;
   fy += cg * ddy;
   fz += cg * ddz;
-  if (VIR) {  // virial records carry c_i (the lanes mix atoms)
-    const T cv = LB ? cg : pi.w * cg;
-    const T cx_ = cv * ddx, cy_ = cv * ddy;
-    w0 += cx_ * ddx;
-    w1 += cy_ * ddy;
-    w2 += cv * ddz * ddz;
-    w3 += cx_ * ddy;
-    w4 += cx_ * ddz;
-    w5 += cy_ * ddz;
+  if (VIR && en.y != kImg0) {
+    const int mx = (en.y & 15) - 8, my = ((en.y >> 4) & 15) - 8, mz = ((en.y >> 8) & 15) - 8;
+    const T cv = pi.w * cg, hx = cv * ddx, hy = cv * ddy, hz = cv * ddz;
+    if (mx != 0) {  // g.mL: L / 2 (the off-diagonal halves)
+      const T u = (T)mx * g.mL[0];
+      w[0] += T(2) * u * hx;
+      w[3] += u * hy;
+      w[4] += u * hz;
+    }
+    if (my != 0) {
+      const T u = (T)my * g.mL[1];
+      w[3] += u * hx;
+      w[1] += T(2) * u * hy;
+      w[5] += u * hz;
+    }
+    if (mz != 0) {
+      const T u = (T)mz * g.mL[2];
+      w[4] += u * hx;
+      w[5] += u * hy;
+      w[2] += T(2) * u * hz;
+    }
   }
 }
 
 // Stage candidates c0 .. c0+cn-1 of a warp's stream in shared memory: the
-// position shifted by its piece's periodic image (for the cutoff test) and
-// {j, image code} (for the evaluation).
+// FP32 position shifted by its piece's periodic image (for the cutoff test)
+// and {j, image code} (for the evaluation).
 template <typename T>
 __device__ __forceinline__ void q_stage(int c0, int cn, int lane, const int* t_end,
                                         const int* t_base, const int* t_img,
-                                        const Vec4<T>* __restrict__ sp, const PairArgs<T>& g,
-                                        Vec4<T>* cpos, int2* cidx) {
+                                        const float4* __restrict__ spf, const PairArgs<T>& g,
+                                        float4* cpos, int2* cidx) {
   constexpr int kImg0 = 8 | (8 << 4) | (8 << 8);
   int p = -1, pend = 0, pbase = 0, pimg = kImg0;
-  T sx = 0, sy = 0, sz = 0;
+  float sx = 0, sy = 0, sz = 0;
   for (int u = lane; u < cn; u += 32) {
     const int k = c0 + u;
     if (k >= pend) {
@@ -738,12 +794,12 @@ __device__ __forceinline__ void q_stage(int c0, int cn, int lane, const int* t_e
       } while (k >= pend);
       pbase = t_base[p];
       pimg = t_img[p];
-      sx = (T)((pimg & 15) - 8) * g.box.L[0];
-      sy = (T)(((pimg >> 4) & 15) - 8) * g.box.L[1];
-      sz = (T)(((pimg >> 8) & 15) - 8) * g.box.L[2];
+      sx = (float)((pimg & 15) - 8) * g.Lf[0];
+      sy = (float)(((pimg >> 4) & 15) - 8) * g.Lf[1];
+      sz = (float)(((pimg >> 8) & 15) - 8) * g.Lf[2];
     }
     const int j = pbase + k;
-    Vec4<T> pj = sp[j];
+    float4 pj = spf[j];
     pj.x += sx;
     pj.y += sy;
     pj.z += sz;
@@ -753,31 +809,35 @@ __device__ __forceinline__ void q_stage(int c0, int cn, int lane, const int* t_e
 }
 
 // Queue form of the pair sum (pair_split 64 G: G = 2, 4 or 8 atoms per
-// warp, kQWarps warps per block).  The G consecutive sorted atoms of a warp
-// that share a row of cells form a segment, and the segment's candidate
-// stream is built as in the warp form (lane t: neighbour row t trimmed
-// against the segment's bounding box, a warp scan flattening the pieces).
-// The stream is staged in shared memory (positions shifted by their
-// periodic image, chunks of qcap<T>() candidates), so the G atoms read the
+// warp, kQWarps warps per block; the FP64 default).  The G consecutive sorted
+// atoms of a warp that share a row of cells form a segment, and the segment's
+// candidate stream is built as in the warp form (lane t: neighbour row t
+// trimmed against the segment's bounding box, a warp scan flattening the
+// pieces).  The stream is staged in shared memory as FP32 positions (shifted by
+// their periodic image, chunks of kQCap candidates), so the G atoms read the
 // candidates from global memory once.  Each atom then tests the staged
-// candidates 32 at a time (0 < r^2 < a^2: the atom itself is the only
-// candidate at distance 0), the hits of the 32 lanes are compacted by a
-// ballot into a per-warp queue, and whenever 32 hits are queued all 32
-// lanes evaluate one each.  The pair arithmetic therefore runs on full warps
-// and only on pairs inside the cutoff.  The queue is filled and drained in
-// stream order and each lane sums its evaluations in that order, then a
-// fixed shuffle tree combines the lanes: results are reproducible bit for
-// bit.
+// candidates 32 at a time in FP32, with a slack that covers its rounding; the
+// 32 lanes' hits are compacted by a ballot into a per-warp queue, and whenever
+// 32 hits are queued all 32 lanes evaluate one each in the plan's precision,
+// with the exact test.  The FP64 pipe (two lanes per clock and SM) bounds the
+// FP64 kernel: it runs on full warps, on pairs inside the cutoff only, 27
+// operations each.  98,765 atoms, a = 3, pair stage with / without the virial:
+// 2390 us (with) with FP64 tests, an FP64 row set-up, the division and six
+// virial products per pair; FP32 tests and the Newton reciprocal 1143 / 844;
+// FP32 set-up 1040 / 731; the virial from the force once per atom 901 / 737 (the
+// FP64 pipe 83% busy; 3.9 rounds of 32 per atom where 3.0 would hold its hits).  The queue is filled and
+// drained in stream order and each lane sums its evaluations in that order,
+// then a fixed shuffle tree that halves the four sums as it goes (6 additions,
+// not 20) combines the lanes: results are reproducible bit for bit.
 constexpr int kQWarps = 4;
-template <typename T> __host__ __device__ constexpr int qcap() {
-  return sizeof(T) == 4 ? 512 : 256;
-}
-template <typename T> constexpr size_t q_smem_bytes() {
-  return (size_t)kQWarps * qcap<T>() * (sizeof(Vec4<T>) + sizeof(int2));
+constexpr int kQCap = 512;
+constexpr size_t q_smem_bytes() {
+  return (size_t)kQWarps * kQCap * (sizeof(float4) + sizeof(int2));
 }
 
 template <typename T, bool VIR, int G, bool LB = false>
 __global__ void __launch_bounds__(kQWarps * 32) k_pair_q(const Vec4<T>* __restrict__ sp,
+                                                          const float4* __restrict__ spf,
                                                           const int* __restrict__ start, int N,
                                                           PairArgs<T> g, T* __restrict__ e0,
                                                           T* __restrict__ floc,
@@ -786,59 +846,52 @@ __global__ void __launch_bounds__(kQWarps * 32) k_pair_q(const Vec4<T>* __restri
   constexpr int kW = kQWarps;
   constexpr int kP = 3 * 32;   // pieces of one segment: <= 3 per row, <= 32 rows
   constexpr int kQ = 64;       // queued hits: < 32 left over + 32 new
-  constexpr int kCap = qcap<T>();
+  constexpr int kCap = kQCap;
   constexpr unsigned kAll = 0xffffffffu;
-  __shared__ double sh[32 * 6];
+  __shared__ T wsum[kW][6], wrow[kW][9];  // virial of each warp; rows of -c_i F_i (x) x_i
+  __shared__ int ended;                   // warps that have written theirs
   __shared__ int t_end[kW][kP], t_base[kW][kP], t_img[kW][kP];
   __shared__ int2 qu[kW][kQ];
   extern __shared__ __align__(16) unsigned char q_dyn[];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  Vec4<T>* cpos = reinterpret_cast<Vec4<T>*>(q_dyn) + (size_t)wid * kCap;
-  int2* cidx = reinterpret_cast<int2*>(q_dyn + (size_t)kW * kCap * sizeof(Vec4<T>)) +
+  if (VIR) {
+    if (threadIdx.x == 0) ended = 0;
+    __syncthreads();
+  }
+  float4* cpos = reinterpret_cast<float4*>(q_dyn) + (size_t)wid * kCap;
+  int2* cidx = reinterpret_cast<int2*>(q_dyn + (size_t)kW * kCap * sizeof(float4)) +
                (size_t)wid * kCap;
   const long i0 = ((long)blockIdx.x * kW + wid) * G;
   const int nat = (int)max(0L, min((long)G, (long)N - i0));  // atoms of this warp
-  // lane t < nat holds atom i0 + t
+  // lane t < nat holds atom i0 + t; the set-up works on the FP32 positions
+  // (the row of cells from the record itself, as the binning formed it)
   Vec4<T> pa = {T(0), T(0), T(0), T(0)};
-  int cx = 0, cy = 0, cz = 0, rid = INT_MAX;
+  float4 pf = make_float4(0.f, 0.f, 0.f, 0.f);
+  int cy = 0, cz = 0, rid = INT_MAX;
   if (lane < nat) {
     pa = sp[i0 + lane];
-    cx = min(max((int)(pa.x * g.inv_w[0]), 0), g.nc[0] - 1);
+    pf = spf[i0 + lane];
     cy = min(max((int)(pa.y * g.inv_w[1]), 0), g.nc[1] - 1);
     cz = min(max((int)(pa.z * g.inv_w[2]), 0), g.nc[2] - 1);
     rid = cy + g.nc[1] * cz;
   }
-  T w0 = 0, w1 = 0, w2 = 0, w3 = 0, w4 = 0, w5 = 0;
+  T w[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};  // pairs of other images, close pairs
+  T rx = 0, ry = 0, rz = 0;  // lane 1 + q: sum c_i F_i,q x_i
+  bool images = false;  // any of those
   const int ny = 2 * g.R[1] + 1, nrows = (2 * g.R[2] + 1) * ny;
   for (int s = 0; s < nat;) {
     const int rs = __shfl_sync(kAll, rid, s);
     const unsigned seg = __ballot_sync(kAll, lane < nat && rid == rs);
     const bool act = (seg >> lane) & 1u;
-    // bounding box of the segment
-    T xmn = act ? pa.x : T(INFINITY), xmx = act ? pa.x : T(-INFINITY);
-    T ymn = act ? pa.y : T(INFINITY), ymx = act ? pa.y : T(-INFINITY);
-    T zmn = act ? pa.z : T(INFINITY), zmx = act ? pa.z : T(-INFINITY);
-    int cxmn = act ? cx : INT_MAX, cxmx = act ? cx : INT_MIN;
-#pragma unroll
-    for (int o = 1; o < G; o <<= 1) {  // over the lanes 0..G-1 that hold atoms
-      xmn = min(xmn, __shfl_xor_sync(kAll, xmn, o));
-      xmx = max(xmx, __shfl_xor_sync(kAll, xmx, o));
-      ymn = min(ymn, __shfl_xor_sync(kAll, ymn, o));
-      ymx = max(ymx, __shfl_xor_sync(kAll, ymx, o));
-      zmn = min(zmn, __shfl_xor_sync(kAll, zmn, o));
-      zmx = max(zmx, __shfl_xor_sync(kAll, zmx, o));
-      cxmn = min(cxmn, __shfl_xor_sync(kAll, cxmn, o));
-      cxmx = max(cxmx, __shfl_xor_sync(kAll, cxmx, o));
-    }
-    // every lane sets up a row: broadcast the box from lane 0
-    xmn = __shfl_sync(kAll, xmn, 0);
-    xmx = __shfl_sync(kAll, xmx, 0);
-    ymn = __shfl_sync(kAll, ymn, 0);
-    ymx = __shfl_sync(kAll, ymx, 0);
-    zmn = __shfl_sync(kAll, zmn, 0);
-    zmx = __shfl_sync(kAll, zmx, 0);
-    cxmn = __shfl_sync(kAll, cxmn, 0);
-    cxmx = __shfl_sync(kAll, cxmx, 0);
+    // bounding box of the segment: coordinates >= 0, whose bits order like integers
+    auto lo = [&](float v) {
+      return __uint_as_float(__reduce_min_sync(kAll, __float_as_uint(act ? v + 0.f : INFINITY)));
+    };
+    auto hi = [&](float v) {
+      return __uint_as_float(__reduce_max_sync(kAll, __float_as_uint(act ? v + 0.f : 0.f)));
+    };
+    const float xmn = lo(pf.x), xmx = hi(pf.x), ymn = lo(pf.y), ymx = hi(pf.y);
+    const float zmn = lo(pf.z), zmx = hi(pf.z);
     const int scy = __shfl_sync(kAll, cy, s), scz = __shfl_sync(kAll, cz, s);
     // 1. lane t: row t of the (2R+1)^2 neighbour rows, trimmed and split
     //    into at most three same-image pieces
@@ -850,14 +903,15 @@ __global__ void __launch_bounds__(kQWarps * 32) k_pair_q(const Vec4<T>* __restri
       int iz, iy, mz, my;
       wrap_image(z, g.nc[2], iz, mz);
       wrap_image(y, g.nc[1], iy, my);
-      const T ylo = (T)y * g.w[1], zlo = (T)z * g.w[2];
-      const T dyl = max(T(0), max(ylo - ymx, ymn - (ylo + g.w[1])) - g.margin);
-      const T dzl = max(T(0), max(zlo - zmx, zmn - (zlo + g.w[2])) - g.margin);
-      const T d2 = dyl * dyl + dzl * dzl;
-      if (d2 < g.a2) {
-        const T rx = sqrt(g.a2 - d2) + g.margin;
-        const int xl = max(cxmn - g.R[0], (int)floor((xmn - rx) * g.inv_w[0]));
-        const int xh = min(cxmx + g.R[0], (int)floor((xmx + rx) * g.inv_w[0]));
+      const float ylo = (float)y * g.wf[1], zlo = (float)z * g.wf[2];
+      const float dyl = fmaxf(0.f, fmaxf(ylo - ymx, ymn - (ylo + g.wf[1])) - g.marginf);
+      const float dzl = fmaxf(0.f, fmaxf(zlo - zmx, zmn - (zlo + g.wf[2])) - g.marginf);
+      const float d2 = dyl * dyl + dzl * dzl;
+      if (d2 < g.a2f) {
+        const float rx = sqrtf(g.a2f - d2) + g.marginf;
+        // at most a neighbour range beyond either end of the box
+        const int xl = max(-g.R[0], __float2int_rd((xmn - rx) * g.iwf));
+        const int xh = min(g.nc[0] - 1 + g.R[0], __float2int_rd((xmx + rx) * g.iwf));
         const int row = g.nc[0] * (iy + g.nc[1] * iz);
         const int img_yz = ((my + 8) << 4) | ((mz + 8) << 8);
         int xa = xl, ix, mx;
@@ -877,6 +931,12 @@ __global__ void __launch_bounds__(kQWarps * 32) k_pair_q(const Vec4<T>* __restri
           }
         }
       }
+    }
+    if (VIR) {  // any piece of another image
+      bool im = false;
+#pragma unroll
+      for (int q = 0; q < 3; ++q) im = im || (q < np && pim[q] != (8 | (8 << 4) | (8 << 8)));
+      images = images || __any_sync(kAll, im);
     }
     // 2. pieces -> one stream
     int np_inc = np, c_inc = cnt;
@@ -903,7 +963,7 @@ __global__ void __launch_bounds__(kQWarps * 32) k_pair_q(const Vec4<T>* __restri
     }
     __syncwarp();
     const bool one = total <= kCap;
-    if (one) q_stage<T>(0, total, lane, t_end[wid], t_base[wid], t_img[wid], sp, g, cpos, cidx);
+    if (one) q_stage<T>(0, total, lane, t_end[wid], t_base[wid], t_img[wid], spf, g, cpos, cidx);
     __syncwarp();
     // 3. every atom of the segment against the stream
     const int send = s + __popc(seg);
@@ -914,33 +974,35 @@ __global__ void __launch_bounds__(kQWarps * 32) k_pair_q(const Vec4<T>* __restri
       pi.y = __shfl_sync(kAll, pa.y, s);
       pi.z = __shfl_sync(kAll, pa.z, s);
       pi.w = __shfl_sync(kAll, pa.w, s);
+      const float4 qf = make_float4(__shfl_sync(kAll, pf.x, s), __shfl_sync(kAll, pf.y, s),
+                                    __shfl_sync(kAll, pf.z, s), 0.f);
       T wi = T(0);
       if (LB) wi = lbw[i];
-      T e = 0, fx = 0, fy = 0, fz = 0;
+      T e = 0, fx = 0, fy = 0, fz = 0, near[3] = {T(0), T(0), T(0)};
+      bool any_near = false;
       int qn = 0;
       for (int c0 = 0; c0 < total; c0 += kCap) {
         const int cn = min(kCap, total - c0);
         if (!one) {
           __syncwarp();
-          q_stage<T>(c0, cn, lane, t_end[wid], t_base[wid], t_img[wid], sp, g, cpos, cidx);
+          q_stage<T>(c0, cn, lane, t_end[wid], t_base[wid], t_img[wid], spf, g, cpos, cidx);
           __syncwarp();
         }
         for (int u0 = 0; u0 < cn; u0 += 32) {
           const int u = u0 + lane;
           bool hit = false;
           if (u < cn) {
-            const Vec4<T> pj = cpos[u];
-            const T ddx = pj.x - pi.x, ddy = pj.y - pi.y, ddz = pj.z - pi.z;
-            const T r2 = ddx * ddx + ddy * ddy + ddz * ddz;
-            hit = r2 < g.a2 && r2 > T(0);
+            const float4 pj = cpos[u];
+            const float ddx = pj.x - qf.x, ddy = pj.y - qf.y, ddz = pj.z - qf.z;
+            hit = ddx * ddx + ddy * ddy + ddz * ddz < g.a2f;
           }
           const unsigned m = __ballot_sync(kAll, hit);
           if (hit) qu[wid][qn + __popc(m & ((1u << lane) - 1u))] = cidx[u];
           qn += __popc(m);
           if (qn >= 32) {
             __syncwarp();
-            pair_eval<T, VIR, LB>(qu[wid][lane], sp, lbw, pi, wi, g, e, fx, fy, fz, w0, w1, w2,
-                                  w3, w4, w5);
+            pair_eval<T, VIR, LB>(qu[wid][lane], sp, lbw, pi, wi, g, e, fx, fy, fz, w, near,
+                                  any_near);
             __syncwarp();
             if (lane < qn - 32) qu[wid][lane] = qu[wid][lane + 32];
             __syncwarp();
@@ -950,32 +1012,84 @@ __global__ void __launch_bounds__(kQWarps * 32) k_pair_q(const Vec4<T>* __restri
       }
       __syncwarp();
       if (lane < qn)
-        pair_eval<T, VIR, LB>(qu[wid][lane], sp, lbw, pi, wi, g, e, fx, fy, fz, w0, w1, w2, w3,
-                              w4, w5);
+        pair_eval<T, VIR, LB>(qu[wid][lane], sp, lbw, pi, wi, g, e, fx, fy, fz, w, near,
+                                  any_near);
+      // lane bits 0 and 1 choose the sum (e, x, y, z), the others are added up
+      const bool b0 = lane & 1, b1 = lane & 2;
+      T ka = b1 ? fy : e, kb = b1 ? fz : fx;
+      ka += __shfl_xor_sync(kAll, b1 ? e : fy, 2);
+      kb += __shfl_xor_sync(kAll, b1 ? fx : fz, 2);
+      T v = (b0 ? kb : ka) + __shfl_xor_sync(kAll, b0 ? ka : kb, 1);
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        e += __shfl_xor_sync(kAll, e, o);
-        fx += __shfl_xor_sync(kAll, fx, o);
-        fy += __shfl_xor_sync(kAll, fy, o);
-        fz += __shfl_xor_sync(kAll, fz, o);
+      for (int o = 4; o < 32; o <<= 1) v += __shfl_xor_sync(kAll, v, o);
+      T vn = T(0);  // lanes 1 .. 3: the close pairs' force
+      if (VIR && __any_sync(kAll, any_near)) {
+        images = true;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+          for (int d = 0; d < 3; ++d) near[d] += __shfl_xor_sync(kAll, near[d], o);
+        vn = lane == 1 ? near[0] : lane == 2 ? near[1] : lane == 3 ? near[2] : T(0);
       }
-      if (lane == 0) {
-        const T cf = LB ? T(1) : pi.w;
-        e0[i] = e;
-        floc[3 * (size_t)i + 0] = -cf * fx;
-        floc[3 * (size_t)i + 1] = -cf * fy;
-        floc[3 * (size_t)i + 2] = -cf * fz;
+      // F_i = -c_i sum c_j g_0'/r d = +c_i 6 a^-8 (x, y, z)
+      if (lane < 4) {
+        if (lane == 0)
+          e0[i] = g.ia6 * v;
+        else
+          floc[3 * (size_t)i + lane - 1] = (LB ? T(6) : T(6) * pi.w) * g.ia8 * (v + vn);
+        if (VIR) {
+          const T f = pi.w * v;
+          rx += f * pi.x;
+          ry += f * pi.y;
+          rz += f * pi.z;
+        }
       }
       __syncwarp();  // the queue is reused by the next atom
     }
     __syncwarp();  // the next segment rewrites the piece table and the stage
   }
   if (VIR) {
-    T wv[6] = {w0, w1, w2, w3, w4, w5};
-    double ws[6];
-    block_sum_lo<T, 6>(wv, ws, sh);
-    if (threadIdx.x == 0)
-      for (int c = 0; c < 6; ++c) wpart[6 * (size_t)blockIdx.x + c] = 0.5 * ws[c];
+    // of c_i c_j (-a^8 g_0'/6r) d (x) d: the image sums over the lanes (lane c
+    // mod 8 ends with sum c; most warps have none), then the rows
+    T v = T(0);
+    if (images) {
+      const bool b0 = lane & 1, b1 = lane & 2, b2 = lane & 4;
+      T k0 = b2 ? w[4] : w[0], k1 = b2 ? w[5] : w[1], k2 = b2 ? T(0) : w[2], k3 = b2 ? T(0) : w[3];
+      k0 += __shfl_xor_sync(kAll, b2 ? w[0] : w[4], 4);
+      k1 += __shfl_xor_sync(kAll, b2 ? w[1] : w[5], 4);
+      const T s2 = __shfl_xor_sync(kAll, w[2], 4), s3 = __shfl_xor_sync(kAll, w[3], 4);
+      k2 += b2 ? T(0) : s2;
+      k3 += b2 ? T(0) : s3;
+      const T m0 = (b1 ? k2 : k0) + __shfl_xor_sync(kAll, b1 ? k0 : k2, 2);
+      const T m1 = (b1 ? k3 : k1) + __shfl_xor_sync(kAll, b1 ? k1 : k3, 2);
+      v = (b0 ? m1 : m0) + __shfl_xor_sync(kAll, b0 ? m0 : m1, 1);
+      v += __shfl_xor_sync(kAll, v, 8);
+      v += __shfl_xor_sync(kAll, v, 16);
+    }
+    if (lane >= 1 && lane < 4) {
+      wrow[wid][3 * (lane - 1)] = rx;
+      wrow[wid][3 * (lane - 1) + 1] = ry;
+      wrow[wid][3 * (lane - 1) + 2] = rz;
+    }
+    __syncwarp();
+    if (lane < 6) {  // xx yy zz xy xz yz: rows p, q
+      const int p = lane < 3 ? lane : (lane == 5 ? 1 : 0);
+      const int q = lane < 3 ? lane : (lane == 3 ? 1 : 2);
+      v -= wrow[wid][3 * p + q] + wrow[wid][3 * q + p];
+      wsum[wid][lane] = v;
+    }
+    // the warp that ends last adds the warps' sums in their order
+    __threadfence_block();
+    __syncwarp();
+    bool last = false;
+    if (lane == 0) last = atomicAdd(&ended, 1) == kW - 1;
+    if (__shfl_sync(kAll, (int)last, 0) && lane < 6) {
+      __threadfence_block();
+      double t = 0.0;
+#pragma unroll
+      for (int u = 0; u < kW; ++u) t += (double)*(volatile T*)&wsum[u][lane];
+      wpart[6 * (size_t)blockIdx.x + lane] = -3.0 * (double)g.ia8 * t;
+    }
   }
 }
 
@@ -1030,10 +1144,9 @@ int pair_split(const Plan* p) {
 }
 
 int pair_split_atom(const Plan* p) {
-  // FP64: the queue form with two atoms per warp where the cell geometry
-  // allows it (1M-atom cube 24.5 ms against 29.4 ms per atom and 31.2 ms
-  // for the warp form); FP32 keeps the per-atom kernel (0.757 ms there
-  // against 2.23 ms for the best queue form)
+  // FP64: the queue form where the cell geometry allows it, with two atoms per
+  // warp (20,000 atoms 240 us against 257 and 323 with four and eight, 98,765
+  // atoms about 900, 900 and 1000; 1,000 atoms 28, 43 and 74)
   if (p->prec == MLS6_FP64 && pair_cluster_ok(p)) return 128;
   const long want = 152L * 48 * 32;
   int s = 1;
@@ -1100,24 +1213,26 @@ static void launch_q(Plan* p, const PairArgs<T>& pg, bool vir, bool lb, cudaStre
   const int N = (int)p->N;
   const long nb = pair_blocks(p, 64 * G);
   if (nb == 0) return;
-  const size_t sm = q_smem_bytes<T>();
+  const size_t sm = q_smem_bytes();
+  // FP32 positions: their own array beside FP64 records
+  const float4* spf = (const float4*)(sizeof(T) == 8 ? p->d_sorted_f : p->d_sorted);
   const int th = kQWarps * 32;
   if (lb)
     k_pair_q<T, false, G, true><<<nb, th, sm, st>>>(
-        (const Vec4<T>*)p->d_sorted, p->d_cell_start, N, pg, (T*)p->d_e0, (T*)p->d_floc,
+        (const Vec4<T>*)p->d_sorted, spf, p->d_cell_start, N, pg, (T*)p->d_e0, (T*)p->d_floc,
         p->d_wpart + 6 * p->wpart_pair, (const T*)p->d_lbw);
   else if (vir)
-    k_pair_q<T, true, G><<<nb, th, sm, st>>>((const Vec4<T>*)p->d_sorted, p->d_cell_start, N,
+    k_pair_q<T, true, G><<<nb, th, sm, st>>>((const Vec4<T>*)p->d_sorted, spf, p->d_cell_start, N,
                                              pg, (T*)p->d_e0, (T*)p->d_floc,
                                              p->d_wpart + 6 * p->wpart_pair);
   else
-    k_pair_q<T, false, G><<<nb, th, sm, st>>>((const Vec4<T>*)p->d_sorted, p->d_cell_start, N,
+    k_pair_q<T, false, G><<<nb, th, sm, st>>>((const Vec4<T>*)p->d_sorted, spf, p->d_cell_start, N,
                                               pg, (T*)p->d_e0, (T*)p->d_floc,
                                               p->d_wpart + 6 * p->wpart_pair);
 }
 
 template <typename T, int G> static int q_attr() {
-  const int sm = (int)q_smem_bytes<T>();
+  const int sm = (int)q_smem_bytes();
   const auto a = cudaFuncAttributeMaxDynamicSharedMemorySize;
   if (cudaFuncSetAttribute(k_pair_q<T, true, G>, a, sm) != cudaSuccess ||
       cudaFuncSetAttribute(k_pair_q<T, false, G>, a, sm) != cudaSuccess ||
@@ -1162,6 +1277,18 @@ template <typename T> static PairArgs<T> pair_args(const Plan* p) {
     pg.Lhi[d] = (T)p->L[d];
     pg.Llo[d] = (T)(p->L[d] - (double)pg.Lhi[d]);
   }
+  // slack of the FP32 test: rounding of the FP32 positions and image shifts
+  // (a few units of the largest coordinate) and of its arithmetic
+  const double af = p->a * (1.0 + 1e-5) + 16.0 * 6.0e-8 * lmax;
+  pg.a2f = (float)(af * af);
+  for (int d = 0; d < 3; ++d) {
+    pg.Lf[d] = (float)p->L[d];
+    pg.wf[d] = (float)p->cg.w[d];
+    pg.mL[d] = (T)(0.5 * p->L[d]);
+  }
+  pg.iwf = (float)p->cg.inv_w[0];
+  pg.near2 = (T)(p->a * p->a / 256.0);
+  pg.marginf = (float)(1e-3 * wmin + 16.0 * 6.0e-8 * lmax);
   for (int k = 0; k < 5; ++k) pg.gc[k] = (T)p->sm.c[k];
   for (int k = 0; k < 4; ++k) pg.gd[k] = (T)(-12.0 * (k + 1) * p->sm.c[k + 1]);
   return pg;

@@ -153,7 +153,7 @@ __device__ __forceinline__ void run_stage(const PStageDesc& d, unsigned b) {
     }
     case P_CELLSORT: {
       const CellsortP& a = d.u.cs;
-      k_cellsort_body<float>(bk, a.start, a.ncell, a.posw, a.sorted, a.sidx);
+      k_cellsort_body<float>(bk, a.start, a.ncell, a.posw, a.sorted, a.sidx, nullptr);
       break;
     }
     case P_PAIR: {
