@@ -402,9 +402,6 @@ int mls6_batch_plan(mls6_batch_t** out, int B, const double* boxes, const int64_
     rc = mls6_plan(&p, boxes + 3 * r, N[r], a, h, levels, order, precision);
     if (rc) break;
     b->plans[r] = reinterpret_cast<Plan*>(p);
-    // replicas keep the per-atom pair forms (the persistent kernel runs
-    // those; the cluster form is for single large systems)
-    b->plans[r]->pair_split = pair_split_atom(b->plans[r]);
     rc = plan_streams(b->plans[r]);
     b->off[r + 1] = b->off[r] + N[r];
     double hh = b->plans[r]->lv[1].h[0];
@@ -436,12 +433,13 @@ int mls6_batch_plan(mls6_batch_t** out, int B, const double* boxes, const int64_
     free_batch(b);
     return rc;
   }
-  // seed: branches from the model (enough chains that the largest replica
-  // bounds the makespan), shapes from each plan's own heuristics
-  const double total = std::accumulate(b->cost.begin(), b->cost.end(), 0.0);
-  const double big = *std::max_element(b->cost.begin(), b->cost.end());
-  int K = (int)std::ceil(total / std::max(big, 1e-12));
-  b->branches = std::max(1, std::min(std::min(K, 32), B));
+  // seed: a chain per replica, up to 48; shapes from each plan's own
+  // heuristics.  A replica alone is a chain of latencies, so every further
+  // chain fills idle SMs until the device is full (whole batch: 12 replicas of
+  // 2k-65k atoms 447 us with 4 chains, 342 with 8; 40 replicas 903 with 16, 849
+  // with 40; 48 of 2k-8k atoms 556 with 13, 436 with 48; 200 replicas 3690-3650
+  // with 24 to 64, 3740 with 128).
+  b->branches = std::min(B, 48);
   assign(b);
   *out = reinterpret_cast<mls6_batch_t*>(b);
   return MLS6_OK;
@@ -512,10 +510,11 @@ static int tune_form(Batch* b, const void* pos, const void* c, void* forces, int
     s.resize(b->B);
     g.resize(b->B);
     for (int r = 0; r < b->B; ++r) {
+      const int def = pair_split(b->plans[r]);
       int x = sb >= 0 ? s0[r] << sb : s0[r] >> -sb;
       // the persistent kernel runs the per-atom pair kernel (1..8 lanes)
       const int smax = (b->mode == 1 || !pair_cluster_ok(b->plans[r])) ? 8 : kPairSplitMax;
-      s[r] = std::max(1, std::min(smax, x));
+      s[r] = sb == 0 && b->mode == 0 && def == kPairTile ? def : std::max(1, std::min(smax, x));
       int y = gb >= 0 ? g0[r] << gb : g0[r] >> -gb;
       g[r] = std::max(1, std::min(4, y));
     }
@@ -637,6 +636,12 @@ int mls6_batch_set_mode(mls6_batch_t* batch, int persistent) {
   if (b->s0 && cudaStreamSynchronize(b->s0) != cudaSuccess) return MLS6_ERR_CUDA;
   b->mode = persistent;
   reset_graph(b);
+  if (persistent)  // the persistent kernel runs the per-atom pair form
+    for (Plan* p : b->plans)
+      if (p->pair_split == kPairTile) {
+        const int rc = mls6_set_tuning(reinterpret_cast<mls6_plan_t*>(p), pair_split_atom(p), 0);
+        if (rc) return rc;
+      }
   return MLS6_OK;
 }
 

@@ -123,3 +123,33 @@ def test_tile_form_default_and_refusals(gpu_lib):
         plan = gpu_lib.Plan(kw["box"], 8192, 3.0, 1.5, 0, precision=kw["precision"])
         with pytest.raises(gpu_lib.MLS6Error):
             gpu_lib.mls6_set_tuning(plan.handle, TILE, 0)
+
+
+def test_tile_form_in_a_batch(gpu_lib):
+    """Replicas take their plan's default form in the kernel chains (bit for
+    bit the single plan's results); the persistent kernel takes the lanes per
+    atom, and stays available."""
+    import torch
+
+    Ns = [8300, 2500]
+    boxes = [(I.cube_side(n, 0.85),) * 3 for n in Ns]
+    parts = [I.uniform_atoms(90 + n, n, b) for n, b in zip(Ns, boxes)]
+    pos = torch.tensor(np.concatenate([np.c_[x, c] for x, c in parts]), dtype=torch.float32,
+                       device="cuda")
+    bt = gpu_lib.Batch(boxes, Ns, 2.5, 1.0, precision="fp32")
+    assert bt.info()["pair_split"][0] == TILE and bt.info()["pair_split"][1] <= 8
+    for persistent in (False, True):
+        gpu_lib.mls6_batch_set_mode(bt.handle, persistent)
+        r = bt.evaluate(pos)
+        torch.cuda.synchronize()
+        info = bt.info()
+        assert gpu_lib.mls6_batch_mode(bt.handle) == int(persistent)
+        assert (info["pair_split"][0] == TILE) != persistent
+        for k in range(2):
+            p = gpu_lib.Plan(boxes[k], Ns[k], 2.5, 1.0, 0, precision="fp32")
+            gpu_lib.mls6_set_tuning(p.handle, info["pair_split"][k], info["stencil_groups"][k])
+            sl = slice(bt.offsets[k], bt.offsets[k + 1])
+            one = p.evaluate(pos[sl].contiguous())
+            torch.cuda.synchronize()
+            assert torch.equal(one["F"], r["F"][sl])
+            assert one["out"][0] == r["E"][k] and torch.equal(one["out"][1:], r["W"][k])
