@@ -13,16 +13,13 @@
 //              (mma.m16n8k16, FP32 accumulation); one warp per 16 atoms, the
 //              accumulator tiles of a layer are repacked in registers as the
 //              A operand of the next
-//   training   BF16 tensor-core backward pass: activation gradients
-//              dZ = (dZ_next W^T) (1 - h^2) per 16-atom warp tile with the
-//              transposed weights as B fragments (mma.m16n8k16, FP32
-//              accumulation, dZ kept as BF16); weight gradients X^T dZ1,
-//              H^T dZ per block of atoms from shared-memory tiles read as
-//              transposed fragments (ldmatrix .trans), bias gradients as
-//              products with a ones operand; per-block partials summed in a
-//              fixed order (results reproducible bit for bit); Adam update of
-//              FP32 master weights, BF16 fragments repacked after every step
+//   training   one kernel per batch: forward, BF16 tensor-core backward pass
+//              and weight gradients of a tile of atoms held in shared memory
+//              (k_mlp_train); per-block partials summed in a fixed order
+//              (results reproducible bit for bit); Adam update of FP32 master
+//              weights, BF16 fragments repacked after every step
 #include <cuda_bf16.h>
+#include <stddef.h>
 #include <stdint.h>
 
 #include <algorithm>
@@ -56,12 +53,6 @@ constexpr int kPk1 = 0, kPk2 = kPk1 + 8 * 8 * 32, kPk3 = kPk2 + 4 * 8 * 32,
 // k-step (K = 8 padded to 16) x 8 tiles, W3^T and W2^T 4 x 8
 constexpr int kPkT4 = kPkN, kPkT3 = kPkT4 + 1 * 8 * 32, kPkT2 = kPkT3 + 4 * 8 * 32,
               kPkAll = kPkT2 + 4 * 8 * 32;
-// weight gradients: blocks of kWB atoms staged in shared memory, at most
-// kWGrid thread blocks (partials), rows padded by 8 BF16 (16 bytes) so the
-// eight rows an ldmatrix reads fall in distinct banks
-constexpr int kWB = 64, kWGrid = 152;
-constexpr int kXS = kNF + 8, kHS = kH + 8;
-constexpr int kWStage = kWB * (kXS + 6 * kHS + kNO);  // BF16 elements per stage
 
 struct Mlp {
   float* d_par = nullptr;   // FP32 master weights
@@ -76,11 +67,8 @@ struct Mlp {
   long cap = 0;
   __nv_bfloat16* d_X = nullptr;   // features for mls6_mlp_apply
   float* d_Y = nullptr;           // outputs
-  __nv_bfloat16* d_H = nullptr;   // 3 x N x 64 activations (training)
-  __nv_bfloat16* d_D = nullptr;   // 3 x N x 64 activation gradients dZ1..dZ3
-  __nv_bfloat16* d_dY = nullptr;  // N x 8 output gradients
-  float* d_part = nullptr;        // blocks x kNPar partial gradients
-  double* d_lpart = nullptr;      // loss partials, one per backward block
+  float* d_part = nullptr;        // kTGrid x kNPar partial gradients
+  double* d_lpart = nullptr;      // loss partials, one per block of k_mlp_train
   float* d_grad = nullptr;        // kNPar
   double* d_loss = nullptr;
 };
@@ -296,22 +284,6 @@ __device__ __forceinline__ void next_a(const float (&acc)[8][4], const float* __
   }
 }
 
-__device__ __forceinline__ void store_act(uint32_t* __restrict__ H, long ra, long rb, bool va,
-                                          bool vb, int c2, const uint32_t (&A)[4][4]) {
-#pragma unroll
-  for (int ks = 0; ks < 4; ++ks) {
-    const int w0 = (16 * ks + c2) >> 1, w1 = (16 * ks + 8 + c2) >> 1;
-    if (va) {
-      H[ra * (kH / 2) + w0] = A[ks][0];
-      H[ra * (kH / 2) + w1] = A[ks][2];
-    }
-    if (vb) {
-      H[rb * (kH / 2) + w0] = A[ks][1];
-      H[rb * (kH / 2) + w1] = A[ks][3];
-    }
-  }
-}
-
 __device__ __forceinline__ void hidden_layer(const uint32_t (&A)[4][4], const uint2* __restrict__ sw,
                                              int lane, float (&acc)[8][4]) {
 #pragma unroll
@@ -327,14 +299,11 @@ __device__ __forceinline__ void hidden_layer(const uint32_t (&A)[4][4], const ui
     }
 }
 
-// Forward pass: Y (N x 8) = network(X); with STORE the three hidden
-// activations (BF16, N x 64 each) are kept for the backward pass.
-template <bool STORE>
+// Forward pass: Y (N x 8) = network(X).
 __global__ void __launch_bounds__(128) k_mlp_fwd(const __nv_bfloat16* __restrict__ X, long N,
                                                  const uint2* __restrict__ pk,
                                                  const float* __restrict__ par,
-                                                 float* __restrict__ Y,
-                                                 __nv_bfloat16* __restrict__ H) {
+                                                 float* __restrict__ Y) {
   __shared__ uint2 sw[kPkN];
   __shared__ float sb[3 * kH + kNO];
   for (int i = threadIdx.x; i < kPkN; i += blockDim.x) sw[i] = pk[i];
@@ -348,7 +317,6 @@ __global__ void __launch_bounds__(128) k_mlp_fwd(const __nv_bfloat16* __restrict
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lane >> 2, c2 = (lane & 3) * 2;
   const uint32_t* Xw = reinterpret_cast<const uint32_t*>(X);
-  uint32_t* Hw = reinterpret_cast<uint32_t*>(H);
   for (long tile = (long)blockIdx.x * 4 + warp; tile * 16 < N; tile += (long)gridDim.x * 4) {
     const long ra = tile * 16 + g, rb = ra + 8;
     const bool va = ra < N, vb = rb < N;
@@ -378,13 +346,10 @@ __global__ void __launch_bounds__(128) k_mlp_fwd(const __nv_bfloat16* __restrict
       }
     uint32_t A[4][4];
     next_a(acc, sb, c2, A);
-    if (STORE) store_act(Hw, ra, rb, va, vb, c2, A);
     hidden_layer(A, sw + kPk2, lane, acc);
     next_a(acc, sb + kH, c2, A);
-    if (STORE) store_act(Hw + N * (kH / 2), ra, rb, va, vb, c2, A);
     hidden_layer(A, sw + kPk3, lane, acc);
     next_a(acc, sb + 2 * kH, c2, A);
-    if (STORE) store_act(Hw + 2 * N * (kH / 2), ra, rb, va, vb, c2, A);
     // output layer: N = 8 (one tile)
     float o[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
@@ -404,141 +369,78 @@ __global__ void __launch_bounds__(128) k_mlp_fwd(const __nv_bfloat16* __restrict
   }
 }
 
-// Backward through the activations on the tensor cores, one warp per
-// 16-atom tile (the forward pass's tiling): dY = 2 (y - t) / N on outputs
-// 0..2 (BF16, stored for the weight gradients), then per layer
-//   dZ3 = (dY W4^T) (1 - h3^2),  dZ2 = (dZ3 W3^T) (1 - h2^2),
-//   dZ1 = (dZ2 W2^T) (1 - h1^2),
-// each product an mma over the transposed-weight fragments with FP32
-// accumulators; the factor (1 - h^2) uses the stored BF16 activations at
-// the accumulator positions, and the result is packed (BF16) both as the
-// next layer's A fragments and into D for the weight gradients.  Loss
-// partials: one per block, summed in a fixed order by k_mlp_reduce.
-__device__ __forceinline__ void act_grad(const float (&acc)[8][4], const uint32_t* __restrict__ Hl,
-                                         long ra, long rb, bool va, bool vb, int c2,
-                                         uint32_t* __restrict__ Dl, uint32_t (&A)[4][4]) {
-#pragma unroll
-  for (int nt = 0; nt < 8; ++nt) {
-    const int w = (8 * nt + c2) >> 1;
-    float ha0 = 0.f, ha1 = 0.f, hb0 = 0.f, hb1 = 0.f;
-    if (va) {
-      const uint32_t u = Hl[ra * (kH / 2) + w];
-      const __nv_bfloat162 h = *reinterpret_cast<const __nv_bfloat162*>(&u);
-      ha0 = __low2float(h);
-      ha1 = __high2float(h);
-    }
-    if (vb) {
-      const uint32_t u = Hl[rb * (kH / 2) + w];
-      const __nv_bfloat162 h = *reinterpret_cast<const __nv_bfloat162*>(&u);
-      hb0 = __low2float(h);
-      hb1 = __high2float(h);
-    }
-    const uint32_t pa = pack_bf16(acc[nt][0] * (1.f - ha0 * ha0), acc[nt][1] * (1.f - ha1 * ha1));
-    const uint32_t pb = pack_bf16(acc[nt][2] * (1.f - hb0 * hb0), acc[nt][3] * (1.f - hb1 * hb1));
-    // tile nt is half (nt & 1) of k-step nt / 2 of the next product
-    A[nt >> 1][(nt & 1) * 2 + 0] = pa;
-    A[nt >> 1][(nt & 1) * 2 + 1] = pb;
-    if (va) Dl[ra * (kH / 2) + w] = pa;
-    if (vb) Dl[rb * (kH / 2) + w] = pb;
-  }
+// ---------------------------------------------------------------- training
+
+// Loss and gradient of a batch in one pass over the rows.  A block of 8 warps
+// takes `per` consecutive tiles of kTA atoms; per tile
+//   - every warp runs the network on its 16 atoms (the tiling of k_mlp_fwd):
+//     activations stay in registers as the next layer's A fragments and go to
+//     shared memory as rows [atom][unit];
+//   - dY = 2 (y - t) / N on outputs 0..2 (BF16), then per layer
+//       dZ3 = (dY W4^T) (1 - h3^2),  dZ2 = (dZ3 W3^T) (1 - h2^2),
+//       dZ1 = (dZ2 W2^T) (1 - h1^2),
+//     each product an mma over the transposed-weight fragments with FP32
+//     accumulators, the result packed (BF16) both as the next product's A
+//     fragments and into shared memory;
+//   - the block adds the tile to its weight gradients,
+//       dW1 = X^T dZ1 (128 x 64), dW2 = H1^T dZ2, dW3 = H2^T dZ3 (64 x 64),
+//       dW4 = H3^T dY (64 x 8), db = column sums of dZ1, dZ2, dZ3, dY,
+//     with the atoms as the K dimension: both operands are read from the rows
+//     in shared memory with ldmatrix .trans.  Warp w owns rows 16w.. of dW1,
+//     rows 16w.. of dW2 and dW4 (w < 4) or of dW3 (w >= 4); the bias sums are
+//     products with an all-ones A (every row of the result is the column
+//     sum), taken by warps 0 (b2), 1 (b4), 4 (b1), 5 (b3) from fragments they
+//     already hold.
+// The features of the next tile are copied (cp.async, 16-byte pieces, rows
+// past N zero) while a tile is used.  Partials go to part[block][*] and
+// lpart[block]; k_mlp_reduce sums them in block order: results are
+// reproducible bit for bit.
+// What bounds it: the chain of dependent mma and tanh of a warp (two warps per
+// scheduler), not memory: X and T are read once.  Three kernels (forward,
+// backward, weight gradients) passed 3 x N x 64 activations and as many
+// gradients through memory instead, 93 us at 65,536 atoms against 37.
+// 128 atoms per tile: 16 per warp, and 226 KB of rows, two feature stages and
+// weight fragments are what one SM holds.
+constexpr int kTA = 128, kTGrid = 152;  // atoms per tile, most blocks (partials)
+constexpr int kHS = kH + 8;             // row pitch: 8 rows of an ldmatrix in distinct banks
+
+struct TrainShared {
+  __nv_bfloat16 x[2][kTA * kNF];  // 16-byte pieces of row r at piece ^ (r & 7)
+  __nv_bfloat16 h[3][kTA * kHS];
+  __nv_bfloat16 d[3][kTA * kHS];
+  __nv_bfloat16 dy[kTA * kNO];
+  uint2 w[kPkAll];
+  float b[3 * kH + kNO];
+  double loss[8];
+};
+static_assert(sizeof(TrainShared) <= 227 * 1024, "shared memory of one block");
+static_assert(offsetof(TrainShared, h) % 16 == 0 && offsetof(TrainShared, d) % 16 == 0 &&
+                  offsetof(TrainShared, dy) % 16 == 0 && offsetof(TrainShared, w) % 16 == 0 &&
+                  offsetof(TrainShared, loss) % 8 == 0,
+              "alignment of the shared-memory rows");
+
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], const void* p) {
+  const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(a)
+               : "memory");
 }
 
-__device__ __forceinline__ void back_product(const uint32_t (&A)[4][4],
-                                             const uint2* __restrict__ sw, int lane,
-                                             float (&acc)[8][4]) {
-#pragma unroll
-  for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-    for (int c = 0; c < 4; ++c) acc[nt][c] = 0.f;
-#pragma unroll
-  for (int ks = 0; ks < 4; ++ks)
-#pragma unroll
-    for (int nt = 0; nt < 8; ++nt) {
-      const uint2 b = sw[(ks * 8 + nt) * 32 + lane];
-      mma16816(acc[nt], A[ks][0], A[ks][1], A[ks][2], A[ks][3], b.x, b.y);
-    }
-}
-
-__global__ void __launch_bounds__(128) k_mlp_bwd(const float* __restrict__ Y,
-                                                 const float* __restrict__ T, long N,
-                                                 float inv_n, const __nv_bfloat16* __restrict__ H,
-                                                 const uint2* __restrict__ pk,
-                                                 __nv_bfloat16* __restrict__ D,
-                                                 __nv_bfloat16* __restrict__ dYb,
-                                                 double* __restrict__ lpart) {
-  constexpr int kT = kPkAll - kPkN;
-  __shared__ uint2 sw[kT];
-  __shared__ double sh[32];
-  for (int i = threadIdx.x; i < kT; i += blockDim.x) sw[i] = pk[kPkN + i];
-  __syncthreads();
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int g = lane >> 2, c2 = (lane & 3) * 2;
-  const uint32_t* Hw = reinterpret_cast<const uint32_t*>(H);
-  uint32_t* Dw = reinterpret_cast<uint32_t*>(D);
-  uint32_t* dYw = reinterpret_cast<uint32_t*>(dYb);
-  double l = 0.0;
-  for (long tile = (long)blockIdx.x * 4 + warp; tile * 16 < N; tile += (long)gridDim.x * 4) {
-    const long ra = tile * 16 + g, rb = ra + 8;
-    const bool va = ra < N, vb = rb < N;
-    float dy[4] = {0.f, 0.f, 0.f, 0.f};  // (ra, c2), (ra, c2+1), (rb, c2), (rb, c2+1)
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const long r = q < 2 ? ra : rb;
-      const int c = c2 + (q & 1);
-      if ((q < 2 ? va : vb) && c < 3) {
-        const float e = Y[r * kNO + c] - T[r * 3 + c];
-        l += (double)e * e;
-        dy[q] = 2.f * e * inv_n;
-      }
-    }
-    const uint32_t da = pack_bf16(dy[0], dy[1]), db = pack_bf16(dy[2], dy[3]);
-    if (va) dYw[ra * (kNO / 2) + (c2 >> 1)] = da;
-    if (vb) dYw[rb * (kNO / 2) + (c2 >> 1)] = db;
-    // dY W4^T: one k-step, columns 8..15 of A are zero
-    float acc[8][4];
-#pragma unroll
-    for (int nt = 0; nt < 8; ++nt) {
-      acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
-      const uint2 b = sw[(kPkT4 - kPkN) + nt * 32 + lane];
-      mma16816(acc[nt], da, db, 0u, 0u, b.x, b.y);
-    }
-    uint32_t A[4][4];
-    act_grad(acc, Hw + 2 * N * (kH / 2), ra, rb, va, vb, c2, Dw + 2 * N * (kH / 2), A);
-    back_product(A, sw + (kPkT3 - kPkN), lane, acc);
-    act_grad(acc, Hw + N * (kH / 2), ra, rb, va, vb, c2, Dw + N * (kH / 2), A);
-    back_product(A, sw + (kPkT2 - kPkN), lane, acc);
-    act_grad(acc, Hw, ra, rb, va, vb, c2, Dw, A);
-  }
-  const double s = block_sum(l, sh);
-  if (threadIdx.x == 0) lpart[blockIdx.x] = s;
-}
-
-// Weight gradients on the tensor cores.  Thread block c sums the atoms of
-// blocks [c per, (c+1) per) of kWB atoms (per = ceil(blocks / kWGrid)):
-//   dW1 = X^T dZ1 (128 x 64), dW2 = H1^T dZ2, dW3 = H2^T dZ3 (64 x 64),
-//   dW4 = H3^T dY (64 x 8), db = column sums of dZ1, dZ2, dZ3, dY.
-// Each block of atoms is copied (cp.async, 16-byte pieces, rows past N
-// zero-filled) into one of two shared-memory stages while the other is
-// used.  Atoms are the K dimension: the A operand (activations transposed)
-// and the B operand (gradients) are both read from row-major [atom][column]
-// tiles with ldmatrix .trans.  Warp w owns rows 16w.. of dW1, rows 16w.. of
-// dW2 and dW4 (w < 4) or of dW3 (w >= 4); the bias sums are mma products
-// with an all-ones A (every row of the result is the column sum), taken by
-// warps 0 (b2), 1 (b4), 4 (b1), 5 (b3) from fragments they already hold.
-// The partial of block c is written to part[c][*]; k_mlp_reduce sums the
-// partials in block order, so the result is reproducible bit for bit.
 __device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], const void* p) {
   const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];\n"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"(a));
+               : "r"(a)
+               : "memory");
 }
 
 __device__ __forceinline__ void ldsm2t(uint32_t (&r)[2], const void* p) {
   const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
   asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];\n"
                : "=r"(r[0]), "=r"(r[1])
-               : "r"(a));
+               : "r"(a)
+               : "memory");
 }
 
 __device__ __forceinline__ void cp_async16(void* dst, const void* src, int bytes) {
@@ -547,65 +449,108 @@ __device__ __forceinline__ void cp_async16(void* dst, const void* src, int bytes
                : "memory");
 }
 
+// Element of the swizzled feature rows: row r, 16-byte piece q.
+__device__ __forceinline__ const __nv_bfloat16* x_piece(const __nv_bfloat16* x, int r, int q) {
+  return x + r * kNF + 8 * (q ^ (r & 7));
+}
+
 // A fragments of rows 16 m0.. (the activation columns) for k-step ks of a
-// stage tile [atom][column] with row stride S: matrices (atoms 0-7 / 8-15)
-// x (columns 0-7 / 8-15) in the order a0 a1 a2 a3 of the mma.
-template <int S>
+// tile [atom][column]: matrices (atoms 0-7 / 8-15) x (columns 0-7 / 8-15) in
+// the order a0 a1 a2 a3 of the mma.
 __device__ __forceinline__ void frag_a(uint32_t (&a)[4], const __nv_bfloat16* t, int ks, int m0,
                                        int lane) {
   const int j = lane >> 3, r = lane & 7;
-  ldsm4t(a, t + (16 * ks + r + 8 * (j >> 1)) * S + 16 * m0 + 8 * (j & 1));
+  ldsm4t(a, t + (16 * ks + r + 8 * (j >> 1)) * kHS + 16 * m0 + 8 * (j & 1));
+}
+
+__device__ __forceinline__ void frag_ax(uint32_t (&a)[4], const __nv_bfloat16* x, int ks, int m0,
+                                        int lane) {
+  const int j = lane >> 3, r = lane & 7;
+  ldsm4t(a, x_piece(x, 16 * ks + r + 8 * (j >> 1), 2 * m0 + (j & 1)));
 }
 
 // B fragments of column tiles nt0, nt0+1 for k-step ks: b[0..1] for nt0,
 // b[2..3] for nt0+1.
-template <int S>
 __device__ __forceinline__ void frag_b2(uint32_t (&b)[4], const __nv_bfloat16* t, int ks, int nt0,
                                         int lane) {
   const int j = lane >> 3, r = lane & 7;
-  ldsm4t(b, t + (16 * ks + r + 8 * (j & 1)) * S + 8 * (nt0 + (j >> 1)));
+  ldsm4t(b, t + (16 * ks + r + 8 * (j & 1)) * kHS + 8 * (nt0 + (j >> 1)));
 }
 
-__global__ void __launch_bounds__(256) k_mlp_wgrad(const __nv_bfloat16* __restrict__ X,
-                                                   const __nv_bfloat16* __restrict__ H,
-                                                   const __nv_bfloat16* __restrict__ D,
-                                                   const __nv_bfloat16* __restrict__ dY, long N,
-                                                   long per, float* __restrict__ part) {
-  extern __shared__ __align__(16) __nv_bfloat16 stg[];  // two stages of kWStage
+// Fragments of a warp's 16 rows (g and g + 8 of row0) as rows of a tile; rows
+// past the batch (va, vb false) are zero, so that they add nothing.
+__device__ __forceinline__ void put_rows(__nv_bfloat16* t, int row0, int g, bool va, bool vb,
+                                         int c2, const uint32_t (&A)[4][4]) {
+  uint32_t* pa = reinterpret_cast<uint32_t*>(t + (row0 + g) * kHS + c2);
+  uint32_t* pb = reinterpret_cast<uint32_t*>(t + (row0 + g + 8) * kHS + c2);
+#pragma unroll
+  for (int ks = 0; ks < 4; ++ks) {
+    pa[8 * ks] = va ? A[ks][0] : 0u;
+    pb[8 * ks] = vb ? A[ks][1] : 0u;
+    pa[8 * ks + 4] = va ? A[ks][2] : 0u;
+    pb[8 * ks + 4] = vb ? A[ks][3] : 0u;
+  }
+}
+
+__device__ __forceinline__ void get_rows(const __nv_bfloat16* t, int row0, int g, int c2,
+                                         uint32_t (&A)[4][4]) {
+  const uint32_t* pa = reinterpret_cast<const uint32_t*>(t + (row0 + g) * kHS + c2);
+  const uint32_t* pb = reinterpret_cast<const uint32_t*>(t + (row0 + g + 8) * kHS + c2);
+#pragma unroll
+  for (int ks = 0; ks < 4; ++ks) {
+    A[ks][0] = pa[8 * ks];
+    A[ks][1] = pb[8 * ks];
+    A[ks][2] = pa[8 * ks + 4];
+    A[ks][3] = pb[8 * ks + 4];
+  }
+}
+
+// v (1 - h^2) for two columns, packed.
+__device__ __forceinline__ uint32_t act_grad2(float v0, float v1, uint32_t h2) {
+  const __nv_bfloat162 h = *reinterpret_cast<const __nv_bfloat162*>(&h2);
+  const float h0 = __low2float(h), h1 = __high2float(h);
+  return pack_bf16(v0 * (1.f - h0 * h0), v1 * (1.f - h1 * h1));
+}
+
+// Column tile nt of acc is half (nt & 1) of k-step nt / 2 of the next product.
+__device__ __forceinline__ void act_grad(const float (&acc)[8][4], const uint32_t (&H)[4][4],
+                                         uint32_t (&A)[4][4]) {
+#pragma unroll
+  for (int nt = 0; nt < 8; ++nt) {
+    const int ks = nt >> 1, o = (nt & 1) * 2;
+    A[ks][o] = act_grad2(acc[nt][0], acc[nt][1], H[ks][o]);
+    A[ks][o + 1] = act_grad2(acc[nt][2], acc[nt][3], H[ks][o + 1]);
+  }
+}
+
+__global__ void __launch_bounds__(256, 1) k_mlp_train(
+    const __nv_bfloat16* __restrict__ X, const float* __restrict__ T, long N, long per,
+    float inv_n, const uint2* __restrict__ pk, const float* __restrict__ par,
+    float* __restrict__ part, double* __restrict__ lpart) {
+  extern __shared__ __align__(16) unsigned char train_smem[];
+  TrainShared& S = *reinterpret_cast<TrainShared*>(train_smem);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lane >> 2, c2 = (lane & 3) * 2;
-  const long nblk = cdiv(N, (long)kWB);
-  const long b0 = (long)blockIdx.x * per, b1 = min(nblk, b0 + per);
-  // stage layout: X [kWB][kXS], H1..H3 [kWB][kHS], dZ1..dZ3 [kWB][kHS], dY [kWB][kNO]
-  auto sx = [&](int st) { return stg + (size_t)st * kWStage; };
-  auto sh = [&](int st, int l) { return sx(st) + kWB * kXS + l * kWB * kHS; };
-  auto sd = [&](int st, int l) { return sx(st) + kWB * kXS + (3 + l) * kWB * kHS; };
-  auto sy = [&](int st) { return sx(st) + kWB * kXS + 6 * kWB * kHS; };
-  auto stage = [&](int st, long blk) {
-    const long r0 = blk * kWB;
-    constexpr int kPieces = kNF / 8 + 6 * (kH / 8) + 1;  // 16-byte pieces per atom row
-    for (int t = threadIdx.x; t < kWB * kPieces; t += blockDim.x) {
-      const int r = t / kPieces, q = t % kPieces;
-      const long i = r0 + r;
+  const long ntile = cdiv(N, (long)kTA);
+  const long t0 = (long)blockIdx.x * per, t1 = min(ntile, t0 + per);
+  auto stage = [&](int st, long tile) {
+    for (int t = threadIdx.x; t < kTA * (kNF / 8); t += blockDim.x) {
+      const int r = t / (kNF / 8), q = t % (kNF / 8);
+      const long i = tile * kTA + r;
       const bool ok = i < N;
-      const long ic = ok ? i : 0;
-      const __nv_bfloat16* src;
-      __nv_bfloat16* dst;
-      if (q < kNF / 8) {
-        src = X + ic * kNF + 8 * q;
-        dst = sx(st) + r * kXS + 8 * q;
-      } else if (q < kNF / 8 + 6 * (kH / 8)) {
-        const int u = q - kNF / 8, l = u / (kH / 8), c = u % (kH / 8);
-        src = (l < 3 ? H + ((long)l * N + ic) * kH : D + ((long)(l - 3) * N + ic) * kH) + 8 * c;
-        dst = (l < 3 ? sh(st, l) : sd(st, l - 3)) + r * kHS + 8 * c;
-      } else {
-        src = dY + ic * kNO;
-        dst = sy(st) + r * kNO;
-      }
-      cp_async16(dst, src, ok ? 16 : 0);
+      cp_async16(const_cast<__nv_bfloat16*>(x_piece(S.x[st], r, q)), X + (ok ? i : 0) * kNF + 8 * q,
+                 ok ? 16 : 0);
     }
     asm volatile("cp.async.commit_group;\n" ::: "memory");
   };
+  if (t0 < t1) stage(0, t0);
+  for (int i = threadIdx.x; i < kPkAll; i += blockDim.x) S.w[i] = pk[i];
+  for (int i = threadIdx.x; i < kH; i += blockDim.x) {
+    S.b[i] = par[kOffB1 + i];
+    S.b[kH + i] = par[kOffB2 + i];
+    S.b[2 * kH + i] = par[kOffB3 + i];
+  }
+  if (threadIdx.x < kNO) S.b[3 * kH + threadIdx.x] = par[kOffB4 + threadIdx.x];
 
   float a1[8][4], a23[8][4], a4[4], ab[8][4];
 #pragma unroll
@@ -615,26 +560,97 @@ __global__ void __launch_bounds__(256) k_mlp_wgrad(const __nv_bfloat16* __restri
 #pragma unroll
   for (int c = 0; c < 4; ++c) a4[c] = 0.f;
   const uint32_t one = 0x3F803F80u;  // two BF16 ones
+  double l = 0.0;
 
-  if (b0 < b1) stage(0, b0);
-  for (long blk = b0; blk < b1; ++blk) {
-    const int st = (int)((blk - b0) & 1);
-    if (blk + 1 < b1) {
-      stage(st ^ 1, blk + 1);
-      asm volatile("cp.async.wait_group 1;\n" ::: "memory");
-    } else {
-      asm volatile("cp.async.wait_group 0;\n" ::: "memory");
-    }
-    __syncthreads();
-    const int l23 = warp < 4 ? 0 : 1;           // dW2 (H1, dZ2) or dW3 (H2, dZ3)
-    const int m23 = warp & 3;
+  for (long tile = t0; tile < t1; ++tile) {
+    const int st = (int)((tile - t0) & 1);
+    asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+    __syncthreads();  // stage st filled; the other stage and all rows are free
+    if (tile + 1 < t1) stage(st ^ 1, tile + 1);
+    const int row0 = 16 * warp;
+    const long ra = tile * kTA + row0 + g, rb = ra + 8;
+    const bool va = ra < N, vb = rb < N;
+    float tg[4];  // targets (ra, c2), (ra, c2 + 1), (rb, c2), (rb, c2 + 1)
 #pragma unroll
-    for (int ks = 0; ks < kWB / 16; ++ks) {
+    for (int q = 0; q < 4; ++q) {
+      const int c = c2 + (q & 1);
+      tg[q] = ((q < 2 ? va : vb) && c < 3) ? T[(q < 2 ? ra : rb) * 3 + c] : 0.f;
+    }
+    // forward
+    float acc[8][4];
+#pragma unroll
+    for (int nt = 0; nt < 8; ++nt)
+#pragma unroll
+      for (int c = 0; c < 4; ++c) acc[nt][c] = 0.f;
+#pragma unroll
+    for (int ks = 0; ks < 8; ++ks) {
+      const int j = lane >> 3, r = lane & 7;
+      uint32_t xa[4];
+      ldsm4(xa, x_piece(S.x[st], row0 + r + 8 * (j & 1), 2 * ks + (j >> 1)));
+#pragma unroll
+      for (int nt = 0; nt < 8; ++nt) {
+        const uint2 b = S.w[kPk1 + (ks * 8 + nt) * 32 + lane];
+        mma16816(acc[nt], xa[0], xa[1], xa[2], xa[3], b.x, b.y);
+      }
+    }
+    uint32_t A[4][4], H[4][4];
+    next_a(acc, S.b, c2, A);
+    put_rows(S.h[0], row0, g, va, vb, c2, A);
+    hidden_layer(A, S.w + kPk2, lane, acc);
+    next_a(acc, S.b + kH, c2, A);
+    put_rows(S.h[1], row0, g, va, vb, c2, A);
+    hidden_layer(A, S.w + kPk3, lane, acc);
+    next_a(acc, S.b + 2 * kH, c2, H);
+    put_rows(S.h[2], row0, g, va, vb, c2, H);
+    float o[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int ks = 0; ks < 4; ++ks) {
+      const uint2 b = S.w[kPk4 + ks * 32 + lane];
+      mma16816(o, H[ks][0], H[ks][1], H[ks][2], H[ks][3], b.x, b.y);
+    }
+    // output gradients and loss
+    float dy[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int c = c2 + (q & 1);
+      if ((q < 2 ? va : vb) && c < 3) {
+        const float e = o[q] + S.b[3 * kH + c] - tg[q];
+        l += (double)e * e;
+        dy[q] = 2.f * e * inv_n;
+      }
+    }
+    const uint32_t da = pack_bf16(dy[0], dy[1]), db = pack_bf16(dy[2], dy[3]);
+    *reinterpret_cast<uint32_t*>(S.dy + (row0 + g) * kNO + c2) = da;
+    *reinterpret_cast<uint32_t*>(S.dy + (row0 + g + 8) * kNO + c2) = db;
+    // backward: dY W4^T is one k-step, columns 8..15 of A are zero
+#pragma unroll
+    for (int nt = 0; nt < 8; ++nt) {
+      acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
+      const uint2 b = S.w[kPkT4 + nt * 32 + lane];
+      mma16816(acc[nt], da, db, 0u, 0u, b.x, b.y);
+    }
+    act_grad(acc, H, A);
+    put_rows(S.d[2], row0, g, va, vb, c2, A);
+    hidden_layer(A, S.w + kPkT3, lane, acc);
+    get_rows(S.h[1], row0, g, c2, H);  // this thread's own words
+    act_grad(acc, H, A);
+    put_rows(S.d[1], row0, g, va, vb, c2, A);
+    hidden_layer(A, S.w + kPkT2, lane, acc);
+    get_rows(S.h[0], row0, g, c2, H);
+    act_grad(acc, H, A);
+    put_rows(S.d[0], row0, g, va, vb, c2, A);
+    __syncthreads();  // the tile's rows are complete
+
+    // weight gradients
+    const int l23 = warp < 4 ? 0 : 1;  // dW2 (H1, dZ2) or dW3 (H2, dZ3)
+    const int m23 = warp & 3;
+#pragma unroll 2
+    for (int ks = 0; ks < kTA / 16; ++ks) {
       uint32_t a[4], b[4][4];
       // dW1 rows 16 warp..: X^T dZ1
-      frag_a<kXS>(a, sx(st), ks, warp, lane);
+      frag_ax(a, S.x[st], ks, warp, lane);
 #pragma unroll
-      for (int q = 0; q < 4; ++q) frag_b2<kHS>(b[q], sd(st, 0), ks, 2 * q, lane);
+      for (int q = 0; q < 4; ++q) frag_b2(b[q], S.d[0], ks, 2 * q, lane);
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         mma16816(a1[2 * q], a[0], a[1], a[2], a[3], b[q][0], b[q][1]);
@@ -647,9 +663,9 @@ __global__ void __launch_bounds__(256) k_mlp_wgrad(const __nv_bfloat16* __restri
           mma16816(ab[2 * q + 1], one, one, one, one, b[q][2], b[q][3]);
         }
       // dW2 (warps 0-3) / dW3 (warps 4-7)
-      frag_a<kHS>(a, sh(st, l23), ks, m23, lane);
+      frag_a(a, S.h[l23], ks, m23, lane);
 #pragma unroll
-      for (int q = 0; q < 4; ++q) frag_b2<kHS>(b[q], sd(st, 1 + l23), ks, 2 * q, lane);
+      for (int q = 0; q < 4; ++q) frag_b2(b[q], S.d[1 + l23], ks, 2 * q, lane);
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         mma16816(a23[2 * q], a[0], a[1], a[2], a[3], b[q][0], b[q][1]);
@@ -665,14 +681,13 @@ __global__ void __launch_bounds__(256) k_mlp_wgrad(const __nv_bfloat16* __restri
         uint32_t by[2];
         {
           const int j = (lane >> 3) & 1, r = lane & 7;
-          ldsm2t(by, sy(st) + (16 * ks + r + 8 * j) * kNO);
+          ldsm2t(by, S.dy + (16 * ks + r + 8 * j) * kNO);
         }
-        frag_a<kHS>(a, sh(st, 2), ks, warp, lane);
+        frag_a(a, S.h[2], ks, warp, lane);
         mma16816(a4, a[0], a[1], a[2], a[3], by[0], by[1]);
         if (warp == 1) mma16816(ab[0], one, one, one, one, by[0], by[1]);  // b4
       }
     }
-    __syncthreads();  // the stage is refilled two iterations later
   }
 
   // partial of this block, parameter order of the master weights
@@ -702,23 +717,43 @@ __global__ void __launch_bounds__(256) k_mlp_wgrad(const __nv_bfloat16* __restri
       P[kOffB4 + c2 + 1] = ab[0][1];
     }
   }
+  l = warp_sum(l);
+  if (lane == 0) S.loss[warp] = l;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < 8; ++w) l += S.loss[w];
+    lpart[blockIdx.x] = l;
+  }
 }
 
-// Fixed-order sums over the chunks: gradient (FP32 out, summed in FP64)
-// and the loss.
-__global__ void k_mlp_reduce(const float* __restrict__ part, int nchunk,
-                             const double* __restrict__ lpart, int nl, double inv_n,
-                             float* __restrict__ grad, double* __restrict__ loss) {
-  const int p = blockIdx.x * blockDim.x + threadIdx.x;
-  if (p < kNPar) {
-    double s = 0.0;
-    for (int c = 0; c < nchunk; ++c) s += (double)part[(long)c * kNPar + p];
+// Fixed-order sums over the blocks' partials: gradient (FP32 out, summed in
+// FP64; also to grad_out where given) and the loss.  32 parameters per block;
+// thread row s adds the partials s, s + 8, ... and the rows' sums are added in
+// order.  One thread per parameter left 85 of the 152 SMs idle, and its block
+// 0 added 1,024 loss partials in one chain: 84 us against 13 at 65,536
+// atoms.
+__global__ void __launch_bounds__(256) k_mlp_reduce(
+    const float* __restrict__ part, int nchunk, const double* __restrict__ lpart, double inv_n,
+    float* __restrict__ grad, float* __restrict__ grad_out, double* __restrict__ loss) {
+  __shared__ double sh[8][32];
+  const int col = threadIdx.x & 31, row = threadIdx.x >> 5;
+  const int p = blockIdx.x * 32 + col;
+  double s = 0.0;
+  if (p < kNPar)
+#pragma unroll 4
+    for (int c = row; c < nchunk; c += 8) s += (double)part[(long)c * kNPar + p];
+  sh[row][col] = s;
+  __syncthreads();
+  if (row == 0 && p < kNPar) {
+    for (int r = 1; r < 8; ++r) s += sh[r][col];
     grad[p] = (float)s;
+    if (grad_out) grad_out[p] = (float)s;
   }
-  if (p == 0) {
-    double s = 0.0;
-    for (int c = 0; c < nl; ++c) s += lpart[c];
-    *loss = s * inv_n;
+  if (blockIdx.x == 0 && row == 1) {  // the loss
+    double v = 0.0;
+    for (int c = col; c < nchunk; c += 32) v += lpart[c];
+    v = warp_sum(v);
+    if (col == 0) *loss = v * inv_n;
   }
 }
 
@@ -765,40 +800,41 @@ static uint64_t splitmix64(uint64_t& s) {
   return z ^ (z >> 31);
 }
 
-// Launch geometry of the training kernels (a function of N only, so the
-// partial sums and hence the results do not depend on the device).
+// Launch geometry: functions of N only, so that the partial sums and hence the
+// results do not depend on the device.
 static long fwd_blocks(long N) { return std::min(cdiv(cdiv(N, 16L), 4L), 152L * 8); }
-static long bwd_blocks(long N) { return fwd_blocks(N); }
-static void wgrad_geometry(long N, long& grid, long& per) {
-  const long nblk = cdiv(N, (long)kWB);
-  per = cdiv(nblk, (long)kWGrid);
-  grid = per > 0 ? cdiv(nblk, per) : 0;
+static void train_geometry(long N, long& grid, long& per) {
+  const long ntile = cdiv(N, (long)kTA);
+  per = cdiv(ntile, (long)kTGrid);
+  grid = per > 0 ? cdiv(ntile, per) : 0;
 }
-constexpr size_t kWSmem = 2 * (size_t)kWStage * sizeof(__nv_bfloat16);
 
+// Buffers of mls6_mlp_apply (features and outputs of N atoms).
 static int grow(Mlp* m, long N) {
   if (N <= m->cap) return MLS6_OK;
-  void* bufs[] = {m->d_X, m->d_Y, m->d_H, m->d_D, m->d_dY, m->d_part, m->d_lpart};
-  for (void* b : bufs)
-    if (b) cudaFree(b);
+  if (m->d_X) cudaFree(m->d_X);
+  if (m->d_Y) cudaFree(m->d_Y);
   m->d_X = nullptr;
   m->d_Y = nullptr;
-  m->d_H = nullptr;
-  m->d_D = nullptr;
-  m->d_dY = nullptr;
-  m->d_part = nullptr;
-  m->d_lpart = nullptr;
   m->cap = 0;
-  const long nbl = bwd_blocks(N);
   if (cudaMalloc((void**)&m->d_X, sizeof(__nv_bfloat16) * kNF * N) != cudaSuccess ||
-      cudaMalloc((void**)&m->d_Y, sizeof(float) * kNO * N) != cudaSuccess ||
-      cudaMalloc((void**)&m->d_H, sizeof(__nv_bfloat16) * 3 * kH * N) != cudaSuccess ||
-      cudaMalloc((void**)&m->d_D, sizeof(__nv_bfloat16) * 3 * kH * N) != cudaSuccess ||
-      cudaMalloc((void**)&m->d_dY, sizeof(__nv_bfloat16) * kNO * N) != cudaSuccess ||
-      cudaMalloc((void**)&m->d_part, sizeof(float) * kNPar * kWGrid) != cudaSuccess ||
-      cudaMalloc((void**)&m->d_lpart, sizeof(double) * nbl) != cudaSuccess)
+      cudaMalloc((void**)&m->d_Y, sizeof(float) * kNO * N) != cudaSuccess)
     return MLS6_ERR_NOMEM;
   m->cap = N;
+  return MLS6_OK;
+}
+
+// Buffers of the gradient (the same for every batch).
+static int grow_train(Mlp* m) {
+  if (!m->d_part &&
+      cudaMalloc((void**)&m->d_part, sizeof(float) * kNPar * kTGrid) != cudaSuccess) {
+    m->d_part = nullptr;
+    return MLS6_ERR_NOMEM;
+  }
+  if (!m->d_lpart && cudaMalloc((void**)&m->d_lpart, sizeof(double) * kTGrid) != cudaSuccess) {
+    m->d_lpart = nullptr;
+    return MLS6_ERR_NOMEM;
+  }
   return MLS6_OK;
 }
 
@@ -808,35 +844,33 @@ static int repack(Mlp* m) {
   return MLS6_OK;
 }
 
-static int forward(Mlp* m, const void* X, long N, float* Y, bool store) {
+static int forward(Mlp* m, const void* X, long N, float* Y) {
   if (N <= 0) return MLS6_OK;
-  const long nb = fwd_blocks(N);
-  if (store)
-    k_mlp_fwd<true><<<nb, 128, 0, m->stream>>>((const __nv_bfloat16*)X, N, m->d_pack, m->d_par,
-                                               Y, m->d_H);
-  else
-    k_mlp_fwd<false><<<nb, 128, 0, m->stream>>>((const __nv_bfloat16*)X, N, m->d_pack,
-                                                m->d_par, Y, nullptr);
+  k_mlp_fwd<<<fwd_blocks(N), 128, 0, m->stream>>>((const __nv_bfloat16*)X, N, m->d_pack, m->d_par,
+                                                  Y);
   CK(cudaGetLastError());
   return MLS6_OK;
 }
 
-static int gradient(Mlp* m, const void* X, const float* T, long N) {
-  int rc = grow(m, N);
+// Loss and gradient into d_loss, d_grad and, where grad is given, grad: by
+// the reduction itself where a kernel can store there, by a copy otherwise.
+static int gradient(Mlp* m, const void* X, const float* T, long N, float* grad) {
+  int rc = grow_train(m);
   if (rc) return rc;
-  rc = forward(m, X, N, m->d_Y, true);
-  if (rc) return rc;
-  const long nbl = bwd_blocks(N);
   long nch, per;
-  wgrad_geometry(N, nch, per);
-  k_mlp_bwd<<<nbl, 128, 0, m->stream>>>(m->d_Y, T, N, 1.0f / (float)N, m->d_H, m->d_pack,
-                                        m->d_D, m->d_dY, m->d_lpart);
-  k_mlp_wgrad<<<nch, 256, kWSmem, m->stream>>>((const __nv_bfloat16*)X, m->d_H, m->d_D, m->d_dY,
-                                               N, per, m->d_part);
-  k_mlp_reduce<<<cdiv(kNPar, 256), 256, 0, m->stream>>>(m->d_part, (int)nch, m->d_lpart,
-                                                       (int)nbl, 1.0 / (double)N, m->d_grad,
-                                                       m->d_loss);
+  train_geometry(N, nch, per);
+  const bool direct =
+      grad && (reinterpret_cast<uintptr_t>(grad) & 3) == 0 && kernel_addressable(grad);
+  k_mlp_train<<<nch, 256, sizeof(TrainShared), m->stream>>>(
+      (const __nv_bfloat16*)X, T, N, per, 1.0f / (float)N, m->d_pack, m->d_par, m->d_part,
+      m->d_lpart);
+  k_mlp_reduce<<<cdiv(kNPar, 32), 256, 0, m->stream>>>(m->d_part, (int)nch, m->d_lpart,
+                                                      1.0 / (double)N, m->d_grad,
+                                                      direct ? grad : nullptr, m->d_loss);
   CK(cudaGetLastError());
+  if (grad && !direct)
+    CK(cudaMemcpyAsync(grad, m->d_grad, sizeof(float) * kNPar, cudaMemcpyDeviceToDevice,
+                       m->stream));
   return MLS6_OK;
 }
 
@@ -849,8 +883,8 @@ static int read_loss(Mlp* m, double* loss) {
 
 static void free_mlp(Mlp* m) {
   if (!m) return;
-  void* bufs[] = {m->d_par, m->d_m, m->d_v, m->d_pack, m->d_norm, m->d_X, m->d_Y, m->d_H,
-                  m->d_D, m->d_dY, m->d_part, m->d_lpart, m->d_grad, m->d_loss};
+  void* bufs[] = {m->d_par, m->d_m, m->d_v, m->d_pack, m->d_norm, m->d_X, m->d_Y, m->d_part,
+                  m->d_lpart, m->d_grad, m->d_loss};
   for (void* b : bufs)
     if (b) cudaFree(b);
   delete m;
@@ -892,9 +926,9 @@ int mls6_mlp_create(mls6_mlp_t** out, uint64_t seed) {
     free_mlp(m);
     return MLS6_ERR_NOMEM;
   }
-  // two shared-memory stages of the weight-gradient kernel (above 48 KB)
-  if (cudaFuncSetAttribute(k_mlp_wgrad, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)kWSmem) != cudaSuccess) {
+  // shared memory of the training kernel (above 48 KB)
+  if (cudaFuncSetAttribute(k_mlp_train, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)sizeof(TrainShared)) != cudaSuccess) {
     free_mlp(m);
     return MLS6_ERR_CUDA;
   }
@@ -981,7 +1015,7 @@ int mls6_mlp_features(mls6_plan_t* plan, const mls6_mlp_t* mm, void* out, int fm
 int mls6_mlp_forward(mls6_mlp_t* mm, const void* X, int64_t N, float* Y) {
   if (!mm || N < 0 || (N > 0 && (!kernel_addressable(X) || !kernel_addressable(Y))))
     return MLS6_ERR_ARG;
-  return forward(reinterpret_cast<Mlp*>(mm), X, N, Y, false);
+  return forward(reinterpret_cast<Mlp*>(mm), X, N, Y);
 }
 
 int mls6_mlp_grad(mls6_mlp_t* mm, const void* X, const float* T, int64_t N, float* grad,
@@ -990,11 +1024,8 @@ int mls6_mlp_grad(mls6_mlp_t* mm, const void* X, const float* T, int64_t N, floa
       (reinterpret_cast<uintptr_t>(X) & 15))
     return MLS6_ERR_ARG;
   Mlp* m = reinterpret_cast<Mlp*>(mm);
-  int rc = gradient(m, X, T, N);
+  int rc = gradient(m, X, T, N, grad);
   if (rc) return rc;
-  if (grad)
-    CK(cudaMemcpyAsync(grad, m->d_grad, sizeof(float) * kNPar, cudaMemcpyDeviceToDevice,
-                       m->stream));
   return read_loss(m, loss);
 }
 
@@ -1004,7 +1035,7 @@ int mls6_mlp_train_step(mls6_mlp_t* mm, const void* X, const float* T, int64_t N
       (reinterpret_cast<uintptr_t>(X) & 15))
     return MLS6_ERR_ARG;
   Mlp* m = reinterpret_cast<Mlp*>(mm);
-  int rc = gradient(m, X, T, N);
+  int rc = gradient(m, X, T, N, nullptr);
   if (rc) return rc;
   m->step += 1;
   const float bc1 = 1.f - (float)std::pow(0.9, (double)m->step);
@@ -1031,7 +1062,7 @@ int mls6_mlp_apply(mls6_plan_t* plan, mls6_mlp_t* mm, void* forces) {
   m->stream = p->stream;
   rc = p->prec == MLS6_FP64 ? features_t<double>(p, m, m->d_X, 0, true, p->stream)
                             : features_t<float>(p, m, m->d_X, 0, true, p->stream);
-  if (!rc) rc = forward(m, m->d_X, N, m->d_Y, false);
+  if (!rc) rc = forward(m, m->d_X, N, m->d_Y);
   m->stream = saved;
   if (rc) return rc;
   if (p->prec == MLS6_FP64)
