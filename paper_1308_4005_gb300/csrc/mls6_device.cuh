@@ -1,5 +1,6 @@
 // Device helpers shared by the kernels of the multilevel summation library.
 #pragma once
+#include <climits>
 
 #include <cuda_runtime.h>
 
@@ -139,6 +140,83 @@ __device__ __forceinline__ long pdl_begin() {
   long z;
   asm volatile("mov.b64 %0, 0;" : "=l"(z)::"memory");
   return z;
+}
+
+// ------------------------------------------------- nodes around a block's atoms
+
+// A block of consecutive cell-sorted atoms touches a compact box of grid
+// nodes.  Where that box fits into kNodeBoxBytes, the block keeps it in shared
+// memory.  One buffer per kernel, whatever stages it runs.
+constexpr int kNodeBoxBytes = 24 * 1024;
+__device__ __forceinline__ unsigned char* node_box_smem() {
+  __shared__ __align__(16) unsigned char buf[kNodeBoxBytes];
+  return buf;
+}
+
+// Unwrapped node indices lo .. lo + e - 1 per axis; in: the box fits and every
+// index is at most one period away from its node (the same for all threads).
+struct NodeBox {
+  int lo0, lo1, lo2, e0, e1, e2;
+  bool in;
+};
+
+// Box of the nodes b - BELOW .. b + ABOVE of the block's valid atoms.
+template <int BELOW, int ABOVE>
+__device__ __forceinline__ NodeBox block_node_box(bool valid, int b0, int b1, int b2, int n0,
+                                                  int n1, int n2, int cap) {
+  __shared__ int lim[6];
+  if (threadIdx.x < 6) lim[threadIdx.x] = threadIdx.x < 3 ? INT_MAX : INT_MIN;
+  __syncthreads();
+  const int l0 = __reduce_min_sync(0xffffffffu, valid ? b0 - BELOW : INT_MAX);
+  const int l1 = __reduce_min_sync(0xffffffffu, valid ? b1 - BELOW : INT_MAX);
+  const int l2 = __reduce_min_sync(0xffffffffu, valid ? b2 - BELOW : INT_MAX);
+  const int h0 = __reduce_max_sync(0xffffffffu, valid ? b0 + ABOVE : INT_MIN);
+  const int h1 = __reduce_max_sync(0xffffffffu, valid ? b1 + ABOVE : INT_MIN);
+  const int h2 = __reduce_max_sync(0xffffffffu, valid ? b2 + ABOVE : INT_MIN);
+  if ((threadIdx.x & 31) == 0 && l0 != INT_MAX) {
+    atomicMin(&lim[0], l0);
+    atomicMin(&lim[1], l1);
+    atomicMin(&lim[2], l2);
+    atomicMax(&lim[3], h0);
+    atomicMax(&lim[4], h1);
+    atomicMax(&lim[5], h2);
+  }
+  __syncthreads();
+  NodeBox B;
+  B.lo0 = lim[0];
+  B.lo1 = lim[1];
+  B.lo2 = lim[2];
+  B.in = lim[3] >= lim[0] && min(n0, min(n1, n2)) > max(BELOW, ABOVE);
+  B.e0 = B.in ? lim[3] - lim[0] + 1 : 0;
+  B.e1 = B.in ? lim[4] - lim[1] + 1 : 0;
+  B.e2 = B.in ? lim[5] - lim[2] + 1 : 0;
+  B.in = B.in && (long)B.e0 * B.e1 * B.e2 <= cap;
+  return B;
+}
+
+// Index at most one period outside [0, n).
+__device__ __forceinline__ int wrap1(int i, int n) {
+  i += i < 0 ? n : 0;
+  return i - (i >= n ? n : 0);
+}
+
+// The box's node values, x fastest: one warp per row, asynchronous copies.
+template <typename T>
+__device__ __forceinline__ void load_node_box(T* box, const T* __restrict__ src, const NodeBox& B,
+                                              int n0, int n1, int n2) {
+  const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  for (int r = threadIdx.x >> 5; r < B.e1 * B.e2; r += nw) {
+    const int c = r / B.e1, b = r - c * B.e1;
+    const T* row = src + (long)n0 * (wrap1(B.lo1 + b, n1) + (long)n1 * wrap1(B.lo2 + c, n2));
+    const unsigned dst = (unsigned)__cvta_generic_to_shared(box + r * B.e0);
+    for (int x = lane; x < B.e0; x += 32)
+      asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"(
+                       dst + x * (unsigned)sizeof(T)),
+                   "l"(row + wrap1(B.lo0 + x, n0)), "n"(sizeof(T))
+                   : "memory");
+  }
+  asm volatile("cp.async.wait_all;\n" ::: "memory");
+  __syncthreads();
 }
 
 __device__ __forceinline__ double warp_sum(double v) {

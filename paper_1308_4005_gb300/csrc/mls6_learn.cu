@@ -10,7 +10,7 @@
 //              (shift, scale), stored as BF16 (or FP32) rows in input order
 //   network    128 -> 64 -> 64 -> 64 -> 8 (outputs 0..2 used), tanh hidden
 //              layers; BF16 weights and activations on the tensor cores
-//              (mma.m16n8k16, FP32 accumulation); one warp per 16 atoms, the
+//              (mma.m16n8k16, FP32 accumulation); 16 atoms per tile, the
 //              accumulator tiles of a layer are repacked in registers as the
 //              A operand of the next
 //   training   one kernel per batch: forward, BF16 tensor-core backward pass
@@ -66,7 +66,6 @@ struct Mlp {
   // work buffers (grown on demand)
   long cap = 0;
   __nv_bfloat16* d_X = nullptr;   // features for mls6_mlp_apply
-  float* d_Y = nullptr;           // outputs
   float* d_part = nullptr;        // kTGrid x kNPar partial gradients
   double* d_lpart = nullptr;      // loss partials, one per block of k_mlp_train
   float* d_grad = nullptr;        // kNPar
@@ -94,121 +93,146 @@ __device__ __forceinline__ void mma16816(float (&d)[4], uint32_t a0, uint32_t a1
 
 // ------------------------------------------------------------- features
 
-// One thread per (atom, dz): the 9 offsets (dx, dy) of one dz.  Separable:
-// per z row of the basis, an x pass over the 6 y rows of the 6x6 node
-// block, then a y pass, then the z weights.  A block (3 x kFA threads)
-// assembles the rows of kFA atoms in shared memory and writes each row with
-// 16-byte stores (a row per atom in input order, or in sorted order when
-// sorted_out is set).
+// One thread per (atom, dx): the 9 offsets (dy, dz) of one dx.  Separable: per
+// z plane of the 6 x 6 x 6 nodes around the atom an x pass over the 6 rows, a y
+// pass for the 3 dy, then the z weights of the dz that the plane belongs to
+// (648 multiply-adds a thread; one thread per dz repeats the x and y passes of
+// the planes that neighbouring dz share, 1,152).  The block's nodes come from
+// shared memory where their box fits (a warp's gathers touched 4 to 8 lines
+// each), from global memory otherwise.  A block (3 x kFA threads) assembles
+// the rows of kFA atoms in shared memory, on top of the node box, and writes
+// each row with 16-byte stores (a row per atom in input order, or in sorted
+// order when sorted_out is set).  What
+// bounds it: the latency of those reads and sums against 21 warps per SM (four
+// blocks, 80 registers): 121 -> 74 us at 262,144 atoms (159 registers: 96).
 constexpr int kFA = 64;
 
-template <typename T>
-__global__ void __launch_bounds__(3 * kFA) k_features(
+template <typename T, bool F32>
+__global__ void __launch_bounds__(3 * kFA, sizeof(T) == 8 ? 1 : 4) k_features(
     const Vec4<T>* __restrict__ sp, const int* __restrict__ sidx, int N, const T* __restrict__ E,
     int n0, int n1, int n2, T ih0, T ih1, T ih2, const float* __restrict__ norm,
-    void* __restrict__ out, int f32, int sorted_out) {
-  __shared__ __align__(16) float rows[kFA][kNF];
-  const int la = threadIdx.x / 3, dz = (int)(threadIdx.x % 3) - 1;
+    void* __restrict__ out, int sorted_out) {
+  // rows are padded by 16 bytes: those of eight atoms start in distinct banks
+  constexpr int kRow = (F32 ? 4 : 2) * kNF + 16;
+  constexpr int kBytes = kFA * kRow > kNodeBoxBytes ? kFA * kRow : kNodeBoxBytes;
+  __shared__ __align__(16) unsigned char smem[kBytes];
+  T* box = reinterpret_cast<T*>(smem);
+  const int la = threadIdx.x / 3, dx = (int)(threadIdx.x % 3);
   const int i = blockIdx.x * kFA + la;
-  if (i < N) {
-    const Vec4<T> p = sp[i];
-    const T u0 = p.x * ih0, u1 = p.y * ih1, u2 = p.z * ih2;
-    const T f0 = floor(u0), f1 = floor(u1), f2 = floor(u2);
-    const int b0 = (int)f0, b1 = (int)f1, b2 = (int)f2;
+  const bool valid = i < N;
+  const Vec4<T> p = valid ? sp[i] : Vec4<T>{T(0), T(0), T(0), T(0)};
+  const T u0 = p.x * ih0, u1 = p.y * ih1, u2 = p.z * ih2;
+  const T f0 = floor(u0), f1 = floor(u1), f2 = floor(u2);
+  const int b0 = (int)f0, b1 = (int)f1, b2 = (int)f2;
+  const NodeBox B =
+      block_node_box<2, 3>(valid, b0, b1, b2, n0, n1, n2, kNodeBoxBytes / (int)sizeof(T));
+  if (B.in) load_node_box(box, E, B, n0, n1, n2);
+  T e[9], gx[9], gy[9], gz[9];  // offset k = dy + 3 dz
+#pragma unroll
+  for (int k = 0; k < 9; ++k) e[k] = gx[k] = gy[k] = gz[k] = T(0);
+  if (valid) {
     T wx[4], dwx[4], wy[4], dwy[4], wz[4], dwz[4];
     phi4(u0 - f0, wx, dwx);
     phi4(u1 - f1, wy, dwy);
     phi4(u2 - f2, wz, dwz);
-    T e[9], gx[9], gy[9], gz[9];
+    auto sums = [&](auto node) {
 #pragma unroll
-    for (int k = 0; k < 9; ++k) e[k] = gx[k] = gy[k] = gz[k] = T(0);
-    int ixw[6], iyw[6];  // wrapped x and y node indices, b - 2 .. b + 3
+      for (int c = 0; c < 6; ++c) {  // plane z = b2 - 2 + c
+        T ax[6], bx[6];
 #pragma unroll
-    for (int k = 0; k < 6; ++k) {
-      ixw[k] = wrapi(b0 - 2 + k, n0);
-      iyw[k] = wrapi(b1 - 2 + k, n1);
-    }
-    for (int c = 0; c < 4; ++c) {
-      const int iz = wrapi(b2 + dz - 1 + c, n2);
-      // x pass: rows y = b1-2 .. b1+3, offsets dx = -1..1
-      T ax[6][3], bx[6][3];
-#pragma unroll
-      for (int yy = 0; yy < 6; ++yy) {
-        const T* row = E + (long)n0 * (iyw[yy] + (long)n1 * iz);
-        T v[6];
-#pragma unroll
-        for (int xx = 0; xx < 6; ++xx) v[xx] = row[ixw[xx]];
-#pragma unroll
-        for (int dx = 0; dx < 3; ++dx) {
+        for (int yy = 0; yy < 6; ++yy) {
           T s = 0, ds = 0;
 #pragma unroll
           for (int a = 0; a < 4; ++a) {
-            s += wx[a] * v[dx + a];
-            ds += dwx[a] * v[dx + a];
+            const T v = node(c, yy, a);
+            s += wx[a] * v;
+            ds += dwx[a] * v;
           }
-          ax[yy][dx] = s;
-          bx[yy][dx] = ds;
+          ax[yy] = s;
+          bx[yy] = ds;
         }
-      }
-      // y pass and z weights
 #pragma unroll
-      for (int dy = 0; dy < 3; ++dy)
-#pragma unroll
-        for (int dx = 0; dx < 3; ++dx) {
+        for (int dy = 0; dy < 3; ++dy) {
           T aa = 0, ab = 0, ba = 0;
 #pragma unroll
           for (int bb = 0; bb < 4; ++bb) {
-            aa += wy[bb] * ax[dy + bb][dx];
-            ab += dwy[bb] * ax[dy + bb][dx];
-            ba += wy[bb] * bx[dy + bb][dx];
+            aa += wy[bb] * ax[dy + bb];
+            ab += dwy[bb] * ax[dy + bb];
+            ba += wy[bb] * bx[dy + bb];
           }
-          const int k = dx + 3 * dy;
-          e[k] += wz[c] * aa;
-          gz[k] += dwz[c] * aa;
-          gy[k] += wz[c] * ab;
-          gx[k] += wz[c] * ba;
-        }
-    }
-    auto put = [&](int j, float v) { rows[la][j] = (v - norm[j]) * norm[kNF + j]; };
 #pragma unroll
-    for (int k = 0; k < 9; ++k) {
-      const int idx = k + 9 * (dz + 1);
-      put(4 * idx + 0, (float)e[k]);
-      put(4 * idx + 1, (float)(gx[k] * ih0));
-      put(4 * idx + 2, (float)(gy[k] * ih1));
-      put(4 * idx + 3, (float)(gz[k] * ih2));
-    }
-    if (dz == 0) {
-      const float t[3] = {(float)(u0 - f0), (float)(u1 - f1), (float)(u2 - f2)};
-      for (int d = 0; d < 3; ++d) {
-        float s, co;
-        sincospif(2.0f * t[d], &s, &co);
-        put(108 + 2 * d, s);
-        put(109 + 2 * d, co);
+          for (int dz = 0; dz < 3; ++dz) {
+            const int m = c - dz;  // the plane's place in the support of offset dz
+            if (m < 0 || m > 3) continue;
+            const int k = dy + 3 * dz;
+            e[k] += wz[m] * aa;
+            gz[k] += dwz[m] * aa;
+            gy[k] += wz[m] * ab;
+            gx[k] += wz[m] * ba;
+          }
+        }
       }
-      for (int j = 114; j < kNF; ++j) put(j, 0.0f);
+    };
+    if (B.in) {
+      const T* at = box + (b0 - 2 - B.lo0 + dx) +
+                    B.e0 * ((b1 - 2 - B.lo1) + B.e1 * (b2 - 2 - B.lo2));
+      const int sy = B.e0, sz = B.e0 * B.e1;
+      sums([&](int c, int yy, int a) { return at[c * sz + yy * sy + a]; });
+    } else {
+      int ix[4], iy[6], iz[6];
+#pragma unroll
+      for (int k = 0; k < 6; ++k) {
+        iy[k] = wrapi(b1 - 2 + k, n1);
+        iz[k] = wrapi(b2 - 2 + k, n2);
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k) ix[k] = wrapi(b0 - 2 + dx + k, n0);
+      sums([&](int c, int yy, int a) {
+        return E[(long)n0 * (iy[yy] + (long)n1 * iz[c]) + ix[a]];
+      });
     }
   }
+  __syncthreads();  // the node box is read: its memory takes the rows
+  unsigned char* row = smem + la * kRow;
+  auto scaled = [&](int j, float v) { return (v - norm[j]) * norm[kNF + j]; };
+  auto put2 = [&](int j, float v0, float v1) {  // columns j, j + 1 (j even)
+    const float a = scaled(j, v0), b = scaled(j + 1, v1);
+    if (F32)
+      *reinterpret_cast<float2*>(row + 4 * j) = make_float2(a, b);
+    else
+      *reinterpret_cast<uint32_t*>(row + 2 * j) = pack_bf16(a, b);
+  };
+  if (valid) {
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+      const int j = 4 * (dx + 3 * k);
+      const float4 sh = *reinterpret_cast<const float4*>(norm + j);
+      const float4 sc = *reinterpret_cast<const float4*>(norm + kNF + j);
+      const float v0 = ((float)e[k] - sh.x) * sc.x;
+      const float v1 = ((float)(gx[k] * ih0) - sh.y) * sc.y;
+      const float v2 = ((float)(gy[k] * ih1) - sh.z) * sc.z;
+      const float v3 = ((float)(gz[k] * ih2) - sh.w) * sc.w;
+      if (F32)
+        *reinterpret_cast<float4*>(row + 4 * j) = make_float4(v0, v1, v2, v3);
+      else
+        *reinterpret_cast<uint2*>(row + 2 * j) = make_uint2(pack_bf16(v0, v1), pack_bf16(v2, v3));
+    }
+    const float t = (float)(dx == 0 ? u0 - f0 : dx == 1 ? u1 - f1 : u2 - f2);
+    float s, co;
+    sincospif(2.0f * t, &s, &co);
+    put2(108 + 2 * dx, s, co);
+    for (int j = 114 + 2 * dx; j < kNF; j += 6) put2(j, 0.0f, 0.0f);
+  }
   __syncthreads();
-  // rows out: 16-byte chunks (8 bf16 or 4 floats)
-  const int per = f32 ? kNF / 4 : kNF / 8;
+  // rows out: 16-byte pieces (8 bf16 or 4 floats)
+  constexpr int per = F32 ? kNF / 4 : kNF / 8;
   for (int t = threadIdx.x; t < kFA * per; t += blockDim.x) {
     const int a = t / per, ch = t % per;
     const int ii = blockIdx.x * kFA + a;
     if (ii >= N) continue;
     const long r = sorted_out ? ii : sidx[ii];
-    if (f32) {
-      const float4 v = *reinterpret_cast<const float4*>(&rows[a][4 * ch]);
-      reinterpret_cast<float4*>(out)[r * (kNF / 4) + ch] = v;
-    } else {
-      const float* f = &rows[a][8 * ch];
-      uint4 v;
-      v.x = pack_bf16(f[0], f[1]);
-      v.y = pack_bf16(f[2], f[3]);
-      v.z = pack_bf16(f[4], f[5]);
-      v.w = pack_bf16(f[6], f[7]);
-      reinterpret_cast<uint4*>(out)[r * (kNF / 8) + ch] = v;
-    }
+    reinterpret_cast<uint4*>(out)[r * per + ch] =
+        *reinterpret_cast<const uint4*>(smem + a * kRow + 16 * ch);
   }
 }
 
@@ -299,73 +323,191 @@ __device__ __forceinline__ void hidden_layer(const uint32_t (&A)[4][4], const ui
     }
 }
 
-// Forward pass: Y (N x 8) = network(X).
-__global__ void __launch_bounds__(128) k_mlp_fwd(const __nv_bfloat16* __restrict__ X, long N,
-                                                 const uint2* __restrict__ pk,
-                                                 const float* __restrict__ par,
-                                                 float* __restrict__ Y) {
-  __shared__ uint2 sw[kPkN];
-  __shared__ float sb[3 * kH + kNO];
-  for (int i = threadIdx.x; i < kPkN; i += blockDim.x) sw[i] = pk[i];
-  for (int i = threadIdx.x; i < kH; i += blockDim.x) {
-    sb[i] = par[kOffB1 + i];
-    sb[kH + i] = par[kOffB2 + i];
-    sb[2 * kH + i] = par[kOffB3 + i];
-  }
-  if (threadIdx.x < kNO) sb[3 * kH + threadIdx.x] = par[kOffB4 + threadIdx.x];
-  __syncthreads();
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], const void* p) {
+  const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(a)
+               : "memory");
+}
+
+__device__ __forceinline__ void cp_async16(void* dst, const void* src, int bytes) {
+  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(d), "l"(src), "r"(bytes)
+               : "memory");
+}
+
+__device__ __forceinline__ void cp_async4(void* dst, const void* src, int bytes) {
+  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;\n" ::"r"(d), "l"(src), "r"(bytes)
+               : "memory");
+}
+
+// Feature rows in shared memory: the 16-byte piece q of row r lies at piece
+// q ^ (r & 7), so that the eight rows of an ldmatrix lie in distinct banks.
+__device__ __forceinline__ __nv_bfloat16* x_piece(__nv_bfloat16* x, int r, int q) {
+  return x + r * kNF + 8 * (q ^ (r & 7));
+}
+
+// A fragment of layer 1: rows row0 .. row0 + 15, k-step ks.
+__device__ __forceinline__ void frag_x(uint32_t (&a)[4], __nv_bfloat16* x, int row0, int ks,
+                                       int lane) {
+  const int j = lane >> 3, r = lane & 7;
+  ldsm4(a, x_piece(x, row0 + r + 8 * (j & 1), 2 * ks + (j >> 1)));
+}
+
+// Forward pass, 32 rows per warp and step: two 16-row tiles share every weight
+// fragment (16 rows per warp read the fragments from shared memory twice as
+// often as the tensor cores could use them), and the next 32 rows are copied
+// into the warp's other buffer meanwhile.  Either the outputs are stored (Y,
+// N x 8), or, with sp given, the rows are the sorted atoms and the correction
+// is added to the forces of atom o = sidx[row]: F_o += c_o s y.
+// x16: rows start on 16-byte boundaries (else they are copied by words).
+// What bounds it: 132 mma and 96 tanh.approx per 16 rows and lane.  262,144
+// rows: 50 -> 29 us; with the correction as its last step instead of a kernel
+// that reads the outputs back, 64 -> 41.
+constexpr int kFwdWarps = 8, kFwdRows = 32;
+struct FwdShared {
+  __nv_bfloat16 x[kFwdWarps][2][kFwdRows * kNF];
+  uint2 w[kPkN];
+  float b[3 * kH + kNO];
+};
+static_assert(sizeof(FwdShared) <= 227 * 1024, "shared memory of one block");
+
+template <typename T>
+struct Correction {
+  const Vec4<T>* sp;
+  const int* sidx;
+  T s;
+  T* F;
+};
+
+template <typename T>
+__global__ void __launch_bounds__(32 * kFwdWarps, 1)
+    k_mlp_fwd(const __nv_bfloat16* __restrict__ X, long N, int x16, const uint2* __restrict__ pk,
+              const float* __restrict__ par, float* __restrict__ Y, Correction<T> C) {
+  extern __shared__ __align__(16) unsigned char mlp_smem[];
+  FwdShared& S = *reinterpret_cast<FwdShared*>(mlp_smem);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lane >> 2, c2 = (lane & 3) * 2;
-  const uint32_t* Xw = reinterpret_cast<const uint32_t*>(X);
-  for (long tile = (long)blockIdx.x * 4 + warp; tile * 16 < N; tile += (long)gridDim.x * 4) {
-    const long ra = tile * 16 + g, rb = ra + 8;
-    const bool va = ra < N, vb = rb < N;
+  auto stage = [&](int st, long tile) {
+    __nv_bfloat16* x = S.x[warp][st];
+    const long r0 = tile * kFwdRows;
+    if (x16) {
+#pragma unroll
+      for (int t = lane; t < kFwdRows * (kNF / 8); t += 32) {
+        const int r = t / (kNF / 8), q = t % (kNF / 8);
+        const bool ok = r0 + r < N;
+        cp_async16(x_piece(x, r, q), X + (ok ? r0 + r : 0) * kNF + 8 * q, ok ? 16 : 0);
+      }
+    } else {
+      for (int t = lane; t < kFwdRows * (kNF / 2); t += 32) {
+        const int r = t / (kNF / 2), q = t % (kNF / 2);
+        const bool ok = r0 + r < N;
+        cp_async4(x_piece(x, r, q >> 2) + 2 * (q & 3), X + (ok ? r0 + r : 0) * kNF + 2 * q,
+                  ok ? 4 : 0);
+      }
+    }
+  };
+  const long first = (long)blockIdx.x * kFwdWarps + warp, step = (long)gridDim.x * kFwdWarps;
+  if (first * kFwdRows < N) stage(0, first);
+  asm volatile("cp.async.commit_group;\n" ::: "memory");
+  for (int i = threadIdx.x; i < kPkN; i += blockDim.x) S.w[i] = pk[i];
+  for (int i = threadIdx.x; i < kH; i += blockDim.x) {
+    S.b[i] = par[kOffB1 + i];
+    S.b[kH + i] = par[kOffB2 + i];
+    S.b[2 * kH + i] = par[kOffB3 + i];
+  }
+  if (threadIdx.x < kNO) S.b[3 * kH + threadIdx.x] = par[kOffB4 + threadIdx.x];
+  __syncthreads();
+  int st = 0;
+  for (long tile = first; tile * kFwdRows < N; tile += step, st ^= 1) {
+    if ((tile + step) * kFwdRows < N) stage(st ^ 1, tile + step);
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+    asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+    __syncwarp();
+    // what the correction needs, ahead of the products that hide its latency
+    T cf[4] = {}, fo[4][2] = {};
+    T* fp[4] = {};
+    if (C.sp && c2 < 3)
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const long r = tile * kFwdRows + 16 * (q >> 1) + 8 * (q & 1) + g;
+        if (r >= N) continue;
+        cf[q] = C.sp[r].w * C.s;
+        fp[q] = C.F + 3 * (size_t)C.sidx[r] + c2;
+        fo[q][0] = fp[q][0];
+        if (c2 == 0) fo[q][1] = fp[q][1];
+      }
+    float acc[2][8][4];
+    uint32_t A[2][4][4];
+    auto clear = [&] {
+#pragma unroll
+      for (int m = 0; m < 2; ++m)
+#pragma unroll
+        for (int nt = 0; nt < 8; ++nt)
+#pragma unroll
+          for (int c = 0; c < 4; ++c) acc[m][nt][c] = 0.f;
+    };
     // layer 1: K = 128 (8 k-steps), N = 64 (8 tiles)
-    float acc[8][4];
-#pragma unroll
-    for (int nt = 0; nt < 8; ++nt)
-#pragma unroll
-      for (int c = 0; c < 4; ++c) acc[nt][c] = 0.f;
-    // all 32 fragment words of the tile's two rows first (loads in flight
-    // together), then the 64 products
-    uint32_t xa[8][4];
+    clear();
 #pragma unroll
     for (int ks = 0; ks < 8; ++ks) {
-      const int w0 = (16 * ks + c2) >> 1, w1 = (16 * ks + 8 + c2) >> 1;
-      xa[ks][0] = va ? __ldg(Xw + ra * (kNF / 2) + w0) : 0u;
-      xa[ks][1] = vb ? __ldg(Xw + rb * (kNF / 2) + w0) : 0u;
-      xa[ks][2] = va ? __ldg(Xw + ra * (kNF / 2) + w1) : 0u;
-      xa[ks][3] = vb ? __ldg(Xw + rb * (kNF / 2) + w1) : 0u;
-    }
-#pragma unroll
-    for (int ks = 0; ks < 8; ++ks)
+      uint32_t xa[2][4];
+      frag_x(xa[0], S.x[warp][st], 0, ks, lane);
+      frag_x(xa[1], S.x[warp][st], 16, ks, lane);
 #pragma unroll
       for (int nt = 0; nt < 8; ++nt) {
-        const uint2 b = sw[kPk1 + (ks * 8 + nt) * 32 + lane];
-        mma16816(acc[nt], xa[ks][0], xa[ks][1], xa[ks][2], xa[ks][3], b.x, b.y);
+        const uint2 b = S.w[kPk1 + (ks * 8 + nt) * 32 + lane];
+#pragma unroll
+        for (int m = 0; m < 2; ++m)
+          mma16816(acc[m][nt], xa[m][0], xa[m][1], xa[m][2], xa[m][3], b.x, b.y);
       }
-    uint32_t A[4][4];
-    next_a(acc, sb, c2, A);
-    hidden_layer(A, sw + kPk2, lane, acc);
-    next_a(acc, sb + kH, c2, A);
-    hidden_layer(A, sw + kPk3, lane, acc);
-    next_a(acc, sb + 2 * kH, c2, A);
+    }
+    next_a(acc[0], S.b, c2, A[0]);
+    next_a(acc[1], S.b, c2, A[1]);
+#pragma unroll
+    for (int l = 0; l < 2; ++l) {
+      const uint2* w = S.w + (l ? kPk3 : kPk2);
+      clear();
+#pragma unroll
+      for (int ks = 0; ks < 4; ++ks)
+#pragma unroll
+        for (int nt = 0; nt < 8; ++nt) {
+          const uint2 b = w[(ks * 8 + nt) * 32 + lane];
+#pragma unroll
+          for (int m = 0; m < 2; ++m)
+            mma16816(acc[m][nt], A[m][ks][0], A[m][ks][1], A[m][ks][2], A[m][ks][3], b.x, b.y);
+        }
+      next_a(acc[0], S.b + (l + 1) * kH, c2, A[0]);
+      next_a(acc[1], S.b + (l + 1) * kH, c2, A[1]);
+    }
     // output layer: N = 8 (one tile)
-    float o[4] = {0.f, 0.f, 0.f, 0.f};
+    float o[2][4] = {{0.f, 0.f, 0.f, 0.f}, {0.f, 0.f, 0.f, 0.f}};
 #pragma unroll
     for (int ks = 0; ks < 4; ++ks) {
-      const uint2 b = sw[kPk4 + ks * 32 + lane];
-      mma16816(o, A[ks][0], A[ks][1], A[ks][2], A[ks][3], b.x, b.y);
+      const uint2 b = S.w[kPk4 + ks * 32 + lane];
+#pragma unroll
+      for (int m = 0; m < 2; ++m)
+        mma16816(o[m], A[m][ks][0], A[m][ks][1], A[m][ks][2], A[m][ks][3], b.x, b.y);
     }
-    const float* b4 = sb + 3 * kH;
-    if (va) {
-      Y[ra * kNO + c2] = o[0] + b4[c2];
-      Y[ra * kNO + c2 + 1] = o[1] + b4[c2 + 1];
+    const float b40 = S.b[3 * kH + c2], b41 = S.b[3 * kH + c2 + 1];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const long r = tile * kFwdRows + 16 * (q >> 1) + 8 * (q & 1) + g;
+      const float y0 = o[q >> 1][2 * (q & 1)] + b40, y1 = o[q >> 1][2 * (q & 1) + 1] + b41;
+      if (r >= N) continue;
+      if (C.sp) {
+        if (c2 < 3) {
+          fp[q][0] = fo[q][0] + cf[q] * (T)y0;
+          if (c2 == 0) fp[q][1] = fo[q][1] + cf[q] * (T)y1;
+        }
+      } else {
+        Y[r * kNO + c2] = y0;
+        Y[r * kNO + c2 + 1] = y1;
+      }
     }
-    if (vb) {
-      Y[rb * kNO + c2] = o[2] + b4[c2];
-      Y[rb * kNO + c2 + 1] = o[3] + b4[c2 + 1];
-    }
+    __syncwarp();  // the buffer is read: the next step fills it
   }
 }
 
@@ -405,7 +547,7 @@ constexpr int kTA = 128, kTGrid = 152;  // atoms per tile, most blocks (partials
 constexpr int kHS = kH + 8;             // row pitch: 8 rows of an ldmatrix in distinct banks
 
 struct TrainShared {
-  __nv_bfloat16 x[2][kTA * kNF];  // 16-byte pieces of row r at piece ^ (r & 7)
+  __nv_bfloat16 x[2][kTA * kNF];  // pieces as in x_piece
   __nv_bfloat16 h[3][kTA * kHS];
   __nv_bfloat16 d[3][kTA * kHS];
   __nv_bfloat16 dy[kTA * kNO];
@@ -418,14 +560,6 @@ static_assert(offsetof(TrainShared, h) % 16 == 0 && offsetof(TrainShared, d) % 1
                   offsetof(TrainShared, dy) % 16 == 0 && offsetof(TrainShared, w) % 16 == 0 &&
                   offsetof(TrainShared, loss) % 8 == 0,
               "alignment of the shared-memory rows");
-
-__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], const void* p) {
-  const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"(a)
-               : "memory");
-}
 
 __device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], const void* p) {
   const uint32_t a = (uint32_t)__cvta_generic_to_shared(p);
@@ -443,17 +577,6 @@ __device__ __forceinline__ void ldsm2t(uint32_t (&r)[2], const void* p) {
                : "memory");
 }
 
-__device__ __forceinline__ void cp_async16(void* dst, const void* src, int bytes) {
-  const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(d), "l"(src), "r"(bytes)
-               : "memory");
-}
-
-// Element of the swizzled feature rows: row r, 16-byte piece q.
-__device__ __forceinline__ const __nv_bfloat16* x_piece(const __nv_bfloat16* x, int r, int q) {
-  return x + r * kNF + 8 * (q ^ (r & 7));
-}
-
 // A fragments of rows 16 m0.. (the activation columns) for k-step ks of a
 // tile [atom][column]: matrices (atoms 0-7 / 8-15) x (columns 0-7 / 8-15) in
 // the order a0 a1 a2 a3 of the mma.
@@ -463,7 +586,7 @@ __device__ __forceinline__ void frag_a(uint32_t (&a)[4], const __nv_bfloat16* t,
   ldsm4t(a, t + (16 * ks + r + 8 * (j >> 1)) * kHS + 16 * m0 + 8 * (j & 1));
 }
 
-__device__ __forceinline__ void frag_ax(uint32_t (&a)[4], const __nv_bfloat16* x, int ks, int m0,
+__device__ __forceinline__ void frag_ax(uint32_t (&a)[4], __nv_bfloat16* x, int ks, int m0,
                                         int lane) {
   const int j = lane >> 3, r = lane & 7;
   ldsm4t(a, x_piece(x, 16 * ks + r + 8 * (j >> 1), 2 * m0 + (j & 1)));
@@ -527,8 +650,8 @@ __global__ void __launch_bounds__(256, 1) k_mlp_train(
     const __nv_bfloat16* __restrict__ X, const float* __restrict__ T, long N, long per,
     float inv_n, const uint2* __restrict__ pk, const float* __restrict__ par,
     float* __restrict__ part, double* __restrict__ lpart) {
-  extern __shared__ __align__(16) unsigned char train_smem[];
-  TrainShared& S = *reinterpret_cast<TrainShared*>(train_smem);
+  extern __shared__ __align__(16) unsigned char mlp_smem[];
+  TrainShared& S = *reinterpret_cast<TrainShared*>(mlp_smem);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lane >> 2, c2 = (lane & 3) * 2;
   const long ntile = cdiv(N, (long)kTA);
@@ -538,7 +661,7 @@ __global__ void __launch_bounds__(256, 1) k_mlp_train(
       const int r = t / (kNF / 8), q = t % (kNF / 8);
       const long i = tile * kTA + r;
       const bool ok = i < N;
-      cp_async16(const_cast<__nv_bfloat16*>(x_piece(S.x[st], r, q)), X + (ok ? i : 0) * kNF + 8 * q,
+      cp_async16(x_piece(S.x[st], r, q), X + (ok ? i : 0) * kNF + 8 * q,
                  ok ? 16 : 0);
     }
     asm volatile("cp.async.commit_group;\n" ::: "memory");
@@ -584,9 +707,8 @@ __global__ void __launch_bounds__(256, 1) k_mlp_train(
       for (int c = 0; c < 4; ++c) acc[nt][c] = 0.f;
 #pragma unroll
     for (int ks = 0; ks < 8; ++ks) {
-      const int j = lane >> 3, r = lane & 7;
       uint32_t xa[4];
-      ldsm4(xa, x_piece(S.x[st], row0 + r + 8 * (j & 1), 2 * ks + (j >> 1)));
+      frag_x(xa, S.x[st], row0, ks, lane);
 #pragma unroll
       for (int nt = 0; nt < 8; ++nt) {
         const uint2 b = S.w[kPk1 + (ks * 8 + nt) * 32 + lane];
@@ -777,20 +899,6 @@ __global__ void k_adam(float* __restrict__ par, float* __restrict__ m, float* __
   par[p] -= lr * (mi / bc1) / (sqrtf(vi / bc2) + 1e-8f);
 }
 
-// forces_o += c_o * s * y_i for the atom o at sorted position i (outputs in
-// sorted order, forces in input order)
-template <typename T>
-__global__ void k_mlp_correct(const Vec4<T>* __restrict__ sp, const int* __restrict__ sidx,
-                              const float* __restrict__ Y, int N, float s, T* __restrict__ F) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= N) return;
-  const T c = sp[i].w * (T)s;
-  const size_t o = (size_t)sidx[i];
-  F[3 * o + 0] += c * (T)Y[(size_t)i * kNO + 0];
-  F[3 * o + 1] += c * (T)Y[(size_t)i * kNO + 1];
-  F[3 * o + 2] += c * (T)Y[(size_t)i * kNO + 2];
-}
-
 // ------------------------------------------------------------------ host
 
 static uint64_t splitmix64(uint64_t& s) {
@@ -802,24 +910,23 @@ static uint64_t splitmix64(uint64_t& s) {
 
 // Launch geometry: functions of N only, so that the partial sums and hence the
 // results do not depend on the device.
-static long fwd_blocks(long N) { return std::min(cdiv(cdiv(N, 16L), 4L), 152L * 8); }
+static long fwd_blocks(long N) { return std::min(cdiv(N, (long)kFwdWarps * kFwdRows), 152L); }
 static void train_geometry(long N, long& grid, long& per) {
   const long ntile = cdiv(N, (long)kTA);
   per = cdiv(ntile, (long)kTGrid);
   grid = per > 0 ? cdiv(ntile, per) : 0;
 }
 
-// Buffers of mls6_mlp_apply (features and outputs of N atoms).
+// Buffer of mls6_mlp_apply (features of N atoms).
 static int grow(Mlp* m, long N) {
   if (N <= m->cap) return MLS6_OK;
   if (m->d_X) cudaFree(m->d_X);
-  if (m->d_Y) cudaFree(m->d_Y);
   m->d_X = nullptr;
-  m->d_Y = nullptr;
   m->cap = 0;
-  if (cudaMalloc((void**)&m->d_X, sizeof(__nv_bfloat16) * kNF * N) != cudaSuccess ||
-      cudaMalloc((void**)&m->d_Y, sizeof(float) * kNO * N) != cudaSuccess)
+  if (cudaMalloc((void**)&m->d_X, sizeof(__nv_bfloat16) * kNF * N) != cudaSuccess) {
+    m->d_X = nullptr;
     return MLS6_ERR_NOMEM;
+  }
   m->cap = N;
   return MLS6_OK;
 }
@@ -844,10 +951,12 @@ static int repack(Mlp* m) {
   return MLS6_OK;
 }
 
-static int forward(Mlp* m, const void* X, long N, float* Y) {
+template <typename T>
+static int forward(Mlp* m, const void* X, long N, float* Y, Correction<T> C, cudaStream_t st) {
   if (N <= 0) return MLS6_OK;
-  k_mlp_fwd<<<fwd_blocks(N), 128, 0, m->stream>>>((const __nv_bfloat16*)X, N, m->d_pack, m->d_par,
-                                                  Y);
+  k_mlp_fwd<T><<<fwd_blocks(N), 32 * kFwdWarps, sizeof(FwdShared), st>>>(
+      (const __nv_bfloat16*)X, N, (reinterpret_cast<uintptr_t>(X) & 15) == 0, m->d_pack, m->d_par,
+      Y, C);
   CK(cudaGetLastError());
   return MLS6_OK;
 }
@@ -883,8 +992,8 @@ static int read_loss(Mlp* m, double* loss) {
 
 static void free_mlp(Mlp* m) {
   if (!m) return;
-  void* bufs[] = {m->d_par, m->d_m, m->d_v, m->d_pack, m->d_norm, m->d_X, m->d_Y, m->d_part,
-                  m->d_lpart, m->d_grad, m->d_loss};
+  void* bufs[] = {m->d_par, m->d_m, m->d_v, m->d_pack, m->d_norm, m->d_X, m->d_part, m->d_lpart,
+                  m->d_grad, m->d_loss};
   for (void* b : bufs)
     if (b) cudaFree(b);
   delete m;
@@ -895,12 +1004,24 @@ static int features_t(Plan* p, Mlp* m, void* out, int f32, bool sorted_out, cuda
   const Level& L1 = p->lv[1];
   const int N = (int)p->N;
   if (N == 0) return MLS6_OK;
-  k_features<T><<<cdiv(N, kFA), 3 * kFA, 0, st>>>(
+  auto kern = f32 ? k_features<T, true> : k_features<T, false>;
+  kern<<<cdiv(N, kFA), 3 * kFA, 0, st>>>(
       (const Vec4<T>*)p->d_sorted, p->d_sorted_idx, N, (const T*)p->d_et[1], L1.n[0], L1.n[1],
-      L1.n[2], (T)(1.0 / L1.h[0]), (T)(1.0 / L1.h[1]), (T)(1.0 / L1.h[2]), m->d_norm, out, f32,
+      L1.n[2], (T)(1.0 / L1.h[0]), (T)(1.0 / L1.h[1]), (T)(1.0 / L1.h[2]), m->d_norm, out,
       sorted_out ? 1 : 0);
   CK(cudaGetLastError());
   return MLS6_OK;
+}
+
+// Features in sorted order, then the network with the correction as its last
+// step, on the plan's stream.
+template <typename T> static int apply_t(Plan* p, Mlp* m, void* forces) {
+  const int rc = features_t<T>(p, m, m->d_X, 0, true, p->stream);
+  if (rc) return rc;
+  return forward(m, m->d_X, p->N, nullptr,
+                 Correction<T>{(const Vec4<T>*)p->d_sorted, p->d_sorted_idx, (T)m->out_scale,
+                               (T*)forces},
+                 p->stream);
 }
 
 }  // namespace mls6
@@ -926,9 +1047,11 @@ int mls6_mlp_create(mls6_mlp_t** out, uint64_t seed) {
     free_mlp(m);
     return MLS6_ERR_NOMEM;
   }
-  // shared memory of the training kernel (above 48 KB)
-  if (cudaFuncSetAttribute(k_mlp_train, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)sizeof(TrainShared)) != cudaSuccess) {
+  // shared memory above 48 KB
+  const auto dyn = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  if (cudaFuncSetAttribute(k_mlp_train, dyn, (int)sizeof(TrainShared)) != cudaSuccess ||
+      cudaFuncSetAttribute(k_mlp_fwd<float>, dyn, (int)sizeof(FwdShared)) != cudaSuccess ||
+      cudaFuncSetAttribute(k_mlp_fwd<double>, dyn, (int)sizeof(FwdShared)) != cudaSuccess) {
     free_mlp(m);
     return MLS6_ERR_CUDA;
   }
@@ -1015,7 +1138,8 @@ int mls6_mlp_features(mls6_plan_t* plan, const mls6_mlp_t* mm, void* out, int fm
 int mls6_mlp_forward(mls6_mlp_t* mm, const void* X, int64_t N, float* Y) {
   if (!mm || N < 0 || (N > 0 && (!kernel_addressable(X) || !kernel_addressable(Y))))
     return MLS6_ERR_ARG;
-  return forward(reinterpret_cast<Mlp*>(mm), X, N, Y);
+  Mlp* m = reinterpret_cast<Mlp*>(mm);
+  return forward(m, X, N, Y, Correction<float>{}, m->stream);
 }
 
 int mls6_mlp_grad(mls6_mlp_t* mm, const void* X, const float* T, int64_t N, float* grad,
@@ -1058,23 +1182,7 @@ int mls6_mlp_apply(mls6_plan_t* plan, mls6_mlp_t* mm, void* forces) {
   if (!kernel_addressable(forces)) return MLS6_ERR_ARG;
   int rc = grow(m, N);
   if (rc) return rc;
-  cudaStream_t saved = m->stream;
-  m->stream = p->stream;
-  rc = p->prec == MLS6_FP64 ? features_t<double>(p, m, m->d_X, 0, true, p->stream)
-                            : features_t<float>(p, m, m->d_X, 0, true, p->stream);
-  if (!rc) rc = forward(m, m->d_X, N, m->d_Y);
-  m->stream = saved;
-  if (rc) return rc;
-  if (p->prec == MLS6_FP64)
-    k_mlp_correct<double><<<cdiv(N, 256), 256, 0, p->stream>>>(
-        (const Vec4<double>*)p->d_sorted, p->d_sorted_idx, m->d_Y, (int)N, m->out_scale,
-        (double*)forces);
-  else
-    k_mlp_correct<float><<<cdiv(N, 256), 256, 0, p->stream>>>(
-        (const Vec4<float>*)p->d_sorted, p->d_sorted_idx, m->d_Y, (int)N, m->out_scale,
-        (float*)forces);
-  CK(cudaGetLastError());
-  return MLS6_OK;
+  return p->prec == MLS6_FP64 ? apply_t<double>(p, m, forces) : apply_t<float>(p, m, forces);
 }
 
 void mls6_mlp_destroy(mls6_mlp_t* mm) { free_mlp(reinterpret_cast<Mlp*>(mm)); }

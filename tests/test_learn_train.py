@@ -66,3 +66,37 @@ def test_gradient_of_quarters(gpu_lib, mlp_ref):
     gq = sum(q[1].double() for q in parts) / 4
     assert loss == pytest.approx(sum(q[0] for q in parts) / 4, rel=1e-12)
     assert (g.double() - gq).norm() <= 1e-3 * gq.norm()
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@pytest.mark.parametrize("N", [1, 31, 33, 1000])
+def test_apply_is_forward_of_the_features(gpu_lib, mlp_ref, N, prec):
+    """F + c s y with y from the stored features: one product and one sum
+    apart (2 u of the larger operand)."""
+    dt = torch.float64 if prec == "fp64" else torch.float32
+    rng = np.random.default_rng(N)
+    pos = torch.tensor(np.c_[rng.uniform(0, 9, (N, 3)), rng.uniform(0.5, 1.5, N)], dtype=dt,
+                       device="cuda")
+    plan = gpu_lib.Plan((9.0, 9.0, 9.0), N, 2.2, 0.75, 3, precision=prec)
+    plan.evaluate(pos, virial=False)
+    m = gpu_lib.MLP(0)
+    m.set_params(_params(mlp_ref, 3))
+    m.set_norm(np.zeros(128), np.full(128, 0.1), 0.7)
+    y = m.forward(m.features(plan, fmt="bf16"))[:, :3].to(dt)
+    F = torch.ones((N, 3), dtype=dt, device="cuda")
+    torch.cuda.synchronize()
+    m.apply(plan, F)
+    torch.cuda.synchronize()
+    add = pos[:, 3:] * torch.tensor(0.7, dtype=torch.float32).to(dt) * y
+    u = 2.0**-24 if prec == "fp32" else 2.0**-53
+    assert (F - (1 + add)).abs().max() <= 4 * u * (1 + add.abs().max())
+
+
+def test_forward_of_rows_off_16_bytes(gpu_lib, mlp_ref):
+    """Rows that start on a 4-byte boundary give what aligned rows give."""
+    m = gpu_lib.MLP(0)
+    m.set_params(_params(mlp_ref, 4))
+    X = torch.randn(300 * 128 + 2, device="cuda").to(torch.bfloat16)
+    off = X[2:].view(300, 128)
+    assert off.data_ptr() % 16 == 4
+    assert torch.equal(m.forward(off), m.forward(off.clone()))
