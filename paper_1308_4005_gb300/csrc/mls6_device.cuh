@@ -146,7 +146,8 @@ __device__ __forceinline__ long pdl_begin() {
 
 // A block of consecutive cell-sorted atoms touches a compact box of grid
 // nodes.  Where that box fits into kNodeBoxBytes, the block keeps it in shared
-// memory.  One buffer per kernel, whatever stages it runs.
+// memory: the anterpolation sums there, the features read there.  One buffer
+// per kernel, whatever stages it runs.
 constexpr int kNodeBoxBytes = 24 * 1024;
 __device__ __forceinline__ unsigned char* node_box_smem() {
   __shared__ __align__(16) unsigned char buf[kNodeBoxBytes];
@@ -355,7 +356,7 @@ template <> struct Fixed<float> {
   using U = unsigned int;
   static constexpr int kBits = 30;
   __device__ static float pow2(int s) { return __int_as_float((127 + s) << 23); }
-  __device__ static I to_fixed(float v, float scale) { return __float2int_rn(v * scale); }
+  __device__ static I to_fixed(float v) { return __float2int_rn(v); }  // v already scaled
   __device__ static float from_fixed(I v, float iscale) { return (float)v * iscale; }
 };
 template <> struct Fixed<double> {
@@ -363,7 +364,7 @@ template <> struct Fixed<double> {
   using U = unsigned long long;
   static constexpr int kBits = 61;
   __device__ static double pow2(int s) { return __longlong_as_double((long long)(1023 + s) << 52); }
-  __device__ static I to_fixed(double v, double scale) { return __double2ll_rn(v * scale); }
+  __device__ static I to_fixed(double v) { return __double2ll_rn(v); }
   __device__ static double from_fixed(I v, double iscale) { return (double)v * iscale; }
 };
 

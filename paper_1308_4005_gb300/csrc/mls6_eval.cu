@@ -412,8 +412,7 @@ static int eval_lb_t(Plan* p, const T* pos, const T* sigma, const T* eps, T* for
   nl += launch_pair<T>(p, false, st, true);
   if (p->spectral) {
     CK(cudaMemsetAsync(p->d_lbq, 0, sizeof(T) * 7 * np1, st));
-    for (int m = 0; m < 7; ++m)
-      nl += launch_anterp<T>(p, st, m, false, (T*)p->d_lbq + (size_t)m * np1);
+    nl += launch_anterp_lb<T>(p, st, p->d_lbq);
     nl += launch_spectral<T>(p, false, true, st);
   }
   for (int m = 0; m < 7 && !p->spectral; ++m) {

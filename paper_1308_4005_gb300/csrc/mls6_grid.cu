@@ -23,89 +23,110 @@ namespace mls6 {
 // overlap of the atoms' supports; otherwise its atoms add to the grid
 // directly.  Both paths add the same integers, so the grid does not depend
 // on the path either.
-constexpr int kAnterpBoxBytes = 24 * 1024;
+// What bounds it: instruction issue (per node a product, a conversion and an
+// atomic), in FP64 also the FP64 pipe (2 lanes per cycle and SM).  The power of
+// two 2^s is folded into the coefficient (exact), not applied per node; the
+// box is cleared by 16-byte stores and flushed with one-period wraps; 64-bit
+// sums in shared memory are two 32-bit atomics with the carry from the first
+// (a 64-bit shared atomic add is a compare-and-swap loop).  Six
+// blocks per SM (40 registers) hide the latencies that four do not.  1M-atom
+// cube 74 -> 66 us (43 without the flush, 52 without the shared atomics),
+// 4M-atom slab 203 -> 162, 98,765 atoms in FP64 74 -> 54.
+// NC = 7: all Lorentz-Berthelot channels in one launch, with the supports and
+// the weights formed once: 97 us at 262,144 atoms, 148 in seven launches.
 
-template <typename T, int NP = 4>
+// Sums of a box in shared memory: 32-bit words, or two planes of them.
+template <typename T> struct BoxSum;
+template <> struct BoxSum<float> {
+  unsigned* w;
+  static constexpr int kCap = kNodeBoxBytes / 4;
+  __device__ explicit BoxSum(unsigned char* m) : w(reinterpret_cast<unsigned*>(m)) {}
+  __device__ void add(int i, int v) const { atomicAdd(w + i, (unsigned)v); }
+  __device__ unsigned take(int i) const { return w[i]; }
+};
+template <> struct BoxSum<double> {
+  unsigned* w;
+  static constexpr int kCap = kNodeBoxBytes / 8;
+  __device__ explicit BoxSum(unsigned char* m) : w(reinterpret_cast<unsigned*>(m)) {}
+  __device__ void add(int i, long long v) const {
+    const unsigned lo = (unsigned)v, hi = (unsigned)((unsigned long long)v >> 32);
+    const unsigned old = atomicAdd(w + i, lo);
+    atomicAdd(w + kCap + i, hi + (old + lo < lo ? 1u : 0u));
+  }
+  __device__ unsigned long long take(int i) const {
+    return (unsigned long long)w[kCap + i] << 32 | w[i];
+  }
+};
+
+struct LbCoef {
+  double c[7];
+};
+
+template <typename T, int NP = 4, int NC = 1>
 __device__ __forceinline__ void k_anterp_body(const Blk bk,
     const Vec4<T>* __restrict__ sp, int N, int n0, int n1, int n2, T ih0, T ih1, T ih2,
     const int* __restrict__ flag, double span, typename Fixed<T>::U* __restrict__ qfx,
-    const T* __restrict__ lbw, int lbm, double lbc) {
+    const T* __restrict__ lbw, int lbm, const LbCoef& lbc) {
   using U = typename Fixed<T>::U;
-  constexpr int kCap = kAnterpBoxBytes / (int)sizeof(U);
-  __shared__ U box[kCap];
-  __shared__ int lo[3], hi[3], sexp;
+  constexpr int B0 = NP / 2 - 1;  // first node of the support below base
+  unsigned char* mem = node_box_smem();
+  const BoxSum<T> box(mem);
+  __shared__ int sexp[NC];
   const long z = pdl_begin();
   sp += z;
   flag += z;
   lbw += z;
   const int i = bk.x * blockDim.x + threadIdx.x;
   const bool valid = i < N;
-  if (threadIdx.x < 3) {
-    lo[threadIdx.x] = INT_MAX;
-    hi[threadIdx.x] = INT_MIN;
+  if (threadIdx.x < NC) {
+    const int m = NC == 1 ? lbm : (int)threadIdx.x;
+    sexp[threadIdx.x] = fixed_exponent<T>(flag, span, m, m < 0 ? 0.0 : lbc.c[m]);
   }
-  if (threadIdx.x == 0) sexp = fixed_exponent<T>(flag, span, lbm, lbc);
-  Vec4<T> p = valid ? sp[i] : Vec4<T>{T(0), T(0), T(0), T(0)};
-  if (valid && lbm >= 0) {  // Lorentz-Berthelot channel: xi_m = lbc sigma^m sqrt(2 eps)
-    T s = T(1);
-    for (int k = 0; k < lbm; ++k) s *= p.w;
-    p.w = (T)lbc * s * lbw[i];
-  }
+  const Vec4<T> p = valid ? sp[i] : Vec4<T>{T(0), T(0), T(0), T(0)};
+  const T lw = valid && (NC > 1 || lbm >= 0) ? lbw[i] : T(0);
   const T u0 = p.x * ih0, u1 = p.y * ih1, u2 = p.z * ih2;
   const T f0 = floor(u0), f1 = floor(u1), f2 = floor(u2);
   const int b0 = (int)f0, b1 = (int)f1, b2 = (int)f2;
-  __syncthreads();
-  {  // bounding box of the block's supports (unwrapped node indices): warp
-     // minima and maxima first, then one shared atomic per warp and axis
-    int l0 = valid ? b0 - (NP / 2 - 1) : INT_MAX, l1 = valid ? b1 - (NP / 2 - 1) : INT_MAX;
-    int l2 = valid ? b2 - (NP / 2 - 1) : INT_MAX;
-    int h0 = valid ? b0 + NP / 2 : INT_MIN, h1 = valid ? b1 + NP / 2 : INT_MIN;
-    int h2 = valid ? b2 + NP / 2 : INT_MIN;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      l0 = min(l0, __shfl_xor_sync(0xffffffffu, l0, o));
-      l1 = min(l1, __shfl_xor_sync(0xffffffffu, l1, o));
-      l2 = min(l2, __shfl_xor_sync(0xffffffffu, l2, o));
-      h0 = max(h0, __shfl_xor_sync(0xffffffffu, h0, o));
-      h1 = max(h1, __shfl_xor_sync(0xffffffffu, h1, o));
-      h2 = max(h2, __shfl_xor_sync(0xffffffffu, h2, o));
+  const NodeBox B =
+      block_node_box<B0, NP / 2>(valid, b0, b1, b2, n0, n1, n2, BoxSum<T>::kCap);
+  const int vol = B.in ? B.e0 * B.e1 * B.e2 : 0;
+  auto clear = [&] {
+    const int words = (vol + 3) >> 2;  // of 16 bytes; kCap is a multiple of 4
+    uint4* m = reinterpret_cast<uint4*>(mem);
+    for (int t = threadIdx.x; t < words; t += blockDim.x) {
+      m[t] = make_uint4(0, 0, 0, 0);
+      if (sizeof(U) == 8) m[BoxSum<T>::kCap / 4 + t] = make_uint4(0, 0, 0, 0);
     }
-    if ((threadIdx.x & 31) == 0 && l0 != INT_MAX) {
-      atomicMin(&lo[0], l0);
-      atomicMin(&lo[1], l1);
-      atomicMin(&lo[2], l2);
-      atomicMax(&hi[0], h0);
-      atomicMax(&hi[1], h1);
-      atomicMax(&hi[2], h2);
+  };
+  clear();
+  __syncthreads();
+  T wx[NP], wy[NP], wz[NP];
+  phiw<NP>(u0 - f0, wx);
+  phiw<NP>(u1 - f1, wy);
+  phiw<NP>(u2 - f2, wz);
+  const int at = B.in ? (b0 - B0 - B.lo0) + B.e0 * ((b1 - B0 - B.lo1) + B.e1 * (b2 - B0 - B.lo2))
+                      : 0;
+  const int sy = B.e0, sz = B.e0 * B.e1;
+  for (int ch = 0; ch < NC; ++ch) {
+    const int m = NC == 1 ? lbm : ch;
+    T w = p.w;
+    if (m >= 0) {  // Lorentz-Berthelot channel: xi_m = lbc sigma^m sqrt(2 eps)
+      T s = T(1);
+      for (int k = 0; k < m; ++k) s *= p.w;
+      w = (T)lbc.c[m] * s * lw;
     }
-  }
-  __syncthreads();
-  const T scale = Fixed<T>::pow2(sexp);
-  const int e0 = hi[0] - lo[0] + 1, e1 = hi[1] - lo[1] + 1, e2 = hi[2] - lo[2] + 1;
-  const long vol = (long)e0 * e1 * e2;
-  const bool in_box = hi[0] >= lo[0] && vol <= kCap;  // the same for the whole block
-  if (in_box)
-    for (int t = threadIdx.x; t < (int)vol; t += blockDim.x) box[t] = 0;
-  __syncthreads();
-  if (valid) {
-    constexpr int B0 = NP / 2 - 1;  // first node of the support below base
-    T wx[NP], wy[NP], wz[NP];
-    phiw<NP>(u0 - f0, wx);
-    phiw<NP>(u1 - f1, wy);
-    phiw<NP>(u2 - f2, wz);
-    if (in_box) {
-      const int x0 = b0 - B0 - lo[0], y0 = b1 - B0 - lo[1], z0 = b2 - B0 - lo[2];
+    w *= Fixed<T>::pow2(sexp[NC == 1 ? 0 : ch]);
+    if (valid && B.in) {
 #pragma unroll
       for (int c = 0; c < NP; ++c)
 #pragma unroll
         for (int b = 0; b < NP; ++b) {
-          const T wyz = p.w * wy[b] * wz[c];
-          const int row = e0 * ((y0 + b) + e1 * (z0 + c)) + x0;
+          const T wyz = w * wy[b] * wz[c];
+          const int row = at + b * sy + c * sz;
 #pragma unroll
-          for (int a = 0; a < NP; ++a)
-            atomicAdd(&box[row + a], (U)Fixed<T>::to_fixed(wyz * wx[a], scale));
+          for (int a = 0; a < NP; ++a) box.add(row + a, Fixed<T>::to_fixed(wyz * wx[a]));
         }
-    } else {
+    } else if (valid) {
       int ix[NP], iy[NP], iz[NP];
 #pragma unroll
       for (int k = 0; k < NP; ++k) {
@@ -117,36 +138,41 @@ __device__ __forceinline__ void k_anterp_body(const Blk bk,
       for (int c = 0; c < NP; ++c)
 #pragma unroll
         for (int b = 0; b < NP; ++b) {
-          const T wyz = p.w * wy[b] * wz[c];
+          const T wyz = w * wy[b] * wz[c];
           const long rowi = (long)n0 * (iy[b] + (long)n1 * iz[c]);
 #pragma unroll
           for (int a = 0; a < NP; ++a)
-            atomicAdd(&qfx[rowi + ix[a]], (U)Fixed<T>::to_fixed(wyz * wx[a], scale));
+            atomicAdd(&qfx[rowi + ix[a]], (U)Fixed<T>::to_fixed(wyz * wx[a]));
         }
     }
-  }
-  if (in_box) {  // flush: one warp per box row (y, z), lanes along x
-    __syncthreads();
-    const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    for (int r = threadIdx.x >> 5; r < e1 * e2; r += nw) {
-      const int y = wrapi(lo[1] + r % e1, n1), zz = wrapi(lo[2] + r / e1, n2);
-      const long row = (long)n0 * (y + (long)n1 * zz);
-      const U* br = box + (size_t)r * e0;
-      for (int x = lane; x < e0; x += 32) {
-        const U v = br[x];
-        if (v == 0) continue;
-        atomicAdd(&qfx[row + wrapi(lo[0] + x, n0)], v);
+    if (B.in) {  // flush: one warp per box row (y, z), lanes along x
+      __syncthreads();
+      const int lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+      for (int r = threadIdx.x >> 5; r < B.e1 * B.e2; r += nw) {
+        const int c = r / B.e1, b = r - c * B.e1;
+        U* row = qfx + (long)n0 * (wrap1(B.lo1 + b, n1) + (long)n1 * wrap1(B.lo2 + c, n2));
+        for (int x = lane; x < B.e0; x += 32) {
+          const U v = box.take(r * B.e0 + x);
+          if (v != 0) atomicAdd(row + wrap1(B.lo0 + x, n0), v);
+        }
+      }
+      if (NC > 1 && ch + 1 < NC) {
+        __syncthreads();
+        clear();
+        __syncthreads();
       }
     }
+    if (NC > 1) qfx += (long)n0 * n1 * n2;
   }
 }
 
-template <typename T, int NP>
-__global__ void __launch_bounds__(kBlock) k_anterp(
+template <typename T, int NP, int NC>
+__global__ void __launch_bounds__(kBlock, sizeof(T) == 8 ? 2 : NP == 6 ? 3 : NC == 7 ? 4 : 6)
+k_anterp(
     const Vec4<T>* __restrict__ sp, int N, int n0, int n1, int n2, T ih0, T ih1, T ih2,
     const int* __restrict__ flag, double span, typename Fixed<T>::U* __restrict__ qfx,
-    const T* __restrict__ lbw, int lbm, double lbc) {
-  k_anterp_body<T, NP>(Blk::self(), sp, N, n0, n1, n2, ih0, ih1, ih2, flag, span, qfx, lbw, lbm, lbc);
+    const T* __restrict__ lbw, int lbm, const __grid_constant__ LbCoef lbc) {
+  k_anterp_body<T, NP, NC>(Blk::self(), sp, N, n0, n1, n2, ih0, ih1, ih2, flag, span, qfx, lbw, lbm, lbc);
 }
 
 // q^1 = fixed-point sums * 2^-s in the plan's precision.
@@ -178,19 +204,35 @@ double lb_coef(int m) {
   static const double binom[7] = {1, 6, 15, 20, 15, 6, 1};
   return m < 0 ? 0.0 : 0.125 * std::sqrt(binom[m]);
 }
-#endif  // MLS6_DEVICE_ONLY
+
+static LbCoef lb_coefs() {
+  LbCoef c;
+  for (int m = 0; m < 7; ++m) c.c[m] = lb_coef(m);
+  return c;
+}
 
 template <typename T> int launch_anterp(Plan* p, cudaStream_t st, int lbm, bool to_grid, void* qfx) {
   const Level& L1 = p->lv[1];
   const int N = (int)p->N;
-  const double span = support_span(p);
-  const double lbc = lb_coef(lbm);
-  launch_pdl(p->order == 5 ? k_anterp<T, 6> : k_anterp<T, 4>, cdiv(N, kBlock), kBlock, 0, st,
+  launch_pdl(p->order == 5 ? k_anterp<T, 6, 1> : k_anterp<T, 4, 1>, cdiv(N, kBlock), kBlock, 0, st,
       (const Vec4<T>*)p->d_sorted, N, L1.n[0], L1.n[1], L1.n[2], (T)(1.0 / L1.h[0]),
-      (T)(1.0 / L1.h[1]), (T)(1.0 / L1.h[2]), p->d_flag, span,
-      (typename Fixed<T>::U*)(qfx ? qfx : p->d_q1fx), (const T*)p->d_lbw, lbm, lbc);
+      (T)(1.0 / L1.h[1]), (T)(1.0 / L1.h[2]), p->d_flag, support_span(p),
+      (typename Fixed<T>::U*)(qfx ? qfx : p->d_q1fx), (const T*)p->d_lbw, lbm, lb_coefs());
   return 1 + (to_grid ? launch_from_fixed<T>(p, st, lbm, qfx) : 0);
 }
+
+// The fixed-point sums of all seven Lorentz-Berthelot channels, one after
+// another in qfx.
+template <typename T> int launch_anterp_lb(Plan* p, cudaStream_t st, void* qfx) {
+  const Level& L1 = p->lv[1];
+  const int N = (int)p->N;
+  launch_pdl(p->order == 5 ? k_anterp<T, 6, 7> : k_anterp<T, 4, 7>, cdiv(N, kBlock), kBlock, 0, st,
+      (const Vec4<T>*)p->d_sorted, N, L1.n[0], L1.n[1], L1.n[2], (T)(1.0 / L1.h[0]),
+      (T)(1.0 / L1.h[1]), (T)(1.0 / L1.h[2]), p->d_flag, support_span(p),
+      (typename Fixed<T>::U*)qfx, (const T*)p->d_lbw, 0, lb_coefs());
+  return 1;
+}
+#endif  // MLS6_DEVICE_ONLY
 
 // q^1 from the fixed-point sums.
 template <typename T> int launch_from_fixed(Plan* p, cudaStream_t st, int lbm, const void* qfx) {
@@ -722,6 +764,12 @@ template <typename T> int launch_prolong(Plan* p, int k, cudaStream_t st) {
 // -1/2 c_i (e0_i + e_i) + 1/2 c_self c_i^2; one energy partial per block.
 // The last block to finish (ticket counter, reset by that block) sums all
 // energy and virial partials in a fixed order into out[0..6].
+// What bounds it: the latency of the gathers and of a block's tail, against
+// the blocks that an SM holds: with several waves of blocks 5 per SM (48
+// registers; 4,194,304 atoms 206 us, 4 per SM 215, 6 spill and take 229), in a
+// single wave 4, which need no spill.
+// Taken back: the block's node box copied into shared memory first (the
+// gathers cost 20 of 67 us on the 1M-atom cube, the copy and its barriers 38).
 struct ReduceArgs {
   const double* wpart;
   long nw;
@@ -742,13 +790,13 @@ __device__ __forceinline__ void k_interp_body(const Blk bk,
   sp += z; sidx += z; et += z; e0 += z; floc += z;
   __shared__ double sh[32 * 7];
   __shared__ bool last;
-  int i = bk.x * blockDim.x + threadIdx.x;
+  const int i = bk.x * blockDim.x + threadIdx.x;
   T ea = T(0);
   if (i < N) {
-    Vec4<T> p = sp[i];
-    T u0 = p.x * ih0, u1 = p.y * ih1, u2 = p.z * ih2;
-    T f0 = floor(u0), f1 = floor(u1), f2 = floor(u2);
-    int b0 = (int)f0, b1 = (int)f1, b2 = (int)f2;
+    const Vec4<T> p = sp[i];
+    const T u0 = p.x * ih0, u1 = p.y * ih1, u2 = p.z * ih2;
+    const T f0 = floor(u0), f1 = floor(u1), f2 = floor(u2);
+    const int b0 = (int)f0, b1 = (int)f1, b2 = (int)f2;
     constexpr int B0 = NP / 2 - 1;
     T wx[NP], wy[NP], wz[NP], dx[NP], dy[NP], dz[NP];
     phid<NP>(u0 - f0, wx, dx);
@@ -764,24 +812,28 @@ __device__ __forceinline__ void k_interp_body(const Blk bk,
     T acc = 0, g0 = 0, g1 = 0, g2 = 0;
 #pragma unroll
     for (int c = 0; c < NP; ++c) {
+      T tv = 0, tx = 0, ty = 0;  // value, d/dx and d/dy in plane c
 #pragma unroll
       for (int b = 0; b < NP; ++b) {
         const T* row = et + (long)n0 * (iy[b] + (long)n1 * iz[c]);
         T sx = 0, sdx = 0;
 #pragma unroll
         for (int a = 0; a < NP; ++a) {
-          T v = row[ix[a]];
+          const T v = row[ix[a]];
           sx += wx[a] * v;
           sdx += dx[a] * v;
         }
-        acc += wy[b] * wz[c] * sx;
-        g0 += wy[b] * wz[c] * sdx;
-        g1 += dy[b] * wz[c] * sx;
-        g2 += wy[b] * dz[c] * sx;
+        tv += wy[b] * sx;
+        tx += wy[b] * sdx;
+        ty += dy[b] * sx;
       }
+      acc += wz[c] * tv;
+      g0 += wz[c] * tx;
+      g1 += wz[c] * ty;
+      g2 += dz[c] * tv;
     }
-    int o = sidx[i];
-    T ci = p.w;
+    const int o = sidx[i];
+    const T ci = p.w;
     forces[3 * (size_t)o + 0] = floc[3 * (size_t)i + 0] + ci * g0 * ih0;
     forces[3 * (size_t)o + 1] = floc[3 * (size_t)i + 1] + ci * g1 * ih1;
     forces[3 * (size_t)o + 2] = floc[3 * (size_t)i + 2] + ci * g2 * ih2;
@@ -826,7 +878,8 @@ __device__ __forceinline__ void k_interp_body(const Blk bk,
 }
 
 template <typename T, bool SLICES, int NP>
-__global__ void __launch_bounds__(kBlock) k_interp(
+__global__ void __launch_bounds__(kBlock, sizeof(T) == 8 ? 2 : NP == 6 ? 3 : SLICES ? 5 : 4)
+k_interp(
     const Vec4<T>* __restrict__ sp, const int* __restrict__ sidx, int N, const T* __restrict__ et,
     int n0, int n1, int n2, T ih0, T ih1, T ih2, const T* __restrict__ e0,
     const T* __restrict__ floc, double cself, T* __restrict__ forces,
@@ -993,6 +1046,7 @@ template <typename T> int prepare_grid_kernels(Plan* p) {
 #ifndef MLS6_DEVICE_ONLY  // host code, left out where another unit includes this file
 #define MLS6_INSTANTIATE(T)                                               \
   template int launch_anterp<T>(Plan*, cudaStream_t, int, bool, void*);   \
+  template int launch_anterp_lb<T>(Plan*, cudaStream_t, void*);           \
   template int launch_from_fixed<T>(Plan*, cudaStream_t, int, const void*); \
   template int launch_lb_weights<T>(Plan*, const T*, cudaStream_t);       \
   template int launch_interp_lb<T>(Plan*, T*, cudaStream_t);              \

@@ -221,6 +221,7 @@ template <typename T> int launch_pair(Plan* p, bool vir, cudaStream_t st, bool l
 // to_grid: also convert the fixed-point sums to q^1; qfx: sums (default d_q1fx)
 template <typename T>
 int launch_anterp(Plan* p, cudaStream_t st, int lbm = -1, bool to_grid = true, void* qfx = nullptr);
+template <typename T> int launch_anterp_lb(Plan* p, cudaStream_t st, void* qfx);
 template <typename T>
 int launch_from_fixed(Plan* p, cudaStream_t st, int lbm = -1, const void* qfx = nullptr);
 // q^1 sums -> e^{1,tot} and the grid part of the virial (lb: the seven channels)

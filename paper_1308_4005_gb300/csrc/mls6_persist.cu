@@ -181,7 +181,7 @@ __device__ __forceinline__ void run_stage(const PStageDesc& d, unsigned b) {
     case P_ANTERP: {
       const AnterpP& a = d.u.an;
       k_anterp_body<float>(bk, a.sp, a.N, a.n0, a.n1, a.n2, a.ih0, a.ih1, a.ih2, a.flag, a.span,
-                           a.qfx, nullptr, -1, 0.0);
+                           a.qfx, nullptr, -1, LbCoef{});
       break;
     }
     case P_FROM_FIXED: {
