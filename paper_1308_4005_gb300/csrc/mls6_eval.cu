@@ -148,7 +148,7 @@ template <typename T> static int upload_tables_t(Plan* p) {
   rc |= A((void**)&p->d_top_T, sizeof(double) * np_top);
   rc |= A((void**)&p->d_top_V, 6 * sizeof(double) * np_top);
   // partial sums: pair blocks | stencil blocks | coarsest nodes
-  p->n_epart = std::max(1L, cdiv(N, kBlock));
+  p->n_epart = std::max(1L, cdiv(N, (long)kBlock / 2));
   // room for the largest lane split, so that the split can be retuned
   // without reallocation; records a smaller split does not write stay zero
   // virial partials of the pair sum: one per warp of the per-atom kernel

@@ -11,6 +11,16 @@ namespace mls6 {
 
 // ------------------------------------------------------------ anterpolation
 
+// Threads per block of the anterpolation and the interpolation.  In FP64 their
+// time is the FP64 pipe's (2 lanes per cycle and SM), so that blocks of 256
+// leave most of the chip idle as long as there are fewer of them than SMs:
+// 1,000 atoms, anterpolation and interpolation, 26 + 34 us with 256, 23 + 22
+// with 128, 29 + 22 with 64.  From one block per SM on the larger block has the
+// fewer node sums to flush: 98,765 atoms 55 + 96 us against 63 + 102.
+template <typename T> inline int atom_block(long N) {
+  return sizeof(T) == 8 && cdiv(N, (long)kBlock) < 152 ? kBlock / 2 : kBlock;
+}
+
 // Eq. (anterpolation): q^1_mu += c_j phi_mu(x_j) over the NP^3 nodes of
 // every atom (NP = p + 1: 4x4x4 for the cubic, 6x6x6 for the quintic).  The contributions are rounded to the fixed-point grid 2^-s
 // and added as integers (Fixed<T>): integer addition is associative, so the
@@ -214,7 +224,8 @@ static LbCoef lb_coefs() {
 template <typename T> int launch_anterp(Plan* p, cudaStream_t st, int lbm, bool to_grid, void* qfx) {
   const Level& L1 = p->lv[1];
   const int N = (int)p->N;
-  launch_pdl(p->order == 5 ? k_anterp<T, 6, 1> : k_anterp<T, 4, 1>, cdiv(N, kBlock), kBlock, 0, st,
+  const int nt = atom_block<T>(N);
+  launch_pdl(p->order == 5 ? k_anterp<T, 6, 1> : k_anterp<T, 4, 1>, cdiv(N, nt), nt, 0, st,
       (const Vec4<T>*)p->d_sorted, N, L1.n[0], L1.n[1], L1.n[2], (T)(1.0 / L1.h[0]),
       (T)(1.0 / L1.h[1]), (T)(1.0 / L1.h[2]), p->d_flag, support_span(p),
       (typename Fixed<T>::U*)(qfx ? qfx : p->d_q1fx), (const T*)p->d_lbw, lbm, lb_coefs());
@@ -226,7 +237,8 @@ template <typename T> int launch_anterp(Plan* p, cudaStream_t st, int lbm, bool 
 template <typename T> int launch_anterp_lb(Plan* p, cudaStream_t st, void* qfx) {
   const Level& L1 = p->lv[1];
   const int N = (int)p->N;
-  launch_pdl(p->order == 5 ? k_anterp<T, 6, 7> : k_anterp<T, 4, 7>, cdiv(N, kBlock), kBlock, 0, st,
+  const int nt = atom_block<T>(N);
+  launch_pdl(p->order == 5 ? k_anterp<T, 6, 7> : k_anterp<T, 4, 7>, cdiv(N, nt), nt, 0, st,
       (const Vec4<T>*)p->d_sorted, N, L1.n[0], L1.n[1], L1.n[2], (T)(1.0 / L1.h[0]),
       (T)(1.0 / L1.h[1]), (T)(1.0 / L1.h[2]), p->d_flag, support_span(p),
       (typename Fixed<T>::U*)qfx, (const T*)p->d_lbw, 0, lb_coefs());
@@ -994,7 +1006,8 @@ int launch_interp(Plan* p, T* forces, double* atom_energy, bool vir, cudaStream_
                   slices ? kReduceGroups : 0};
   auto kern = p->order == 5 ? (slices ? k_interp<T, true, 6> : k_interp<T, false, 6>)
                             : (slices ? k_interp<T, true, 4> : k_interp<T, false, 4>);
-  launch_pdl(kern, cdiv(N, kBlock), kBlock, 0, st,
+  const int nt = atom_block<T>(N);
+  launch_pdl(kern, cdiv(N, nt), nt, 0, st,
       (const Vec4<T>*)p->d_sorted, p->d_sorted_idx, N, (const T*)p->d_et[1], L1.n[0], L1.n[1],
       L1.n[2], (T)(1.0 / L1.h[0]), (T)(1.0 / L1.h[1]), (T)(1.0 / L1.h[2]), (const T*)p->d_e0,
       (const T*)p->d_floc, p->c_self, forces, atom_energy, p->d_epart, R);

@@ -130,3 +130,32 @@ def test_interpolation_of_several_waves(gpu_lib, h):
     ref = c[:, None].astype(np.float64) * g / h
     err = np.abs(F.double().cpu().numpy() - ref).max()
     assert err <= 64 * 2.0**-24 * np.abs(e).max() * c.max() / h, err
+
+
+def test_fp64_block_size_rule(gpu_lib):
+    """152 blocks of 256 atoms are the first that keep the larger block; atoms
+    of coefficient zero, there or left out, change nothing but the block size."""
+    import torch
+
+    N, L = 152 * 256, 36.0
+    rng = np.random.default_rng(3)
+    m = 34  # jittered lattice, no two atoms close
+    at = np.stack(np.meshgrid(*[np.arange(m)] * 3, indexing="ij"), -1).reshape(-1, 3)[:N]
+    x = (at + 0.5 + rng.uniform(-0.1, 0.1, at.shape)) * (L / m)
+    q = np.c_[x, rng.uniform(0.5, 1.5, N)]
+    q = np.concatenate([q, [[0.0, 0.0, 0.0, 0.0]]])
+    r = []
+    for n in (N - 256, N, N + 1):
+        p = np.concatenate([q[:N], q[N:]])[:n] if n >= N else q[:n]
+        plan = gpu_lib.Plan((L, L, L), n, 2.5, 1.0, 3, precision="fp64")
+        g = plan.evaluate(torch.tensor(p, device="cuda"), virial=True)
+        r.append((g["out"].cpu().numpy(), g["F"].cpu().numpy()))
+    assert np.abs(r[1][0] - r[2][0]).max() <= 1e-12 * np.abs(r[1][0]).max()
+    assert np.abs(r[1][1] - r[2][1][:N]).max() <= 1e-11 * np.abs(r[1][1]).max()
+    # the 128-thread blocks: the last 256 atoms' coefficients zero against left out
+    plan = gpu_lib.Plan((L, L, L), N, 2.5, 1.0, 3, precision="fp64")
+    z = q[:N].copy()
+    z[N - 256:, 3] = 0.0
+    g = plan.evaluate(torch.tensor(z, device="cuda"), virial=True)
+    assert np.abs(g["out"].cpu().numpy() - r[0][0]).max() <= 1e-12 * np.abs(r[0][0]).max()
+    assert np.abs(g["F"].cpu().numpy()[: N - 256] - r[0][1]).max() <= 1e-11 * np.abs(r[0][1]).max()
