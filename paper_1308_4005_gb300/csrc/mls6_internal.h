@@ -184,18 +184,23 @@ struct Plan {
   bool use_graph = true;
   cudaGraphExec_t gexec = nullptr;
   struct GraphKey {
-    const void *pos, *c, *forces, *energy, *virial, *atom_energy;
-    bool vir, prof;
+    const void *pos, *c, *forces, *atom_energy;
+    bool energy, virial, both, vir, prof;
     bool operator==(const GraphKey& o) const {
-      return pos == o.pos && c == o.c && forces == o.forces && energy == o.energy &&
-             virial == o.virial && atom_energy == o.atom_energy && vir == o.vir && prof == o.prof;
+      return pos == o.pos && c == o.c && forces == o.forces && atom_energy == o.atom_energy &&
+             energy == o.energy && virial == o.virial && both == o.both && vir == o.vir &&
+             prof == o.prof;
     }
   } gkey = {};
+  cudaGraph_t graph = nullptr;         // what gexec was made from (its copy nodes' handles)
+  cudaGraphNode_t gout[2] = {};        // copies of energy (and virial) and of the virial
+  double* gdst[2] = {};                // their present targets
 
   size_t elem() const { return prec == MLS6_FP64 ? sizeof(double) : sizeof(float); }
 };
 
 // host helpers (mls6_plan.cpp)
+void drop_graph(Plan* p);  // mls6_eval.cu
 Smooth smooth_coefficients(int continuity);
 double gamma_fn(const Smooth& s, double rho);
 double dgamma_over_rho(const Smooth& s, double rho);  // gamma'(rho)/rho

@@ -279,7 +279,7 @@ static void free_plan(Plan* p) {
     if (p->ev_s[i]) cudaEventDestroy(p->ev_s[i]);
     if (p->ev_e[i]) cudaEventDestroy(p->ev_e[i]);
   }
-  if (p->gexec) cudaGraphExecDestroy(p->gexec);
+  drop_graph(p);
   cudaEvent_t evs[] = {p->ev_in, p->ev_out, p->ev_fork, p->ev_join};
   for (cudaEvent_t e : evs)
     if (e) cudaEventDestroy(e);
@@ -490,10 +490,7 @@ int mls6_set_tuning(mls6_plan_t* plan, int split, int groups) {
   if (p->cs2 && cudaStreamSynchronize(p->cs2) != cudaSuccess) return MLS6_ERR_CUDA;
   p->pair_split = s2;
   p->stencil_groups = g2;
-  if (p->gexec) {
-    cudaGraphExecDestroy(p->gexec);
-    p->gexec = nullptr;
-  }
+  drop_graph(p);
   return MLS6_OK;
 }
 
