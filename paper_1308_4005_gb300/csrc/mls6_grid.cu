@@ -792,7 +792,7 @@ struct ReduceArgs {
   int ng;
 };
 
-template <typename T, bool SLICES, int NP = 4>
+template <typename T, int NP = 4>
 __device__ __forceinline__ void k_interp_body(const Blk bk,
     const Vec4<T>* __restrict__ sp, const int* __restrict__ sidx, int N, const T* __restrict__ et,
     int n0, int n1, int n2, T ih0, T ih1, T ih2, const T* __restrict__ e0,
@@ -856,22 +856,25 @@ __device__ __forceinline__ void k_interp_body(const Blk bk,
   T ev[1] = {ea};
   double s[1];
   block_sum_lo<T, 1>(ev, s, sh);
-  // With several waves of blocks, warp 0 of each of the first ng blocks sums
+  // From kReduceGroups blocks on, warp 0 of each of the first ng blocks sums
   // one contiguous slice of the virial records (fixed order) and the last
-  // block adds the ng slice sums instead of every record (one block summing
-  // ~7,600 records in FP64 took 22 us on a 1M-atom cube).  In a single wave
-  // the slices would lengthen the kernel instead, and ng is 0.
-  if (SLICES && R.vir && (int)bk.x < R.ng && threadIdx.x < 32) {
+  // block adds the ng slice sums instead of every record: one block's FP64
+  // pipe takes 22 us for the ~7,600 records of a 1M-atom cube; 131,072 atoms
+  // of order 5 (512 blocks) 167 -> 155 us, 65,536 92.6 -> 90.5, 98,765 in FP64
+  // 1094 -> 1072 (whole evaluations).  Fewer blocks leave it to the last one.
+  if (R.vir && (int)bk.x < R.ng && threadIdx.x < 32) {
     const long per = (R.nw + R.ng - 1) / R.ng, k0 = (long)bk.x * per;
     const long k1 = min(R.nw, k0 + per);
     double v[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
     for (long k = k0 + threadIdx.x; k < k1; k += 32)
 #pragma unroll
       for (int c = 0; c < 6; ++c) v[c] += R.wpart[6 * k + c];
+    const double t = warp_sums(v);
 #pragma unroll
-    for (int c = 0; c < 6; ++c) v[c] = warp_sum(v[c]);
-    if (threadIdx.x == 0)
-      for (int c = 0; c < 6; ++c) R.gsum[6 * bk.x + c] = v[c];
+    for (int c = 0; c < 6; ++c) {  // stored by the thread whose ticket follows
+      const double w = __shfl_sync(0xffffffffu, t, 4 * c);
+      if (threadIdx.x == 0) R.gsum[6 * bk.x + c] = w;
+    }
   }
   if (threadIdx.x == 0) {
     epart[bk.x] = s[0];
@@ -881,22 +884,20 @@ __device__ __forceinline__ void k_interp_body(const Blk bk,
   __syncthreads();
   if (last) {
     __threadfence();
-    if (SLICES)
-      final_reduce(epart, bk.n, R.gsum, R.ng, R.vir, R.out, sh);
-    else
-      final_reduce(epart, bk.n, R.wpart, R.nw, R.vir, R.out, sh);
+    final_reduce(epart, bk.n, R.ng > 0 ? R.gsum : R.wpart, R.ng > 0 ? R.ng : R.nw, R.vir, R.out,
+                 sh);
     if (threadIdx.x == 0) *R.ticket = 0u;
   }
 }
 
-template <typename T, bool SLICES, int NP>
-__global__ void __launch_bounds__(kBlock, sizeof(T) == 8 ? 2 : NP == 6 ? 3 : SLICES ? 5 : 4)
+template <typename T, bool WAVES, int NP>
+__global__ void __launch_bounds__(kBlock, sizeof(T) == 8 ? 2 : NP == 6 ? 3 : WAVES ? 5 : 4)
 k_interp(
     const Vec4<T>* __restrict__ sp, const int* __restrict__ sidx, int N, const T* __restrict__ et,
     int n0, int n1, int n2, T ih0, T ih1, T ih2, const T* __restrict__ e0,
     const T* __restrict__ floc, double cself, T* __restrict__ forces,
     double* __restrict__ atom_energy, double* __restrict__ epart, ReduceArgs R) {
-  k_interp_body<T, SLICES, NP>(Blk::self(), sp, sidx, N, et, n0, n1, n2, ih0, ih1, ih2, e0, floc, cself, forces, atom_energy, epart, R);
+  k_interp_body<T, NP>(Blk::self(), sp, sidx, N, et, n0, n1, n2, ih0, ih1, ih2, e0, floc, cself, forces, atom_energy, epart, R);
 }
 
 // Lorentz-Berthelot interpolation: the seven channel potentials e^{(m),tot}
@@ -981,6 +982,9 @@ __global__ void __launch_bounds__(kBlock) k_interp_lb(
   }
 }
 
+// Blocks that pre-reduce slices of the virial records.
+inline int reduce_groups(long blocks) { return blocks >= kReduceGroups ? kReduceGroups : 0; }
+
 template <typename T> int launch_interp_lb(Plan* p, T* forces, cudaStream_t st) {
   const Level& L1 = p->lv[1];
   const int N = (int)p->N;
@@ -998,15 +1002,13 @@ template <typename T>
 int launch_interp(Plan* p, T* forces, double* atom_energy, bool vir, cudaStream_t st) {
   const Level& L1 = p->lv[1];
   const int N = (int)p->N;
-  // slice sums only for interpolations of several waves: the single-wave
-  // instantiation keeps the smaller kernel (one final-reduction copy)
-  const bool slices = cdiv(N, kBlock) >= 4L * 152;
+  const bool waves = cdiv(N, kBlock) >= 4L * 152;  // several waves of blocks
+  const int nt = atom_block<T>(N);
   ReduceArgs R = {p->d_wpart, wpart_used(p), vir ? 1 : 0, p->d_out,
                   reinterpret_cast<unsigned*>(p->d_flag + 1), p->d_out + 8,
-                  slices ? kReduceGroups : 0};
-  auto kern = p->order == 5 ? (slices ? k_interp<T, true, 6> : k_interp<T, false, 6>)
-                            : (slices ? k_interp<T, true, 4> : k_interp<T, false, 4>);
-  const int nt = atom_block<T>(N);
+                  reduce_groups(cdiv(N, nt))};
+  auto kern = p->order == 5 ? (waves ? k_interp<T, true, 6> : k_interp<T, false, 6>)
+                            : (waves ? k_interp<T, true, 4> : k_interp<T, false, 4>);
   launch_pdl(kern, cdiv(N, nt), nt, 0, st,
       (const Vec4<T>*)p->d_sorted, p->d_sorted_idx, N, (const T*)p->d_et[1], L1.n[0], L1.n[1],
       L1.n[2], (T)(1.0 / L1.h[0]), (T)(1.0 / L1.h[1]), (T)(1.0 / L1.h[2]), (const T*)p->d_e0,

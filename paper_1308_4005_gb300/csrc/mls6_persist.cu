@@ -81,7 +81,7 @@ struct ProlongP { const float* ef; int f0, f1, f2; const float* etc_; int c0, c1
 struct InterpP {
   const Vec4<float>* sp; const int* sidx; int N; const float* et; int n0, n1, n2;
   float ih0, ih1, ih2; const float* e0; const float* floc; double cself; float* forces;
-  double* epart; ReduceArgs R; int slices;
+  double* epart; ReduceArgs R;
 };
 struct OutP { const double* out; const int* flag; double* ew; int* flagdst; };
 
@@ -211,13 +211,8 @@ __device__ __forceinline__ void run_stage(const PStageDesc& d, unsigned b) {
     case P_SPEC_INV: spec_inv_body<float, 19>(bk, 0, d.u.sp, persist_smem); break;
     case P_INTERP: {
       const InterpP& a = d.u.in;
-      if (a.slices)
-        k_interp_body<float, true>(bk, a.sp, a.sidx, a.N, a.et, a.n0, a.n1, a.n2, a.ih0, a.ih1,
-                                   a.ih2, a.e0, a.floc, a.cself, a.forces, nullptr, a.epart, a.R);
-      else
-        k_interp_body<float, false>(bk, a.sp, a.sidx, a.N, a.et, a.n0, a.n1, a.n2, a.ih0, a.ih1,
-                                    a.ih2, a.e0, a.floc, a.cself, a.forces, nullptr, a.epart,
-                                    a.R);
+      k_interp_body<float>(bk, a.sp, a.sidx, a.N, a.et, a.n0, a.n1, a.n2, a.ih0, a.ih1, a.ih2,
+                           a.e0, a.floc, a.cself, a.forces, nullptr, a.epart, a.R);
       break;
     }
     case P_OUT: {
@@ -416,15 +411,14 @@ static void replica_stages(Plan* p, const float* pos, const float* cc, float* fo
     }
   }
   {
-    const bool slices = cdiv(N, kBlock) >= 4L * 152;
     PStageDesc& d = add(P_INTERP, cdiv(N, kBlock));
     ReduceArgs R = {p->d_wpart, wpart_used(p), vir ? 1 : 0, p->d_out,
                     reinterpret_cast<unsigned*>(p->d_flag + 1), p->d_out + 8,
-                    slices ? kReduceGroups : 0};
+                    reduce_groups(cdiv(N, kBlock))};
     d.u.in = InterpP{(const Vec4<float>*)p->d_sorted, p->d_sorted_idx, N, (const float*)p->d_et[1],
                      L1.n[0], L1.n[1], L1.n[2], (float)(1.0 / L1.h[0]), (float)(1.0 / L1.h[1]),
                      (float)(1.0 / L1.h[2]), (const float*)p->d_e0, (const float*)p->d_floc,
-                     p->c_self, forces, p->d_epart, R, slices ? 1 : 0};
+                     p->c_self, forces, p->d_epart, R};
   }
   {
     PStageDesc& d = add(P_OUT, 1);
