@@ -515,7 +515,7 @@ __global__ void __launch_bounds__(32 * kFwdWarps, 1)
 
 // Loss and gradient of a batch in one pass over the rows.  A block of 8 warps
 // takes `per` consecutive tiles of kTA atoms; per tile
-//   - every warp runs the network on its 16 atoms (the tiling of k_mlp_fwd):
+//   - every warp runs the network on its 16 atoms:
 //     activations stay in registers as the next layer's A fragments and go to
 //     shared memory as rows [atom][unit];
 //   - dY = 2 (y - t) / N on outputs 0..2 (BF16), then per layer
