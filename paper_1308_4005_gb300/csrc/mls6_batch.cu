@@ -279,6 +279,7 @@ static int launch(Batch* b, const void* pos, const void* c, void* forces, bool v
     int rc = capture(b, pos, c, forces, vir);
     if (rc) return rc;
   }
+  for (Plan* p : b->plans) p->lb_last = false;
   CK(cudaEventRecord(b->ev_in, b->stream));
   CK(cudaStreamWaitEvent(b->s0, b->ev_in, 0));
   CK(cudaGraphLaunch(b->gexec, b->s0));

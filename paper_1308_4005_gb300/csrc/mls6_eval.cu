@@ -239,7 +239,6 @@ static int enqueue(Plan* p, const T* pos, const T* cc, T* forces, double* energy
     if (p->prof) CK(cudaEventRecordWithFlags(p->ev_e[i], s, evf)); \
   } while (0)
   int nl = 0;
-  p->lb_last = false;
   BEGIN(0, st);
   // flags, tickets, maxima (see Plan::d_flag), cell counts, anterpolation sums
   CK(cudaMemsetAsync(p->d_zero, 0, p->zero_bytes, st));
@@ -367,6 +366,7 @@ static int eval_t(Plan* p, const void* pos_, const void* c_, void* forces_, doub
   double* virial_dev = (virial && is_device_ptr(virial)) ? virial : nullptr;
   const bool host_sync = (energy && !energy_dev) || (virial && !virial_dev);
 
+  p->lb_last = false;  // here, not in enqueue: a replay of the graph does not pass through it
   CK(cudaEventRecord(p->ev_in, p->stream));
   CK(cudaStreamWaitEvent(p->cs, p->ev_in, 0));
   if (p->use_graph) {
