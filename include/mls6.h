@@ -245,7 +245,8 @@ int mls6_plan_info(const mls6_plan_t* p, int* n_grid, double* h_actual, int* lev
 /* Copy one grid of the last evaluation to host memory as doubles (x fastest):
  * which = 0: xi^k (anterpolated / restricted coefficients),
  *         1: e^k (level evaluation), 2: e^{k,tot} (after prolongation).
- * level: 1..l.  Synchronises the plan's stream.  A plan that evaluates by
+ * level: 1..l.  After mls6_eval_lb the grids are those of its last channel,
+ * xi_6.  Synchronises the plan's stream.  A plan that evaluates by
  * transforms keeps only xi^1 (fixed point) and e^{1,tot}; the other grids are
  * formed by this call, with the plan's stencil kernel. */
 int mls6_debug_grid(mls6_plan_t* p, int level, int which, double* host_out);
@@ -485,8 +486,9 @@ int mls6_mlp_set_params(mls6_mlp_t* m, const float* host, int n);
 /* Feature normalisation (host arrays of 128) and output scale s. */
 int mls6_mlp_set_norm(mls6_mlp_t* m, const float* shift, const float* scale, float out_scale);
 
-/* Normalised features of the plan's last evaluation, written to the device
- * array out (N x 128, fmt 0 = bf16, 1 = float), input order. */
+/* Normalised features of the plan's last evaluation (after mls6_eval_lb, of
+ * its channel xi_6), written to the device array out (N x 128, fmt 0 = bf16,
+ * 1 = float), input order. */
 int mls6_mlp_features(mls6_plan_t* p, const mls6_mlp_t* m, void* out, int fmt);
 
 /* Network outputs Y (device, N x 8 floats) for features X (device, N x 128

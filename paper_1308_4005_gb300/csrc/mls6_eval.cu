@@ -561,7 +561,10 @@ template <typename T> static int debug_grid_t(Plan* p, int level, int which, dou
     for (int k = p->levels - 1; k >= 2; --k) launch_prolong<T>(p, k, st);
     if (cudaStreamSynchronize(st) != cudaSuccess) return MLS6_ERR_CUDA;
   }
-  const void* src = which == 0 ? p->d_q[level] : which == 1 ? p->d_e[level] : p->d_et[level];
+  const void* src = have         ? level1_potential(p)
+                    : which == 0 ? p->d_q[level]
+                    : which == 1 ? p->d_e[level]
+                                 : p->d_et[level];
   std::vector<T> tmp((size_t)Lk.np);
   if (cudaStreamSynchronize(p->stream) != cudaSuccess) return MLS6_ERR_CUDA;
   if (cudaMemcpy(tmp.data(), src, sizeof(T) * Lk.np, cudaMemcpyDeviceToHost) != cudaSuccess)

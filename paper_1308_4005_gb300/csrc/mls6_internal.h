@@ -199,6 +199,13 @@ struct Plan {
   size_t elem() const { return prec == MLS6_FP64 ? sizeof(double) : sizeof(float); }
 };
 
+// e^{1,tot} of the last evaluation; of a Lorentz-Berthelot one, channel 6, the
+// last (the spectral form writes the channels to d_lbpot only).
+inline const void* level1_potential(const Plan* p) {
+  return p->lb_last ? (const char*)p->d_lbpot + 6 * (size_t)p->lv[1].np * p->elem()
+                    : (const char*)p->d_et[1];
+}
+
 // host helpers (mls6_plan.cpp)
 void drop_graph(Plan* p);  // mls6_eval.cu
 Smooth smooth_coefficients(int continuity);

@@ -1006,7 +1006,7 @@ static int features_t(Plan* p, Mlp* m, void* out, int f32, bool sorted_out, cuda
   if (N == 0) return MLS6_OK;
   auto kern = f32 ? k_features<T, true> : k_features<T, false>;
   kern<<<cdiv(N, kFA), 3 * kFA, 0, st>>>(
-      (const Vec4<T>*)p->d_sorted, p->d_sorted_idx, N, (const T*)p->d_et[1], L1.n[0], L1.n[1],
+      (const Vec4<T>*)p->d_sorted, p->d_sorted_idx, N, (const T*)level1_potential(p), L1.n[0], L1.n[1],
       L1.n[2], (T)(1.0 / L1.h[0]), (T)(1.0 / L1.h[1]), (T)(1.0 / L1.h[2]), m->d_norm, out,
       sorted_out ? 1 : 0);
   CK(cudaGetLastError());

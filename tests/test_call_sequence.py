@@ -67,3 +67,31 @@ def test_grids_after_a_replay_behind_lorentz_berthelot(gpu_lib, form):
     got = _grids(gpu_lib, plan)
     for k in ref:
         assert np.array_equal(got[k], ref[k]), k
+
+
+@pytest.mark.parametrize("before", [False, True], ids=["first_call", "behind_evaluate"])
+def test_grids_and_features_after_lorentz_berthelot(gpu_lib, orc, before):
+    """After mls6_eval_lb the grids and the features are those of channel
+    xi_6, also as the plan's first call.  FP64 grids: 1e-12 of the maximum,
+    as for the other grids; features in FP32: u = 6e-8 of the values (a
+    potential and its gradient, |.| <= 4 max |e|) through the FP32 output."""
+    import torch
+
+    from oracle import lb
+
+    x, c, s, e = _system()
+    xi6 = lb.xi(s, e)[6]
+    plan = gpu_lib.Plan(BOX, N, A, H, LEVELS)
+    if before:
+        plan.evaluate(_dev(np.c_[x, c]))
+    _lb(gpu_lib, plan, _dev(x), _dev(s), _dev(e))
+    G = orc.grids(BOX, A, orc.grid_dims(BOX, H, LEVELS), LEVELS, x, xi6)
+    for (k, w), got in _grids(gpu_lib, plan).items():
+        assert np.abs(got - G[k - 1][w]).max() <= 1e-12 * np.abs(G[k - 1][w]).max(), (k, w)
+    net = gpu_lib.MLP(seed=1)
+    X = net.features(plan, "f32")
+    other = gpu_lib.Plan(BOX, N, A, H, LEVELS)
+    other.evaluate(_dev(np.c_[x, xi6]))
+    Y = net.features(other, "f32")
+    torch.cuda.synchronize()
+    assert float((X - Y).abs().max()) <= 6e-8 * 4 * G[0][2].max()
