@@ -456,16 +456,10 @@ static int eval_lb_t(Plan* p, const T* pos, const T* sigma, const T* eps, T* for
   int rc = ensure_streams(p);
   if (rc) return rc;
   const long np1 = p->lv[1].np;
-  if (!p->d_lbw) {
-    if (cudaMalloc(&p->d_lbw, sizeof(T) * N) != cudaSuccess) return MLS6_ERR_NOMEM;
-    if (cudaMalloc(&p->d_lbpot, sizeof(T) * 7 * np1) != cudaSuccess) return MLS6_ERR_NOMEM;
-    if (p->spectral) {
-      const int* n = p->lv[1].n;
-      const size_t ns = (size_t)n[1] * (n[0] / 2 + 1) * n[2];
-      if (cudaMalloc(&p->d_lbq, sizeof(T) * 7 * np1) != cudaSuccess ||
-          cudaMalloc(&p->d_lbs, 2 * sizeof(T) * 2 * 7 * ns) != cudaSuccess)
-        return MLS6_ERR_NOMEM;
-    }
+  if (!lb_workspace(p, [](void** q, size_t b) { return cudaMalloc(q, b) == cudaSuccess; },
+                    [](void* q) { cudaFree(q); })) {
+    cudaGetLastError();
+    return MLS6_ERR_NOMEM;
   }
   cudaStream_t st = p->cs;
   const int l = p->levels;

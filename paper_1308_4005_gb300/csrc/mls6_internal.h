@@ -206,6 +206,34 @@ inline const void* level1_potential(const Plan* p) {
                     : (const char*)p->d_et[1];
 }
 
+// Buffers of Lorentz-Berthelot evaluations, all of them or (false) none, so
+// that a call after a failed one allocates anew: alloc(void**, bytes) -> bool.
+template <class Alloc, class Free> bool lb_workspace(Plan* p, Alloc alloc, Free release) {
+  if (p->d_lbw) return true;
+  const size_t e = p->elem(), np1 = (size_t)p->lv[1].np;
+  const int* n = p->lv[1].n;
+  const size_t ns = (size_t)n[1] * (n[0] / 2 + 1) * n[2];
+  struct {
+    void** ptr;
+    size_t bytes;
+  } const bufs[] = {{&p->d_lbw, e * (size_t)p->N},
+                    {&p->d_lbpot, e * 7 * np1},
+                    {&p->d_lbq, p->spectral ? e * 7 * np1 : 0},
+                    {&p->d_lbs, p->spectral ? 2 * e * 2 * 7 * ns : 0}};
+  bool ok = true;
+  for (const auto& b : bufs)
+    if (ok && b.bytes > 0 && !alloc(b.ptr, b.bytes)) {
+      *b.ptr = nullptr;
+      ok = false;
+    }
+  for (const auto& b : bufs)
+    if (!ok && *b.ptr) {
+      release(*b.ptr);
+      *b.ptr = nullptr;
+    }
+  return ok;
+}
+
 // host helpers (mls6_plan.cpp)
 void drop_graph(Plan* p);  // mls6_eval.cu
 Smooth smooth_coefficients(int continuity);
