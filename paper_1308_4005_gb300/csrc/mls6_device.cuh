@@ -147,12 +147,19 @@ __device__ __forceinline__ long pdl_begin() {
 // A block of consecutive cell-sorted atoms touches a compact box of grid
 // nodes.  Where that box fits into kNodeBoxBytes, the block keeps it in shared
 // memory: the anterpolation sums there, the features read there.  One buffer
-// per kernel, whatever stages it runs.
+// per kernel, whatever stages it runs; in the persistent kernel the start of
+// its dynamic shared memory, of which the transforms take up to 200 KB (beside
+// 24 KB of static memory that is more than a block may have).
 constexpr int kNodeBoxBytes = 24 * 1024;
+#ifdef MLS6_DEVICE_ONLY
+extern __shared__ __align__(16) unsigned char persist_smem[];
+__device__ __forceinline__ unsigned char* node_box_smem() { return persist_smem; }
+#else
 __device__ __forceinline__ unsigned char* node_box_smem() {
   __shared__ __align__(16) unsigned char buf[kNodeBoxBytes];
   return buf;
 }
+#endif
 
 // Unwrapped node indices lo .. lo + e - 1 per axis; in: the box fits and every
 // index is at most one period away from its node (the same for all threads).

@@ -118,8 +118,6 @@ struct PExecArgs {
   long long total, limit, withhold;
 };
 
-extern __shared__ __align__(16) unsigned char persist_smem[];  // the stencil's and the transforms'
-
 template <bool VIR>
 __device__ __forceinline__ void run_stage(const PStageDesc& d, unsigned b) {
   const Blk bk{b, d.nb};
@@ -487,7 +485,7 @@ int persist_build(PersistExec** out, Plan* const* plans, int B, const int64_t* o
       first[i + 1] = first[i] + st[(size_t)order[k] * S + s].nb;
     }
   x->total = first.back();
-  size_t smem = 0;
+  size_t smem = kNodeBoxBytes;
   for (int r = 0; r < B; ++r) {
     const Plan* p = plans[r];
     const int* n = p->lv[1].n;

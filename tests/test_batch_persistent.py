@@ -1,0 +1,32 @@
+"""The persistent form of a batch over the grids that it accepts."""
+import numpy as np
+import pytest
+
+from paper_1308_4005_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("box,levels", [((136.0, 180.0, 8.0), 3), ((192.0, 128.0, 16.0), 4)],
+                         ids=["136x180", "192x128"])
+def test_largest_planes(gpu_lib, box, levels):
+    """x-y planes that leave a block of the transforms less than 30 KB of
+    shared memory: one persistent launch, equal to the kernel chains bit for
+    bit (the same bodies)."""
+    import torch
+
+    N = [700, 500]
+    boxes = [box, (12.0, 12.0, 12.0)]
+    at = [I.uniform_atoms(80 + r, n, b) for r, (n, b) in enumerate(zip(N, boxes))]
+    pos = torch.tensor(np.concatenate([np.c_[x, c] for x, c in at]), dtype=torch.float32,
+                       device="cuda")
+    bt = gpu_lib.Batch(boxes, N, 2.0, 1.0, levels, precision="fp32")
+    res = []
+    for mode in (True, False):
+        gpu_lib.mls6_batch_set_mode(bt.handle, mode)
+        r = bt.evaluate(pos)
+        torch.cuda.synchronize()
+        assert gpu_lib.mls6_batch_mode(bt.handle) == int(mode)
+        res.append([r[k].cpu().numpy() for k in ("E", "W", "F")])
+    for a, b in zip(*res):
+        assert np.array_equal(a, b)
