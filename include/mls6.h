@@ -148,6 +148,13 @@ int mls6_plan(mls6_plan_t** out, const double box[3], int64_t N, double a, doubl
  * restriction, every level, the coarsest level and prolongation are products
  * in the discrete Fourier transform of the finest grid, in the plan's
  * precision (the coarsest level in FP64); the same periodic sums, reassociated.
+ * Their rounding is relative to the largest potential in the box.  An
+ * evaluation whose atoms have thin surroundings beside dense ones (a vapour
+ * beside a liquid: the 3 x 3 x 3 cells around the densest occupied cell hold
+ * more than 16 times the atoms of those around the thinnest, weighted by the
+ * largest over the least nonzero |c|) runs the direct kernels on the CUDA cores
+ * instead, whose rounding is relative to each node's own potential; the device
+ * chooses, call by call.
  * Out-of-range values return MLS6_ERR_ARG. */
 typedef struct {
   int continuity;

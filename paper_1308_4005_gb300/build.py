@@ -21,7 +21,7 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 SOURCES = ["mls6_plan.cpp", "mls6_eval.cu", "mls6_bin.cu", "mls6_pair.cu",
            "mls6_pair_tile.cu", "mls6_grid.cu", "mls6_spectral.cu",
            "mls6_noalloc.cu", "mls6_batch.cu", "mls6_stencil_tc.cu",
-           "mls6_learn.cu", "mls6_peaks.cu", "mls6_stencil_mma.cu", "mls6_persist.cu"]
+           "mls6_learn.cu", "mls6_peaks.cu", "mls6_stencil_mma.cu", "mls6_persist.cu", "mls6_direct.cu"]
 
 
 def _nvcc() -> str:

@@ -19,7 +19,8 @@ template <typename T> struct BinArgs {
 
 // Also keeps, for the fixed-point anterpolation, the largest |c| in
 // flag[4..5] (a double; one atomic maximum per block on its bits, which
-// order like the value for non-negative doubles), and, when tsum is given
+// order like the value for non-negative doubles), the least nonzero |c| in
+// flag[kThinC..] (for k_thin), and, when tsum is given
 // (at most kScanDirect tiles), adds the block's atoms per scan tile of
 // kScanTile cells to tsum (a shared-memory histogram first, then one
 // integer atomic per touched tile).  count, flag and tsum start at zero (one
@@ -33,7 +34,7 @@ __device__ __forceinline__ void k_bin_body(const Blk bk,const T* __restrict__ po
                       int ntiles) {
   const long z = pdl_begin();
   pos += z; cc += z;
-  __shared__ T wmax[32];
+  __shared__ T wmax[32], wmin[32];
   __shared__ int hist[kScanDirect];
   const int i = bk.x * blockDim.x + threadIdx.x;
   if (tsum)
@@ -65,14 +66,24 @@ __device__ __forceinline__ void k_bin_body(const Blk bk,const T* __restrict__ po
     if (tsum) atomicAdd(&hist[cell / kScanTile], 1);
     cabs = fabs(c);
   }
-  for (int o = 16; o > 0; o >>= 1) cabs = fmax(cabs, __shfl_xor_sync(0xffffffffu, cabs, o));
-  if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = cabs;
+  T cmin = cabs > T(0) ? cabs : T(INFINITY);
+  warp_range(cmin, cabs);
+  if ((threadIdx.x & 31) == 0) {
+    wmax[threadIdx.x >> 5] = cabs;
+    wmin[threadIdx.x >> 5] = cmin;
+  }
   __syncthreads();
   if (threadIdx.x == 0) {
-    T m = T(0);
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) m = fmax(m, wmax[w]);
-    atomicMax(reinterpret_cast<unsigned long long*>(flag + 4),
-              (unsigned long long)__double_as_longlong((double)m));
+    T m = T(0), lo = T(INFINITY);
+    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+      m = fmax(m, wmax[w]);
+      lo = fmin(lo, wmin[w]);
+    }
+    raise_to(reinterpret_cast<unsigned long long*>(flag + 4),
+             (unsigned long long)__double_as_longlong((double)m));
+    if (lo <= m)  // else no atom with a coefficient
+      raise_to(reinterpret_cast<unsigned long long*>(flag + kThinC),
+               ~(unsigned long long)__double_as_longlong((double)lo));
   }
   if (tsum)
     for (int t = threadIdx.x; t < ntiles; t += blockDim.x)
@@ -326,11 +337,78 @@ __device__ __forceinline__ void k_cellsort_body(const Blk bk,const int* __restri
   for (int i = b; i < e; ++i) put(i, posw[sidx[i]]);
 }
 
+// Which form the grid part takes.  A transform spreads the rounding of the
+// largest potentials over the whole box, where the direct kernels round each
+// node's sum relative to itself: with atoms in a thin phase beside a dense one
+// (a vapour, far from a droplet or a slab) their forces from transforms would
+// be 5 to 9 times further off (relative to themselves; atoms near others are
+// dominated by the rounding of the pair sum).  So the direct kernels run where
+// the densest surroundings of an occupied cell (atoms in the 3 x 3 x 3 cells
+// around it) exceed the thinnest kThinRatio times, each weighted by the
+// extreme coefficients.  Surfaces of slabs reach 5 (with C6 in 0.5 .. 1.5: 8),
+// single atoms of a vapour 20 to 100.  Lorentz-Berthelot: C grows like sigma^3
+// sqrt(eps) of either atom.  One thread per cell, in blocks of their own beside
+// the cell sort's; the anterpolation decides (k_anterp_body).
+struct ThinArgs {
+  int nc[3];
+};
+
+__device__ __forceinline__ void k_thin_body(const Blk bk, const int* __restrict__ start, long ncell,
+                                            ThinArgs g, int* __restrict__ flag) {
+  const long z0 = pdl_begin();
+  start += z0;
+  __shared__ int smax[32], smin[32];
+  const long cell = (long)bk.x * blockDim.x + threadIdx.x;
+  const bool occ = cell < ncell && start[cell + 1] > start[cell];
+  int n = 0;
+  if (occ) {
+    int x, y, z;
+    if (ncell <= 0x7fffffff) {  // 64-bit divisions are long
+      const unsigned c = (unsigned)cell, q = c / (unsigned)g.nc[0];
+      x = (int)(c - q * (unsigned)g.nc[0]);
+      y = (int)(q % (unsigned)g.nc[1]);
+      z = (int)(q / (unsigned)g.nc[1]);
+    } else {
+      const long q = cell / g.nc[0];
+      x = (int)(cell - q * g.nc[0]);
+      y = (int)(q % g.nc[1]);
+      z = (int)(q / g.nc[1]);
+    }
+    n = atoms_around(start, g.nc, x, y, z);
+  }
+  const int mx = __reduce_max_sync(0xffffffffu, n);
+  const int mn = __reduce_max_sync(0xffffffffu, occ ? kThinMany - n : 0);
+  if ((threadIdx.x & 31) == 0) {
+    smax[threadIdx.x >> 5] = mx;
+    smin[threadIdx.x >> 5] = mn;
+  }
+  __syncthreads();
+  if (threadIdx.x > 0) return;
+  int hi = 0, lo = 0;
+  for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
+    hi = max(hi, smax[w]);
+    lo = max(lo, smin[w]);
+  }
+  if (hi > 0) {
+    raise_to(flag + kThinMax, hi);
+    raise_to(flag + kThinMin, lo);
+  }
+}
+
+// nsort blocks sort, the others (if any) choose the form of the grid part.
 template <typename T>
 __global__ void k_cellsort(const int* __restrict__ start, long ncell,
                            const Vec4<T>* __restrict__ posw, Vec4<T>* __restrict__ sorted,
-                           int* __restrict__ sidx, float4* __restrict__ sortedf) {
-  k_cellsort_body<T>(Blk::self(), start, ncell, posw, sorted, sidx, sortedf);
+                           int* __restrict__ sidx, float4* __restrict__ sortedf, int nsort,
+                           ThinArgs g, int* __restrict__ flag) {
+  if ((int)blockIdx.x < nsort)
+    k_cellsort_body<T>(Blk::self(), start, ncell, posw, sorted, sidx, sortedf);
+  else
+    k_thin_body(Blk{blockIdx.x - nsort, gridDim.x - nsort}, start, ncell, g, flag);
+}
+
+static ThinArgs thin_args(const Plan* p) {
+  return ThinArgs{{p->cg.nc[0], p->cg.nc[1], p->cg.nc[2]}};
 }
 
 // Arguments of the binning kernel for a plan.
@@ -345,7 +423,8 @@ template <typename T> static BinArgs<T> bin_args(const Plan* p) {
   return bg;
 }
 
-template <typename T> int launch_bin(Plan* p, const T* pos, const T* cc, cudaStream_t st) {
+template <typename T>
+int launch_bin(Plan* p, const T* pos, const T* cc, cudaStream_t st) {
   const int N = (int)p->N;
   const BinArgs<T> bg = bin_args<T>(p);
   const long ncell = p->cg.ncell;
@@ -363,9 +442,10 @@ template <typename T> int launch_bin(Plan* p, const T* pos, const T* cc, cudaStr
              p->d_cell_start, direct ? 1 : 0, p->d_flag);
   launch_pdl(k_scatter, cdiv(N, kBlock), kBlock, 0, st, (const int2*)p->d_cell_of, N,
              (const int*)p->d_cell_start, p->d_sorted_idx);
-  launch_pdl(k_cellsort<T>, cdiv(ncell, kBlock), kBlock, 0, st, (const int*)p->d_cell_start, ncell,
-             (const Vec4<T>*)p->d_pos_w, (Vec4<T>*)p->d_sorted, p->d_sorted_idx,
-             (float4*)p->d_sorted_f);
+  const int nsort = (int)cdiv(ncell, kBlock);
+  launch_pdl(k_cellsort<T>, p->spectral ? 2 * nsort : nsort, kBlock, 0, st, (const int*)p->d_cell_start,
+             ncell, (const Vec4<T>*)p->d_pos_w, (Vec4<T>*)p->d_sorted, p->d_sorted_idx,
+             (float4*)p->d_sorted_f, nsort, thin_args(p), p->d_flag);
   return direct ? 4 : 5;
 }
 

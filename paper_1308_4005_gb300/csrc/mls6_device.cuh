@@ -142,6 +142,19 @@ __device__ __forceinline__ long pdl_begin() {
   return z;
 }
 
+// ------------------------------------------------- work queues of persistent kernels
+
+struct PQueue {
+  unsigned long long ticket;  // next item
+  int error;                  // bit 0: a bounded wait ran out
+};
+
+__device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
+  unsigned v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+
 // ------------------------------------------------- nodes around a block's atoms
 
 // A block of consecutive cell-sorted atoms touches a compact box of grid
@@ -230,6 +243,25 @@ __device__ __forceinline__ void load_node_box(T* box, const T* __restrict__ src,
 __device__ __forceinline__ double warp_sum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
   return v;
+}
+
+// *w = max(*w, v); most blocks find it reached already, which spares them the
+// atomic (thousands on one word take microseconds).
+template <typename I> __device__ __forceinline__ void raise_to(I* w, I v) {
+  if (*(volatile I*)w < v) atomicMax(w, v);
+}
+
+// Least and largest over the warp of values >= 0 (FP32: their bits order like
+// unsigned integers, one instruction each instead of five exchanges).
+__device__ __forceinline__ void warp_range(float& lo, float& hi) {
+  lo = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(lo)));
+  hi = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(hi)));
+}
+__device__ __forceinline__ void warp_range(double& lo, double& hi) {
+  for (int o = 16; o > 0; o >>= 1) {
+    lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+    hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+  }
 }
 
 // Sums over a warp of NV = 5..8 values per lane: lane l returns the sum of
@@ -381,6 +413,24 @@ __device__ __forceinline__ double lb_coef_d(int k) {
   const double b = (k == 0 || k == 6) ? 1.0 : (k == 1 || k == 5) ? 6.0 : (k == 2 || k == 4) ? 15.0
                                                                                            : 20.0;
   return 0.125 * sqrt(b);
+}
+
+// The choice of the grid part's form (see k_thin_body): the direct kernels
+// where the densest surroundings of an occupied cell exceed the thinnest
+// kThinRatio times, weighted by the extreme coefficients.
+constexpr double kThinRatio = 16.0;
+
+__device__ __forceinline__ double thin_range(const int* flag, int most, int least) {
+  const double hi = __longlong_as_double(*(volatile const long long*)(flag + most));
+  const unsigned long long k = *(volatile const unsigned long long*)(flag + least);
+  return k ? hi / __longlong_as_double((long long)~k) : 1.0;
+}
+__device__ __forceinline__ int thin_choice(const int* flag, bool lb) {
+  const int most = *(volatile const int*)(flag + kThinMax);
+  const int least = kThinMany - *(volatile const int*)(flag + kThinMin);
+  double r = thin_range(flag, 4, kThinC);
+  if (lb) r = r * r * r * thin_range(flag, 6, kThinW);
+  return (double)most * r > kThinRatio * (double)least ? 1 : 0;
 }
 
 // Fixed-point accumulation of the anterpolation: 32-bit integers for the

@@ -70,22 +70,10 @@ template <typename T> static int upload_tables_t(Plan* p) {
     return cudaMalloc(ptr, bytes) == cudaSuccess ? 0 : MLS6_ERR_NOMEM;
   };
   int rc = 0;
+  size_t all_bytes = 0;  // of the region at d_zero
   rc |= A(&p->d_pos_w, sizeof(Vec4<T>) * N);
   rc |= A((void**)&p->d_cell_of, sizeof(int2) * N);
   rc |= A((void**)&p->d_cell_start, sizeof(int) * (p->cg.ncell + 1));
-  {
-    auto up = [](size_t b) { return (b + 255) & ~size_t(255); };
-    const size_t flag = up(sizeof(int) * 8);
-    const size_t scan = up(sizeof(int) * std::max(1L, cdiv(p->cg.ncell, kScanTile)));
-    const size_t count = up(sizeof(int) * p->cg.ncell);
-    const size_t q1 = up(e * p->lv[1].np);  // int32 (FP32 modes) or int64 sums
-    p->zero_bytes = flag + scan + count + q1;
-    if (A((void**)&p->d_zero, p->zero_bytes)) return MLS6_ERR_NOMEM;
-    p->d_flag = (int*)p->d_zero;
-    p->d_scan = (int*)(p->d_zero + flag);
-    p->d_cell_count = (int*)(p->d_zero + flag + scan);
-    p->d_q1fx = p->d_zero + flag + scan + count;
-  }
   rc |= A(&p->d_sorted, sizeof(Vec4<T>) * (N + 3));  // 3 padding records (pair kernel loads)
   if (e == 8) rc |= A(&p->d_sorted_f, sizeof(float4) * N);
   rc |= A((void**)&p->d_sorted_idx, sizeof(int) * N);
@@ -157,12 +145,30 @@ template <typename T> static int upload_tables_t(Plan* p) {
   p->n_pair_blocks =
       std::max(1L, std::max(cdiv(N * 8, (long)kBlock) * (kBlock / 32), cdiv(N * kPairSplitMax, kBlock)));
   p->wpart_stencil = 0;
-  p->wpart_top = p->stencil_blocks;
+  p->wpart_top = std::max(p->stencil_blocks, p->spectral ? direct_records(p) : 0L);
+  p->wpart_spec = p->wpart_top + np_top;
   // (spectral form: one record per set of frequencies, i.e. coarsest node)
-  p->wpart_pair = p->spectral ? np_top : p->wpart_top + np_top;
-  p->n_wpart = p->wpart_top + np_top + p->n_pair_blocks;
+  p->wpart_pair = p->wpart_spec + (p->spectral ? np_top : 0);
+  p->n_wpart = p->wpart_pair + p->n_pair_blocks;
   rc |= A((void**)&p->d_epart, sizeof(double) * p->n_epart);
-  rc |= A((void**)&p->d_wpart, 6 * sizeof(double) * p->n_wpart);
+  {
+    auto up = [](size_t b) { return (b + 255) & ~size_t(255); };
+    const size_t flag = up(sizeof(int) * kFlagWords);
+    const size_t scan = up(sizeof(int) * std::max(1L, cdiv(p->cg.ncell, kScanTile)));
+    const size_t count = up(sizeof(int) * p->cg.ncell);
+    const size_t q1 = up(e * p->lv[1].np);  // int32 (FP32 modes) or int64 sums
+    const size_t queue = p->spectral ? up(direct_queue_bytes(p)) : 0;
+    const size_t at = flag + scan + count + q1 + queue;
+    p->zero_bytes = at + (p->spectral ? 6 * sizeof(double) * p->wpart_pair : 0);
+    all_bytes = at + 6 * sizeof(double) * p->n_wpart;
+    if (A((void**)&p->d_zero, all_bytes)) return MLS6_ERR_NOMEM;
+    p->d_flag = (int*)p->d_zero;
+    p->d_scan = (int*)(p->d_zero + flag);
+    p->d_cell_count = (int*)(p->d_zero + flag + scan);
+    p->d_q1fx = p->d_zero + flag + scan + count;
+    p->d_direct_queue = p->d_zero + flag + scan + count + q1;
+    p->d_wpart = (double*)(p->d_zero + at);
+  }
   rc |= A((void**)&p->d_out, (8 + 6 * kReduceGroups) * sizeof(double));
   if (rc) return MLS6_ERR_NOMEM;
   if (cudaMallocHost((void**)&p->h_out, 8 * sizeof(double)) != cudaSuccess) return MLS6_ERR_NOMEM;
@@ -188,9 +194,8 @@ template <typename T> static int upload_tables_t(Plan* p) {
   CK(cudaMemcpy(p->d_top_T, p->h_top_T.data(), sizeof(double) * np_top, cudaMemcpyHostToDevice));
   CK(cudaMemcpy(p->d_top_V, p->h_top_V.data(), 6 * sizeof(double) * np_top,
                 cudaMemcpyHostToDevice));
-  CK(cudaMemset(p->d_zero, 0, p->zero_bytes));
-  CK(cudaMemset(p->d_wpart, 0, 6 * sizeof(double) * p->n_wpart));
-  return MLS6_OK;
+  CK(cudaMemset(p->d_zero, 0, all_bytes));
+  return p->spectral ? prepare_direct<T>(p, false) : MLS6_OK;
 }
 
 int upload_tables(Plan* p) {
@@ -269,7 +274,8 @@ static int enqueue(Plan* p, const T* pos, const T* cc, T* forces, double* energy
     for (int k = 1; k < l; ++k) nl += launch_restrict<T>(p, k, st);
   END(3, st);
   BEGIN(4, st);
-  nl += p->spectral ? launch_spectral<T>(p, vir, false, st) : launch_stencil<T>(p, vir, st);
+  nl += p->spectral ? launch_spectral<T>(p, vir, false, st) + launch_direct<T>(p, vir, false, st)
+                    : launch_stencil<T>(p, vir, st);
   END(4, st);
   BEGIN(5, st);
   if (!p->spectral) nl += launch_top<T>(p, vir, st);
@@ -461,6 +467,10 @@ static int eval_lb_t(Plan* p, const T* pos, const T* sigma, const T* eps, T* for
     cudaGetLastError();
     return MLS6_ERR_NOMEM;
   }
+  if (p->spectral && !p->direct[1][1].d_stages) {
+    rc = prepare_direct<T>(p, true);
+    if (rc) return rc;
+  }
   cudaStream_t st = p->cs;
   const int l = p->levels;
   p->lb_last = true;
@@ -477,6 +487,7 @@ static int eval_lb_t(Plan* p, const T* pos, const T* sigma, const T* eps, T* for
     CK(cudaMemsetAsync(p->d_lbq, 0, sizeof(T) * 7 * np1, st));
     nl += launch_anterp_lb<T>(p, st, p->d_lbq);
     nl += launch_spectral<T>(p, false, true, st);
+    nl += launch_direct<T>(p, false, true, st);
   }
   for (int m = 0; m < 7 && !p->spectral; ++m) {
     if (m > 0) CK(cudaMemsetAsync(p->d_q1fx, 0, sizeof(T) * np1, st));

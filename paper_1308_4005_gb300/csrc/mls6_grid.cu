@@ -75,7 +75,7 @@ struct LbCoef {
 template <typename T, int NP = 4, int NC = 1>
 __device__ __forceinline__ void k_anterp_body(const Blk bk,
     const Vec4<T>* __restrict__ sp, int N, int n0, int n1, int n2, T ih0, T ih1, T ih2,
-    const int* __restrict__ flag, double span, typename Fixed<T>::U* __restrict__ qfx,
+    int* __restrict__ flag, double span, typename Fixed<T>::U* __restrict__ qfx,
     const T* __restrict__ lbw, int lbm, const LbCoef& lbc) {
   using U = typename Fixed<T>::U;
   constexpr int B0 = NP / 2 - 1;  // first node of the support below base
@@ -92,6 +92,7 @@ __device__ __forceinline__ void k_anterp_body(const Blk bk,
     const int m = NC == 1 ? lbm : (int)threadIdx.x;
     sexp[threadIdx.x] = fixed_exponent<T>(flag, span, m, m < 0 ? 0.0 : lbc.c[m]);
   }
+  if (bk.x == 0 && threadIdx.x == blockDim.x - 1) flag[kThin] = thin_choice(flag, NC > 1);
   const Vec4<T> p = valid ? sp[i] : Vec4<T>{T(0), T(0), T(0), T(0)};
   const T lw = valid && (NC > 1 || lbm >= 0) ? lbw[i] : T(0);
   const T u0 = p.x * ih0, u1 = p.y * ih1, u2 = p.z * ih2;
@@ -180,7 +181,7 @@ template <typename T, int NP, int NC>
 __global__ void __launch_bounds__(kBlock, sizeof(T) == 8 ? 2 : NP == 6 ? 3 : NC == 7 ? 4 : 6)
 k_anterp(
     const Vec4<T>* __restrict__ sp, int N, int n0, int n1, int n2, T ih0, T ih1, T ih2,
-    const int* __restrict__ flag, double span, typename Fixed<T>::U* __restrict__ qfx,
+    int* __restrict__ flag, double span, typename Fixed<T>::U* __restrict__ qfx,
     const T* __restrict__ lbw, int lbm, const __grid_constant__ LbCoef lbc) {
   k_anterp_body<T, NP, NC>(Blk::self(), sp, N, n0, n1, n2, ih0, ih1, ih2, flag, span, qfx, lbw, lbm, lbc);
 }
@@ -258,29 +259,40 @@ template <typename T> int launch_from_fixed(Plan* p, cudaStream_t st, int lbm, c
 
 // sqrt(2 eps) of the atoms in sorted order, and its largest value
 // (flag[6..7] as a double; one atomic per block on the value's bits, which
-// order like the integers for non-negative doubles).
+// order like the integers for non-negative doubles) and least nonzero one
+// (flag[kThinW..]).
 template <typename T>
 __global__ void k_lb_weights(const T* __restrict__ eps, const int* __restrict__ sidx, int N,
                              T* __restrict__ lbw, int* __restrict__ flag) {
   const long z = pdl_begin();
   eps += z; sidx += z;
-  __shared__ double wmax[32];
+  __shared__ T wmax[32], wmin[32];
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  double m = 0.0;
+  T m = T(0);
   if (i < N) {
     const T e = eps[sidx[i]];
     const T w = sqrt(T(2) * (e > T(0) ? e : T(0)));
     lbw[i] = w;
-    m = (double)w;
-    if (!isfinite(m)) atomicOr(flag, 1);
+    if (!isfinite(w)) atomicOr(flag, 1);
+    m = fmax(w, T(0));  // NaN counts as none
   }
-  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = m;
+  T lo = m > T(0) ? m : T(INFINITY);
+  warp_range(lo, m);
+  if ((threadIdx.x & 31) == 0) {
+    wmax[threadIdx.x >> 5] = m;
+    wmin[threadIdx.x >> 5] = lo;
+  }
   __syncthreads();
   if (threadIdx.x == 0) {
-    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) m = fmax(m, wmax[w]);
-    atomicMax(reinterpret_cast<unsigned long long*>(flag + 6),
-              (unsigned long long)__double_as_longlong(m));
+    for (int w = 1; w < (int)(blockDim.x >> 5); ++w) {
+      m = fmax(m, wmax[w]);
+      lo = fmin(lo, wmin[w]);
+    }
+    raise_to(reinterpret_cast<unsigned long long*>(flag + 6),
+             (unsigned long long)__double_as_longlong((double)m));
+    if (lo <= m)  // else no atom with a depth
+      raise_to(reinterpret_cast<unsigned long long*>(flag + kThinW),
+               ~(unsigned long long)__double_as_longlong((double)lo));
   }
 }
 
@@ -531,12 +543,12 @@ __global__ void __launch_bounds__(kStencilThreads * G) k_stencil(StencilArgs<T> 
 // and tap table exceed the shared-memory budget (large 2a/h): one thread per
 // node, periodic indices, taps read from global memory (warp-uniform).
 template <typename T, bool VIR>
-__global__ void __launch_bounds__(kBlock) k_stencil_global(StencilArgs<T> A,
-                                                           double* __restrict__ wpart,
-                                                           long nodes_total) {
+__device__ __forceinline__ void k_stencil_global_body(const Blk bk, const StencilArgs<T>& A,
+                                                      double* __restrict__ wpart,
+                                                      long nodes_total) {
   pdl_begin();
   __shared__ double red[32 * 6];
-  const long gid = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  const long gid = (long)bk.x * blockDim.x + threadIdx.x;
   // level of this node (levels are concatenated)
   long off = 0;
   int k = 0;
@@ -587,8 +599,15 @@ __global__ void __launch_bounds__(kBlock) k_stencil_global(StencilArgs<T> A,
     double w6[6];
     block_sum_lo<T, 6>(v6, w6, red);
     if (threadIdx.x == 0)
-      for (int c = 0; c < 6; ++c) wpart[6 * (size_t)blockIdx.x + c] = 0.5 * A.hc[c] * w6[c];
+      for (int c = 0; c < 6; ++c) wpart[6 * (size_t)bk.x + c] = 0.5 * A.hc[c] * w6[c];
   }
+}
+
+template <typename T, bool VIR>
+__global__ void __launch_bounds__(kBlock) k_stencil_global(StencilArgs<T> A,
+                                                           double* __restrict__ wpart,
+                                                           long nodes_total) {
+  k_stencil_global_body<T, VIR>(Blk::self(), A, wpart, nodes_total);
 }
 
 template <typename T> static StencilArgs<T> stencil_args(Plan* p) {

@@ -35,6 +35,38 @@ constexpr int kPairSplitMax = 32;  // pair-kernel blocks are at most N * kPairSp
 
 __host__ __device__ inline long cdiv(long a, long b) { return (a + b - 1) / b; }
 
+// Words of Plan::d_flag that choose the form of the grid part (thin_choice): most
+// and (as kThinMany minus it) fewest atoms around an occupied cell, least
+// nonzero |c| and sqrt(2 eps) (doubles, complement of their bits), and the
+// choice (1: the direct kernels).
+constexpr int kFlagWords = 16, kThinMax = 8, kThinMin = 9, kThinC = 10, kThinW = 12, kThin = 14;
+constexpr int kThinMany = 0x7fffffff;
+
+// Atoms in the up to 3 x 3 x 3 cells (periodic, each once) around cell (x, y, z).
+__host__ __device__ inline int atoms_around(const int* start, const int (&nc)[3], int x, int y,
+                                            int z) {
+  // the x range within the row, and beyond its end
+  const int a = nc[0] <= 3 || x == 0 ? 0 : x - 1, b = nc[0] <= 3 || x + 2 > nc[0] ? nc[0] : x + 2;
+  const bool wrap = nc[0] > 3 && (x == 0 || x == nc[0] - 1);
+  const int w = x == 0 ? nc[0] - 1 : 0;
+  int sum = 0;
+#ifdef __CUDA_ARCH__
+#pragma unroll
+#endif
+  for (int k = 0; k < 9; ++k) {  // rows (y + k % 3 - 1, z + k / 3 - 1)
+    const int dy = k % 3 - 1, dz = k / 3 - 1;
+    if ((dy < 0 && nc[1] < 3) || (dy > 0 && nc[1] < 2) || (dz < 0 && nc[2] < 3) ||
+        (dz > 0 && nc[2] < 2))
+      continue;
+    const int yy = y + dy < 0 ? nc[1] - 1 : y + dy >= nc[1] ? 0 : y + dy;
+    const int zz = z + dz < 0 ? nc[2] - 1 : z + dz >= nc[2] ? 0 : z + dz;
+    const int* row = start + (long)nc[0] * (yy + (long)nc[1] * zz);
+    sum += row[b] - row[a];
+    if (wrap) sum += row[w + 1] - row[w];
+  }
+  return sum;
+}
+
 // A caller's array that kernels read or write: device (or managed) memory,
 // or page-locked host memory that the device addresses through the same
 // pointer (unified addressing; kernels then reach it over the host link).
@@ -125,7 +157,8 @@ struct Plan {
   void* d_pos_w = nullptr;     // Vec4<T>[N]: wrapped positions + c, input order
   int2* d_cell_of = nullptr;   // [N]: cell, place among the cell's atoms
   // what every evaluation starts from zero, one region (zero_bytes):
-  // d_flag | d_scan | d_cell_count | d_q1fx
+  // d_flag | d_scan | d_cell_count | d_q1fx | queue of the direct grid part |
+  // virial records of the grid part; those of the pair sum follow
   char* d_zero = nullptr;
   size_t zero_bytes = 0;
   int* d_cell_count = nullptr; // int[ncell]
@@ -150,6 +183,16 @@ struct Plan {
   void* d_spec_tab = nullptr;  // restriction factors per axis | level-1 factors, 7 octants
   double* d_spec_top = nullptr;// coarsest-level factors, 7 grids
   void* d_spec_s = nullptr;    // transforms of q^1 and of e^{1,tot}
+  // the direct grid part in one launch, for thin phases (mls6_direct.cu): the
+  // stages of an evaluation [0] and of a Lorentz-Berthelot one [1] for blocks of
+  // two and of four stencil thread groups, and their queue
+  struct DirectGrid {
+    void* d_stages = nullptr;
+    int stages = 0;
+    long long items = 0;
+    int blocks[2] = {};        // without, with the virial
+  } direct[2][2];
+  char* d_direct_queue = nullptr;
   void* d_q[kMaxLevels + 1] = {};
   void* d_e[kMaxLevels + 1] = {};
   void* d_et[kMaxLevels + 1] = {};
@@ -158,16 +201,18 @@ struct Plan {
   double* d_top_T = nullptr;
   double* d_top_V = nullptr;
   double* d_epart = nullptr;   // energy partials (interpolation blocks)
-  double* d_wpart = nullptr;   // virial partials: pair blocks | stencil blocks | top nodes
+  double* d_wpart = nullptr;   // virial partials: stencil blocks | top nodes | transforms | pair
+                               // blocks; the part before the pair blocks starts from zero
   long n_epart = 0, n_wpart = 0, n_pair_blocks = 0;
   // virial partials, in 6-double records: stencil blocks | coarsest nodes |
   // pair blocks (room for the largest lane split; only the records of the
   // current split are written and summed)
-  long wpart_stencil = 0, wpart_top = 0, wpart_pair = 0;
+  long wpart_stencil = 0, wpart_top = 0, wpart_spec = 0, wpart_pair = 0;
   double* d_out = nullptr;     // [0] energy, [1..6] virial; [8..] kReduceGroups slice sums of 6
   int* d_flag = nullptr;       // [0] bit 0 non-finite, bit 1 wait timeout, [1] interpolation ticket, [2] tile-pass ticket,
                                // [3] max cell population, [4..5] max |c| (double),
-                               // [6..7] max sqrt(2 eps) (double, Lorentz-Berthelot)
+                               // [6..7] max sqrt(2 eps) (double, Lorentz-Berthelot),
+                               // and the kThin* words
   double* h_out = nullptr;     // pinned host staging of d_out
 
   // per-stage event timing (mls6_profile): start/end event per stage
@@ -268,6 +313,11 @@ int launch_from_fixed(Plan* p, cudaStream_t st, int lbm = -1, const void* qfx = 
 bool spectral_eligible(const Plan* p);
 template <typename T> int prepare_spectral(Plan* p);
 template <typename T> int launch_spectral(Plan* p, bool vir, bool lb, cudaStream_t st);
+// the direct grid part where thin_choice fell on it (mls6_direct.cu)
+size_t direct_queue_bytes(const Plan* p);
+long direct_records(const Plan* p);  // virial records of its stencil
+template <typename T> int prepare_direct(Plan* p, bool lb);
+template <typename T> int launch_direct(Plan* p, bool vir, bool lb, cudaStream_t st);
 template <typename T> int launch_lb_weights(Plan* p, const T* eps, cudaStream_t st);
 template <typename T> int launch_interp_lb(Plan* p, T* forces, cudaStream_t st);
 template <typename T> int launch_restrict(Plan* p, int k, cudaStream_t st);

@@ -50,7 +50,7 @@
 namespace mls6 {
 
 enum PStage : int {
-  P_ZERO, P_BIN, P_SCAN_TILES, P_SCAN_FINAL, P_SCATTER, P_CELLSORT, P_PAIR, P_ANTERP,
+  P_ZERO, P_BIN, P_SCAN_TILES, P_SCAN_FINAL, P_SCATTER, P_CELLSORT, P_THIN, P_PAIR, P_ANTERP,
   P_FROM_FIXED, P_RESTRICT, P_STENCIL, P_PROLONG, P_SPEC_FWD, P_SPEC_Z, P_SPEC_TREE, P_SPEC_IZ,
   P_SPEC_INV, P_INTERP, P_OUT
 };
@@ -66,12 +66,13 @@ struct ScatterP { const int2* cell_of; int N; const int* start; int* sidx; };
 struct CellsortP {
   const int* start; long ncell; const Vec4<float>* posw; Vec4<float>* sorted; int* sidx;
 };
+struct ThinP { const int* start; long ncell; ThinArgs g; int* flag; };
 struct PairP {
   const Vec4<float>* sp; const int* start; int N; PairArgs<float> g; float* e0; float* floc;
   double* wpart; int S;
 };
 struct AnterpP {
-  const Vec4<float>* sp; int N, n0, n1, n2; float ih0, ih1, ih2; const int* flag; double span;
+  const Vec4<float>* sp; int N, n0, n1, n2; float ih0, ih1, ih2; int* flag; double span;
   unsigned* qfx;
 };
 struct FromFixedP { const unsigned* qfx; long np; const int* flag; double span; float* q; };
@@ -90,22 +91,24 @@ struct OutP { const double* out; const int* flag; double* ew; int* flagdst; };
 // the anterpolation does not wait for the pair sum (the two only read the
 // sorted atoms) and the interpolation waits for both the grid chain and the
 // pair sum.
+// A replica with both forms of the grid part lists the stages of both; gate is
+// its choice (1: direct) and want the value for which the stage runs.  The
+// items of the direct ones, which run only for thin phases, are `chunk` blocks
+// each.
 struct PStageDesc {
   int kind;
   unsigned nb;
+  unsigned blocks, chunk;
+  const int* gate;
+  int want;
   int dep, dep2;            // stage indices waited for (-1: none)
   unsigned dep_nb, dep2_nb; // their block counts
   union U {
-    ZeroP z; BinP bin; ScanTilesP st; ScanFinalP sf; ScatterP sc; CellsortP cs; PairP pair;
-    AnterpP an; FromFixedP ff; RestrictP re; StencilP sten; ProlongP pr; SpecArgs<float> sp;
+    ZeroP z; BinP bin; ScanTilesP st; ScanFinalP sf; ScatterP sc; CellsortP cs; ThinP th;
+    PairP pair; AnterpP an; FromFixedP ff; RestrictP re; StencilP sten; ProlongP pr; SpecArgs<float> sp;
     InterpP in; OutP out;
     U() {}
   } u;
-};
-
-struct PQueue {
-  unsigned long long ticket;  // next item
-  int error;                  // bit 0: a bounded wait ran out
 };
 
 struct PExecArgs {
@@ -119,8 +122,8 @@ struct PExecArgs {
 };
 
 template <bool VIR>
-__device__ __forceinline__ void run_stage(const PStageDesc& d, unsigned b) {
-  const Blk bk{b, d.nb};
+__device__ __forceinline__ void run_block(const PStageDesc& d, unsigned b) {
+  const Blk bk{b, d.blocks};
   switch (d.kind) {
     case P_ZERO: {
       const ZeroP& a = d.u.z;
@@ -152,6 +155,11 @@ __device__ __forceinline__ void run_stage(const PStageDesc& d, unsigned b) {
     case P_CELLSORT: {
       const CellsortP& a = d.u.cs;
       k_cellsort_body<float>(bk, a.start, a.ncell, a.posw, a.sorted, a.sidx, nullptr);
+      break;
+    }
+    case P_THIN: {
+      const ThinP& a = d.u.th;
+      k_thin_body(bk, a.start, a.ncell, a.g, a.flag);
       break;
     }
     case P_PAIR: {
@@ -223,10 +231,14 @@ __device__ __forceinline__ void run_stage(const PStageDesc& d, unsigned b) {
   }
 }
 
-__device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
-  unsigned v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
+template <bool VIR>
+__device__ __forceinline__ void run_stage(const PStageDesc& d, unsigned b) {
+  if (d.gate && *(volatile const int*)d.gate != d.want) return;
+  const unsigned end = min(d.blocks, (b + 1) * d.chunk);
+  for (unsigned k = b * d.chunk; k < end; ++k) {
+    if (k > b * d.chunk) __syncthreads();  // the shared memory is the next block's
+    run_block<VIR>(d, k);
+  }
 }
 
 template <bool VIR>
@@ -319,7 +331,10 @@ static void replica_stages(Plan* p, const float* pos, const float* cc, float* fo
     out.emplace_back();
     PStageDesc& d = out.back();
     d.kind = kind;
-    d.nb = (unsigned)std::max(0L, nb);
+    d.blocks = d.nb = (unsigned)std::max(0L, nb);
+    d.chunk = 1;
+    d.gate = nullptr;
+    d.want = 0;
     d.dep = d.dep2 = -1;
     d.dep_nb = d.dep2_nb = 0;
     return d;
@@ -355,6 +370,19 @@ static void replica_stages(Plan* p, const float* pos, const float* cc, float* fo
     d.u.cs = CellsortP{p->d_cell_start, ncell, (const Vec4<float>*)p->d_pos_w,
                        (Vec4<float>*)p->d_sorted, p->d_sorted_idx};
   }
+  const bool sp = p->spectral;
+  // a stage of the form that runs when the choice is `want`
+  auto gated = [&](PStageDesc& d, int want, unsigned chunk) {
+    if (!sp) return;
+    d.gate = p->d_flag + kThin;
+    d.want = want;
+    d.chunk = chunk;
+    d.nb = (unsigned)cdiv(d.blocks, chunk);
+  };
+  {
+    PStageDesc& d = add(P_THIN, sp ? cdiv(ncell, kBlock) : 0);
+    d.u.th = ThinP{p->d_cell_start, ncell, thin_args(p), p->d_flag};
+  }
   {
     PStageDesc& d = add(P_PAIR, cdiv((long)N * p->pair_split, kBlock));
     d.u.pair = PairP{(const Vec4<float>*)p->d_sorted, p->d_cell_start, N, pair_args<float>(p),
@@ -368,14 +396,15 @@ static void replica_stages(Plan* p, const float* pos, const float* cc, float* fo
                      (float)(1.0 / L1.h[0]), (float)(1.0 / L1.h[1]), (float)(1.0 / L1.h[2]),
                      p->d_flag, span, (unsigned*)p->d_q1fx};
   }
-  const bool sp = p->spectral;
   {
-    PStageDesc& d = add(P_FROM_FIXED, sp ? 0 : cdiv(L1.np, kBlock));
+    PStageDesc& d = add(P_FROM_FIXED, cdiv(L1.np, kBlock));
     d.u.ff = FromFixedP{(const unsigned*)p->d_q1fx, L1.np, p->d_flag, span, (float*)p->d_q[1]};
+    gated(d, 1, 16);
   }
   for (int k = 1; k < lmax; ++k) {  // restriction slots (empty beyond this replica's levels)
-    const bool on = k < l && !sp;
+    const bool on = k < l;
     PStageDesc& d = add(P_RESTRICT, on ? cdiv(p->lv[k + 1].np, kBlock) : 0);
+    gated(d, 1, 4);
     if (on) {
       const Level &F = p->lv[k], &C = p->lv[k + 1];
       d.u.re = RestrictP{(const float*)p->d_q[k], F.n[0], F.n[1], F.n[2], (float*)p->d_q[k + 1],
@@ -384,14 +413,16 @@ static void replica_stages(Plan* p, const float* pos, const float* cc, float* fo
   }
   {
     const int warps = kStencilThreads * 2 / 32;
-    PStageDesc& d = add(P_STENCIL, sp ? 0 : p->stencil_blocks + cdiv(p->lv[l].np, warps));
+    PStageDesc& d = add(P_STENCIL, p->stencil_blocks + cdiv(p->lv[l].np, warps));
+    gated(d, 1, 4);
     d.u.sten.A = stencil_args<float>(p);
     d.u.sten.wpart = p->d_wpart + 6 * p->wpart_stencil;
   }
   for (int j = 0; j < lmax - 1; ++j) {  // prolongation slots, coarse to fine
     const int k = l - 1 - j;
-    const bool on = k >= 1 && !sp;
+    const bool on = k >= 1;
     PStageDesc& d = add(P_PROLONG, on ? cdiv(p->lv[k].np, kBlock) : 0);
+    gated(d, 1, 16);
     if (on) {
       const Level &F = p->lv[k], &C = p->lv[k + 1];
       d.u.pr = ProlongP{(const float*)p->d_e[k], F.n[0], F.n[1], F.n[2],
@@ -406,6 +437,7 @@ static void replica_stages(Plan* p, const float* pos, const float* cc, float* fo
     for (int k = 0; k < 5; ++k) {
       PStageDesc& d = add(P_SPEC_FWD + k, nb[k]);
       if (sp) d.u.sp = spec_args<float>(p, false);
+      gated(d, 0, 1);
     }
   }
   {
@@ -489,10 +521,10 @@ int persist_build(PersistExec** out, Plan* const* plans, int B, const int64_t* o
   for (int r = 0; r < B; ++r) {
     const Plan* p = plans[r];
     const int* n = p->lv[1].n;
-    smem = std::max(smem, p->spectral ? std::max({spec_plane_smem<float>(n[0], n[1], (n[0] / 2 + 1) | 1),
-                                                  spec_z_smem<float>(n[2]),
-                                                  spec_tree_smem<float>(p->levels)})
-                                      : p->stencil_smem);
+    smem = std::max(smem, p->stencil_smem);
+    if (p->spectral)
+      smem = std::max({smem, spec_plane_smem<float>(n[0], n[1], (n[0] / 2 + 1) | 1),
+                       spec_z_smem<float>(n[2]), spec_tree_smem<float>(p->levels)});
   }
   x->smem = smem;
   int rc = MLS6_OK;

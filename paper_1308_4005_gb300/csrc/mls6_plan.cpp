@@ -264,9 +264,10 @@ static void free_plan(Plan* p) {
   if (!p) return;
   void* ptrs[] = {p->d_pos_w, p->d_cell_of, p->d_zero, p->d_cell_start, p->d_sorted,
                   p->d_sorted_f, p->d_sorted_idx, p->d_e0, p->d_floc, p->d_rows, p->d_wv, p->d_top_T,
-                  p->d_top_V, p->d_epart, p->d_wpart, p->d_out, p->d_tcw, p->d_lbw, p->d_lbpot, p->d_mma_rows, p->d_mma_bv,
+                  p->d_top_V, p->d_epart, p->d_out, p->d_tcw, p->d_lbw, p->d_lbpot, p->d_mma_rows, p->d_mma_bv,
                   p->d_mma_be, p->d_lbq, p->d_lbs, p->d_spec_tw, p->d_spec_tab, p->d_spec_top,
-                  p->d_spec_s};
+                  p->d_spec_s, p->direct[0][0].d_stages, p->direct[0][1].d_stages,
+                  p->direct[1][0].d_stages, p->direct[1][1].d_stages};
   for (void* q : ptrs)
     if (q) cudaFree(q);
   for (int k = 1; k <= kMaxLevels; ++k) {

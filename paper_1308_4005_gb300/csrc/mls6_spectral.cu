@@ -13,7 +13,10 @@
 //                  the transform of the taps g_k'/r r_a r_b
 // The direct kernels (mls6_grid.cu, the tensor-core stencils) compute the same
 // grids node by node; they stay for grids this form does not take, for plans
-// that ask for a stencil kernel, and for mls6_debug_grid.
+// that ask for a stencil kernel, for mls6_debug_grid, and for evaluations with
+// thin phases, whose potentials the transforms would round too coarsely: there
+// (k_thin_body, mls6_bin.cu) every kernel here returns at once and the direct
+// form runs in one launch behind them (mls6_direct.cu).
 //
 // Why: the direct stencils cost ~1000 taps per node (14 operations each with
 // the virial) and the hierarchy 2 l launches of ever smaller grids; the
@@ -66,7 +69,7 @@ template <typename T> struct SpecArgs {
   unsigned long long rad[3];      // radices, 5 bits each (x: of M), lowest first
   const Cx<T>* tw[3];             // exp(-2 pi i j / n_d), j < n_d
   const typename Fixed<T>::U* qfx;
-  const int* flag;
+  const int* flag;                // flag[kThin]: the direct kernels run instead
   double span;
   int lb;                         // Lorentz-Berthelot: channel = grid y index
   double lbc[7];
@@ -442,29 +445,34 @@ __device__ __forceinline__ void spec_tree_body(const Blk bk, int ch, const SpecA
 }
 
 #ifndef MLS6_DEVICE_ONLY
+template <typename T> __device__ __forceinline__ bool spec_off(const SpecArgs<T>& A) {
+  pdl_begin();
+  return *(volatile const int*)(A.flag + kThin) != 0;
+}
+
 template <typename T, int MAXR>
 __global__ void __launch_bounds__(spec_plane_threads<T, MAXR>()) k_spec_fwd(SpecArgs<T> A) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  pdl_begin();
+  if (spec_off(A)) return;
   spec_fwd_body<T, MAXR>(Blk::self(), blockIdx.y, A, smem_raw);
 }
 template <typename T, int MAXR>
 __global__ void __launch_bounds__(kSpecThreads, MAXR == 8 && sizeof(T) == 4 ? 4 : 1)
     k_spec_z(SpecArgs<T> A, T sg) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  pdl_begin();
+  if (spec_off(A)) return;
   spec_z_body<T, MAXR>(Blk::self(), blockIdx.y, A, sg, smem_raw);
 }
 template <typename T, bool VIR>
 __global__ void __launch_bounds__(kSpecThreads) k_spec_tree(SpecArgs<T> A) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  pdl_begin();
+  if (spec_off(A)) return;
   spec_tree_body<T, VIR>(Blk::self(), blockIdx.y, A, smem_raw);
 }
 template <typename T, int MAXR>
 __global__ void __launch_bounds__(spec_plane_threads<T, MAXR>()) k_spec_inv(SpecArgs<T> A) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  pdl_begin();
+  if (spec_off(A)) return;
   spec_inv_body<T, MAXR>(Blk::self(), blockIdx.y, A, smem_raw);
 }
 #endif  // MLS6_DEVICE_ONLY
@@ -506,7 +514,7 @@ template <typename T> static SpecArgs<T> spec_args(const Plan* p, bool lb) {
   A.S = reinterpret_cast<Cx<T>*>(lb ? p->d_lbs : p->d_spec_s);
   A.R = A.S + (lb ? 7 : 1) * A.ns;
   A.et = reinterpret_cast<T*>(lb ? p->d_lbpot : p->d_et[1]);
-  A.wpart = p->d_wpart;
+  A.wpart = p->d_wpart + 6 * p->wpart_spec;
   A.inv_n = (T)(1.0 / (double)L1.np);
   return A;
 }
