@@ -385,7 +385,8 @@ __device__ __forceinline__ void spec_tree_body(const Blk bk, int ch, const SpecA
     __syncthreads();
     off = o1;
   }
-  // coarsest level in FP64
+  // coarsest level in FP64, its virial added to the record behind the levels' sum
+  double wt[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};  // (thread 0)
   T wv[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
   const int npt = A.m[0] * A.m[1] * A.m[2];
   if (threadIdx.x == 0) {
@@ -393,7 +394,7 @@ __device__ __forceinline__ void spec_tree_body(const Blk bk, int ch, const SpecA
     if (VIR) {
       const double p = 0.5 / npt * ((double)v.x * v.x + (double)v.y * v.y);
 #pragma unroll
-      for (int c = 0; c < 6; ++c) wv[c] = (T)(p * A.Kt[(size_t)(c + 1) * npt + bk.x]);
+      for (int c = 0; c < 6; ++c) wt[c] = p * A.Kt[(size_t)(c + 1) * npt + bk.x];
     }
     const double t = A.Kt[bk.x];
     q[off] = Cx<T>{(T)(t * v.x), (T)(t * v.y)};
@@ -440,7 +441,7 @@ __device__ __forceinline__ void spec_tree_body(const Blk bk, int ch, const SpecA
     double ws[6];
     block_sum_lo<T, 6>(wv, ws, red);
     if (threadIdx.x == 0)
-      for (int c = 0; c < 6; ++c) A.wpart[6 * (size_t)bk.x + c] = ws[c];
+      for (int c = 0; c < 6; ++c) A.wpart[6 * (size_t)bk.x + c] = ws[c] + wt[c];
   }
 }
 
