@@ -416,7 +416,7 @@ __device__ __forceinline__ void spec_tree_body(const Blk bk, int ch, const SpecA
       const Vec4<T> Ka = K[0];
       const Cx<T> v = q[off + e];
       if (VIR) {
-        const T p = hs * (v.x * v.x + v.y * v.y);
+        const T p = (hs * v.x) * v.x + (hs * v.y) * v.y;  // |v|^2 ~ (N c)^2 alone may overflow
         const Vec4<T> Kb = K[1];
         wv[0] += p * Ka.y;
         wv[1] += p * Ka.z;

@@ -42,3 +42,22 @@ def test_coarsest_virial_is_kept_in_fp64(gpu_lib, a):
     k = _k1(a)
     want = W["fp64"] + 32.0 * (float(np.float32(k)) - k)
     assert np.abs(W["fp32"] - want).max() <= 1e-13 * np.abs(W["fp64"]).max()
+
+
+@pytest.mark.parametrize("shift", [56, -32])
+def test_virial_scales_with_large_and_small_coefficients(gpu_lib, shift):
+    """c 2^s gives the virial times 2^(2s), bit for bit: every operation on the
+    way is exact under powers of two as long as none leaves the FP32 range.
+    c^2 times the sums of a system of 400 atoms, 2^112 x 10^3, is inside it; the
+    square of a transform's entry, (N c)^2 times the nodes, is not."""
+    import torch
+
+    box = (8.0, 8.0, 16.0)
+    x, c = I.uniform_atoms(41, 400, box)
+    plan = gpu_lib.Plan(box, 400, 2.0, 1.0, 2, precision="fp32")
+    W = []
+    for s in (0, shift):
+        pos = torch.tensor(np.c_[x, c], dtype=torch.float32, device="cuda")
+        pos[:, 3] *= 2.0 ** s
+        W.append(plan.evaluate(pos)["out"].cpu().numpy()[1:])
+    assert np.all(np.isfinite(W[1])) and np.array_equal(W[1], W[0] * 2.0 ** (2 * shift))
