@@ -272,9 +272,12 @@ __global__ void k_scatter(const int2* __restrict__ cell_of, int N, const int* __
 // the atomics of the binning.  Cells of up to 8 atoms (nearly all at liquid
 // densities with cells of width a/2) sort 64-bit keys (the bits of x >= 0 over
 // the index) in registers by an odd-even transposition network and only then
-// copy the records; larger cells use an insertion sort of the indices in
-// global memory; cells above 256 atoms are left in scatter order (results stay
-// correct, only bitwise reproducibility is lost for them).  FP64 plans also get
+// copy the records; in larger cells every atom counts the smaller keys of its
+// cell (one thread per atom, the cell's keys from L1); cells above 256 atoms
+// are left in scatter order (results stay correct, only bitwise reproducibility
+// is lost for them).  Threads that count are those of the block that has the
+// cells, or, from kSlotAtoms atoms per cell on, of blocks of their own (a block
+// of 256 cells would take thousands of atoms).  FP64 plans also get
 // the positions in FP32, for the cutoff test of the pair sum's queue form.
 template <typename T>
 __device__ __forceinline__ unsigned long long record_key(const Vec4<T>* __restrict__ posw, int i) {
@@ -283,27 +286,51 @@ __device__ __forceinline__ unsigned long long record_key(const Vec4<T>* __restri
   return k;
 }
 
+// slots: scatter-order indices, sidx: the cell order's.  big: the block also
+// takes its cells of more than 8 atoms.
+template <typename T>
+__device__ __forceinline__ void put_record(Vec4<T>* sorted, float4* sortedf, int k, const Vec4<T>& v) {
+  sorted[k] = v;
+  if constexpr (sizeof(T) == 8)
+    sortedf[k] = make_float4((float)v.x, (float)v.y, (float)v.z, 0.f);
+}
+
+// The atom in slot k, if its cell has more than 8: its place among the cell's.
+template <typename T>
+__device__ __forceinline__ void rank_in_cell(const int* __restrict__ start,
+                           const int2* __restrict__ cell_of, const Vec4<T>* __restrict__ posw,
+                           Vec4<T>* __restrict__ sorted, const int* __restrict__ slots,
+                           int* __restrict__ sidx, float4* __restrict__ sortedf, int k) {
+  const int i = slots[k];
+  const int c = cell_of[i].x;
+  const int b = start[c], e = start[c + 1];
+  if (e - b <= 8) return;
+  int at = k;
+  if (e - b <= 256) {
+    const unsigned long long key = record_key(posw, i);
+    at = b;
+#pragma unroll 4
+    for (int j = b; j < e; ++j) at += record_key(posw, slots[j]) < key ? 1 : 0;
+  }
+  sidx[at] = i;
+  put_record(sorted, sortedf, at, posw[i]);
+}
+
 template <typename T>
 __device__ __forceinline__ void k_cellsort_body(const Blk bk,const int* __restrict__ start, long ncell,
-                           const Vec4<T>* __restrict__ posw, Vec4<T>* __restrict__ sorted,
-                           int* __restrict__ sidx, float4* __restrict__ sortedf) {
+                           const int2* __restrict__ cell_of, const Vec4<T>* __restrict__ posw,
+                           Vec4<T>* __restrict__ sorted, const int* __restrict__ slots,
+                           int* __restrict__ sidx, float4* __restrict__ sortedf, bool big) {
   const long z = pdl_begin();
-  start += z; posw += z;
-  auto put = [&](int k, const Vec4<T>& v) {
-    sorted[k] = v;
-    if constexpr (sizeof(T) == 8)
-      sortedf[k] = make_float4((float)v.x, (float)v.y, (float)v.z, 0.f);
-  };
-  const long cell = (long)bk.x * blockDim.x + threadIdx.x;
-  if (cell >= ncell) return;
-  const int b = start[cell], e = start[cell + 1];
-  const int n = e - b;
+  start += z; posw += z; cell_of += z; slots += z;
+  const long first = (long)bk.x * blockDim.x, cell = first + threadIdx.x;
+  const int b = cell < ncell ? start[cell] : 0, n = cell < ncell ? start[cell + 1] - b : 0;
   if (n <= 8) {
     unsigned long long key[8];
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
       key[k] = ~0ull;
-      if (k < n) key[k] = record_key(posw, sidx[b + k]);
+      if (k < n) key[k] = record_key(posw, slots[b + k]);
     }
 #pragma unroll
     for (int r = 0; r < 8; ++r)
@@ -319,22 +346,14 @@ __device__ __forceinline__ void k_cellsort_body(const Blk bk,const int* __restri
       if (k < n) {
         const int i = (int)(unsigned)key[k];
         sidx[b + k] = i;
-        put(b + k, posw[i]);
+        put_record(sorted, sortedf, b + k, posw[i]);
       }
-    return;
   }
-  if (n <= 256)
-    for (int i = b + 1; i < e; ++i) {
-      const int id = sidx[i];
-      const unsigned long long key = record_key(posw, id);
-      int j = i - 1;
-      while (j >= b && record_key(posw, sidx[j]) > key) {
-        sidx[j + 1] = sidx[j];
-        --j;
-      }
-      sidx[j + 1] = id;
-    }
-  for (int i = b; i < e; ++i) put(i, posw[sidx[i]]);
+  if (big && __syncthreads_or(n > 8)) {
+    const int lo = start[first], hi = start[min(ncell, first + (long)blockDim.x)];
+    for (int k = lo + threadIdx.x; k < hi; k += blockDim.x)
+      rank_in_cell<T>(start, cell_of, posw, sorted, slots, sidx, sortedf, k);
+  }
 }
 
 // Which form the grid part takes.  A transform spreads the rounding of the
@@ -395,21 +414,42 @@ __device__ __forceinline__ void k_thin_body(const Blk bk, const int* __restrict_
   }
 }
 
-// nsort blocks sort, the others (if any) choose the form of the grid part.
+// Blocks: cells, atoms of large cells (if any blocks are theirs), the choice of
+// the grid part's form (if any).
 template <typename T>
 __global__ void k_cellsort(const int* __restrict__ start, long ncell,
-                           const Vec4<T>* __restrict__ posw, Vec4<T>* __restrict__ sorted,
-                           int* __restrict__ sidx, float4* __restrict__ sortedf, int nsort,
-                           ThinArgs g, int* __restrict__ flag) {
-  if ((int)blockIdx.x < nsort)
-    k_cellsort_body<T>(Blk::self(), start, ncell, posw, sorted, sidx, sortedf);
-  else
-    k_thin_body(Blk{blockIdx.x - nsort, gridDim.x - nsort}, start, ncell, g, flag);
+                           const int2* __restrict__ cell_of, const Vec4<T>* __restrict__ posw,
+                           Vec4<T>* __restrict__ sorted, const int* __restrict__ slots,
+                           int* __restrict__ sidx, float4* __restrict__ sortedf, int N, int ncells,
+                           int nslots, ThinArgs g, int* __restrict__ flag) {
+  const int b = (int)blockIdx.x - ncells;
+  if (b < 0) {
+    k_cellsort_body<T>(Blk::self(), start, ncell, cell_of, posw, sorted, slots, sidx, sortedf,
+                       nslots == 0);
+  } else if (b < nslots) {
+    const long z = pdl_begin();
+    const int k = b * blockDim.x + threadIdx.x;
+    if (k < N)
+      rank_in_cell<T>(start + z, cell_of + z, posw + z, sorted, slots + z, sidx, sortedf, k);
+  } else {
+    k_thin_body(Blk{(unsigned)(b - nslots), gridDim.x - ncells - nslots}, start, ncell, g, flag);
+  }
 }
 
 static ThinArgs thin_args(const Plan* p) {
   return ThinArgs{{p->cg.nc[0], p->cg.nc[1], p->cg.nc[2]}};
 }
+
+// Atoms per cell from which the atoms of large cells get blocks of their own.
+// Binning stage, 100,000 atoms in FP32, with an insertion sort per cell (one
+// thread, two dependent loads per comparison) -> here: 6.8 atoms per cell
+// (a = 4) 39 -> 19 us (30 without blocks of their own), 13 (a = 5) 92 -> 21, 54
+// (a = 8) 911 -> 26; cells of 370 atoms, copied by one thread each, 2588 -> 26.
+// Between 4 and 6 atoms per cell the two agree.
+constexpr long kSlotAtoms = 6;
+
+// Scatter-order indices: in the pair sum's output, which is written later.
+static int* scatter_slots(const Plan* p) { return reinterpret_cast<int*>(p->d_floc); }
 
 // Arguments of the binning kernel for a plan.
 template <typename T> static BinArgs<T> bin_args(const Plan* p) {
@@ -440,12 +480,15 @@ int launch_bin(Plan* p, const T* pos, const T* cc, cudaStream_t st) {
                p->d_cell_start, p->d_flag);
   launch_pdl(k_scan_final, ntiles, kBlock, 0, st, (const int*)p->d_cell_count, ncell, (const int*)p->d_scan,
              p->d_cell_start, direct ? 1 : 0, p->d_flag);
+  int* slots = scatter_slots(p);
   launch_pdl(k_scatter, cdiv(N, kBlock), kBlock, 0, st, (const int2*)p->d_cell_of, N,
-             (const int*)p->d_cell_start, p->d_sorted_idx);
-  const int nsort = (int)cdiv(ncell, kBlock);
-  launch_pdl(k_cellsort<T>, p->spectral ? 2 * nsort : nsort, kBlock, 0, st, (const int*)p->d_cell_start,
-             ncell, (const Vec4<T>*)p->d_pos_w, (Vec4<T>*)p->d_sorted, p->d_sorted_idx,
-             (float4*)p->d_sorted_f, nsort, thin_args(p), p->d_flag);
+             (const int*)p->d_cell_start, slots);
+  const int ncells = (int)cdiv(ncell, kBlock);
+  const int nslots = N >= kSlotAtoms * ncell ? (int)cdiv(N, kBlock) : 0;
+  launch_pdl(k_cellsort<T>, ncells + nslots + (p->spectral ? ncells : 0), kBlock, 0, st,
+             (const int*)p->d_cell_start, ncell, (const int2*)p->d_cell_of,
+             (const Vec4<T>*)p->d_pos_w, (Vec4<T>*)p->d_sorted, (const int*)slots,
+             p->d_sorted_idx, (float4*)p->d_sorted_f, N, ncells, nslots, thin_args(p), p->d_flag);
   return direct ? 4 : 5;
 }
 

@@ -64,7 +64,8 @@ struct ScanTilesP { const int* count; long n; int* tsum; int* start; int* flag; 
 struct ScanFinalP { const int* count; long n; const int* tsum; int* start; int direct; int* flag; };
 struct ScatterP { const int2* cell_of; int N; const int* start; int* sidx; };
 struct CellsortP {
-  const int* start; long ncell; const Vec4<float>* posw; Vec4<float>* sorted; int* sidx;
+  const int* start; long ncell; const int2* cell_of; const Vec4<float>* posw;
+  Vec4<float>* sorted; const int* slots; int* sidx;
 };
 struct ThinP { const int* start; long ncell; ThinArgs g; int* flag; };
 struct PairP {
@@ -154,7 +155,8 @@ __device__ __forceinline__ void run_block(const PStageDesc& d, unsigned b) {
     }
     case P_CELLSORT: {
       const CellsortP& a = d.u.cs;
-      k_cellsort_body<float>(bk, a.start, a.ncell, a.posw, a.sorted, a.sidx, nullptr);
+      k_cellsort_body<float>(bk, a.start, a.ncell, a.cell_of, a.posw, a.sorted, a.slots, a.sidx,
+                             nullptr, true);
       break;
     }
     case P_THIN: {
@@ -363,12 +365,12 @@ static void replica_stages(Plan* p, const float* pos, const float* cc, float* fo
   }
   {
     PStageDesc& d = add(P_SCATTER, cdiv(N, kBlock));
-    d.u.sc = ScatterP{p->d_cell_of, N, p->d_cell_start, p->d_sorted_idx};
+    d.u.sc = ScatterP{p->d_cell_of, N, p->d_cell_start, scatter_slots(p)};
   }
   {
     PStageDesc& d = add(P_CELLSORT, cdiv(ncell, kBlock));
-    d.u.cs = CellsortP{p->d_cell_start, ncell, (const Vec4<float>*)p->d_pos_w,
-                       (Vec4<float>*)p->d_sorted, p->d_sorted_idx};
+    d.u.cs = CellsortP{p->d_cell_start, ncell, p->d_cell_of, (const Vec4<float>*)p->d_pos_w,
+                       (Vec4<float>*)p->d_sorted, scatter_slots(p), p->d_sorted_idx};
   }
   const bool sp = p->spectral;
   // a stage of the form that runs when the choice is `want`
