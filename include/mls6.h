@@ -419,9 +419,9 @@ int mls6_batch_size(const mls6_batch_t* b, int* B, int64_t* offsets);
  * replica's previous stage has counted all its blocks (bounded waits, see
  * mls6_batch_set_wait), run the same kernel body as the per-stage launch,
  * and count the item done.  Results equal mls6_eval's on each replica's
- * plan bit for bit.  Setting it gives replicas that have the tile form of the
- * pair sum (their default from 8,192 atoms on) the lanes per atom instead, and
- * they keep those.  persistent = 0 (default), or an ineligible batch: the
+ * plan bit for bit.  Setting it on an eligible batch gives replicas that
+ * have the tile form of the pair sum (their default from 8,192 atoms on) the
+ * lanes per atom instead, and they keep those.  persistent = 0 (default), or an ineligible batch: the
  * graph of per-replica kernel chains described above.  Waits for the
  * batch's work; the next evaluation re-captures. */
 int mls6_batch_set_mode(mls6_batch_t* b, int persistent);

@@ -583,11 +583,7 @@ int mls6_batch_tune(mls6_batch_t* batch, const void* pos, const void* c, void* f
   // FP32 batches whose plans the persistent kernel can run: tune the other
   // launch form too and keep the faster
   // (the persistent form is tuned with 1..8 lanes per atom, which it runs)
-  bool other = b->prec == MLS6_FP32;
-  for (const Plan* p : b->plans)
-    other = other && p->N > 0 && p->levels >= 2 && !p->stencil_global && !p->stencil_mma &&
-            !p->stencil_tc && p->sm.n == 2 && p->order == 3;
-  if (other) {
+  if (std::all_of(b->plans.begin(), b->plans.end(), persist_possible)) {
     const int m0 = b->mode, k0 = b->branches;
     std::vector<int> s0(b->B), g0(b->B);
     for (int r = 0; r < b->B; ++r) {
@@ -637,7 +633,9 @@ int mls6_batch_set_mode(mls6_batch_t* batch, int persistent) {
   if (b->s0 && cudaStreamSynchronize(b->s0) != cudaSuccess) return MLS6_ERR_CUDA;
   b->mode = persistent;
   reset_graph(b);
-  if (persistent)  // the persistent kernel runs the per-atom pair form
+  // the persistent kernel runs the per-atom pair form; a batch that it cannot
+  // run keeps its own
+  if (persistent && std::all_of(b->plans.begin(), b->plans.end(), persist_possible))
     for (Plan* p : b->plans)
       if (p->pair_split == kPairTile) {
         const int rc = mls6_set_tuning(reinterpret_cast<mls6_plan_t*>(p), pair_split_atom(p), 0);

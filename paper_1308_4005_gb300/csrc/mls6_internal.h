@@ -358,6 +358,7 @@ int prepare_stencil_tc(Plan* p);
 int launch_stencil_tc(Plan* p, bool vir, bool fuse_top, cudaStream_t st);
 // persistent batch execution (mls6_persist.cu)
 struct PersistExec;
+bool persist_possible(const Plan* p);  // with the per-atom form of the pair sum
 bool persist_eligible(const Plan* p);
 int persist_build(PersistExec** out, Plan* const* plans, int B, const int64_t* off,
                   const double* cost, const void* pos, const void* c, void* forces, double* ew,

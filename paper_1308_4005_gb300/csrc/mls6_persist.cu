@@ -316,10 +316,14 @@ struct PersistExec {
   size_t smem = 0;
 };
 
-bool persist_eligible(const Plan* p) {
+bool persist_possible(const Plan* p) {
   return p->prec == MLS6_FP32 && p->N > 0 && p->levels >= 2 && !p->stencil_global &&
-         !p->stencil_mma && !p->stencil_tc && p->pair_split >= 1 && p->pair_split <= 8 &&
-         p->sm.n == 2 && p->order == 3 && p->levels <= kMaxLevels;
+         !p->stencil_mma && !p->stencil_tc && p->sm.n == 2 && p->order == 3 &&
+         p->levels <= kMaxLevels;
+}
+
+bool persist_eligible(const Plan* p) {
+  return persist_possible(p) && p->pair_split >= 1 && p->pair_split <= 8;
 }
 
 // The stage list of one replica (mirrors the launch sequence of a single

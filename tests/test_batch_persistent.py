@@ -30,3 +30,15 @@ def test_largest_planes(gpu_lib, box, levels):
         res.append([r[k].cpu().numpy() for k in ("E", "W", "F")])
     for a, b in zip(*res):
         assert np.array_equal(a, b)
+
+
+def test_mode_leaves_a_batch_that_cannot_run_it(gpu_lib):
+    """A batch with a replica without atoms, or in mixed precision, runs its
+    chains whatever the mode: its pair sums stay as they were."""
+    for prec, N in (("mixed", [9000, 9000]), ("fp32", [9000, 0])):
+        bt = gpu_lib.Batch([(24.0, 24.0, 24.0)] * 2, N, 2.5, 1.0, 3, precision=prec)
+        before = bt.info()["pair_split"]
+        assert before[0] == 2048  # the tile form
+        gpu_lib.mls6_batch_set_mode(bt.handle, True)
+        assert gpu_lib.mls6_batch_mode(bt.handle) == 0
+        assert bt.info()["pair_split"] == before
