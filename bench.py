@@ -57,8 +57,17 @@ EXACT_R = 20.0          # radius of the direct sums behind the exact sampled for
 TRAFFIC = {
 }
 
-# arithmetic of each precision mode (pair/grid transfers; level stencils)
+# arithmetic of each precision mode (pair/grid transfers; level stencils, where
+# a mixed plan has them on the tensor cores and no transforms in their place)
 DTYPE = {"fp64": "f64", "fp32": "f32", "mixed": "f32+bf16x3"}
+
+
+def dtype_label(precision, info):
+    if precision == "mixed" and (info["transforms"] or info["stencil_kind"] not in (2, 3)):
+        return DTYPE["fp32"]
+    return DTYPE[precision]
+
+
 DEFAULT_PREC = {"cube1m": "mixed", "slab4m": "fp32"}
 
 
@@ -507,16 +516,13 @@ def stage_work(info, N, n_pairs, prec, vir):
 GRID_STAGES = ("restrict", "coarsest", "prolongate")
 
 
-def grid_part_transformed(stage_ms):
-    return all(stage_ms.get(k) is not None and stage_ms[k] < 0.0035 for k in GRID_STAGES)
-
-
-def rooflines(stage_ms, work, peaks, prec, stencil_kind, workload, vir, work_grid=0.0):
+def rooflines(stage_ms, work, peaks, prec, stencil_kind, workload, vir, work_grid=None):
     """One entry per stage: achieved rate (algorithmic work / stage time)
-    against the stage's peak."""
+    against the stage's peak.  work_grid: bytes of the grid part where the
+    evaluation ran it by transforms."""
     hbm, bf16, hbm_src = peaks["hbm"], peaks["bf16"], peaks["src"]
     out = {}
-    if grid_part_transformed(stage_ms):
+    if work_grid is not None:
         # all levels in the stencil stage, by transforms of the finest grid;
         # the other stages are empty (two events back to back)
         work = {k: v for k, v in work.items() if k not in GRID_STAGES}
@@ -884,6 +890,7 @@ def run_ours(args):
     # ------------------------------------- per-kernel times (serialised pass)
     stage_ms = b.stages(args.steps, flush)
     F_main = b.forces()
+    transformed = mls6.mls6_grid_form(b.plan.handle)[1]  # by the last evaluation
     b.close()
 
     # ------------------------------------------------------------- roofline
@@ -891,18 +898,17 @@ def run_ours(args):
     work = stage_work(info, N, n_pairs, args.precision, vir)
     nodes = math.prod(info["n_grid"][0])
     roofs = rooflines(stage_ms, work, peaks, args.precision, info["stencil_kind"], w.name, vir,
-                      nodes * (16.0 if args.precision == "fp64" else 8.0))
+                      nodes * (16.0 if args.precision == "fp64" else 8.0) if transformed else None)
     dom = max(roofs, key=lambda k: roofs[k]["avg_launch_ms"])
     roof = dict(roofs[dom], kernel=dom,
                 timing=("CUDA events on the launching stream around the stage, averaged over a "
                         "serialised pass of the same steps right after the timed region"))
-    if (dom == "stencil" and info["stencil_kind"] in (2, 3)
-            and not grid_part_transformed(stage_ms)):
+    if dom == "stencil" and info["stencil_kind"] in (2, 3) and not transformed:
         roof["issued_over_useful"] = "32/13 Toeplitz band x 3 split products (energy channel)"
     line = {"metric": "atom-evals/s", "value": value, "unit": "atom-evals/s", "n_gpus": world,
             "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms_per_step,
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-            "dtype": DTYPE[args.precision], "data": "synthetic",
+            "dtype": dtype_label(args.precision, info), "data": "synthetic",
             "config": config_of(w, args, world),
             "e2e": {"value": e2e_value, "unit": "atom-evals/s",
                     "h2d_bytes_per_step": int(b.pos_h.numel() * b.pos_h.element_size()),
@@ -1155,12 +1161,13 @@ def run_batch(args):
             stage_acc[name] = stage_acc.get(name, 0.0) + ms
         lv = pinfo["n_grid"]
         work_pair += count_pairs(x[sl], np.array(w.box), w.a) * (FLOP_PAIR + FLOP_PAIR_VIR)
-        work_sten += sum(n[0] * n[1] * n[2] for n in lv[:-1]) * pinfo["ntaps"] * \
-            (FLOP_TAP + FLOP_TAP_VIR)
+        if not pinfo["transforms"]:  # else the stage is not the taps
+            work_sten += sum(n[0] * n[1] * n[2] for n in lv[:-1]) * pinfo["ntaps"] * \
+                (FLOP_TAP + FLOP_TAP_VIR)
     dom = max(stage_acc, key=lambda k: stage_acc[k])
     fp32_peak = mls6.mls6_fma_peak("fp32")
     roof = None
-    if dom in ("pair", "stencil"):
+    if dom == "pair" or (dom == "stencil" and work_sten):
         amount = (work_pair if dom == "pair" else work_sten) / 1e12
         ach = amount / (stage_acc[dom] / 1e3)
         roof = {"kernel": dom, "bound": "alu", "achieved": ach, "peak": fp32_peak,
@@ -1173,7 +1180,7 @@ def run_batch(args):
     line = {"metric": "atom-evals/s", "value": value, "unit": "atom-evals/s", "n_gpus": world,
             "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms_per_step,
             "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-            "dtype": DTYPE[args.precision], "data": "synthetic",
+            "dtype": dtype_label(args.precision, pinfo), "data": "synthetic",
             "config": {"workload": args.workload, "replicas": nrep, "atoms_per_gpu": Ntot,
                        "N_min": int(min(w.N for w in ws)), "N_max": int(max(w.N for w in ws)),
                        "a": ws[0].a, "h": ws[0].h, "levels": "auto per replica",

@@ -65,11 +65,13 @@ typedef enum {
   MLS6_FP64 = 0,  /* every step in double precision */
   MLS6_FP32 = 1,  /* pair kernel and grids in float; coarsest level, energy
                      and virial accumulation in double */
-  MLS6_MIXED = 2  /* as MLS6_FP32, but the level stencils run on the tensor
-                     cores with BF16 hi+lo split operands and FP32
-                     accumulation (relative error of a stencil product
-                     <= 3 * 2^-18); used when every tap row spans at most 8
-                     nodes either side (2a/h_1 < 9), else the FP32 stencil */
+  MLS6_MIXED = 2  /* as MLS6_FP32, but where the levels are evaluated node by
+                     node (mls6_plan_options: not where the transforms apply)
+                     their stencils may run on the tensor cores with BF16
+                     hi+lo split operands and FP32 accumulation (relative
+                     error of a stencil product <= 3 * 2^-18); used when every
+                     tap row spans at most 8 nodes either side (2a/h_1 < 9),
+                     else the FP32 stencil */
 } mls6_precision;
 
 /* Finest-grid size for a box (per axis the multiple of 2^(levels-1) nearest
@@ -324,6 +326,12 @@ int mls6_set_tuning(mls6_plan_t* p, int pair_split, int stencil_groups);
  * with the accumulators in tensor memory (MLS6_MIXED, 2a/h_1 < 9, see
  * mls6_plan_options), -1 none (l = 1). */
 int mls6_stencil_kind(const mls6_plan_t* p);
+
+/* How the plan evaluates its grid part: 0 by the direct kernels, 1 by
+ * transforms unless an evaluation's atoms have a thin phase (see
+ * mls6_plan_options).  last (may be NULL): what the last evaluation ran, 0 or 1
+ * (waits for the plan's stream). */
+int mls6_grid_form(const mls6_plan_t* p, int* last);
 int mls6_get_tuning(const mls6_plan_t* p, int* pair_split, int* stencil_groups);
 
 /* ---------------------------------------------------------------------

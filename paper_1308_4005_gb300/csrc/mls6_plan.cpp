@@ -508,6 +508,20 @@ int mls6_stencil_kind(const mls6_plan_t* plan) {
   return p->stencil_mma ? 3 : p->stencil_tc ? 2 : (p->stencil_global ? 1 : 0);
 }
 
+int mls6_grid_form(const mls6_plan_t* plan, int* last) {
+  if (!plan) return MLS6_ERR_ARG;
+  const Plan* p = reinterpret_cast<const Plan*>(plan);
+  if (last) {
+    int thin = 0;
+    if (p->spectral && (cudaStreamSynchronize(p->stream) != cudaSuccess ||
+                        cudaMemcpy(&thin, p->d_flag + kThin, sizeof(int),
+                                   cudaMemcpyDeviceToHost) != cudaSuccess))
+      return MLS6_ERR_CUDA;
+    *last = p->spectral && !thin ? 1 : 0;
+  }
+  return p->spectral ? 1 : 0;
+}
+
 int mls6_get_tuning(const mls6_plan_t* plan, int* split, int* groups) {
   if (!plan) return MLS6_ERR_ARG;
   const Plan* p = reinterpret_cast<const Plan*>(plan);

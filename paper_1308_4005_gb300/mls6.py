@@ -37,7 +37,8 @@ EXPORTS = ("mls6_grid_dims", "mls6_coarse_tables", "mls6_plan", "mls6_plan_ex",
            "mls6_set_graph", "mls6_eval",
            "mls6_eval_atoms", "mls6_eval_lb", "mls6_last_error", "mls6_plan_info", "mls6_debug_grid",
            "mls6_profile", "mls6_stage_times", "mls6_stage_name", "mls6_auto_levels",
-           "mls6_set_tuning", "mls6_get_tuning", "mls6_stencil_kind", "mls6_cost_model", "mls6_lpt_assign",
+           "mls6_set_tuning", "mls6_get_tuning", "mls6_stencil_kind", "mls6_grid_form",
+           "mls6_cost_model", "mls6_lpt_assign",
            "mls6_batch_plan", "mls6_batch_set_stream", "mls6_batch_eval", "mls6_batch_tune",
            "mls6_batch_set_config", "mls6_batch_info", "mls6_batch_size", "mls6_batch_replica",
            "mls6_batch_destroy", "mls6_batch_set_mode", "mls6_batch_mode", "mls6_batch_set_wait",
@@ -115,6 +116,8 @@ def load(path: str = LIB_PATH):
     L.mls6_set_tuning.restype = C.c_int
     L.mls6_stencil_kind.argtypes = [C.c_void_p]
     L.mls6_stencil_kind.restype = C.c_int
+    L.mls6_grid_form.argtypes = [C.c_void_p, _ip]
+    L.mls6_grid_form.restype = C.c_int
     L.mls6_get_tuning.argtypes = [C.c_void_p, _ip, _ip]
     L.mls6_get_tuning.restype = C.c_int
     L.mls6_cost_model.argtypes = [_dp, C.c_int64, C.c_double, C.c_double, C.c_int, _dp, _dp]
@@ -286,7 +289,8 @@ def mls6_plan_info(plan):
     _check(L.mls6_plan_info(C.c_void_p(plan), ng, h, None, None), "mls6_plan_info")
     dims = [tuple(ng[3 * k: 3 * k + 3]) for k in range(lev.value)]
     return dict(levels=lev.value, n_grid=dims, h=tuple(h), ntaps=nt.value,
-                stencil_kind=L.mls6_stencil_kind(C.c_void_p(plan)))
+                stencil_kind=L.mls6_stencil_kind(C.c_void_p(plan)),
+                transforms=L.mls6_grid_form(C.c_void_p(plan), None) == 1)
 
 
 def mls6_debug_grid(plan, level, which):
@@ -339,6 +343,15 @@ def mls6_set_tuning(plan, pair_split=0, stencil_groups=0):
 
 def mls6_stencil_kind(plan):
     return load().mls6_stencil_kind(C.c_void_p(plan))
+
+
+def mls6_grid_form(plan):
+    """(transforms apply to the plan, the last evaluation ran them)."""
+    last = C.c_int()
+    rc = load().mls6_grid_form(C.c_void_p(plan), C.byref(last))
+    if rc < 0:
+        _check(rc, "mls6_grid_form")
+    return bool(rc), bool(last.value)
 
 
 def mls6_get_tuning(plan):

@@ -227,3 +227,23 @@ def test_thin_phase_lorentz_berthelot(gpu_lib, groups):
             out.append((F.cpu().numpy(), float(E[0])))
     for F, E in out[1:]:
         assert np.array_equal(F, out[0][0]) and E == out[0][1]
+
+
+@pytest.mark.gpu
+def test_grid_form_query(gpu_lib):
+    """Which form the plan has and which the last evaluation ran."""
+    import torch
+
+    box, x, _, nd = _droplet()
+    y = x.copy()  # the vapour's atoms moved into the droplet
+    y[nd:] = np.array(box) / 2 + np.random.default_rng(36).uniform(-4.0, 4.0, (len(x) - nd, 3))
+    for prec in ("fp32", "fp64", "mixed"):
+        plan = gpu_lib.Plan(box, len(x), A, 1.0, 3, precision=prec)
+        for at, last in ((x, False), (y, True), (x, False)):
+            plan.evaluate(torch.tensor(np.c_[at, np.ones(len(x))], device="cuda",
+                                       dtype=torch.float64 if prec == "fp64" else torch.float32))
+            assert gpu_lib.mls6_grid_form(plan.handle) == (True, last)
+        assert plan.info()["transforms"]
+    for kw in (dict(levels=3, precision="mixed", stencil="cuda"), dict(levels=1)):
+        plan = gpu_lib.Plan((16.0, 16.0, 16.0), 10, A, 1.0, **kw)
+        assert gpu_lib.mls6_grid_form(plan.handle) == (False, False)
