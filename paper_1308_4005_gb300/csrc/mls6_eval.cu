@@ -114,8 +114,6 @@ template <typename T> static int upload_tables_t(Plan* p) {
     stencil_mma_geometry(p);
     p->stencil_mma = true;
     p->stencil_global = false;
-    rc = prepare_stencil_mma(p);
-    if (rc) return rc;
   } else if (p->stencil_req == 2 && stencil_tc_eligible(p)) {  // mma.sync stencil tiles
     tc_geometry(p);
     p->stencil_tc = true;
@@ -124,10 +122,8 @@ template <typename T> static int upload_tables_t(Plan* p) {
     if (rc) return rc;
   }
   p->spectral = spectral_eligible(p);
-  if (p->spectral) {
-    rc = prepare_spectral<T>(p);
-    if (rc) return rc;
-  }
+  rc = p->spectral ? prepare_spectral<T>(p) : p->stencil_mma ? prepare_stencil_mma(p) : 0;
+  if (rc) return rc;
   if (l >= 2) {
     rc |= A((void**)&p->d_rows, sizeof(int) * 4 * p->nrows);
     rc |= A(&p->d_wv, sizeof(Vec4<T>) * p->ntaps);
@@ -558,6 +554,8 @@ template <typename T> static int debug_grid_t(Plan* p, int level, int which, dou
   if (p->spectral && !have) {
     cudaStream_t st = p->cs ? p->cs : p->stream;
     if (cudaStreamSynchronize(p->stream) != cudaSuccess) return MLS6_ERR_CUDA;
+    if (p->stencil_mma && !p->d_mma_rows)
+      if (const int rc = prepare_stencil_mma(p)) return rc;
     launch_from_fixed<T>(p, st, p->lb_last ? 6 : -1,
                          p->lb_last ? (const T*)p->d_lbq + (size_t)6 * p->lv[1].np : nullptr);
     for (int k = 1; k < p->levels; ++k) launch_restrict<T>(p, k, st);

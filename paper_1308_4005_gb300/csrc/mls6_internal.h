@@ -180,7 +180,8 @@ struct Plan {
   bool lb_last = false;        // the last evaluation was a Lorentz-Berthelot one
   unsigned long long spec_rad[3] = {};  // radices per axis (x: of n/2)
   void* d_spec_tw = nullptr;   // exp(-2 pi i j / n) per axis
-  void* d_spec_tab = nullptr;  // restriction factors per axis | level-1 factors, 7 octants
+  void* d_spec_tab = nullptr;  // level-1 factors, 8 values per frequency of an octant |
+                               // restriction factors per axis
   double* d_spec_top = nullptr;// coarsest-level factors, 7 grids
   void* d_spec_s = nullptr;    // transforms of q^1 and of e^{1,tot}
   // the direct grid part in one launch, for thin phases (mls6_direct.cu): the

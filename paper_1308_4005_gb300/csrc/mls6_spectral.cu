@@ -568,12 +568,11 @@ bool spectral_eligible(const Plan* p) {
 // (dy, dz) with dx contiguous (Plan::h_rows, h_wv).  Seven factors per
 // frequency of one octant: g_1, then g_1'/r r_a r_b for xx yy zz xy xz yz (an
 // off-diagonal tap is odd along two axes: -sin sin).
-static void spec_level_tables(const Plan* p, std::vector<double>& K) {
+// Records of 8 (one or two 32-byte sectors) per frequency, x fastest.
+template <typename T> static void spec_level_tables(const Plan* p, T* tab) {
   const int* n = p->lv[1].n;
   const double* h = p->lv[1].h;
   const int o0 = n[0] / 2 + 1, o1 = n[1] / 2 + 1, o2 = n[2] / 2 + 1;
-  const size_t noct = (size_t)o0 * o1 * o2;
-  K.assign(7 * noct, 0.0);
   std::vector<double> cs[3], sn[3];
   for (int d = 0; d < 3; ++d) {
     cs[d].resize(n[d]);
@@ -590,12 +589,14 @@ static void spec_level_tables(const Plan* p, std::vector<double>& K) {
   for (int r = 0; r < p->nrows; ++r)
     if (p->h_rows[4 * r] >= 0 && p->h_rows[4 * r + 1] >= 0)
       by_z[p->h_rows[4 * r + 1]].push_back(r);
+  // per dz the sums over dx and dy: seven planes each
   const size_t pl = (size_t)o0 * o1;
-  std::vector<double> A(4 * (size_t)o0), Pz(7 * pl);
-  for (int dz = 0; dz <= P; ++dz) {
-    if (by_z[dz].empty()) continue;
-    std::fill(Pz.begin(), Pz.end(), 0.0);
-    for (int r : by_z[dz]) {
+  std::vector<int> zs;
+  for (int dz = 0; dz <= P; ++dz)
+    if (!by_z[dz].empty()) zs.push_back(dz);
+  std::vector<double> A(4 * (size_t)o0), Pz(7 * pl * zs.size(), 0.0);
+  for (size_t iz = 0; iz < zs.size(); ++iz)
+    for (int r : by_z[zs[iz]]) {
       const int dy = p->h_rows[4 * r], R = p->h_rows[4 * r + 2];
       const double* wv = &p->h_wv[4 * (size_t)p->h_rows[4 * r + 3]];
       std::fill(A.begin(), A.end(), 0.0);
@@ -612,7 +613,7 @@ static void spec_level_tables(const Plan* p, std::vector<double>& K) {
       for (int k1 = 0; k1 < o1; ++k1) {
         const int i = at(1, k1, dy);
         const double c = (dy ? 2.0 : 1.0) * cs[1][i], s = dy * 2.0 * sn[1][i];
-        double* q = &Pz[(size_t)k1 * o0];
+        double* q = &Pz[7 * pl * iz + (size_t)k1 * o0];
         for (int k = 0; k < o0; ++k) {
           const double g = A[k], G = A[o0 + k], G2 = A[2 * o0 + k], G1 = A[3 * o0 + k];
           q[k] += g * c;
@@ -625,18 +626,26 @@ static void spec_level_tables(const Plan* p, std::vector<double>& K) {
         }
       }
     }
-    for (int k2 = 0; k2 < o2; ++k2) {
-      const int i = at(2, k2, dz);
-      const double c = (dz ? 2.0 : 1.0) * cs[2][i], s = dz * 2.0 * sn[2][i];
-      const double f[7] = {c, c * h[0] * h[0], c * h[1] * h[1], c * dz * dz * h[2] * h[2],
-                           -c * h[0] * h[1], -s * h[0] * h[2], -s * h[1] * h[2]};
-      for (int ch = 0; ch < 7; ++ch) {
-        double* q = &K[ch * noct + (size_t)k2 * pl];
-        const double* a = &Pz[ch * pl];
-        for (size_t k = 0; k < pl; ++k) q[k] += f[ch] * a[k];
+  // sums over dz, one row of frequencies at a time
+  std::vector<double> row((size_t)7 * o0);
+  for (int k2 = 0; k2 < o2; ++k2)
+    for (int k1 = 0; k1 < o1; ++k1) {
+      std::fill(row.begin(), row.end(), 0.0);
+      for (size_t iz = 0; iz < zs.size(); ++iz) {
+        const int dz = zs[iz], i = at(2, k2, dz);
+        const double c = (dz ? 2.0 : 1.0) * cs[2][i], s = dz * 2.0 * sn[2][i];
+        const double f[7] = {c, c * h[0] * h[0], c * h[1] * h[1], c * dz * dz * h[2] * h[2],
+                             -c * h[0] * h[1], -s * h[0] * h[2], -s * h[1] * h[2]};
+        for (int ch = 0; ch < 7; ++ch) {
+          const double* a = &Pz[pl * (7 * iz + ch) + (size_t)k1 * o0];
+          double* q = &row[(size_t)ch * o0];
+          for (int k = 0; k < o0; ++k) q[k] += f[ch] * a[k];
+        }
       }
+      T* out = tab + 8 * ((size_t)k2 * pl + (size_t)k1 * o0);
+      for (int k = 0; k < o0; ++k)
+        for (int ch = 0; ch < 7; ++ch) out[8 * (size_t)k + ch] = (T)row[(size_t)ch * o0 + k];
     }
-  }
 }
 
 // The same for the coarsest level's periodic tables (whole grid).
@@ -649,6 +658,12 @@ static void spec_top_tables(const Plan* p, std::vector<double>& Kt) {
   static const bool odd[7][3] = {{false, false, false}, {false, false, false}, {false, false, false},
                                  {false, false, false}, {true, true, false},   {true, false, true},
                                  {false, true, true}};
+  std::vector<double> wave[2][3];  // cosines, sines of 2 pi j / n
+  for (int d = 0; d < 3; ++d)
+    for (int j = 0; j < n[d]; ++j) {
+      wave[0][d].push_back(std::cos(2.0 * M_PI * j / n[d]));
+      wave[1][d].push_back(std::sin(2.0 * M_PI * j / n[d]));
+    }
   for (int ch = 0; ch < 7; ++ch) {
     for (long i = 0; i < L.np; ++i)
       a[i] = ch ? p->h_top_V[(size_t)(ch - 1) * L.np + i] : p->h_top_T[i];
@@ -657,11 +672,9 @@ static void spec_top_tables(const Plan* p, std::vector<double>& Kt) {
       for (long i = 0; i < L.np; ++i) {
         const int k = (int)(i / st % n[d]);
         const long base = i - k * st;
+        const std::vector<double>& w = wave[odd[ch][d]][d];
         double s = 0.0;
-        for (int m = 0; m < n[d]; ++m) {
-          const double t = 2.0 * M_PI * ((long)k * m % n[d]) / n[d];
-          s += a[base + m * st] * (odd[ch][d] ? std::sin(t) : std::cos(t));
-        }
+        for (int m = 0; m < n[d]; ++m) s += a[base + m * st] * w[(long)k * m % n[d]];
         b[i] = s;
       }
       a.swap(b);
@@ -693,13 +706,12 @@ template <typename T> int prepare_spectral(Plan* p) {
   for (int d = 0; d < 3; ++d)
     for (int j = 0; j < n[d]; ++j)
       tw.push_back(Cx<T>{(T)std::cos(2.0 * M_PI * j / n[d]), (T)-std::sin(2.0 * M_PI * j / n[d])});
-  std::vector<double> K, Kt;
-  spec_level_tables(p, K);
+  std::vector<double> Kt;
   spec_top_tables(p, Kt);
-  const size_t noct = K.size() / 7;
-  tab.resize(8 * noct, T(0));  // records of 8 (one or two 32-byte sectors) per frequency
-  for (size_t i = 0; i < noct; ++i)
-    for (int c = 0; c < 7; ++c) tab[8 * i + c] = (T)K[c * noct + i];
+  const size_t noct = (size_t)(n[0] / 2 + 1) * (n[1] / 2 + 1) * (n[2] / 2 + 1);
+  tab.reserve(8 * noct + ntw);
+  tab.resize(8 * noct, T(0));
+  spec_level_tables<T>(p, tab.data());
   // Phi at half-integer offsets 1/2, 3/2 (5/2)
   static const double w3[3] = {0.5625, -0.0625, 0.0};
   static const double w5[3] = {150.0 / 256.0, -25.0 / 256.0, 3.0 / 256.0};

@@ -514,7 +514,8 @@ template <bool VIR> static std::vector<uint8_t> weight_matrices(const Plan* p, i
   return out;
 }
 
-// Upload the weight matrices and the padded row table (plan creation).
+// Upload the weight matrices and the padded row table: at plan creation, or at
+// the first mls6_debug_grid of a plan that evaluates by transforms.
 int prepare_stencil_mma(Plan* p) {
   const int RBv = mma_rows_per_chunk<true>(), RBe = mma_rows_per_chunk<false>();
   p->mma_rows_pad_v = (int)cdiv(p->nrows, RBv) * RBv;
@@ -525,15 +526,24 @@ int prepare_stencil_mma(Plan* p) {
     for (int j = 0; j < 4; ++j) rows[4 * r + j] = p->h_rows[4 * r + j];
   std::vector<uint8_t> bv = weight_matrices<true>(p, p->mma_rows_pad_v);
   std::vector<uint8_t> be = weight_matrices<false>(p, p->mma_rows_pad_e);
+  auto undo = [&](int rc) {  // all three, or none
+    cudaFree(p->d_mma_rows);
+    cudaFree(p->d_mma_bv);
+    cudaFree(p->d_mma_be);
+    p->d_mma_rows = nullptr;
+    p->d_mma_bv = p->d_mma_be = nullptr;
+    cudaGetLastError();
+    return rc;
+  };
   if (cudaMalloc((void**)&p->d_mma_rows, sizeof(int) * rows.size()) != cudaSuccess ||
       cudaMalloc((void**)&p->d_mma_bv, bv.size()) != cudaSuccess ||
       cudaMalloc((void**)&p->d_mma_be, be.size()) != cudaSuccess)
-    return MLS6_ERR_NOMEM;
+    return undo(MLS6_ERR_NOMEM);
   if (cudaMemcpy(p->d_mma_rows, rows.data(), sizeof(int) * rows.size(),
                  cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(p->d_mma_bv, bv.data(), bv.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
       cudaMemcpy(p->d_mma_be, be.data(), be.size(), cudaMemcpyHostToDevice) != cudaSuccess)
-    return MLS6_ERR_CUDA;
+    return undo(MLS6_ERR_CUDA);
   const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
   if (cudaFuncSetAttribute(k_stencil_mma<true>, attr, (int)mma_smem<true>(p->P)) != cudaSuccess ||
       cudaFuncSetAttribute(k_stencil_mma<false>, attr, (int)mma_smem<false>(p->P)) != cudaSuccess)
