@@ -354,7 +354,9 @@ typedef struct mls6_batch_t mls6_batch_t;
  *   coef[0] (a^3 N/V) N + coef[1] (a/h)^3 (V/h^3) 8/7 + coef[2] N
  *   + coef[3] N_l^2 + coef[4] (8 + 2(l-1)).
  * coef: 5 doubles or NULL for the built-in values (from GB300 stage
- * timings).  Host only. */
+ * timings of the direct kernels).  Batches price a replica that evaluates by
+ * transforms by another formula: the same local and per-atom terms, one per
+ * node of the finest grid and a latency of 13 launches.  Host only. */
 int mls6_cost_model(const double box[3], int64_t N, double a, double h, int levels,
                     const double* coef, double* cost);
 

@@ -11,8 +11,9 @@
 // captures all their kernel sequences into a single graph whose replicas are
 // spread over K independent chains ("branches"), so that kernels of small
 // replicas, which cannot fill the GPU alone, run side by side.  Replicas are
-// assigned to branches by longest-processing-time-first on a cost model
-// (Sec. IV, Eq. cost: C_local (a/d)^3 N + C_grids (a/h)^3 V/h^3, plus the
+// assigned to branches by longest-processing-time-first on a cost model (by
+// transforms: transform_cost; by the direct kernels:
+// Sec. IV, Eq. cost: C_local (a/d)^3 N + C_grids (a/h)^3 V/h^3, plus the
 // per-atom transfers, the coarsest product and a per-launch latency that
 // dominate small replicas), and the autotuner picks the branch count and the
 // per-replica kernel shapes (pair-kernel lanes per atom, stencil thread
@@ -68,8 +69,8 @@ struct Batch {
 };
 
 // Cost model coefficients (seconds), from stage timings of a 65,536-atom
-// slab (a = 3, h = 1.25) on GB300: per neighbour-pair volume term, per
-// tap x node, per atom (binning, anterpolation, interpolation, transfers),
+// slab (a = 3, h = 1.25) on GB300 by the direct kernels: per neighbour-pair
+// volume term, per tap x node, per atom (binning, anterpolation, interpolation, transfers),
 // per coarsest-node pair, per kernel launch.
 static const double kCostDefault[5] = {1.6e-10, 4.0e-11, 1.7e-9, 3.4e-10, 2.5e-6};
 
@@ -84,6 +85,17 @@ static double model_cost(const double box[3], int64_t N, double a, double h, int
   top = nl * nl;
   const int launches = 8 + 2 * (levels - 1);
   return k[0] * local + k[1] * grids + k[2] * (double)N + k[3] * top + k[4] * launches;
+}
+
+// The same of a replica that evaluates by transforms: no taps and no coarsest
+// product, a term per node of the finest grid and 13 launches.  From stage
+// timings of the 1,048,576-atom cube (pair 524, transforms 86, per atom 187 us)
+// and of small systems (37 us where nothing but latency counts); 65,536-atom
+// slab 66 us here, 88 measured.
+static double transform_cost(const Plan* p) {
+  const double V = p->L[0] * p->L[1] * p->L[2], N = (double)p->N;
+  return 2.2e-11 * N * (p->a * p->a * p->a * N / V) + 1.8e-10 * N + 6e-11 * (double)p->lv[1].np +
+         13 * 2.8e-6;
 }
 
 // Longest processing time first: replicas in decreasing cost, each to the
@@ -406,7 +418,9 @@ int mls6_batch_plan(mls6_batch_t** out, int B, const double* boxes, const int64_
     rc = plan_streams(b->plans[r]);
     b->off[r + 1] = b->off[r] + N[r];
     double hh = b->plans[r]->lv[1].h[0];
-    b->cost[r] = model_cost(boxes + 3 * r, N[r], a, hh, b->plans[r]->levels, nullptr);
+    b->cost[r] = b->plans[r]->spectral
+                     ? transform_cost(b->plans[r])
+                     : model_cost(boxes + 3 * r, N[r], a, hh, b->plans[r]->levels, nullptr);
   }
   if (rc == MLS6_OK) {
     auto fail = [&](cudaError_t e) {
