@@ -171,7 +171,11 @@ int mls6_plan_ex(mls6_plan_t** out, const double box[3], int64_t N, double a, do
  * default stream).  Internally an evaluation runs on two streams owned by
  * the plan (the pair sum in parallel with the grid chain); they wait for
  * the caller's stream at the start and the caller's stream waits for them
- * at the end, so ordering is as if all work ran on the caller's stream. */
+ * at the end, so ordering is as if all work ran on the caller's stream.
+ * The pair sum's stream has the default priority, the grid chain's the next
+ * higher one: kernels that the caller runs meanwhile on streams of default
+ * priority are placed behind the grid chain's, those on streams of higher
+ * priority before them. */
 int mls6_set_stream(mls6_plan_t* p, void* stream);
 
 /* Graph execution (default on): the first evaluation with a given set of
@@ -526,7 +530,7 @@ int mls6_mlp_train_step(mls6_mlp_t* m, const void* X, const float* T, int64_t N,
 
 /* Correct the forces of the plan's last evaluation in place (device, N x 3
  * of the plan precision, input order): features, network, then
- * F_i += c_i * s * y_i.  Three kernels on the plan's stream. */
+ * F_i += c_i * s * y_i.  Two kernels on the plan's stream. */
 int mls6_mlp_apply(mls6_plan_t* p, mls6_mlp_t* m, void* forces);
 
 void mls6_mlp_destroy(mls6_mlp_t* m);

@@ -302,10 +302,11 @@ static int ensure_streams(Plan* p) {
   // the chain's small and latency-bound kernels run in between (65,536-atom
   // slab 108 -> 98 us, 1M-atom cube 778 -> 768).  Graphs of single plans keep
   // the priorities; a batch's graph does not (its chains fill each other's
-  // gaps: 40 replicas 845 us without, 887 with them).
+  // gaps: 40 replicas 845 us without, 887 with them).  One step above the
+  // default, so that a caller's streams of higher priority still go first.
   int lowest = 0, highest = 0;
   CK(cudaDeviceGetStreamPriorityRange(&lowest, &highest));
-  CK(cudaStreamCreateWithPriority(&p->cs, cudaStreamNonBlocking, highest));
+  CK(cudaStreamCreateWithPriority(&p->cs, cudaStreamNonBlocking, std::max(highest, lowest - 1)));
   CK(cudaStreamCreateWithPriority(&p->cs2, cudaStreamNonBlocking, lowest));
   CK(cudaEventCreateWithFlags(&p->ev_in, cudaEventDisableTiming));
   CK(cudaEventCreateWithFlags(&p->ev_out, cudaEventDisableTiming));
