@@ -20,9 +20,8 @@ template <typename T> struct PairArgs {
   T margin;  // absolute slack of the row trimming (covers rounding of x, x/w)
   T Lhi[3], Llo[3];  // box length as an unevaluated sum hi + lo (exact image shifts)
   // queue form, FP32 set-up and test: box, (a + slack)^2, cells, slack of the
-  // row trimming; half the box (virial)
+  // row trimming
   float Lf[3], a2f, wf[3], iwf, marginf;
-  T mL[3], near2;  // and (a/16)^2
   // smoothing function of continuity other than C^2 (GEN kernels):
   // gamma = sum gc[k] u^k, u = rho^12; gamma'(rho)/rho = -12 rho^10 ... as
   // g_0'/r = -6 r^-8 + a^-8 rho^10 sum gd[k] u^k with gd[k] = -12 (k+1) gc[k+1]
@@ -690,17 +689,15 @@ __device__ __forceinline__ bool q_inside(double r2, double a2) {
 // (x_i - Lhi for m = +1, x_j - Lhi for m = -1), where the subtraction is
 // exact: an image pair carries no rounding of the box length or of the
 // absolute coordinates.
-// Virial: d = x_j - x_i + m L, and a pair is met from both atoms with opposite
-// d and m, so the sum of c_i f (x) d over all pairs (f = C (...) d) is -2
-// sum_i c_i F_i (x) x_i, formed once per atom, plus c_i f (x) m L for pairs of
-// other images (symmetrised; usually one axis).  The product with x_i loses
-// |x_i| / r of a pair's precision, so pairs closer than a/16 (none in a
-// liquid) stay out of it: they have sums of their own, f and d (x) d.
+// Virial: c_i C (...) d (x) d of the pairs met from their first atom (sorted
+// order; an atom's own images: from the first of the two).  A pair is met from
+// both atoms, and the stream holds the earlier atoms of the rows first, so that
+// about half of the rounds of 32 have none to add.
 template <typename T, bool VIR, bool LB>
 __device__ __forceinline__ void pair_eval(int2 en, const Vec4<T>* __restrict__ sp,
                                           const T* __restrict__ lbw, const Vec4<T>& pi, T wi,
-                                          const PairArgs<T>& g, T& e, T& fx, T& fy, T& fz,
-                                          T (&w)[6], T (&near)[3], bool& any_near) {
+                                          const PairArgs<T>& g, int i, T& e, T& fx, T& fy, T& fz,
+                                          T (&w)[6]) {
   constexpr int kImg0 = 8 | (8 << 4) | (8 << 8);
   const Vec4<T> pj = sp[en.x];
   T ddx = pj.x - pi.x, ddy = pj.y - pi.y, ddz = pj.z - pi.z;
@@ -733,44 +730,17 @@ __device__ __forceinline__ void pair_eval(int2 en, const Vec4<T>* __restrict__ s
   }
   e += cj * g0;
   const T cg = cj * gp;
-  if (VIR && q_inside(r2, g.near2)) {
-    const T hx = cg * ddx, hy = cg * ddy, hz = cg * ddz;
-    any_near = true;
-    near[0] += hx;
-    near[1] += hy;
-    near[2] += hz;
-    w[0] += pi.w * hx * ddx;
-    w[1] += pi.w * hy * ddy;
-    w[2] += pi.w * hz * ddz;
-    w[3] += pi.w * hx * ddy;
-    w[4] += pi.w * hx * ddz;
-    w[5] += pi.w * hy * ddz;
-    return;
-  }
   fx += cg * ddx;
   fy += cg * ddy;
   fz += cg * ddz;
-  if (VIR && en.y != kImg0) {
-    const int mx = (en.y & 15) - 8, my = ((en.y >> 4) & 15) - 8, mz = ((en.y >> 8) & 15) - 8;
-    const T cv = pi.w * cg, hx = cv * ddx, hy = cv * ddy, hz = cv * ddz;
-    if (mx != 0) {  // g.mL: L / 2 (the off-diagonal halves)
-      const T u = (T)mx * g.mL[0];
-      w[0] += T(2) * u * hx;
-      w[3] += u * hy;
-      w[4] += u * hz;
-    }
-    if (my != 0) {
-      const T u = (T)my * g.mL[1];
-      w[3] += u * hx;
-      w[1] += T(2) * u * hy;
-      w[5] += u * hz;
-    }
-    if (mz != 0) {
-      const T u = (T)mz * g.mL[2];
-      w[4] += u * hx;
-      w[5] += u * hy;
-      w[2] += T(2) * u * hz;
-    }
+  if (VIR && (en.x > i || (en.x == i && en.y > kImg0))) {
+    const T cv = pi.w * cg, hx = cv * ddx, hy = cv * ddy;
+    w[0] += hx * ddx;
+    w[1] += hy * ddy;
+    w[2] += cv * ddz * ddz;
+    w[3] += hx * ddy;
+    w[4] += hx * ddz;
+    w[5] += hy * ddz;
   }
 }
 
@@ -824,8 +794,10 @@ __device__ __forceinline__ void q_stage(int c0, int cn, int lane, const int* t_e
 // operations each.  98,765 atoms, a = 3, pair stage with / without the virial:
 // 2390 us (with) with FP64 tests, an FP64 row set-up, the division and six
 // virial products per pair; FP32 tests and the Newton reciprocal 1143 / 844;
-// FP32 set-up 1040 / 731; the virial from the force once per atom 901 / 737 (the
-// FP64 pipe 83% busy; 3.9 rounds of 32 per atom where 3.0 would hold its hits).  The queue is filled and
+// FP32 set-up 1040 / 731; the virial of a pair from one of its atoms 890 / 737
+// (from the force times the position, once per atom, 901, but without |x| / r of
+// a pair's precision).  The FP64 pipe is 83% busy; 3.9 rounds of 32 per atom
+// where 3.0 would hold its hits.  The queue is filled and
 // drained in stream order and each lane sums its evaluations in that order,
 // then a fixed shuffle tree that halves the four sums as it goes (6 additions,
 // not 20) combines the lanes: results are reproducible bit for bit.
@@ -848,7 +820,7 @@ __global__ void __launch_bounds__(kQWarps * 32) k_pair_q(const Vec4<T>* __restri
   constexpr int kQ = 64;       // queued hits: < 32 left over + 32 new
   constexpr int kCap = kQCap;
   constexpr unsigned kAll = 0xffffffffu;
-  __shared__ T wsum[kW][6], wrow[kW][9];  // virial of each warp; rows of -c_i F_i (x) x_i
+  __shared__ T wsum[kW][6];               // virial of each warp
   __shared__ int ended;                   // warps that have written theirs
   __shared__ int t_end[kW][kP], t_base[kW][kP], t_img[kW][kP];
   __shared__ int2 qu[kW][kQ];
@@ -875,9 +847,7 @@ __global__ void __launch_bounds__(kQWarps * 32) k_pair_q(const Vec4<T>* __restri
     cz = min(max((int)(pa.z * g.inv_w[2]), 0), g.nc[2] - 1);
     rid = cy + g.nc[1] * cz;
   }
-  T w[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};  // pairs of other images, close pairs
-  T rx = 0, ry = 0, rz = 0;  // lane 1 + q: sum c_i F_i,q x_i
-  bool images = false;  // any of those
+  T w[6] = {T(0), T(0), T(0), T(0), T(0), T(0)};
   const int ny = 2 * g.R[1] + 1, nrows = (2 * g.R[2] + 1) * ny;
   for (int s = 0; s < nat;) {
     const int rs = __shfl_sync(kAll, rid, s);
@@ -932,12 +902,6 @@ __global__ void __launch_bounds__(kQWarps * 32) k_pair_q(const Vec4<T>* __restri
         }
       }
     }
-    if (VIR) {  // any piece of another image
-      bool im = false;
-#pragma unroll
-      for (int q = 0; q < 3; ++q) im = im || (q < np && pim[q] != (8 | (8 << 4) | (8 << 8)));
-      images = images || __any_sync(kAll, im);
-    }
     // 2. pieces -> one stream
     int np_inc = np, c_inc = cnt;
 #pragma unroll
@@ -978,8 +942,7 @@ __global__ void __launch_bounds__(kQWarps * 32) k_pair_q(const Vec4<T>* __restri
                                     __shfl_sync(kAll, pf.z, s), 0.f);
       T wi = T(0);
       if (LB) wi = lbw[i];
-      T e = 0, fx = 0, fy = 0, fz = 0, near[3] = {T(0), T(0), T(0)};
-      bool any_near = false;
+      T e = 0, fx = 0, fy = 0, fz = 0;
       int qn = 0;
       for (int c0 = 0; c0 < total; c0 += kCap) {
         const int cn = min(kCap, total - c0);
@@ -1001,8 +964,7 @@ __global__ void __launch_bounds__(kQWarps * 32) k_pair_q(const Vec4<T>* __restri
           qn += __popc(m);
           if (qn >= 32) {
             __syncwarp();
-            pair_eval<T, VIR, LB>(qu[wid][lane], sp, lbw, pi, wi, g, e, fx, fy, fz, w, near,
-                                  any_near);
+            pair_eval<T, VIR, LB>(qu[wid][lane], sp, lbw, pi, wi, g, i, e, fx, fy, fz, w);
             __syncwarp();
             if (lane < qn - 32) qu[wid][lane] = qu[wid][lane + 32];
             __syncwarp();
@@ -1012,8 +974,7 @@ __global__ void __launch_bounds__(kQWarps * 32) k_pair_q(const Vec4<T>* __restri
       }
       __syncwarp();
       if (lane < qn)
-        pair_eval<T, VIR, LB>(qu[wid][lane], sp, lbw, pi, wi, g, e, fx, fy, fz, w, near,
-                                  any_near);
+        pair_eval<T, VIR, LB>(qu[wid][lane], sp, lbw, pi, wi, g, i, e, fx, fy, fz, w);
       // lane bits 0 and 1 choose the sum (e, x, y, z), the others are added up
       const bool b0 = lane & 1, b1 = lane & 2;
       T ka = b1 ? fy : e, kb = b1 ? fz : fx;
@@ -1022,62 +983,31 @@ __global__ void __launch_bounds__(kQWarps * 32) k_pair_q(const Vec4<T>* __restri
       T v = (b0 ? kb : ka) + __shfl_xor_sync(kAll, b0 ? ka : kb, 1);
 #pragma unroll
       for (int o = 4; o < 32; o <<= 1) v += __shfl_xor_sync(kAll, v, o);
-      T vn = T(0);  // lanes 1 .. 3: the close pairs' force
-      if (VIR && __any_sync(kAll, any_near)) {
-        images = true;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-          for (int d = 0; d < 3; ++d) near[d] += __shfl_xor_sync(kAll, near[d], o);
-        vn = lane == 1 ? near[0] : lane == 2 ? near[1] : lane == 3 ? near[2] : T(0);
-      }
       // F_i = -c_i sum c_j g_0'/r d = +c_i 6 a^-8 (x, y, z)
-      if (lane < 4) {
-        if (lane == 0)
-          e0[i] = g.ia6 * v;
-        else
-          floc[3 * (size_t)i + lane - 1] = (LB ? T(6) : T(6) * pi.w) * g.ia8 * (v + vn);
-        if (VIR) {
-          const T f = pi.w * v;
-          rx += f * pi.x;
-          ry += f * pi.y;
-          rz += f * pi.z;
-        }
-      }
+      if (lane == 0)
+        e0[i] = g.ia6 * v;
+      else if (lane < 4)
+        floc[3 * (size_t)i + lane - 1] = (LB ? T(6) : T(6) * pi.w) * g.ia8 * v;
       __syncwarp();  // the queue is reused by the next atom
     }
     __syncwarp();  // the next segment rewrites the piece table and the stage
   }
   if (VIR) {
-    // of c_i c_j (-a^8 g_0'/6r) d (x) d: the image sums over the lanes (lane c
-    // mod 8 ends with sum c; most warps have none), then the rows
-    T v = T(0);
-    if (images) {
-      const bool b0 = lane & 1, b1 = lane & 2, b2 = lane & 4;
-      T k0 = b2 ? w[4] : w[0], k1 = b2 ? w[5] : w[1], k2 = b2 ? T(0) : w[2], k3 = b2 ? T(0) : w[3];
-      k0 += __shfl_xor_sync(kAll, b2 ? w[0] : w[4], 4);
-      k1 += __shfl_xor_sync(kAll, b2 ? w[1] : w[5], 4);
-      const T s2 = __shfl_xor_sync(kAll, w[2], 4), s3 = __shfl_xor_sync(kAll, w[3], 4);
-      k2 += b2 ? T(0) : s2;
-      k3 += b2 ? T(0) : s3;
-      const T m0 = (b1 ? k2 : k0) + __shfl_xor_sync(kAll, b1 ? k0 : k2, 2);
-      const T m1 = (b1 ? k3 : k1) + __shfl_xor_sync(kAll, b1 ? k1 : k3, 2);
-      v = (b0 ? m1 : m0) + __shfl_xor_sync(kAll, b0 ? m0 : m1, 1);
-      v += __shfl_xor_sync(kAll, v, 8);
-      v += __shfl_xor_sync(kAll, v, 16);
-    }
-    if (lane >= 1 && lane < 4) {
-      wrow[wid][3 * (lane - 1)] = rx;
-      wrow[wid][3 * (lane - 1) + 1] = ry;
-      wrow[wid][3 * (lane - 1) + 2] = rz;
-    }
-    __syncwarp();
-    if (lane < 6) {  // xx yy zz xy xz yz: rows p, q
-      const int p = lane < 3 ? lane : (lane == 5 ? 1 : 0);
-      const int q = lane < 3 ? lane : (lane == 3 ? 1 : 2);
-      v -= wrow[wid][3 * p + q] + wrow[wid][3 * q + p];
-      wsum[wid][lane] = v;
-    }
+    // sums of c_i c_j (-a^8 g_0'/6r) d (x) d over the lanes: lane c mod 8 ends with
+    // sum c
+    const bool b0 = lane & 1, b1 = lane & 2, b2 = lane & 4;
+    T k0 = b2 ? w[4] : w[0], k1 = b2 ? w[5] : w[1], k2 = b2 ? T(0) : w[2], k3 = b2 ? T(0) : w[3];
+    k0 += __shfl_xor_sync(kAll, b2 ? w[0] : w[4], 4);
+    k1 += __shfl_xor_sync(kAll, b2 ? w[1] : w[5], 4);
+    const T s2 = __shfl_xor_sync(kAll, w[2], 4), s3 = __shfl_xor_sync(kAll, w[3], 4);
+    k2 += b2 ? T(0) : s2;
+    k3 += b2 ? T(0) : s3;
+    const T m0 = (b1 ? k2 : k0) + __shfl_xor_sync(kAll, b1 ? k0 : k2, 2);
+    const T m1 = (b1 ? k3 : k1) + __shfl_xor_sync(kAll, b1 ? k1 : k3, 2);
+    T v = (b0 ? m1 : m0) + __shfl_xor_sync(kAll, b0 ? m0 : m1, 1);
+    v += __shfl_xor_sync(kAll, v, 8);
+    v += __shfl_xor_sync(kAll, v, 16);
+    if (lane < 6) wsum[wid][lane] = v;
     // the warp that ends last adds the warps' sums in their order
     __threadfence_block();
     __syncwarp();
@@ -1088,7 +1018,7 @@ __global__ void __launch_bounds__(kQWarps * 32) k_pair_q(const Vec4<T>* __restri
       double t = 0.0;
 #pragma unroll
       for (int u = 0; u < kW; ++u) t += (double)*(volatile T*)&wsum[u][lane];
-      wpart[6 * (size_t)blockIdx.x + lane] = -3.0 * (double)g.ia8 * t;
+      wpart[6 * (size_t)blockIdx.x + lane] = -6.0 * (double)g.ia8 * t;
     }
   }
 }
@@ -1284,10 +1214,8 @@ template <typename T> static PairArgs<T> pair_args(const Plan* p) {
   for (int d = 0; d < 3; ++d) {
     pg.Lf[d] = (float)p->L[d];
     pg.wf[d] = (float)p->cg.w[d];
-    pg.mL[d] = (T)(0.5 * p->L[d]);
   }
   pg.iwf = (float)p->cg.inv_w[0];
-  pg.near2 = (T)(p->a * p->a / 256.0);
   pg.marginf = (float)(1e-3 * wmin + 16.0 * 6.0e-8 * lmax);
   for (int k = 0; k < 5; ++k) pg.gc[k] = (T)p->sm.c[k];
   for (int k = 0; k < 4; ++k) pg.gd[k] = (T)(-12.0 * (k + 1) * p->sm.c[k + 1]);
