@@ -438,10 +438,10 @@ static int eval_t(Plan* p, const void* pos_, const void* c_, void* forces_, doub
 int plan_streams(Plan* p) { return ensure_streams(p); }
 
 // Lorentz-Berthelot mixing (Sec. II.D): the local part with the exact pair
-// coefficients, then the grid part once per channel m = 0..6 (anterpolation
-// of xi_m, restriction, level stencils, coarsest level, prolongation; the
-// level-1 total potential of each channel kept), and one interpolation that
-// pairs channel m with xi_{6-m}.  Launched eagerly on the plan's main stream.
+// coefficients on the second stream, the grid part of the channels m = 0..6 of
+// xi_m beside it (all seven in each launch of the transforms; channel by
+// channel where the plan has the direct kernels only), and one interpolation
+// that pairs channel m with xi_{6-m}.  Launched eagerly.
 template <typename T>
 static int eval_lb_t(Plan* p, const T* pos, const T* sigma, const T* eps, T* forces,
                      double* energy) {

@@ -222,15 +222,15 @@ static LbCoef lb_coefs() {
   return c;
 }
 
-template <typename T> int launch_anterp(Plan* p, cudaStream_t st, int lbm, bool to_grid, void* qfx) {
+template <typename T> int launch_anterp(Plan* p, cudaStream_t st, int lbm, bool to_grid) {
   const Level& L1 = p->lv[1];
   const int N = (int)p->N;
   const int nt = atom_block<T>(N);
   launch_pdl(p->order == 5 ? k_anterp<T, 6, 1> : k_anterp<T, 4, 1>, cdiv(N, nt), nt, 0, st,
       (const Vec4<T>*)p->d_sorted, N, L1.n[0], L1.n[1], L1.n[2], (T)(1.0 / L1.h[0]),
       (T)(1.0 / L1.h[1]), (T)(1.0 / L1.h[2]), p->d_flag, support_span(p),
-      (typename Fixed<T>::U*)(qfx ? qfx : p->d_q1fx), (const T*)p->d_lbw, lbm, lb_coefs());
-  return 1 + (to_grid ? launch_from_fixed<T>(p, st, lbm, qfx) : 0);
+      (typename Fixed<T>::U*)p->d_q1fx, (const T*)p->d_lbw, lbm, lb_coefs());
+  return 1 + (to_grid ? launch_from_fixed<T>(p, st, lbm) : 0);
 }
 
 // The fixed-point sums of all seven Lorentz-Berthelot channels, one after
@@ -1079,7 +1079,7 @@ template <typename T> int prepare_grid_kernels(Plan* p) {
 
 #ifndef MLS6_DEVICE_ONLY  // host code, left out where another unit includes this file
 #define MLS6_INSTANTIATE(T)                                               \
-  template int launch_anterp<T>(Plan*, cudaStream_t, int, bool, void*);   \
+  template int launch_anterp<T>(Plan*, cudaStream_t, int, bool);          \
   template int launch_anterp_lb<T>(Plan*, cudaStream_t, void*);           \
   template int launch_from_fixed<T>(Plan*, cudaStream_t, int, const void*); \
   template int launch_lb_weights<T>(Plan*, const T*, cudaStream_t);       \

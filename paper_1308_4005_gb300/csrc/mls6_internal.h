@@ -304,9 +304,8 @@ int enqueue_eval(Plan* p, const void* pos, const void* c, void* forces, double* 
 // kernel launchers; each returns the number of kernels it launched
 template <typename T> int launch_bin(Plan* p, const T* pos, const T* c, cudaStream_t st);
 template <typename T> int launch_pair(Plan* p, bool vir, cudaStream_t st, bool lb = false);
-// to_grid: also convert the fixed-point sums to q^1; qfx: sums (default d_q1fx)
-template <typename T>
-int launch_anterp(Plan* p, cudaStream_t st, int lbm = -1, bool to_grid = true, void* qfx = nullptr);
+// to_grid: also convert the fixed-point sums to q^1
+template <typename T> int launch_anterp(Plan* p, cudaStream_t st, int lbm = -1, bool to_grid = true);
 template <typename T> int launch_anterp_lb(Plan* p, cudaStream_t st, void* qfx);
 template <typename T>
 int launch_from_fixed(Plan* p, cudaStream_t st, int lbm = -1, const void* qfx = nullptr);

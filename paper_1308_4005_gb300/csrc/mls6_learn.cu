@@ -104,7 +104,8 @@ __device__ __forceinline__ void mma16816(float (&d)[4], uint32_t a0, uint32_t a1
 // each row with 16-byte stores (a row per atom in input order, or in sorted
 // order when sorted_out is set).  What
 // bounds it: the latency of those reads and sums against 21 warps per SM (four
-// blocks, 80 registers): 121 -> 74 us at 262,144 atoms (159 registers: 96).
+// blocks, 80 registers, of which 450 bytes of running sums spill): 121 -> 74 us
+// at 262,144 atoms (159 registers, no spills, two blocks: 96).
 constexpr int kFA = 64;
 
 template <typename T, bool F32>

@@ -71,7 +71,7 @@ struct TileArgs {
 constexpr int kTileAtoms = 8;
 constexpr int kTileWarps = 4;
 constexpr int kTileBlocks = 6;  // per SM: 80 registers a thread
-constexpr int kTileCap = 384;   // candidates of a list (315 on average at a = 3, density 0.85)
+constexpr int kTileCap = 384;   // candidates of a list (298 on average at a = 3, density 0.85)
 constexpr int kTileRuns = 3 * 25;
 constexpr float kTileFar = 1e10f;  // an absent atom or candidate: always outside the cutoff
 
