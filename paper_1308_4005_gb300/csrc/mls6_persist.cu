@@ -94,8 +94,8 @@ struct OutP { const double* out; const int* flag; double* ew; int* flagdst; };
 // pair sum.
 // A replica with both forms of the grid part lists the stages of both; gate is
 // its choice (1: direct) and want the value for which the stage runs.  The
-// items of the direct ones, which run only for thin phases, are `chunk` blocks
-// each.
+// direct ones, which run only for thin phases, have few items of `chunk` blocks
+// each: an item that is skipped still costs its ticket and its wait.
 struct PStageDesc {
   int kind;
   unsigned nb;
@@ -377,13 +377,14 @@ static void replica_stages(Plan* p, const float* pos, const float* cc, float* fo
                        (Vec4<float>*)p->d_sorted, scatter_slots(p), p->d_sorted_idx};
   }
   const bool sp = p->spectral;
-  // a stage of the form that runs when the choice is `want`
-  auto gated = [&](PStageDesc& d, int want, unsigned chunk) {
-    if (!sp) return;
+  // a stage of the form that runs when the choice is `want`, in at most `items`
+  // items
+  auto gated = [&](PStageDesc& d, int want, long items) {
+    if (!sp || d.blocks == 0) return;
     d.gate = p->d_flag + kThin;
     d.want = want;
-    d.chunk = chunk;
-    d.nb = (unsigned)cdiv(d.blocks, chunk);
+    d.chunk = (unsigned)cdiv(d.blocks, items);
+    d.nb = (unsigned)cdiv(d.blocks, d.chunk);
   };
   {
     PStageDesc& d = add(P_THIN, sp ? cdiv(ncell, kBlock) : 0);
@@ -405,7 +406,7 @@ static void replica_stages(Plan* p, const float* pos, const float* cc, float* fo
   {
     PStageDesc& d = add(P_FROM_FIXED, cdiv(L1.np, kBlock));
     d.u.ff = FromFixedP{(const unsigned*)p->d_q1fx, L1.np, p->d_flag, span, (float*)p->d_q[1]};
-    gated(d, 1, 16);
+    gated(d, 1, 4);
   }
   for (int k = 1; k < lmax; ++k) {  // restriction slots (empty beyond this replica's levels)
     const bool on = k < l;
@@ -420,7 +421,7 @@ static void replica_stages(Plan* p, const float* pos, const float* cc, float* fo
   {
     const int warps = kStencilThreads * 2 / 32;
     PStageDesc& d = add(P_STENCIL, p->stencil_blocks + cdiv(p->lv[l].np, warps));
-    gated(d, 1, 4);
+    gated(d, 1, 24);
     d.u.sten.A = stencil_args<float>(p);
     d.u.sten.wpart = p->d_wpart + 6 * p->wpart_stencil;
   }
@@ -428,7 +429,7 @@ static void replica_stages(Plan* p, const float* pos, const float* cc, float* fo
     const int k = l - 1 - j;
     const bool on = k >= 1;
     PStageDesc& d = add(P_PROLONG, on ? cdiv(p->lv[k].np, kBlock) : 0);
-    gated(d, 1, 16);
+    gated(d, 1, 8);
     if (on) {
       const Level &F = p->lv[k], &C = p->lv[k + 1];
       d.u.pr = ProlongP{(const float*)p->d_e[k], F.n[0], F.n[1], F.n[2],
@@ -443,7 +444,7 @@ static void replica_stages(Plan* p, const float* pos, const float* cc, float* fo
     for (int k = 0; k < 5; ++k) {
       PStageDesc& d = add(P_SPEC_FWD + k, nb[k]);
       if (sp) d.u.sp = spec_args<float>(p, false);
-      gated(d, 0, 1);
+      gated(d, 0, d.blocks);
     }
   }
   {
