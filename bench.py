@@ -55,6 +55,11 @@ EXACT_R = 20.0          # radius of the direct sums behind the exact sampled for
 # named workload and precision, virial on; a kernel changed since its
 # capture has no entry and reports null.
 TRAFFIC = {
+    ("cube1m", "mixed", "bin"): 53743360,          # k_bin, scans, k_scatter, k_cellsort
+    ("cube1m", "mixed", "pair"): 18405632,         # k_pair_tile
+    ("cube1m", "mixed", "anterpolate"): 22436864,  # k_anterp
+    ("cube1m", "mixed", "stencil"): 34640384,      # the transforms' five kernels, k_direct
+    ("cube1m", "mixed", "interpolate"): 48607232,  # k_interp (+ final reduction)
 }
 
 # arithmetic of each precision mode (pair/grid transfers; level stencils, where
@@ -492,8 +497,9 @@ def stage_work(info, N, n_pairs, prec, vir):
     fp_tap = FLOP_TAP + (FLOP_TAP_VIR if vir else 0)
     fx = 8 if prec == "fp64" else 4  # fixed-point sums
     w = {
-        "bin": ("hbm", N * 80.0, "B", "per atom: input 16 B read, record 16 B + cell 4 B "
-                "written, scatter 20 B read + 20 B written, order 4 B"),
+        "bin": ("hbm", N * 92.0, "B", "per atom: input 16 B read, record 16 B + cell and place "
+                "8 B written; scatter 8 B read, 4 B written; order: index 4 B + record 16 B "
+                "read, 20 B written"),
         "pair": ("alu", n_pairs * float(fp_pair), "flop",
                  f"{n_pairs} ordered pairs inside a x {fp_pair} flop"),
         "anterpolate": ("hbm", N * 16.0 + np_[0] * float(fx), "B",
