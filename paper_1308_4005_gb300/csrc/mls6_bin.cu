@@ -286,8 +286,6 @@ __device__ __forceinline__ unsigned long long record_key(const Vec4<T>* __restri
   return k;
 }
 
-// slots: scatter-order indices, sidx: the cell order's.  big: the block also
-// takes its cells of more than 8 atoms.
 template <typename T>
 __device__ __forceinline__ void put_record(Vec4<T>* sorted, float4* sortedf, int k, const Vec4<T>& v) {
   sorted[k] = v;
@@ -296,6 +294,7 @@ __device__ __forceinline__ void put_record(Vec4<T>* sorted, float4* sortedf, int
 }
 
 // The atom in slot k, if its cell has more than 8: its place among the cell's.
+// slots: scatter-order indices, sidx: the cell order's.
 template <typename T>
 __device__ __forceinline__ void rank_in_cell(const int* __restrict__ start,
                            const int2* __restrict__ cell_of, const Vec4<T>* __restrict__ posw,
@@ -316,6 +315,7 @@ __device__ __forceinline__ void rank_in_cell(const int* __restrict__ start,
   put_record(sorted, sortedf, at, posw[i]);
 }
 
+// big: the block also takes the atoms of its cells of more than 8.
 template <typename T>
 __device__ __forceinline__ void k_cellsort_body(const Blk bk,const int* __restrict__ start, long ncell,
                            const int2* __restrict__ cell_of, const Vec4<T>* __restrict__ posw,

@@ -34,10 +34,10 @@ namespace mls6 {
 // has nothing to do: with the choice it costs 2 of 54 us at 3,001 atoms, 3 of 88
 // at 65,536, 10 of 760 at 1,048,576 (on a stream of its own beside the
 // transforms, or behind the pair sum: the same or more).  With a vapour, whole
-// evaluations, the launches of mls6_grid.cu (and 8 lanes per atom or the
-// per-atom pair sum) -> here: 3,001-atom slab 88 -> 98 us (the transforms'
-// launches that return at once), 65,536 atoms 162 -> 140, FP64 20,000 788 -> 450,
-// 1,000,000 atoms 1232 -> 1111.  Bound like those by latency on small grids and
+// evaluations, with the separate launches (and the pair sums of that time) ->
+// here: 3,001-atom slab 88 -> 98 us (the transforms' launches that return at
+// once), 65,536 atoms 162 -> 140, FP64 20,000 788 -> 450, 1,000,000 atoms 1232 ->
+// 1111.  Bound like those by latency on small grids and
 // by the stencil's FP32 pipe on large ones, so 64 registers, as its kernel has
 // (128: 65,536 atoms 172).  The level stencils' tensor-core forms stay out: they
 // round coarser.
