@@ -414,25 +414,26 @@ __device__ __forceinline__ void k_thin_body(const Blk bk, const int* __restrict_
   }
 }
 
-// Blocks: cells, atoms of large cells (if any blocks are theirs), the choice of
-// the grid part's form (if any).
+// Blocks: what the choice of the grid part's form needs (if any; first, so that
+// their loads run beside the sort's), cells, atoms of large cells (if any blocks
+// are theirs).
 template <typename T>
 __global__ void k_cellsort(const int* __restrict__ start, long ncell,
                            const int2* __restrict__ cell_of, const Vec4<T>* __restrict__ posw,
                            Vec4<T>* __restrict__ sorted, const int* __restrict__ slots,
-                           int* __restrict__ sidx, float4* __restrict__ sortedf, int N, int ncells,
-                           int nslots, ThinArgs g, int* __restrict__ flag) {
-  const int b = (int)blockIdx.x - ncells;
+                           int* __restrict__ sidx, float4* __restrict__ sortedf, int N, int nthin,
+                           int ncells, int nslots, ThinArgs g, int* __restrict__ flag) {
+  const int b = (int)blockIdx.x - nthin;
   if (b < 0) {
-    k_cellsort_body<T>(Blk::self(), start, ncell, cell_of, posw, sorted, slots, sidx, sortedf,
-                       nslots == 0);
-  } else if (b < nslots) {
+    k_thin_body(Blk{blockIdx.x, (unsigned)nthin}, start, ncell, g, flag);
+  } else if (b < ncells) {
+    k_cellsort_body<T>(Blk{(unsigned)b, (unsigned)ncells}, start, ncell, cell_of, posw, sorted,
+                       slots, sidx, sortedf, nslots == 0);
+  } else {
     const long z = pdl_begin();
-    const int k = b * blockDim.x + threadIdx.x;
+    const int k = (b - ncells) * blockDim.x + threadIdx.x;
     if (k < N)
       rank_in_cell<T>(start + z, cell_of + z, posw + z, sorted, slots + z, sidx, sortedf, k);
-  } else {
-    k_thin_body(Blk{(unsigned)(b - nslots), gridDim.x - ncells - nslots}, start, ncell, g, flag);
   }
 }
 
@@ -485,10 +486,11 @@ int launch_bin(Plan* p, const T* pos, const T* cc, cudaStream_t st) {
              (const int*)p->d_cell_start, slots);
   const int ncells = (int)cdiv(ncell, kBlock);
   const int nslots = N >= kSlotAtoms * ncell ? (int)cdiv(N, kBlock) : 0;
-  launch_pdl(k_cellsort<T>, ncells + nslots + (p->spectral ? ncells : 0), kBlock, 0, st,
-             (const int*)p->d_cell_start, ncell, (const int2*)p->d_cell_of,
-             (const Vec4<T>*)p->d_pos_w, (Vec4<T>*)p->d_sorted, (const int*)slots,
-             p->d_sorted_idx, (float4*)p->d_sorted_f, N, ncells, nslots, thin_args(p), p->d_flag);
+  const int nthin = p->spectral ? ncells : 0;
+  launch_pdl(k_cellsort<T>, nthin + ncells + nslots, kBlock, 0, st, (const int*)p->d_cell_start,
+             ncell, (const int2*)p->d_cell_of, (const Vec4<T>*)p->d_pos_w,
+             (Vec4<T>*)p->d_sorted, (const int*)slots, p->d_sorted_idx, (float4*)p->d_sorted_f, N,
+             nthin, ncells, nslots, thin_args(p), p->d_flag);
   return direct ? 4 : 5;
 }
 

@@ -31,9 +31,10 @@
 namespace mls6 {
 
 // One launch, because it is part of every evaluation and mostly finds that it
-// has nothing to do: with the choice it costs 2 of 54 us at 3,001 atoms, 3 of 88
-// at 65,536, 10 of 760 at 1,048,576 (on a stream of its own beside the
-// transforms, or behind the pair sum: the same or more).  With a vapour, whole
+// has nothing to do: with the choice it costs 1 of 53 us at 3,001 atoms, 2 of 87
+// at 65,536, 12 of 765 at 1,048,576, where its blocks wait for room beside the
+// pair sum's (on a stream of its own beside the transforms, or behind the pair
+// sum: the same or more).  With a vapour, whole
 // evaluations, with the separate launches (and the pair sums of that time) ->
 // here: 3,001-atom slab 88 -> 98 us (the transforms' launches that return at
 // once), 65,536 atoms 162 -> 140, FP64 20,000 788 -> 450, 1,000,000 atoms 1232 ->
