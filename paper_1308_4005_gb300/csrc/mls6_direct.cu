@@ -36,9 +36,9 @@ namespace mls6 {
 // pair sum's (on a stream of its own beside the transforms, or behind the pair
 // sum: the same or more).  With a vapour, whole
 // evaluations, with the separate launches (and the pair sums of that time) ->
-// here: 3,001-atom slab 88 -> 98 us (the transforms' launches that return at
-// once), 65,536 atoms 162 -> 140, FP64 20,000 788 -> 450, 1,000,000 atoms 1232 ->
-// 1111.  Bound like those by latency on small grids and
+// here: 3,001-atom slab 88 -> 99 us (the transforms' launches that return at
+// once), 65,536 atoms 162 -> 140, FP64 20,000 788 -> 427, 1,000,000 atoms 1232 ->
+// 1096.  Bound like those by latency on small grids and
 // by the stencil's FP32 pipe on large ones, so 64 registers, as its kernel has
 // (128: 65,536 atoms 172).  The level stencils' tensor-core forms stay out: they
 // round coarser.
@@ -239,7 +239,8 @@ template <typename T> static int prepare_direct_list(Plan* p, bool lb, int i) {
           lb && k == 1 ? (void*)((T*)p->d_lbpot + (size_t)m * L1.np) : p->d_et[k], p->lv[k],
           p->lv[k + 1]);
   }
-  // blocks: what the device holds, at most what a stage has
+  // blocks: up to two per SM, at most what a stage has (four per SM: 1,000,000
+  // atoms with a vapour 1127 us against 1096; one: 1650, 65,536 atoms 152 against 140)
   unsigned most = 1;
   for (const GStage& s : st) most = std::max(most, s.nb);
   int dev = 0, sms = 0;
@@ -254,7 +255,7 @@ template <typename T> static int prepare_direct_list(Plan* p, bool lb, int i) {
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, nt, G.smem) != cudaSuccess ||
         per_sm < 1)
       return MLS6_ERR_CUDA;
-    g.blocks[v] = (int)std::min<long>((long)most, (long)per_sm * sms);
+    g.blocks[v] = (int)std::min<long>((long)most, (long)std::min(per_sm, 2) * sms);
   }
   void* d_st = nullptr;
   const size_t bytes = sizeof(GStage) * st.size();
